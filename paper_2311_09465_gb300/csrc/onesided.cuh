@@ -1,0 +1,170 @@
+// Eigenpairs of the symmetric positive definite (2N-1) x (2N-1) matrices of
+// eq. (3D-tau) in FP32, one matrix per group of N lanes, entirely in registers:
+// M = L L^T (Cholesky), then one-sided Jacobi (Hestenes 1958; on a Cholesky
+// factor: Veselic & Hari 1989) on the columns of L.  Plane rotations from the
+// right, L J = F, make the columns of F orthogonal; then M = F F^T gives the
+// eigenvectors f_a / |f_a| and the eigenvalues |f_a|^2, so only one matrix is
+// rotated (the two-sided form rotates rows and columns of M and accumulates V).
+//
+// Layout: NM = 2N-1 columns in a line of slots 0..2N-2; lane p of a group
+// holds slot 2p-1 in x and slot 2p in y (lane 0: only y, its x stays zero).
+// Odd-even ordering (every pair of columns meets once in NM rounds): a round
+// rotates neighbouring slots and exchanges them.  The pairs (2p-1, 2p) are in
+// one lane; for the pairs (2p, 2p+1) the right lane's x moves over and one
+// column moves back, so a round costs one column of shuffles on average.
+// Lanes without a partner do a rotation by a right angle with a zero column,
+// which leaves their column in its slot without any select.
+//
+// What bounds it: 128 FP32 lanes and 32 shuffle lanes a clock and SM; a round
+// is about 90 FP32 instructions and 14 shuffles a lane at N = 7, with no
+// shared memory in the loop.
+#pragma once
+#include "common.cuh"
+
+namespace ts {
+
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// 1/sqrt(x) with one Newton step on the hardware approximation
+__device__ __forceinline__ float rsqrt_newton(float x) {
+  const float r = rsqrt_ftz(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.f), r);
+}
+
+// rotation that makes X and Y orthogonal: X' = X - s (Y + ta X), Y' = Y + s (X - ta Y);
+// ax, ay: their squared norms, g: their product; t = s/c is returned for the norms
+__device__ __forceinline__ void rotation_of(float ax, float ay, float g, float& s, float& ta, float& t) {
+  const float d = ay - ax;
+  const float h2 = fmaf(2.f * g, 2.f * g, d * d);
+  const float h = h2 * rsqrt_ftz(h2);
+  t = 2.f * g * rcp_ftz(d + copysignf(h, d));
+  if (!(h2 > 1e-36f)) t = 0.f;
+  const float c = rsqrt_ftz(fmaf(t, t, 1.f));
+  s = t * c;
+  ta = s * rcp_ftz(1.f + c);
+}
+
+// Cholesky factor of the group's matrix in place: on entry x, y hold the full
+// columns 2p-1 and 2p, on return the columns of L (zeros above the diagonal).
+// base: the group's first lane.  floor: a lower bound of the eigenvalues, hence
+// of the exact pivots; rounding may take a computed pivot below it.
+template <int N>
+__device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, int base,
+                                                 float floor) {
+  constexpr int NM = 2 * N - 1;
+#pragma unroll
+  for (int k = 0; k < NM; ++k) {
+    const int src = base + (k + 1) / 2;
+    float l[NM];
+#pragma unroll
+    for (int i = k; i < NM; ++i) l[i] = __shfl_sync(0xffffffffu, (k & 1) ? x[i] : y[i], src);
+    const float rd = rsqrt_newton(fmaxf(l[k], floor));
+    // the pivot column itself becomes l; a column j > k loses l l_j, l_j = rd A_jk
+    const int jx = 2 * p - 1, jy = 2 * p;
+    const float mx = jx > k ? x[k] * rd * rd : 0.f;
+    const float my = jy > k ? y[k] * rd * rd : 0.f;
+    const bool ox = jx == k, oy = jy == k;
+#pragma unroll
+    for (int i = k + 1; i < NM; ++i) {
+      const float sx = fmaf(-l[i], mx, x[i]), sy = fmaf(-l[i], my, y[i]);
+      x[i] = ox ? l[i] * rd : sx;
+      y[i] = oy ? l[i] * rd : sy;
+    }
+    const float dk = fmaxf(l[k], floor) * rd;
+    if (jx >= k) x[k] = ox ? dk : 0.f;
+    if (jy >= k) y[k] = oy ? dk : 0.f;
+  }
+}
+
+// One-sided Jacobi on the group's columns.  Returns whether this lane's pairs
+// were orthogonal to ORTHO2 (squared cosine) before the last sweep's rotations;
+// that sweep then leaves cosines of the order of their squares (1e-8).
+constexpr float ORTHO2 = 1e-8f;
+constexpr int ONESIDED_SWEEPS = 15;
+
+template <int N>
+__device__ __forceinline__ bool onesided_jacobi(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, int lane) {
+  constexpr int NM = 2 * N - 1;
+  if constexpr (N == 1) return true;
+  const int up = (lane + 31) & 31, down = (lane + 1) & 31;
+  const bool first = p == 0, last = p == N - 1;
+  bool rotated = true;
+#pragma unroll 1
+  for (int sweep = 0; sweep < ONESIDED_SWEEPS; ++sweep) {
+    float ax = 0.f, ay = 0.f;
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      ax = fmaf(x[i], x[i], ax);
+      ay = fmaf(y[i], y[i], ay);
+    }
+    rotated = false;
+#pragma unroll 1
+    for (int rr = 0; rr < N; ++rr) {
+      float g = 0.f, s, ta, t;
+      // pairs (2p-1, 2p)
+      {
+        float g0 = 0.f, g1 = 0.f;
+#pragma unroll
+        for (int i = 0; i < NM; i += 2) g0 = fmaf(x[i], y[i], g0);
+#pragma unroll
+        for (int i = 1; i < NM; i += 2) g1 = fmaf(x[i], y[i], g1);
+        g = g0 + g1;
+      }
+      rotation_of(ax, ay, g, s, ta, t);
+      rotated |= g * g > ORTHO2 * ax * ay;
+      if (first) s = -1.f, ta = -1.f;
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        const float nx = fmaf(-s, fmaf(ta, x[i], y[i]), x[i]);
+        const float ny = fmaf(s, fmaf(-ta, y[i], x[i]), y[i]);
+        x[i] = ny;
+        y[i] = nx;
+      }
+      {
+        const float na = fmaf(-t, g, ax), nb = fmaf(t, g, ay);
+        ax = first ? 0.f : nb;
+        ay = first ? ay : na;
+      }
+      // pairs (2p, 2p+1)
+      float z[NM];
+#pragma unroll
+      for (int i = 0; i < NM; ++i) z[i] = __shfl_sync(0xffffffffu, x[i], down);
+      float az = __shfl_sync(0xffffffffu, ax, down);
+      {
+        float g0 = 0.f, g1 = 0.f;
+#pragma unroll
+        for (int i = 0; i < NM; i += 2) g0 = fmaf(y[i], z[i], g0);
+#pragma unroll
+        for (int i = 1; i < NM; i += 2) g1 = fmaf(y[i], z[i], g1);
+        g = g0 + g1;
+      }
+      rotation_of(ay, az, g, s, ta, t);
+      rotated |= g * g > ORTHO2 * ay * az;
+      if (last) s = 1.f, ta = 1.f;
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        const float nx = fmaf(-s, fmaf(ta, y[i], z[i]), y[i]);
+        const float ny = fmaf(s, fmaf(-ta, z[i], y[i]), z[i]);
+        y[i] = ny;
+        x[i] = __shfl_sync(0xffffffffu, nx, up);
+      }
+      {
+        const float na = last ? 0.f : fmaf(-t, g, ay), nb = last ? ay : fmaf(t, g, az);
+        ay = nb;
+        ax = __shfl_sync(0xffffffffu, na, up);
+      }
+    }
+    if (!__any_sync(0xffffffffu, rotated)) break;
+  }
+  return !rotated;
+}
+
+}  // namespace ts

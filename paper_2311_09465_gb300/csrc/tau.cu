@@ -12,9 +12,12 @@
 // parallel cyclic Jacobi (round-robin ordering, N disjoint rotations per
 // round, one per lane), padded with a decoupled dummy row to size 2N.
 // tau = V diag(lambda^{-1/2}) V^T is written as a packed upper triangle.
+#include <algorithm>
+
 #include "common.cuh"
 #include "jacobi.cuh"
 #include "kernels.h"
+#include "onesided.cuh"
 
 namespace ts {
 
@@ -154,35 +157,308 @@ __global__ void __launch_bounds__(128) tau_kernel(const int4* __restrict__ tets,
   }
 }
 
+// ---------------------------------------------------------------------------
+// FP32 tau.  A group of N lanes owns a point (GPW points a warp); lane p holds
+// two columns of every matrix in registers: 2p-1 and 2p, i.e. Re and Im of
+// mode p (lane 0: the mean).  Steps: w_m at the point, the columns of C_m
+// (gathered from a zero-padded table of the modes of w_m), M = sum C_m C_m +
+// c I with C_m read back row by row from shared memory (a 16-byte broadcast
+// feeds eight multiply-adds), Cholesky and one-sided Jacobi (onesided.cuh),
+// tau = sum_a f_a f_a^T / |f_a|^3, and 16-byte stores through shared memory.
+// The point is scaled by a power of two (sum_m beta_m + sqrt(c) <= 1, beta_m a
+// bound of |C_m|), undone exactly at the end.
+//
+// Bound by FP32 issue: at N = 7 about 10 k instructions a lane and group of
+// four points.
+template <int N>
+struct Tau32Layout {
+  static constexpr int NM = 2 * N - 1, C = 2 * N, L = N - 1, GPW = 32 / N;
+  static constexpr int LDC = (2 * N + 3) & ~3;        // matrix row, 16-byte multiple
+  static constexpr int TW = 3 * N;                    // modes -(N-1) .. 2(N-1), zero beyond N-1 (+ pad)
+  static constexpr int T = 0;                         // [3][2][TW] re, im of the modes of w_m
+  static constexpr int CM = (3 * 2 * TW + 3) & ~3;    // [3][NM][LDC]; then the scaled f_a [NM][LDC]
+  static constexpr int OUTP = CM + NM * LDC;          // packed tau, over the later C_m (N > 1)
+  static constexpr int RAW = CM + 3 * NM * LDC + (N == 1 ? 4 : 0);
+  // 16-byte reads of the warp's groups fall into different banks: stride 4 mod 32 words
+  static constexpr int GROUP = RAW + ((4 - RAW) % 32 + 32) % 32;
+  static constexpr int WARP = GPW * GROUP;
+  static_assert(OUTP + Dims<N>::NT_PAD <= GROUP, "packed tau fits over the matrices");
+};
+
+// a 16-byte aligned row of W floats (W a multiple of 4) to registers
+template <int W>
+__device__ __forceinline__ void load_row(const float* src, float (&dst)[W]) {
+#pragma unroll
+  for (int j = 0; j < W / 4; ++j) {
+    const float4 v = reinterpret_cast<const float4*>(src)[j];
+    dst[4 * j] = v.x;
+    dst[4 * j + 1] = v.y;
+    dst[4 * j + 2] = v.z;
+    dst[4 * j + 3] = v.w;
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(128) tau32_kernel(const int4* __restrict__ tets, const float* __restrict__ geo,
+                                                    const float* __restrict__ y, int64_t n_qp,
+                                                    float* __restrict__ tau_out, float nu, float C_I,
+                                                    unsigned* __restrict__ n_unconverged,
+                                                    float* __restrict__ eig_out) {
+  using D = Dims<N>;
+  using Lt = Tau32Layout<N>;
+  constexpr int NM = D::NM, C = D::C, LDC = Lt::LDC, GPW = Lt::GPW, TW = Lt::TW, L = N - 1;
+  extern __shared__ __align__(16) float tau32_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane / N, p = lane - (lane / N) * N;
+  const bool in_group = g < GPW;
+  float* base = tau32_smem + warp * Lt::WARP + (in_group ? g : 0) * Lt::GROUP;
+  float* tw = base + Lt::T;
+  float* cm = base + Lt::CM;
+  const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t qb = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * GPW; qb < n_qp; qb += warps_total * GPW) {
+    const bool live = in_group && qb + g < n_qp;
+    const int64_t gq = live ? qb + g : qb;     // idle lanes redo the warp's first point, unstored
+    const int64_t e = gq >> 2;
+    const int q = (int)(gq & 3);
+    // w_m = sum_i L_im u_i for mode p
+    float w[3][2];
+    float diff;
+    {
+      const float* gg = geo + e * GEO_STRIDE + GEO_G;
+      const float gxx = gg[0], gxy = gg[1], gxz = gg[2], gyy = gg[3], gyz = gg[4], gzz = gg[5];
+      const float l00 = sqrtf(gxx), l10 = gxy / l00, l20 = gxz / l00;
+      const float l11 = sqrtf(gyy - l10 * l10), l21 = (gyz - l20 * l10) / l11;
+      const float l22 = sqrtf(gzz - l20 * l20 - l21 * l21);
+      const float GG = gxx * gxx + gyy * gyy + gzz * gzz + 2.f * (gxy * gxy + gxz * gxz + gyz * gyz);
+      diff = C_I * nu * nu * GG;
+      const int4 nd = tets[e];
+      const int node[4] = {nd.x, nd.y, nd.z, nd.w};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float u[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const float lam = (float)qp_bary(q, a);
+          const float* ya = y + (int64_t)node[a] * 4 * C + 2 * p + h;
+#pragma unroll
+          for (int i = 0; i < 3; ++i) u[i] += lam * ya[i * C];
+        }
+        if (p == 0 && h == 1) u[0] = u[1] = u[2] = 0.f;
+        w[0][h] = l00 * u[0] + l10 * u[1] + l20 * u[2];
+        w[1][h] = l11 * u[1] + l21 * u[2];
+        w[2][h] = l22 * u[2];
+      }
+    }
+    // |C_m| <= beta_m = |w_0| + 2 sum |w_n|; 2^-ex scales the point
+    float bound = 0.f;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) bound += (fabsf(w[m][0]) + fabsf(w[m][1])) * (p == 0 ? 1.f : 2.f);
+    if constexpr (N > 1) {
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < N; ++j) sum += __shfl_sync(0xffffffffu, bound, (in_group ? g * N : 0) + j);
+      bound = sum;
+    }
+    bound = 1.0001f * (bound + sqrtf(diff));
+    const bool finite = bound < 1e37f && bound > 1e-37f;
+    int ex = 0;
+    if (finite) frexpf(bound, &ex);
+    const float sc = ldexpf(1.f, -ex);
+    const float cd = diff * sc * sc;
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      float* tr = tw + m * 2 * TW + L;        // mode k at tr[k], im at tr[TW + k]
+      const float re = w[m][0] * sc, im = w[m][1] * sc;
+      if (in_group) {
+        tr[p] = re;
+        tr[TW + p] = im;
+        if (p > 0) {
+          tr[-p] = re;
+          tr[TW - p] = -im;
+          tr[L + p] = 0.f;
+          tr[TW + L + p] = 0.f;
+        }
+      }
+    }
+    __syncwarp();
+    float x[NM], yy[NM];
+#pragma unroll
+    for (int i = 0; i < NM; ++i) x[i] = yy[i] = 0.f;
+    // the lane's columns of C_m (Re p, Im p; lane 0: the mean) to shared memory
+    float* colx = cm + (2 * p - 1) * LDC;
+    float* coly = cm + (2 * p) * LDC;
+#pragma unroll 1
+    for (int m = 0; m < 3; ++m) {
+      const float* tr = tw + m * 2 * TW + L;
+      const float* ti = tr + TW;
+      float cx[NM], cy[NM];
+      constexpr float S2 = Real<float>::SQRT2;
+      cx[0] = S2 * tr[p];
+      cy[0] = p == 0 ? tr[0] : S2 * ti[p];
+#pragma unroll
+      for (int k = 1; k < N; ++k) {
+        const float pl = tr[k - p], ph = tr[k + p], ql = ti[k - p], qh = ti[k + p];
+        cx[2 * k - 1] = pl + ph;
+        cx[2 * k] = ql + qh;
+        cy[2 * k - 1] = p == 0 ? S2 * pl : qh - ql;
+        cy[2 * k] = p == 0 ? S2 * ql : pl - ph;
+      }
+      if (in_group) {
+        float* dx = colx + m * NM * LDC;
+        float* dy = coly + m * NM * LDC;
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          if (p > 0) dx[i] = cx[i];
+          dy[i] = cy[i];
+        }
+      }
+      __syncwarp();
+      // M's columns: row i of the symmetric C_m is a 16-byte broadcast stream
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        float row[LDC], sx = x[i], sy = yy[i];
+        load_row<LDC>(cm + (m * NM + i) * LDC, row);
+#pragma unroll
+        for (int j = 0; j < NM; ++j) {
+          sx = fmaf(row[j], cx[j], sx);
+          sy = fmaf(row[j], cy[j], sy);
+        }
+        x[i] = sx;
+        yy[i] = sy;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      x[i] += i == 2 * p - 1 ? cd : 0.f;
+      yy[i] += i == 2 * p ? cd : 0.f;
+      if (p == 0 || !in_group) x[i] = 0.f;
+      if (!in_group) yy[i] = 0.f;
+    }
+    cholesky_columns<N>(x, yy, in_group ? p : 64, g * N, fmaxf(cd, 1e-30f));
+    const bool conv = onesided_jacobi<N>(x, yy, p, lane);
+    {
+      const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);
+      const unsigned mine = N == 32 ? ~0u : ((1u << N) - 1u) << (in_group ? g * N : 0);
+      if (live && p == 0 && (bad & mine)) atomicAdd(n_unconverged, 1u);
+    }
+    float ax = 0.f, ay = 0.f;
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      ax = fmaf(x[i], x[i], ax);
+      ay = fmaf(yy[i], yy[i], ay);
+    }
+    // eigenpairs for the derivative of tau (exact tangent), when asked: the
+    // lane's two vectors are columns 2p-1 and 2p of the cache
+    if (live && eig_out) {
+      float* eo = eig_out + gq * D::EIG;
+      const float back = ldexpf(1.f, 2 * ex);
+      const float ix = rsqrt_newton(ax), iy = rsqrt_newton(ay);
+      if (p > 0) {
+#pragma unroll
+        for (int i = 0; i < NM; ++i) eo[i * NM + 2 * p - 1] = x[i] * ix;
+        eo[NM * NM + 2 * p - 1] = ax * back;
+      }
+#pragma unroll
+      for (int i = 0; i < NM; ++i) eo[i * NM + 2 * p] = yy[i] * iy;
+      eo[NM * NM + 2 * p] = ay * back;
+    }
+    // h_a = f_a / |f_a|^{3/2} (so that tau = sum_a h_a h_a^T), stored one float
+    // off so that a lane's two entries are an aligned pair
+    __syncwarp();
+    {
+      const float rx = rsqrt_newton(ax), ry = rsqrt_newton(ay);
+      const float hx = rx * sqrtf(rx), hy = ry * sqrtf(ry);
+      if (in_group) {
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          if (p > 0) colx[i + 1] = x[i] * hx;
+          coly[i + 1] = yy[i] * hy;
+        }
+        if (p == 0)
+          for (int a = 0; a < NM; ++a) cm[a * LDC] = 0.f;
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NM; ++i) x[i] = yy[i] = 0.f;
+#pragma unroll 1
+    for (int a = 0; a < NM; ++a) {
+      const float* ha = cm + a * LDC;
+      const float2 own = *reinterpret_cast<const float2*>(ha + 2 * p);   // entries 2p-1 and 2p
+      float row[LDC];
+      load_row<LDC>(ha, row);
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        x[i] = fmaf(row[i + 1], own.x, x[i]);
+        yy[i] = fmaf(row[i + 1], own.y, yy[i]);
+      }
+    }
+    // packed upper triangle through shared memory
+    float* op = base + Lt::OUTP;
+    const float un = finite ? sc : __int_as_float(0x7fc00000);
+    __syncwarp();
+    if (in_group) {
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        if (p > 0 && i <= 2 * p - 1) op[packed_index(i, 2 * p - 1, NM)] = x[i] * un;
+        if (i <= 2 * p) op[packed_index(i, 2 * p, NM)] = yy[i] * un;
+      }
+      if (p == 0)
+        for (int t = D::NT; t < D::NT_PAD; ++t) op[t] = 0.f;
+    }
+    __syncwarp();
+    if (live) {
+      float4* out = reinterpret_cast<float4*>(tau_out + gq * D::NT_PAD);
+      for (int t = p; t < D::NT_PAD / 4; t += N) out[t] = *reinterpret_cast<const float4*>(op + 4 * t);
+    }
+    __syncwarp();
+  }
+}
+
+template <int N>
+size_t tau32_smem(int* warps) {
+  using L = Tau32Layout<N>;
+  *warps = 4;
+  while (*warps > 1 && (size_t)*warps * L::WARP * sizeof(float) > 100 * 1024) *warps >>= 1;
+  return (size_t)*warps * L::WARP * sizeof(float);
+}
+
 template <typename T, int N>
 int launch_tau(const int4* tets, const T* geo, const T* y, int64_t n_elem, T* tau_out, T nu,
                T C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out) {
-  using L = TauLayout<N>;
-  const int warps = 4;
-  size_t smem = (size_t)warps * L::WARP * sizeof(T);
-  cudaFuncSetAttribute(tau_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int64_t n_qp = n_elem * 4;
-  int64_t groups = (n_qp + L::GPW - 1) / L::GPW;
-  int64_t blocks = (groups + warps - 1) / warps;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  if (blocks < 1) blocks = 1;
-  const int sweeps = sizeof(T) == 4 ? 12 : 20;
-  const T tol2 = sizeof(T) == 4 ? T(1e-12) : T(1e-28);
-  count_launches(1);
-  tau_kernel<T, N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, nu, C_I,
-                                                          sweeps, tol2, n_unconverged, eig_out);
+  const int64_t n_qp = n_elem * 4, groups = (n_qp + 32 / N - 1) / (32 / N);
+  if constexpr (sizeof(T) == 4) {
+    int warps;
+    const size_t smem = tau32_smem<N>(&warps);
+    if (cudaFuncSetAttribute(tau32_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return -2;
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, 152 * 64));
+    count_launches(1);
+    tau32_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, nu, C_I, n_unconverged, eig_out);
+  } else {
+    using L = TauLayout<N>;
+    const int warps = 4;
+    const size_t smem = (size_t)warps * L::WARP * sizeof(T);
+    cudaFuncSetAttribute(tau_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, 152 * 64));
+    count_launches(1);
+    tau_kernel<T, N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, nu, C_I,
+                                                            20, T(1e-28), n_unconverged, eig_out);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
-// Loads tau_kernel<T, N> into the current device's context without launching
+// Loads the FP32 tau kernel into the current device's context without launching
 // it (with lazy module loading a kernel is otherwise loaded at its first launch).
 template <typename T, int N>
 int preload_tau() {
-  using L = TauLayout<N>;
+  static_assert(sizeof(T) == 4, "FP32 only");
+  int warps;
+  const size_t smem = tau32_smem<N>(&warps);
   cudaFuncAttributes a;
-  if (cudaFuncGetAttributes(&a, tau_kernel<T, N>) != cudaSuccess) return -2;
-  const size_t smem = (size_t)4 * L::WARP * sizeof(T);
-  return cudaFuncSetAttribute(tau_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+  if (cudaFuncGetAttributes(&a, tau32_kernel<N>) != cudaSuccess) return -2;
+  return cudaFuncSetAttribute(tau32_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
                  cudaSuccess ? 0 : -2;
 }
 
