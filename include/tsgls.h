@@ -77,16 +77,9 @@ extern "C" {
 #define TS_ELEMENT64_NATIVE 0  /*   FP64 instructions                                     */
 #define TS_ELEMENT64_DOUBLEFLOAT 1 /* double-float pairs on the FP32 pipe (FP64 storage;  */
                                    /* default): meets the FP64 bar, 1.5x faster           */
-#define TS_OPT_TAU_WARM     4  /* 0 (default): every FP64 residual with TS_TAU64_DOUBLEFLOAT */
-                               /* computes tau from scratch; 1: its FP32 Jacobi sweeps     */
-                               /* start from each quadrature point's eigenvectors of the   */
-                               /* previous evaluation on this problem (cached, (2N-1)^2    */
-                               /* floats per point, allocated on first use), so they stop  */
-                               /* early when the state moved little.  The refinement makes */
-                               /* tau independent of the start up to rounding (about 1e-15 */
-                               /* relative), not bitwise.  Setting the key drops the cache; */
-                               /* ts_solve uses 1 for its own residuals and restores the   */
-                               /* caller's value on return.                                */
+#define TS_OPT_TAU_WARM     4  /* 0 (default) or 1.  Accepted and without effect: tau is    */
+                               /* computed from scratch at every residual, faster than a   */
+                               /* start from stored eigenvectors was                        */
 
 typedef struct ts_mesh ts_mesh;
 typedef struct ts_problem ts_problem;

@@ -393,7 +393,7 @@ class GLSProblem:
 
     def option(self, tau64=None, fp32_tangent=None, element64=None, tau_warm=None):
         """tau64: "refine" | "doublefloat" | "jacobi"; fp32_tangent: "single" | "coloured";
-        element64: "native" | "doublefloat"; tau_warm: bool (warm-started tau eigensolve)."""
+        element64: "native" | "doublefloat"; tau_warm: bool (accepted, without effect)."""
         if tau_warm is not None:
             ts_problem_option(self.prob, TS_OPT_TAU_WARM, int(bool(tau_warm)))
         if element64 is not None:

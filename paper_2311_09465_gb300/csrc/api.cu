@@ -70,6 +70,7 @@ struct LinState {
   T* tau = nullptr;     // [E][4][NT_PAD]
   T* t0 = nullptr;      // [E][4][3][C] tau L at the state
   T* dft = nullptr;     // forward [K][C] then inverse [C][K]
+  float2* udd = nullptr;   // [V][4][C] u0 as double-float pairs (FP64 state only)
   T* u0t = nullptr;     // [V][K][4] u0 velocity sampled in time (FP32 fast path)
   T* vt = nullptr;      // [V][K][4] scratch of the FP32 fast path: the product's input sampled
   T* bneg = nullptr;    // [backflow points][NT_PAD] |A_n|_- (section 2.6)
@@ -131,9 +132,6 @@ struct ts_problem {
   float *d_v32 = nullptr, *d_w32 = nullptr;
   double *d_D = nullptr, *d_t = nullptr;      // preconditioner diagonal (inverted), temp
   float* d_binv = nullptr;                    // inverted nodal blocks [V][8N][8N] (block Jacobi)
-  int tau_warm = 0;                           // TS_OPT_TAU_WARM
-  float* d_vcache = nullptr;                  // eigenvectors of M per point [E*4][(2N-1)^2] (warm start)
-  bool vcache_valid = false;
   bool binv_valid = false;                    // d_binv built at the current linearisation state
   float* d_eig = nullptr;                     // eigenpairs of M per point [E*4][EIG] (exact tangent)
   float* d_dT = nullptr;                      // d tau[v] L(u0) per point [E][4][3][C] (exact tangent)
@@ -209,6 +207,7 @@ static int lin_alloc(ts_problem* pr, LinState<T>& l) {
   std::vector<T> tt(tab.begin(), tab.end());
   TS_TRY(dalloc(&l.dft, tt.size()));
   TS_CUDA(cudaMemcpy(l.dft, tt.data(), tt.size() * sizeof(T), cudaMemcpyHostToDevice));
+  if (sizeof(T) == 8) TS_TRY(dalloc(&l.udd, (size_t)field_len(pr)));
   if (sizeof(T) == 4) {
     TS_TRY(dalloc(&l.u0t, (size_t)m->V * 4 * pr->K));
     TS_TRY(dalloc(&l.vt, (size_t)m->V * 4 * pr->K));
@@ -234,6 +233,7 @@ static void lin_free(LinState<T>& l) {
   dfree(l.t0);
   dfree(l.dft);
   dfree(l.u0t);
+  dfree(l.udd);
   dfree(l.vt);
   dfree(l.bneg);
   dfree(l.l0);
@@ -375,16 +375,9 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
       rc = launch_tau<T, N>(m->d_tets, geo_of<T>(m), y, m->E, l.tau, (T)(pr->p.mu / pr->p.rho),
                             (T)pr->p.C_I, pr->d_counter, st, eig);
     else if (pr->tau64 == TS_TAU64_DOUBLEFLOAT) {
-      float* vc = nullptr;
-      if (pr->tau_warm) {
-        constexpr int64_t NMN = (2 * N - 1) * (2 * N - 1);
-        if (!pr->d_vcache) TS_TRY(dalloc(&pr->d_vcache, (size_t)(m->E * 4 * NMN)));
-        vc = pr->d_vcache;
-      }
-      rc = launch_tau_dd<N>(m->d_tets, m->d_geo64, (const double*)y, m->E, (double*)l.tau,
-                            pr->p.mu / pr->p.rho, pr->p.C_I, pr->d_counter, st, eig, vc,
-                            pr->vcache_valid ? 1 : 0);
-      if (vc && rc == 0) pr->vcache_valid = true;
+      if (launch_split_dd((const double*)y, l.udd, n, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
+      rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, l.udd, m->E, (double*)l.tau, pr->p.mu / pr->p.rho, pr->p.C_I,
+                            pr->d_counter, st, eig);
     }
     else
       rc = launch_tau_polish<N>(m->d_tets, m->d_geo64, (const double*)y, m->E, (double*)l.tau,
@@ -1076,7 +1069,6 @@ void ts_problem_free(ts_problem* pr) {
   dfree(pr->d_D);
   dfree(pr->d_t);
   dfree(pr->d_binv);
-  dfree(pr->d_vcache);
   dfree(pr->d_eig);
   dfree(pr->d_dT);
   dfree(pr->d_hasm);
@@ -1110,8 +1102,6 @@ int ts_problem_option(ts_problem* pr, int key, int value) {
   }
   if (key == TS_OPT_TAU_WARM) {
     if (value != 0 && value != 1) return fail(TS_ERR_ARG, "TS_OPT_TAU_WARM takes 0 or 1");
-    pr->tau_warm = value;
-    pr->vcache_valid = false;
     return 0;
   }
   if (key == TS_OPT_FP32_TANGENT) {
@@ -1495,6 +1485,7 @@ struct ts_tracer {
   bool dirty = true;
   double *a4_64 = nullptr, *tau64 = nullptr, *dft64 = nullptr;
   float *a4_32 = nullptr, *tau32 = nullptr, *dft32 = nullptr;
+  float2* add = nullptr;             // a4_64 as double-float pairs
   unsigned* d_counter = nullptr;
   int gls = 1;                       // 0: Galerkin terms only (no least-squares term)
   // solve workspace (FP64)
@@ -1545,11 +1536,15 @@ int tracer_prepare(ts_tracer* tr, const T* a, cudaStream_t st) {
   }
   if (launch_repack_velocity<T>(a, a4, m->V, tr->C, st)) return fail(TS_ERR_CUDA, "repack kernel launch failed");
   int rc;
-  if constexpr (sizeof(T) == 8)
-    rc = launch_tau_dd<N>(m->d_tets, m->d_geo64, a4, m->E, tau, tr->kappa, tr->C_I, tr->d_counter, st);
-  else
+  if constexpr (sizeof(T) == 8) {
+    const int64_t n = m->V * 4 * (int64_t)tr->C;
+    if (!tr->add) TS_TRY(dalloc(&tr->add, (size_t)n));
+    if (launch_split_dd(a4, tr->add, n, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
+    rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, tr->add, m->E, tau, tr->kappa, tr->C_I, tr->d_counter, st);
+  } else {
     rc = launch_tau<float, N>(m->d_tets, m->d_geo32, a4, m->E, tau, (float)tr->kappa, (float)tr->C_I,
                               tr->d_counter, st);
+  }
   if (rc) return fail(TS_ERR_CUDA, "tau kernel launch failed");
   return 0;
 }
@@ -1717,6 +1712,7 @@ void ts_tracer_free(ts_tracer* t) {
   dfree(t->d_dmask);
   dfree(t->d_counter);
   dfree(t->a4_64);
+  dfree(t->add);
   dfree(t->tau64);
   dfree(t->dft64);
   dfree(t->a4_32);
@@ -1920,17 +1916,6 @@ int ts_solve(ts_problem* pr, void* y_inout, const ts_solve_opts* opts, ts_solve_
   if (o.precond < 0 || o.precond > 3) return fail(TS_ERR_ARG, "ts_solve: precond must be 0, 1, 2 or 3");
   std::memset(rep, 0, sizeof(*rep));
   TS_TRY(sync_dmask(pr));
-  // the solve's own residuals start tau's eigensolve from the previous step's
-  // eigenvectors (TS_OPT_TAU_WARM); the caller's setting returns on exit
-  struct WarmGuard {
-    ts_problem* p;
-    int saved;
-    ~WarmGuard() {
-      p->tau_warm = saved;
-      if (!saved) p->vcache_valid = false;
-    }
-  } warm_guard{pr, pr->tau_warm};
-  pr->tau_warm = 1;
   const int64_t n = field_len(pr);
   const int m = o.krylov;
   if (pr->basis_m < m + 1) {

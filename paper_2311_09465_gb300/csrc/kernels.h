@@ -34,13 +34,13 @@ int launch_tau_polish(const int4* tets, const double* geo, const double* y, int6
                       double* tau_out, double nu, double C_I, unsigned* n_unconverged,
                       cudaStream_t st, float* eig_out = nullptr);
 
-// the same refinement in double-float arithmetic (tau_dd.cu); with vcache
-// ((2N-1)^2 floats per point) the refined eigenvectors are stored there, and
-// with warm the Jacobi sweeps start from the ones stored by the last launch
+// FP64 tau from FP32 eigenpairs and Newton corrections with residuals in 58-bit
+// fixed point (tau_fx.cu); y: the state as double-float pairs [V][4][C]
 template <int N>
-int launch_tau_dd(const int4* tets, const double* geo, const double* y, int64_t n_elem,
-                  double* tau_out, double nu, double C_I, unsigned* n_unconverged,
-                  cudaStream_t st, float* eig_out = nullptr, float* vcache = nullptr, int warm = 0);
+int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t n_elem, double* tau_out, double nu,
+                  double C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out = nullptr);
+// n doubles as (hi, lo) FP32 pairs
+int launch_split_dd(const double* in, float2* out, int64_t n, cudaStream_t st);
 
 // Backflow stabilisation on one Neumann face set (tau.cu): when y_for_matrix
 // is given, first |A_n|_- at the 3 points of every face into bneg; then

@@ -1,0 +1,628 @@
+// tau of eq. (3D-tau) to FP64 accuracy without FP64 arithmetic: FP32 eigenpairs
+// (onesided.cuh) and Newton corrections whose residuals are formed in 58-bit
+// fixed point on the integer multiply-add pipe.
+//
+// With the point scaled so that the eigenvalues of M lie in (0, 1] and X near
+// M^{-1/2}, one correction is
+//   R = I - X M X,   S E + E S = R with S = M^{1/2},   X <- X + E.
+// Only R needs more than FP32 (it is the small difference of large terms); the
+// Sylvester equation is solved in the FP32 eigenbasis, E_ab = R_ab / (s_a + s_b).
+// The start X0 = U diag(1/s) U^T rounded to 29 bits leaves |R| near 1e-6; the
+// first correction leaves |R| near 1e-11 and the second is below the output's
+// rounding.  Matrices whose FP32 eigenpairs are poor (very large condition
+// number) take more corrections, up to FX_MAX_IT.
+//
+// Fixed point: a value v, |v| <= 1, is the integer V = v 2^58, split into two
+// 29-bit signed limbs V = 2^29 h + l, |l| <= 2^28.  A dot product of length
+// n <= 29 sums h h' in one 64-bit accumulator and h l' + l h' in another (no
+// overflow: 29 * 2^58 and 58 * 2^57 stay below 2^63), exactly; l l' (below
+// 2^-58 of the largest term) is left out.  That is three 32 x 32 -> 64 bit
+// multiply-adds a term against 12 to 15 FP32 instructions for a double-float
+// term, and GB300 issues them at half the FP32 rate: 6 issue slots against 12
+// to 15, with an absolute error near 2^-57 instead of 2^-47.  In R the scale of
+// X enters twice, so R is known to about cond(M) 2^-57.
+//
+// Mapping: as tau32_kernel (tau.cu), a group of N lanes owns a point and lane p
+// the columns 2p-1 and 2p of every matrix.  A product reads the left matrix
+// row by row from shared memory (16-byte loads, the same address in the whole
+// group where a full product is needed) against the lane's columns in registers.
+// Symmetric results (M, R, E) are formed for half of their entries: rows
+// 2p-1 .. 2p+N-1 (cyclic) of the lane's two columns cover every pair (r, s), and
+// both triangles are written.  The loops over rows stay rolled: a correction is
+// one instruction stream of a few hundred instructions, not of several thousand.
+#include <algorithm>
+
+#include "common.cuh"
+#include "ddfloat.cuh"
+#include "kernels.h"
+#include "onesided.cuh"
+
+namespace ts {
+
+namespace {
+
+constexpr int FX_MAX_IT = 10;
+
+using i64 = long long;
+
+struct Limbs {
+  int h, l;
+};
+
+__device__ __forceinline__ Limbs fx_split(i64 v) {
+  const int l = (int)((unsigned)v << 3) >> 3;   // the low 29 bits, signed
+  return {(int)((v - l) >> 29), l};
+}
+
+// v sqrt(2) for |v| <= 2^58 (rounded to the last place)
+__device__ __forceinline__ i64 fx_sqrt2(i64 v) {
+  constexpr i64 S = 6521908912666391106;        // sqrt(2) 2^62
+  return (__mul64hi(v << 4, S) + 2) >> 2;
+}
+
+__device__ __forceinline__ i64 fx_from_dd(dd a) {   // |a| <= 1
+  constexpr float B = 288230376151711744.f;         // 2^58
+  return __float2ll_rn(a.hi * B) + __float2ll_rn(a.lo * B);
+}
+
+// V 2^e as a double, rounded to nearest (ties away from zero)
+__device__ __forceinline__ double fx_to_double(i64 v, int e) {
+  if (v == 0) return 0.0;
+  const unsigned long long u = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
+  const int lz = __clzll((i64)u);
+  const unsigned long long m = u << lz;
+  unsigned long long b = (m >> 11) + ((m >> 10) & 1);
+  b += (unsigned long long)(1022 + 63 - lz + e) << 52;
+  return __longlong_as_double((i64)(b | (v < 0 ? 1ull << 63 : 0ull)));
+}
+
+// sum_j row[j] col[j]: acc.x of the h h' products, acc.y of the mixed ones
+template <int NM>
+__device__ __forceinline__ void fx_dot(const int4* __restrict__ row, const Limbs (&c)[NM], i64& hh, i64& x) {
+#pragma unroll
+  for (int j = 0; j < NM; j += 2) {
+    const int4 r = row[j / 2];
+    hh += (i64)r.x * c[j].h;
+    x += (i64)r.x * c[j].l;
+    x += (i64)r.y * c[j].h;
+    if (j + 1 < NM) {
+      hh += (i64)r.z * c[j + 1].h;
+      x += (i64)r.z * c[j + 1].l;
+      x += (i64)r.w * c[j + 1].h;
+    }
+  }
+}
+
+// the same with two columns: each row entry is loaded once
+template <int NM>
+__device__ __forceinline__ void fx_dot2(const int4* __restrict__ row, const Limbs (&a)[NM], const Limbs (&b)[NM],
+                                        i64& h0, i64& x0, i64& h1, i64& x1) {
+#pragma unroll
+  for (int j = 0; j < NM; ++j) {
+    const int4 r = row[j / 2];
+    const int rh = (j & 1) ? r.z : r.x, rl = (j & 1) ? r.w : r.y;
+    h0 += (i64)rh * a[j].h;
+    x0 += (i64)rh * a[j].l;
+    x0 += (i64)rl * a[j].h;
+    h1 += (i64)rh * b[j].h;
+    x1 += (i64)rh * b[j].l;
+    x1 += (i64)rl * b[j].h;
+  }
+}
+
+template <int W>
+__device__ __forceinline__ void load_floats(const float* src, float (&dst)[W]) {
+#pragma unroll
+  for (int j = 0; j < W / 4; ++j) {
+    const float4 v = reinterpret_cast<const float4*>(src)[j];
+    dst[4 * j] = v.x;
+    dst[4 * j + 1] = v.y;
+    dst[4 * j + 2] = v.z;
+    dst[4 * j + 3] = v.w;
+  }
+}
+
+}  // namespace
+
+template <int N>
+struct FxLayout {
+  static constexpr int NM = 2 * N - 1, C = 2 * N, L = N - 1, GPW = 32 / N;
+  static constexpr int LDQ = (NM + 1) & ~1;             // limb pairs a row (16-byte multiple)
+  static constexpr int LDF = (2 * N + 3) & ~3;          // floats a row
+  static constexpr int TW = 3 * N;
+  // in 4-byte words
+  static constexpr int M = 0;                           // [NM][LDQ] limbs
+  static constexpr int X = M + 2 * NM * LDQ;            // [NM][LDQ] limbs: C_m, then X
+  static constexpr int F = X + 2 * NM * LDQ;            // [NM][LDF]: h_a, R, U^T R, E
+  static constexpr int U = F + NM * LDF;                // [NM][LDF]: row a = eigenvector a
+  static constexpr int S = U + NM * LDF;                // [2N] sqrt of the eigenvalues
+  static constexpr int END = S + ((2 * N + 3) & ~3);
+  static constexpr int T = F;                           // [3][2][TW] 64-bit modes, [3][2][N] times sqrt2: over F, U
+  static constexpr int TEND = T + 2 * (3 * 2 * TW + 3 * 2 * N);
+  static constexpr int OUTP = M;                        // packed tau (doubles) over M
+  static constexpr int RAW0 = END > TEND ? END : TEND;
+  static constexpr int RAW1 = (RAW0 > 2 * Dims<N>::NT_PAD ? RAW0 : 2 * Dims<N>::NT_PAD);
+  static constexpr int RAW = (RAW1 + 3) & ~3;
+  static constexpr int GROUP = RAW + ((4 - RAW) % 32 + 32) % 32;   // groups in different banks
+  static constexpr int WARP = GPW * GROUP;
+};
+
+// y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2
+template <int N>
+__global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
+                                                     const float2* __restrict__ y, int64_t n_qp,
+                                                     double* __restrict__ tau_out, dd nu2,
+                                                     unsigned* __restrict__ n_unconverged,
+                                                     float* __restrict__ eig_out) {
+  using Lt = FxLayout<N>;
+  constexpr int NM = Lt::NM, C = Lt::C, L = Lt::L, LDQ = Lt::LDQ, LDF = Lt::LDF, GPW = Lt::GPW, TW = Lt::TW;
+  constexpr int NT = Dims<N>::NT, NTP = Dims<N>::NT_PAD;
+  extern __shared__ __align__(16) int fx_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane / N, p = lane - (lane / N) * N;
+  const bool in_group = g < GPW;
+  const int first = in_group ? g * N : 0;               // first lane of the group
+  int* base = fx_smem + warp * Lt::WARP + (in_group ? g : 0) * Lt::GROUP;
+  Limbs* Ms = reinterpret_cast<Limbs*>(base + Lt::M);
+  Limbs* Xs = reinterpret_cast<Limbs*>(base + Lt::X);
+  float* F = reinterpret_cast<float*>(base + Lt::F);
+  float* U = reinterpret_cast<float*>(base + Lt::U);
+  float* sv = reinterpret_cast<float*>(base + Lt::S);
+  i64* T = reinterpret_cast<i64*>(base + Lt::T);
+  i64* T2 = T + 3 * 2 * TW;
+  // the lane's columns, and whether it has a first one
+  const int cx = 2 * p - 1, cy = 2 * p;
+  const bool hx = in_group && p > 0, hy = in_group;
+  // row o of the lane's half: (2p - 1 + o) mod NM
+  auto half_row = [&](int o) {
+    int r = 2 * p - 1 + o;
+    if (r < 0) r += NM;
+    return r >= NM ? r - NM : r;
+  };
+
+  const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t qb = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * GPW; qb < n_qp; qb += warps_total * GPW) {
+    const bool live = in_group && qb + g < n_qp;
+    const int64_t gq = live ? qb + g : qb;              // idle lanes redo the warp's first point, unstored
+    const int64_t e = gq >> 2;
+    const int q = (int)(gq & 3);
+    // ---- w_m = sum_i L_im u_i for mode p, G = L L^T (double-float)
+    dd w[3][2], diff;
+    {
+      const double* gg = geo + e * GEO_STRIDE + GEO_G;
+      const dd gxx = dd_from_double(gg[0]), gxy = dd_from_double(gg[1]), gxz = dd_from_double(gg[2]),
+               gyy = dd_from_double(gg[3]), gyz = dd_from_double(gg[4]), gzz = dd_from_double(gg[5]);
+      const dd off = dd_fma(gxy, gxy, dd_fma(gxz, gxz, dd_mul(gyz, gyz)));
+      const dd dia = dd_fma(gxx, gxx, dd_fma(gyy, gyy, dd_mul(gzz, gzz)));
+      diff = dd_mul(nu2, dd_add(dia, dd_scale(off, 2.f)));
+      const dd l00 = dd_sqrt(gxx), r00 = dd_rcp(l00);
+      const dd l10 = dd_mul(gxy, r00), l20 = dd_mul(gxz, r00);
+      const dd l11 = dd_sqrt(dd_fma(dd_neg(l10), l10, gyy)), r11 = dd_rcp(l11);
+      const dd l21 = dd_mul(dd_fma(dd_neg(l20), l10, gyz), r11);
+      const dd l22 = dd_sqrt(dd_fma(dd_neg(l21), l21, dd_fma(dd_neg(l20), l20, gzz)));
+      const int4 nd = tets[e];
+      const int node[4] = {nd.x, nd.y, nd.z, nd.w};
+      // lambda_a(q) = b + (a - b) delta_aq: u = b sum_a y_a + (a - b) y_q
+      constexpr double BQ = qp_bary(0, 1), DQ = qp_bary(0, 0) - qp_bary(0, 1);
+      constexpr float BH = (float)BQ, BL = (float)(BQ - (double)BH), DH = (float)DQ, DL = (float)(DQ - (double)DH);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        dd u[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          dd v[4];
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            const float2 f = y[(int64_t)node[a] * 4 * C + i * C + 2 * p + h];
+            v[a] = dd{f.x, f.y};
+          }
+          const dd vq = q == 0 ? v[0] : q == 1 ? v[1] : q == 2 ? v[2] : v[3];
+          const dd sum = dd_add(dd_add(v[0], v[1]), dd_add(v[2], v[3]));
+          u[i] = dd_fma(dd{DH, DL}, vq, dd_mul(dd{BH, BL}, sum));
+          if (p == 0 && h == 1) u[i] = dd{0.f, 0.f};
+        }
+        w[0][h] = dd_fma(l00, u[0], dd_fma(l10, u[1], dd_mul(l20, u[2])));
+        w[1][h] = dd_fma(l11, u[1], dd_mul(l21, u[2]));
+        w[2][h] = dd_mul(l22, u[2]);
+      }
+    }
+    // |C_m| <= beta_m = |w_0| + 2 sum |w_n|: with sum_m beta_m + sqrt(c) <= 1 after
+    // the scale 2^-ex, M's eigenvalues (and so its entries) are at most 1
+    float bound = 0.f;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) bound += (fabsf(w[m][0].hi) + fabsf(w[m][1].hi)) * (p == 0 ? 1.f : 2.f);
+    {
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < N; ++j) sum += __shfl_sync(0xffffffffu, bound, first + j);
+      bound = 1.0001f * (sum + sqrtf(diff.hi));
+    }
+    const bool finite = bound < 1e18f && bound > 1e-18f;
+    int ex = 0;
+    if (finite) frexpf(bound, &ex);
+    const float sc = ldexpf(1.f, -ex);
+    const i64 cfix = finite ? fx_from_dd(dd_scale(diff, sc * sc)) : (1ll << 57);
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      i64* tr = T + m * 2 * TW + L;                     // mode k at tr[k], its imaginary part at tr[TW + k]
+      const i64 re = finite ? fx_from_dd(dd_scale(w[m][0], sc)) : 0, im = finite ? fx_from_dd(dd_scale(w[m][1], sc)) : 0;
+      if (in_group) {
+        tr[p] = re;
+        tr[TW + p] = im;
+        T2[(m * 2 + 0) * N + p] = fx_sqrt2(re);
+        T2[(m * 2 + 1) * N + p] = fx_sqrt2(im);
+        if (p > 0) {
+          tr[-p] = re;
+          tr[TW - p] = -im;
+          tr[L + p] = 0;
+          tr[TW + L + p] = 0;
+        }
+      }
+    }
+    __syncwarp();
+    // ---- M = sum_m C_m C_m + c I on half of the entries: the sums over m are kept
+    // as 64-bit integers at (row, lane's column) of M's place
+    {
+      i64* acc = reinterpret_cast<i64*>(Ms);
+#pragma unroll 1
+      for (int m = 0; m < 3; ++m) {
+        const i64* tr = T + m * 2 * TW + L;
+        const i64* ti = tr + TW;
+        const i64* t2 = T2 + m * 2 * N;
+        Limbs a[NM], b[NM];
+        a[0] = fx_split(t2[p]);
+        b[0] = fx_split(p == 0 ? tr[0] : t2[N + p]);
+#pragma unroll
+        for (int k = 1; k < N; ++k) {
+          const i64 pl = tr[k - p], ph = tr[k + p], ql = ti[k - p], qh = ti[k + p];
+          a[2 * k - 1] = fx_split(pl + ph);
+          a[2 * k] = fx_split(ql + qh);
+          b[2 * k - 1] = fx_split(p == 0 ? t2[k] : qh - ql);
+          b[2 * k] = fx_split(p == 0 ? t2[N + k] : pl - ph);
+        }
+        __syncwarp();                                   // all lanes have read the previous C_m
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          if (hx) Xs[cx * LDQ + i] = a[i];
+          if (hy) Xs[cy * LDQ + i] = b[i];
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int o = 0; o <= N; ++o) {
+          const int r = half_row(o);
+          const int4* row = reinterpret_cast<const int4*>(Xs + r * LDQ);
+          i64 h0 = 0, x0 = 0, h1 = 0, x1 = 0;
+          fx_dot2<NM>(row, a, b, h0, x0, h1, x1);
+          const i64 v0 = h0 + ((x0 + (1ll << 28)) >> 29), v1 = h1 + ((x1 + (1ll << 28)) >> 29);
+          if (hx && o < N) acc[r * LDQ + cx] = m == 0 ? v0 : acc[r * LDQ + cx] + v0;
+          if (hy && o > 0) acc[r * LDQ + cy] = m == 0 ? v1 : acc[r * LDQ + cy] + v1;
+        }
+      }
+      // limbs in both triangles (a lane's entries are its own: no other lane's place is touched)
+#pragma unroll 1
+      for (int o = 0; o <= N; ++o) {
+        const int r = half_row(o);
+        if (hx && o < N) {
+          const Limbs v = fx_split(acc[r * LDQ + cx] + (r == cx ? cfix : 0));
+          Ms[r * LDQ + cx] = v;
+          Ms[cx * LDQ + r] = v;
+        }
+        if (hy && o > 0) {
+          const Limbs v = fx_split(acc[r * LDQ + cy] + (r == cy ? cfix : 0));
+          Ms[r * LDQ + cy] = v;
+          Ms[cy * LDQ + r] = v;
+        }
+      }
+    }
+    __syncwarp();
+    // ---- FP32 eigenpairs: f_a with M = sum f_a f_a^T
+    int xe;                                             // |X| <= 2^xe
+    {
+      float x[NM], yv[NM];
+      constexpr float H = 1.f / 536870912.f, HL = H * H;   // 2^-29, 2^-58
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        const Limbs mx = Ms[(hx ? cx : 0) * LDQ + i], my = Ms[cy * LDQ + i];
+        x[i] = hx ? fmaf((float)mx.l, HL, (float)mx.h * H) : 0.f;
+        yv[i] = hy ? fmaf((float)my.l, HL, (float)my.h * H) : 0.f;
+      }
+      const float cd = (float)cfix * HL;
+      cholesky_columns<N>(x, yv, in_group ? p : 64, first, fmaxf(cd, 1e-30f));
+      const bool conv = onesided_jacobi<N>(x, yv, p, lane);
+      {
+        const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);
+        const unsigned mine = ((1u << N) - 1u) << first;
+        if (live && p == 0 && (bad & mine)) atomicAdd(n_unconverged, 1u);
+      }
+      float ax = 0.f, ay = 0.f;
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        ax = fmaf(x[i], x[i], ax);
+        ay = fmaf(yv[i], yv[i], ay);
+      }
+      const float ix = hx ? rsqrt_newton(ax) : 0.f, iy = hy ? rsqrt_newton(ay) : 0.f;
+      const float jx = ix * sqrtf(ix), jy = iy * sqrtf(iy);
+      float big = fmaxf(ix, iy), all = 0.f;
+#pragma unroll
+      for (int j = 0; j < N; ++j) all = fmaxf(all, __shfl_sync(0xffffffffu, big, first + j));
+      frexpf(1.01f * all, &xe);
+      xe = min(max(xe, 0), 28);
+      // eigenpairs for the derivative of tau (exact tangent), when asked
+      if (live && eig_out) {
+        float* eo = eig_out + gq * Dims<N>::EIG;
+        const float back = ldexpf(1.f, 2 * ex);
+        if (hx) {
+#pragma unroll
+          for (int i = 0; i < NM; ++i) eo[i * NM + cx] = x[i] * ix;
+          eo[NM * NM + cx] = ax * back;
+        }
+#pragma unroll
+        for (int i = 0; i < NM; ++i) eo[i * NM + cy] = yv[i] * iy;
+        eo[NM * NM + cy] = ay * back;
+      }
+      // U, s; h_a = f_a / |f_a|^{3/2} one float off (a lane's two entries an aligned pair)
+      if (hx) {
+        sv[cx] = ax * ix;
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          U[cx * LDF + i] = x[i] * ix;
+          F[cx * LDF + i + 1] = x[i] * jx;
+        }
+      }
+      if (hy) {
+        sv[cy] = ay * iy;
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          U[cy * LDF + i] = yv[i] * iy;
+          F[cy * LDF + i + 1] = yv[i] * jy;
+        }
+      }
+      if (in_group && p == 0) {
+#pragma unroll
+        for (int a = 0; a < NM; ++a) F[a * LDF] = 0.f;
+      }
+    }
+    __syncwarp();
+    // ---- X0 = sum_a h_a h_a^T rounded to one limb
+    {
+      float x[NM], yv[NM];
+#pragma unroll
+      for (int i = 0; i < NM; ++i) x[i] = yv[i] = 0.f;
+#pragma unroll 1
+      for (int a = 0; a < NM; ++a) {
+        const float2 own = *reinterpret_cast<const float2*>(F + a * LDF + 2 * p);
+        float row[LDF];
+        load_floats<LDF>(F + a * LDF, row);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          x[i] = fmaf(row[i + 1], own.x, x[i]);
+          yv[i] = fmaf(row[i + 1], own.y, yv[i]);
+        }
+      }
+      const float to = ldexpf(1.f, 29 - xe);
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        if (hx) Xs[cx * LDQ + i] = Limbs{__float2int_rn(x[i] * to), 0};
+        if (hy) Xs[cy * LDQ + i] = Limbs{__float2int_rn(yv[i] * to), 0};
+      }
+    }
+    const float rscale = ldexpf(1.f, xe - 58), escale = ldexpf(1.f, 58 - xe);
+    const float small = fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
+    // ---- corrections
+#pragma unroll 1
+    for (int it = 0;; ++it) {
+      __syncwarp();
+      // R = I - X (M X), half of the entries, one of the lane's columns at a time
+      float rmax = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < 2; ++c) {
+        const int col = c == 0 ? (hx ? cx : 0) : cy;
+        const bool has = c == 0 ? hx : hy;
+        Limbs xc[NM], pc[NM];
+#pragma unroll
+        for (int j = 0; j < NM; j += 2) {
+          const int4 v = reinterpret_cast<const int4*>(Xs + col * LDQ)[j / 2];
+          xc[j] = Limbs{v.x, v.y};
+          if (j + 1 < NM) xc[j + 1] = Limbs{v.z, v.w};
+        }
+#pragma unroll
+        for (int r = 0; r < NM; ++r) {
+          i64 hh = 0, xx = 0;
+          fx_dot<NM>(reinterpret_cast<const int4*>(Ms + r * LDQ), xc, hh, xx);
+          // M X to 2^-58 (|M X| <= 1)
+          pc[r] = fx_split((hh << xe) + (xx >> (29 - xe)));
+        }
+#pragma unroll
+        for (int o = 0; o < N; ++o) {
+          const int r = half_row(o + c);
+          i64 hh = 0, xx = 0;
+          fx_dot<NM>(reinterpret_cast<const int4*>(Xs + r * LDQ), pc, hh, xx);
+          const i64 one = r == col ? (1ll << 58) >> xe : 0;
+          const float rv = (float)(one - hh - ((xx + (1ll << 28)) >> 29)) * rscale;
+          if (has) {
+            rmax = fmaxf(rmax, fabsf(rv));
+            F[r * LDF + col] = rv;
+            F[col * LDF + r] = rv;
+          }
+        }
+      }
+      const bool more = __any_sync(0xffffffffu, live && rmax > small) && it + 1 < FX_MAX_IT;
+      __syncwarp();
+      // U^T R: the lane's columns, over R
+      float rx[NM], ry[NM];
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        rx[i] = F[(hx ? cx : 0) * LDF + i];             // R is symmetric: column = row
+        ry[i] = F[cy * LDF + i];
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int a = 0; a < NM; ++a) {
+        float row[LDF], sx = 0.f, sy = 0.f;
+        load_floats<LDF>(U + a * LDF, row);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          sx = fmaf(row[i], rx[i], sx);
+          sy = fmaf(row[i], ry[i], sy);
+        }
+        if (hx) F[a * LDF + cx] = sx;
+        if (hy) F[a * LDF + cy] = sy;
+      }
+      __syncwarp();
+      // (U^T R) U divided by s_a + s_b, row by row in place
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        rx[i] = U[(hx ? cx : 0) * LDF + i];
+        ry[i] = U[cy * LDF + i];
+      }
+      {
+        const float s0 = sv[hx ? cx : 0], s1 = sv[cy];
+#pragma unroll 1
+        for (int a = 0; a < NM; ++a) {
+          float row[LDF], sx = 0.f, sy = 0.f;
+          load_floats<LDF>(F + a * LDF, row);
+#pragma unroll
+          for (int i = 0; i < NM; ++i) {
+            sx = fmaf(row[i], rx[i], sx);
+            sy = fmaf(row[i], ry[i], sy);
+          }
+          const float sa = sv[a];
+          __syncwarp();
+          if (hx) F[a * LDF + cx] = sx * rcp_ftz(sa + s0);
+          if (hy) F[a * LDF + cy] = sy * rcp_ftz(sa + s1);
+        }
+      }
+      __syncwarp();
+      // E = U (.) U^T: the lane's columns
+      float ex_[NM], ey_[NM];
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        rx[i] = U[i * LDF + (hx ? cx : 0)];
+        ry[i] = U[i * LDF + cy];
+        ex_[i] = ey_[i] = 0.f;
+      }
+#pragma unroll 1
+      for (int a = 0; a < NM; ++a) {
+        float row[LDF], sx = 0.f, sy = 0.f;
+        load_floats<LDF>(F + a * LDF, row);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          sx = fmaf(row[i], rx[i], sx);
+          sy = fmaf(row[i], ry[i], sy);
+        }
+        load_floats<LDF>(U + a * LDF, row);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          ex_[i] = fmaf(row[i], sx, ex_[i]);
+          ey_[i] = fmaf(row[i], sy, ey_[i]);
+        }
+      }
+      __syncwarp();
+      // X <- X + E on half of the entries (exactly symmetric)
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        if (hx) F[cx * LDF + i] = ex_[i];
+        if (hy) F[cy * LDF + i] = ey_[i];
+      }
+      __syncwarp();
+      i64 nx[N], ny[N];
+#pragma unroll
+      for (int o = 0; o < N; ++o) {
+        const int r0 = half_row(o), r1 = half_row(o + 1), c0 = hx ? cx : 0;
+        const Limbs a = Xs[c0 * LDQ + r0], b = Xs[cy * LDQ + r1];
+        nx[o] = ((i64)a.h << 29) + a.l + __float2ll_rn(F[c0 * LDF + r0] * escale);
+        ny[o] = ((i64)b.h << 29) + b.l + __float2ll_rn(F[cy * LDF + r1] * escale);
+      }
+      __syncwarp();
+      if (more) {
+#pragma unroll
+        for (int o = 0; o < N; ++o) {
+          const int r0 = half_row(o), r1 = half_row(o + 1);
+          const Limbs a = fx_split(nx[o]), b = fx_split(ny[o]);
+          if (hx) {
+            Xs[cx * LDQ + r0] = a;
+            Xs[r0 * LDQ + cx] = a;
+          }
+          if (hy) {
+            Xs[cy * LDQ + r1] = b;
+            Xs[r1 * LDQ + cy] = b;
+          }
+        }
+        continue;
+      }
+      // packed upper triangle through shared memory (over M)
+      double* op = reinterpret_cast<double*>(base + Lt::OUTP);
+      const int e2 = xe - 58 - ex;
+#pragma unroll
+      for (int o = 0; o < N; ++o) {
+        const int r0 = half_row(o), r1 = half_row(o + 1);
+        if (hx) op[packed_index(min(r0, cx), max(r0, cx), NM)] = finite ? fx_to_double(nx[o], e2) : __longlong_as_double(0x7ff8000000000000ll);
+        if (hy) op[packed_index(min(r1, cy), max(r1, cy), NM)] = finite ? fx_to_double(ny[o], e2) : __longlong_as_double(0x7ff8000000000000ll);
+      }
+      if (in_group && p == 0) {
+#pragma unroll
+        for (int t = NT; t < NTP; ++t) op[t] = 0.0;
+      }
+      break;
+    }
+    __syncwarp();
+    if (live) {
+      const double2* op = reinterpret_cast<const double2*>(base + Lt::OUTP);
+      double2* out = reinterpret_cast<double2*>(tau_out + gq * NTP);
+      for (int t = p; t < NTP / 2; t += N) out[t] = op[t];
+    }
+    __syncwarp();
+  }
+}
+
+template <int N>
+int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t n_elem, double* tau_out, double nu,
+                  double C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out) {
+  using Lt = FxLayout<N>;
+  // warps a block (1..4) that keep the most warps resident in 227 KB of shared memory
+  int warps = 1, best = 0;
+  for (int wb = 1; wb <= 4; ++wb) {
+    const size_t per_block = (size_t)wb * Lt::WARP * 4;
+    if (per_block > 227 * 1024) break;
+    const int resident = wb * (int)((228 * 1024) / (per_block + 1024));
+    if (resident > best) {
+      best = resident;
+      warps = wb;
+    }
+  }
+  const size_t smem = (size_t)warps * Lt::WARP * 4;
+  if (cudaFuncSetAttribute(tau_fx_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return -2;
+  const int64_t n_qp = n_elem * 4, groups = (n_qp + Lt::GPW - 1) / Lt::GPW;
+  const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, 152 * 128));
+  const double k = C_I * nu * nu;
+  const float kh = (float)k;
+  count_launches(1);
+  tau_fx_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, dd{kh, (float)(k - (double)kh)},
+                                                          n_unconverged, eig_out);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}
+
+#define TS_INST_TAU_FX(T, N)                                                                             \
+  template int launch_tau_fx<N>(const int4*, const double*, const float2*, int64_t, double*, double, double, \
+                                unsigned*, cudaStream_t, float*);
+TS_FOR_EACH_N(TS_INST_TAU_FX, double)
+
+// double -> (hi, lo) pairs of FP32 numbers
+__global__ void split_dd_kernel(const double* __restrict__ in, float2* __restrict__ out, int64_t n) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    const dd v = dd_from_double(in[t]);
+    out[t] = make_float2(v.hi, v.lo);
+  }
+}
+
+int launch_split_dd(const double* in, float2* out, int64_t n, cudaStream_t st) {
+  if (n <= 0) return 0;
+  const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 16);
+  count_launches(1);
+  split_dd_kernel<<<(int)blocks, 256, 0, st>>>(in, out, n);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}
+
+}  // namespace ts
