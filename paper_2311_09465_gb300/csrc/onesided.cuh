@@ -84,14 +84,14 @@ __device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&
   }
 }
 
-// One-sided Jacobi on the group's columns.  Returns whether this lane's pairs
-// were orthogonal to ORTHO2 (squared cosine) before the last sweep's rotations;
-// that sweep then leaves cosines of the order of their squares (1e-8).
-constexpr float ORTHO2 = 1e-8f;
+// One-sided Jacobi on the group's columns.  Sweeps until every pair of the warp
+// had a squared cosine of at most ortho2 before its rotation; that last sweep
+// leaves cosines of the order of ortho2.  Returns whether this lane's pairs had.
 constexpr int ONESIDED_SWEEPS = 15;
 
 template <int N>
-__device__ __forceinline__ bool onesided_jacobi(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, int lane) {
+__device__ __forceinline__ bool onesided_jacobi(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, int lane,
+                                                float ortho2) {
   constexpr int NM = 2 * N - 1;
   if constexpr (N == 1) return true;
   const int up = (lane + 31) & 31, down = (lane + 1) & 31;
@@ -119,7 +119,7 @@ __device__ __forceinline__ bool onesided_jacobi(float (&x)[2 * N - 1], float (&y
         g = g0 + g1;
       }
       rotation_of(ax, ay, g, s, ta, t);
-      rotated |= g * g > ORTHO2 * ax * ay;
+      rotated |= g * g > ortho2 * ax * ay;
       if (first) s = -1.f, ta = -1.f;
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
@@ -147,7 +147,7 @@ __device__ __forceinline__ bool onesided_jacobi(float (&x)[2 * N - 1], float (&y
         g = g0 + g1;
       }
       rotation_of(ay, az, g, s, ta, t);
-      rotated |= g * g > ORTHO2 * ay * az;
+      rotated |= g * g > ortho2 * ay * az;
       if (last) s = 1.f, ta = 1.f;
 #pragma unroll
       for (int i = 0; i < NM; ++i) {

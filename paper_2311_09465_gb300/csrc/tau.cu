@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(128) tau32_kernel(const int4* __restrict__ tet
       if (!in_group) yy[i] = 0.f;
     }
     cholesky_columns<N>(x, yy, in_group ? p : 64, g * N, fmaxf(cd, 1e-30f));
-    const bool conv = onesided_jacobi<N>(x, yy, p, lane);
+    const bool conv = onesided_jacobi<N>(x, yy, p, lane, 1e-8f);
     {
       const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);
       const unsigned mine = N == 32 ? ~0u : ((1u << N) - 1u) << (in_group ? g * N : 0);

@@ -42,8 +42,14 @@ namespace ts {
 namespace {
 
 constexpr int FX_MAX_IT = 10;
+constexpr float FX_ORTHO2 = 1e-6f;   // leaves cosines near 1e-6: the corrections absorb them
 
 using i64 = long long;
+
+// acc += a b; written out because a reassociated sum of products costs 64-bit adds
+__device__ __forceinline__ void fx_mad(i64& acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
 
 struct Limbs {
   int h, l;
@@ -76,38 +82,25 @@ __device__ __forceinline__ double fx_to_double(i64 v, int e) {
   return __longlong_as_double((i64)(b | (v < 0 ? 1ull << 63 : 0ull)));
 }
 
-// sum_j row[j] col[j]: acc.x of the h h' products, acc.y of the mixed ones
-template <int NM>
-__device__ __forceinline__ void fx_dot(const int4* __restrict__ row, const Limbs (&c)[NM], i64& hh, i64& x) {
-#pragma unroll
-  for (int j = 0; j < NM; j += 2) {
-    const int4 r = row[j / 2];
-    hh += (i64)r.x * c[j].h;
-    x += (i64)r.x * c[j].l;
-    x += (i64)r.y * c[j].h;
-    if (j + 1 < NM) {
-      hh += (i64)r.z * c[j + 1].h;
-      x += (i64)r.z * c[j + 1].l;
-      x += (i64)r.w * c[j + 1].h;
-    }
-  }
-}
-
-// the same with two columns: each row entry is loaded once
+// sums over j of row[j] a[j] and row[j] b[j]; row: limb pairs stored one place
+// off (entry j at j + 1), so that a lane's columns 2p-1 and 2p are one int4
 template <int NM>
 __device__ __forceinline__ void fx_dot2(const int4* __restrict__ row, const Limbs (&a)[NM], const Limbs (&b)[NM],
                                         i64& h0, i64& x0, i64& h1, i64& x1) {
+  i64 y0 = 0, y1 = 0;
 #pragma unroll
   for (int j = 0; j < NM; ++j) {
-    const int4 r = row[j / 2];
-    const int rh = (j & 1) ? r.z : r.x, rl = (j & 1) ? r.w : r.y;
-    h0 += (i64)rh * a[j].h;
-    x0 += (i64)rh * a[j].l;
-    x0 += (i64)rl * a[j].h;
-    h1 += (i64)rh * b[j].h;
-    x1 += (i64)rh * b[j].l;
-    x1 += (i64)rl * b[j].h;
+    const int4 r = row[(j + 1) / 2];
+    const int rh = (j & 1) ? r.x : r.z, rl = (j & 1) ? r.y : r.w;
+    fx_mad(h0, rh, a[j].h);
+    fx_mad(x0, rh, a[j].l);
+    fx_mad(y0, rl, a[j].h);
+    fx_mad(h1, rh, b[j].h);
+    fx_mad(x1, rh, b[j].l);
+    fx_mad(y1, rl, b[j].h);
   }
+  x0 += y0;
+  x1 += y1;
 }
 
 template <int W>
@@ -122,13 +115,40 @@ __device__ __forceinline__ void load_floats(const float* src, float (&dst)[W]) {
   }
 }
 
+// a row from registers (times f), one place off
+template <int NM, int W>
+__device__ __forceinline__ void store_floats(float* dst, const float (&v)[NM], float f) {
+#pragma unroll
+  for (int j = 0; j < W / 4; ++j) {
+    if (4 * j > NM) break;
+    float t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = 4 * j + k - 1;
+      t[k] = i >= 0 && i < NM ? v[i < 0 ? 0 : i >= NM ? NM - 1 : i] * f : 0.f;
+    }
+    reinterpret_cast<float4*>(dst)[j] = make_float4(t[0], t[1], t[2], t[3]);
+  }
+}
+template <int NM>
+__device__ __forceinline__ void store_limbs(Limbs* dst, const Limbs (&v)[NM]) {
+#pragma unroll
+  for (int j = 0; j <= NM; j += 2) {
+    const Limbs lo = j == 0 ? Limbs{0, 0} : v[j == 0 ? 0 : j - 1], hi = j < NM ? v[j < NM ? j : 0] : Limbs{0, 0};
+    *reinterpret_cast<int4*>(dst + j) = make_int4(lo.h, lo.l, hi.h, hi.l);
+  }
+}
+
 }  // namespace
 
 template <int N>
 struct FxLayout {
   static constexpr int NM = 2 * N - 1, C = 2 * N, L = N - 1, GPW = 32 / N;
-  static constexpr int LDQ = (NM + 1) & ~1;             // limb pairs a row (16-byte multiple)
-  static constexpr int LDF = (2 * N + 3) & ~3;          // floats a row
+  // entry i of a row is stored at i + 1; a row is an odd number of 16-byte units,
+  // so that 16-byte reads of different rows by the lanes of a group spread over the banks
+  static constexpr int LDQ = (N & 1) ? 2 * N : 2 * N + 2;            // limb pairs a row
+  static constexpr int LDF0 = (2 * N + 3) & ~3;
+  static constexpr int LDF = (LDF0 / 4) & 1 ? LDF0 : LDF0 + 4;       // floats a row
   static constexpr int TW = 3 * N;
   // in 4-byte words
   static constexpr int M = 0;                           // [NM][LDQ] limbs
@@ -264,7 +284,7 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
     // ---- M = sum_m C_m C_m + c I on half of the entries: the sums over m are kept
     // as 64-bit integers at (row, lane's column) of M's place
     {
-      i64* acc = reinterpret_cast<i64*>(Ms);
+      i64* acc = reinterpret_cast<i64*>(Ms) + 1;
 #pragma unroll 1
       for (int m = 0; m < 3; ++m) {
         const i64* tr = T + m * 2 * TW + L;
@@ -282,11 +302,9 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
           b[2 * k] = fx_split(p == 0 ? t2[N + k] : pl - ph);
         }
         __syncwarp();                                   // all lanes have read the previous C_m
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-          if (hx) Xs[cx * LDQ + i] = a[i];
-          if (hy) Xs[cy * LDQ + i] = b[i];
-        }
+        // C_m's columns as rows (symmetric)
+        if (hx) store_limbs<NM>(Xs + cx * LDQ, a);
+        if (hy) store_limbs<NM>(Xs + cy * LDQ, b);
         __syncwarp();
 #pragma unroll 1
         for (int o = 0; o <= N; ++o) {
@@ -305,13 +323,13 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
         const int r = half_row(o);
         if (hx && o < N) {
           const Limbs v = fx_split(acc[r * LDQ + cx] + (r == cx ? cfix : 0));
-          Ms[r * LDQ + cx] = v;
-          Ms[cx * LDQ + r] = v;
+          Ms[r * LDQ + cx + 1] = v;
+          Ms[cx * LDQ + r + 1] = v;
         }
         if (hy && o > 0) {
           const Limbs v = fx_split(acc[r * LDQ + cy] + (r == cy ? cfix : 0));
-          Ms[r * LDQ + cy] = v;
-          Ms[cy * LDQ + r] = v;
+          Ms[r * LDQ + cy + 1] = v;
+          Ms[cy * LDQ + r + 1] = v;
         }
       }
     }
@@ -323,13 +341,13 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
       constexpr float H = 1.f / 536870912.f, HL = H * H;   // 2^-29, 2^-58
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
-        const Limbs mx = Ms[(hx ? cx : 0) * LDQ + i], my = Ms[cy * LDQ + i];
-        x[i] = hx ? fmaf((float)mx.l, HL, (float)mx.h * H) : 0.f;
-        yv[i] = hy ? fmaf((float)my.l, HL, (float)my.h * H) : 0.f;
+        const int4 mm = *reinterpret_cast<const int4*>(Ms + i * LDQ + 2 * p);   // (i, 2p-1) and (i, 2p)
+        x[i] = hx ? fmaf((float)mm.y, HL, (float)mm.x * H) : 0.f;
+        yv[i] = hy ? fmaf((float)mm.w, HL, (float)mm.z * H) : 0.f;
       }
       const float cd = (float)cfix * HL;
       cholesky_columns<N>(x, yv, in_group ? p : 64, first, fmaxf(cd, 1e-30f));
-      const bool conv = onesided_jacobi<N>(x, yv, p, lane);
+      const bool conv = onesided_jacobi<N>(x, yv, p, lane, FX_ORTHO2);
       {
         const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);
         const unsigned mine = ((1u << N) - 1u) << first;
@@ -361,26 +379,16 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
         for (int i = 0; i < NM; ++i) eo[i * NM + cy] = yv[i] * iy;
         eo[NM * NM + cy] = ay * back;
       }
-      // U, s; h_a = f_a / |f_a|^{3/2} one float off (a lane's two entries an aligned pair)
+      // U, s, and h_a = f_a / |f_a|^{3/2}
       if (hx) {
         sv[cx] = ax * ix;
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-          U[cx * LDF + i] = x[i] * ix;
-          F[cx * LDF + i + 1] = x[i] * jx;
-        }
+        store_floats<NM, LDF>(U + cx * LDF, x, ix);
+        store_floats<NM, LDF>(F + cx * LDF, x, jx);
       }
       if (hy) {
         sv[cy] = ay * iy;
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-          U[cy * LDF + i] = yv[i] * iy;
-          F[cy * LDF + i + 1] = yv[i] * jy;
-        }
-      }
-      if (in_group && p == 0) {
-#pragma unroll
-        for (int a = 0; a < NM; ++a) F[a * LDF] = 0.f;
+        store_floats<NM, LDF>(U + cy * LDF, yv, iy);
+        store_floats<NM, LDF>(F + cy * LDF, yv, jy);
       }
     }
     __syncwarp();
@@ -403,8 +411,8 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
       const float to = ldexpf(1.f, 29 - xe);
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
-        if (hx) Xs[cx * LDQ + i] = Limbs{__float2int_rn(x[i] * to), 0};
-        if (hy) Xs[cy * LDQ + i] = Limbs{__float2int_rn(yv[i] * to), 0};
+        const int4 v = make_int4(hx ? __float2int_rn(x[i] * to) : 0, 0, __float2int_rn(yv[i] * to), 0);
+        if (hy) *reinterpret_cast<int4*>(Xs + i * LDQ + 2 * p) = v;
       }
     }
     const float rscale = ldexpf(1.f, xe - 58), escale = ldexpf(1.f, 58 - xe);
@@ -413,158 +421,165 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
 #pragma unroll 1
     for (int it = 0;; ++it) {
       __syncwarp();
-      // R = I - X (M X), half of the entries, one of the lane's columns at a time
+      // R = I - X (M X), half of the entries
       float rmax = 0.f;
+      {
+        Limbs pa[NM], pb[NM];
+        {
+          // M X: M is symmetric, so row j of M times X_j,col adds to all rows of the column
+          i64 ha[NM], xa[NM], hb[NM], xb[NM];
+#pragma unroll
+          for (int r = 0; r < NM; ++r) ha[r] = xa[r] = hb[r] = xb[r] = 0;
 #pragma unroll 1
-      for (int c = 0; c < 2; ++c) {
-        const int col = c == 0 ? (hx ? cx : 0) : cy;
-        const bool has = c == 0 ? hx : hy;
-        Limbs xc[NM], pc[NM];
+          for (int j = 0; j < NM; ++j) {
+            const int4* row = reinterpret_cast<const int4*>(Ms + j * LDQ);
+            const int4 v = *reinterpret_cast<const int4*>(Xs + j * LDQ + 2 * p);
+            int mh[NM], ml[NM];
 #pragma unroll
-        for (int j = 0; j < NM; j += 2) {
-          const int4 v = reinterpret_cast<const int4*>(Xs + col * LDQ)[j / 2];
-          xc[j] = Limbs{v.x, v.y};
-          if (j + 1 < NM) xc[j + 1] = Limbs{v.z, v.w};
+            for (int r = 0; r < NM; ++r) {
+              const int4 w4 = row[(r + 1) / 2];
+              mh[r] = (r & 1) ? w4.x : w4.z;
+              ml[r] = (r & 1) ? w4.y : w4.w;
+            }
+            // in this order no multiply-add waits for the one before it
+#pragma unroll
+            for (int r = 0; r < NM; ++r) {
+              fx_mad(ha[r], mh[r], v.x);
+              fx_mad(hb[r], mh[r], v.z);
+            }
+#pragma unroll
+            for (int r = 0; r < NM; ++r) {
+              fx_mad(xa[r], mh[r], v.y);
+              fx_mad(xb[r], mh[r], v.w);
+            }
+#pragma unroll
+            for (int r = 0; r < NM; ++r) {
+              fx_mad(xa[r], ml[r], v.x);
+              fx_mad(xb[r], ml[r], v.z);
+            }
+          }
+          // to 2^-58 (|M X| <= 1)
+#pragma unroll
+          for (int r = 0; r < NM; ++r) {
+            pa[r] = fx_split((ha[r] << xe) + (xa[r] >> (29 - xe)));
+            pb[r] = fx_split((hb[r] << xe) + (xb[r] >> (29 - xe)));
+          }
         }
-#pragma unroll
-        for (int r = 0; r < NM; ++r) {
-          i64 hh = 0, xx = 0;
-          fx_dot<NM>(reinterpret_cast<const int4*>(Ms + r * LDQ), xc, hh, xx);
-          // M X to 2^-58 (|M X| <= 1)
-          pc[r] = fx_split((hh << xe) + (xx >> (29 - xe)));
-        }
-#pragma unroll
-        for (int o = 0; o < N; ++o) {
-          const int r = half_row(o + c);
-          i64 hh = 0, xx = 0;
-          fx_dot<NM>(reinterpret_cast<const int4*>(Xs + r * LDQ), pc, hh, xx);
-          const i64 one = r == col ? (1ll << 58) >> xe : 0;
-          const float rv = (float)(one - hh - ((xx + (1ll << 28)) >> 29)) * rscale;
-          if (has) {
-            rmax = fmaxf(rmax, fabsf(rv));
-            F[r * LDF + col] = rv;
-            F[col * LDF + r] = rv;
+        const i64 one = (1ll << 58) >> xe;
+#pragma unroll 1
+        for (int o = 0; o <= N; ++o) {
+          const int r = half_row(o);
+          i64 h0 = 0, x0 = 0, h1 = 0, x1 = 0;
+          fx_dot2<NM>(reinterpret_cast<const int4*>(Xs + r * LDQ), pa, pb, h0, x0, h1, x1);
+          const float r0 = (float)((r == cx ? one : 0) - h0 - ((x0 + (1ll << 28)) >> 29)) * rscale;
+          const float r1 = (float)((r == cy ? one : 0) - h1 - ((x1 + (1ll << 28)) >> 29)) * rscale;
+          if (hx && o < N) {
+            rmax = fmaxf(rmax, fabsf(r0));
+            F[r * LDF + cx + 1] = r0;
+            F[cx * LDF + r + 1] = r0;
+          }
+          if (hy && o > 0) {
+            rmax = fmaxf(rmax, fabsf(r1));
+            F[r * LDF + cy + 1] = r1;
+            F[cy * LDF + r + 1] = r1;
           }
         }
       }
       const bool more = __any_sync(0xffffffffu, live && rmax > small) && it + 1 < FX_MAX_IT;
       __syncwarp();
-      // U^T R: the lane's columns, over R
-      float rx[NM], ry[NM];
-#pragma unroll
-      for (int i = 0; i < NM; ++i) {
-        rx[i] = F[(hx ? cx : 0) * LDF + i];             // R is symmetric: column = row
-        ry[i] = F[cy * LDF + i];
-      }
+      // E = U [(U^T R U)_ab / (s_a + s_b)] U^T, row by row; R is symmetric (column = row)
+      float rx[LDF], ry[LDF];
+      load_floats<LDF>(F + (hx ? cx : 0) * LDF, rx);
+      load_floats<LDF>(F + cy * LDF, ry);
       __syncwarp();
 #pragma unroll 1
-      for (int a = 0; a < NM; ++a) {
+      for (int a = 0; a < NM; ++a) {                    // U^T R over R
         float row[LDF], sx = 0.f, sy = 0.f;
         load_floats<LDF>(U + a * LDF, row);
 #pragma unroll
-        for (int i = 0; i < NM; ++i) {
+        for (int i = 1; i <= NM; ++i) {
           sx = fmaf(row[i], rx[i], sx);
           sy = fmaf(row[i], ry[i], sy);
         }
-        if (hx) F[a * LDF + cx] = sx;
-        if (hy) F[a * LDF + cy] = sy;
+        if (hy) *reinterpret_cast<float2*>(F + a * LDF + 2 * p) = make_float2(sx, sy);
       }
       __syncwarp();
-      // (U^T R) U divided by s_a + s_b, row by row in place
-#pragma unroll
-      for (int i = 0; i < NM; ++i) {
-        rx[i] = U[(hx ? cx : 0) * LDF + i];
-        ry[i] = U[cy * LDF + i];
-      }
+      load_floats<LDF>(U + (hx ? cx : 0) * LDF, rx);
+      load_floats<LDF>(U + cy * LDF, ry);
       {
         const float s0 = sv[hx ? cx : 0], s1 = sv[cy];
 #pragma unroll 1
-        for (int a = 0; a < NM; ++a) {
+        for (int a = 0; a < NM; ++a) {                  // times U, divided, in place
           float row[LDF], sx = 0.f, sy = 0.f;
           load_floats<LDF>(F + a * LDF, row);
 #pragma unroll
-          for (int i = 0; i < NM; ++i) {
+          for (int i = 1; i <= NM; ++i) {
             sx = fmaf(row[i], rx[i], sx);
             sy = fmaf(row[i], ry[i], sy);
           }
           const float sa = sv[a];
           __syncwarp();
-          if (hx) F[a * LDF + cx] = sx * rcp_ftz(sa + s0);
-          if (hy) F[a * LDF + cy] = sy * rcp_ftz(sa + s1);
+          if (hy)
+            *reinterpret_cast<float2*>(F + a * LDF + 2 * p) = make_float2(sx * rcp_ftz(sa + s0), sy * rcp_ftz(sa + s1));
         }
       }
       __syncwarp();
-      // E = U (.) U^T: the lane's columns
-      float ex_[NM], ey_[NM];
+      {
+        float ea[NM], eb[NM];
 #pragma unroll
-      for (int i = 0; i < NM; ++i) {
-        rx[i] = U[i * LDF + (hx ? cx : 0)];
-        ry[i] = U[i * LDF + cy];
-        ex_[i] = ey_[i] = 0.f;
-      }
+        for (int i = 0; i < NM; ++i) {
+          const float2 v = *reinterpret_cast<const float2*>(U + i * LDF + 2 * p);
+          rx[i + 1] = v.x;
+          ry[i + 1] = v.y;
+          ea[i] = eb[i] = 0.f;
+        }
 #pragma unroll 1
-      for (int a = 0; a < NM; ++a) {
-        float row[LDF], sx = 0.f, sy = 0.f;
-        load_floats<LDF>(F + a * LDF, row);
+        for (int a = 0; a < NM; ++a) {
+          float row[LDF], sx = 0.f, sy = 0.f;
+          load_floats<LDF>(F + a * LDF, row);
 #pragma unroll
-        for (int i = 0; i < NM; ++i) {
-          sx = fmaf(row[i], rx[i], sx);
-          sy = fmaf(row[i], ry[i], sy);
-        }
-        load_floats<LDF>(U + a * LDF, row);
-#pragma unroll
-        for (int i = 0; i < NM; ++i) {
-          ex_[i] = fmaf(row[i], sx, ex_[i]);
-          ey_[i] = fmaf(row[i], sy, ey_[i]);
-        }
-      }
-      __syncwarp();
-      // X <- X + E on half of the entries (exactly symmetric)
-#pragma unroll
-      for (int i = 0; i < NM; ++i) {
-        if (hx) F[cx * LDF + i] = ex_[i];
-        if (hy) F[cy * LDF + i] = ey_[i];
-      }
-      __syncwarp();
-      i64 nx[N], ny[N];
-#pragma unroll
-      for (int o = 0; o < N; ++o) {
-        const int r0 = half_row(o), r1 = half_row(o + 1), c0 = hx ? cx : 0;
-        const Limbs a = Xs[c0 * LDQ + r0], b = Xs[cy * LDQ + r1];
-        nx[o] = ((i64)a.h << 29) + a.l + __float2ll_rn(F[c0 * LDF + r0] * escale);
-        ny[o] = ((i64)b.h << 29) + b.l + __float2ll_rn(F[cy * LDF + r1] * escale);
-      }
-      __syncwarp();
-      if (more) {
-#pragma unroll
-        for (int o = 0; o < N; ++o) {
-          const int r0 = half_row(o), r1 = half_row(o + 1);
-          const Limbs a = fx_split(nx[o]), b = fx_split(ny[o]);
-          if (hx) {
-            Xs[cx * LDQ + r0] = a;
-            Xs[r0 * LDQ + cx] = a;
+          for (int i = 1; i <= NM; ++i) {
+            sx = fmaf(row[i], rx[i], sx);
+            sy = fmaf(row[i], ry[i], sy);
           }
-          if (hy) {
-            Xs[cy * LDQ + r1] = b;
-            Xs[r1 * LDQ + cy] = b;
+          load_floats<LDF>(U + a * LDF, row);
+#pragma unroll
+          for (int i = 0; i < NM; ++i) {
+            ea[i] = fmaf(row[i + 1], sx, ea[i]);
+            eb[i] = fmaf(row[i + 1], sy, eb[i]);
           }
         }
-        continue;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < NM; ++i)
+          if (hy) *reinterpret_cast<float2*>(F + i * LDF + 2 * p) = make_float2(ea[i], eb[i]);
       }
-      // packed upper triangle through shared memory (over M)
-      double* op = reinterpret_cast<double*>(base + Lt::OUTP);
+      __syncwarp();
+      // X <- X + E on half of the entries, both triangles written (a pair (r, c) is one lane's)
       const int e2 = xe - 58 - ex;
-#pragma unroll
-      for (int o = 0; o < N; ++o) {
-        const int r0 = half_row(o), r1 = half_row(o + 1);
-        if (hx) op[packed_index(min(r0, cx), max(r0, cx), NM)] = finite ? fx_to_double(nx[o], e2) : __longlong_as_double(0x7ff8000000000000ll);
-        if (hy) op[packed_index(min(r1, cy), max(r1, cy), NM)] = finite ? fx_to_double(ny[o], e2) : __longlong_as_double(0x7ff8000000000000ll);
+      double* op = reinterpret_cast<double*>(base + Lt::OUTP);
+#pragma unroll 1
+      for (int o = 0; o <= N; ++o) {
+        const int r = half_row(o);
+        const int4 v = *reinterpret_cast<const int4*>(Xs + r * LDQ + 2 * p);
+        const float2 ev = *reinterpret_cast<const float2*>(F + r * LDF + 2 * p);
+        const i64 n0 = ((i64)v.x << 29) + v.y + __float2ll_rn(ev.x * escale);
+        const i64 n1 = ((i64)v.z << 29) + v.w + __float2ll_rn(ev.y * escale);
+        if (more) {
+          if (hx && o < N) Xs[r * LDQ + cx + 1] = Xs[cx * LDQ + r + 1] = fx_split(n0);
+          if (hy && o > 0) Xs[r * LDQ + cy + 1] = Xs[cy * LDQ + r + 1] = fx_split(n1);
+        } else {
+          // packed upper triangle through shared memory (over M)
+          const double bad = __longlong_as_double(0x7ff8000000000000ll);
+          if (hx && o < N) op[packed_index(min(r, cx), max(r, cx), NM)] = finite ? fx_to_double(n0, e2) : bad;
+          if (hy && o > 0) op[packed_index(min(r, cy), max(r, cy), NM)] = finite ? fx_to_double(n1, e2) : bad;
+        }
       }
-      if (in_group && p == 0) {
+      if (!more) break;
+    }
+    if (in_group && p == 0) {
 #pragma unroll
-        for (int t = NT; t < NTP; ++t) op[t] = 0.0;
-      }
-      break;
+      for (int t = NT; t < NTP; ++t) reinterpret_cast<double*>(base + Lt::OUTP)[t] = 0.0;
     }
     __syncwarp();
     if (live) {
