@@ -70,7 +70,15 @@ struct LinState {
   T* tau = nullptr;     // [E][4][NT_PAD]
   T* t0 = nullptr;      // [E][4][3][C] tau L at the state
   T* dft = nullptr;     // forward [K][C] then inverse [C][K]
-  float2* udd = nullptr;   // [V][4][C] u0 as double-float pairs (FP64 state only)
+  // operands of the one-launch element operator (element.cuh); for T = double the
+  // values are double-float pairs of the same size
+  T* trig = nullptr;    // cos, sin of 2 pi n k / K: [2][N][K/2 + 1]
+  T* uc = nullptr;      // [V][4][C] u0 without Im(mode 0)
+  T* us = nullptr;      // [V][3][K] its velocity on samples
+  T* vc = nullptr;      // the same of a product's operand
+  T* vs = nullptr;
+  T* rows = nullptr;    // [E][4][4][C] element rows
+  bool prepared = false;   // uc, us belong to u0
   T* u0t = nullptr;     // [V][K][4] u0 velocity sampled in time (FP32 fast path)
   T* vt = nullptr;      // [V][K][4] scratch of the FP32 fast path: the product's input sampled
   T* bneg = nullptr;    // [backflow points][NT_PAD] |A_n|_- (section 2.6)
@@ -207,7 +215,6 @@ static int lin_alloc(ts_problem* pr, LinState<T>& l) {
   std::vector<T> tt(tab.begin(), tab.end());
   TS_TRY(dalloc(&l.dft, tt.size()));
   TS_CUDA(cudaMemcpy(l.dft, tt.data(), tt.size() * sizeof(T), cudaMemcpyHostToDevice));
-  if (sizeof(T) == 8) TS_TRY(dalloc(&l.udd, (size_t)field_len(pr)));
   if (sizeof(T) == 4) {
     TS_TRY(dalloc(&l.u0t, (size_t)m->V * 4 * pr->K));
     TS_TRY(dalloc(&l.vt, (size_t)m->V * 4 * pr->K));
@@ -233,7 +240,13 @@ static void lin_free(LinState<T>& l) {
   dfree(l.t0);
   dfree(l.dft);
   dfree(l.u0t);
-  dfree(l.udd);
+  dfree(l.trig);
+  dfree(l.uc);
+  dfree(l.us);
+  dfree(l.vc);
+  dfree(l.vs);
+  dfree(l.rows);
+  l.prepared = false;
   dfree(l.vt);
   dfree(l.bneg);
   dfree(l.l0);
@@ -282,6 +295,107 @@ static Phys<T> phys_of(const ts_problem* pr, bool with_mass) {
   return ph;
 }
 
+// resistance outlets: the terms of v added to out
+template <typename T>
+static int outlet_terms(ts_problem* pr, const T* v, int mask_input, T* out, cudaStream_t st) {
+  for (auto& o : pr->outlets)
+    if (launch_outlet<T>(o.d_nodes, outlet_w<T>(o), (int)o.nodes.size(), (T)o.R, v, pr->d_dmask, mask_input, out,
+                         pr->C, st))
+      return fail(TS_ERR_CUDA, "outlet kernel launch failed");
+  return 0;
+}
+
+// ---- the one-launch element operator
+template <typename T>
+struct PairOf;
+template <>
+struct PairOf<float> {
+  using V = float;
+  static V of(double x) { return (float)x; }
+};
+template <>
+struct PairOf<double> {
+  using V = float2;
+  static V of(double x) {
+    const float h = (float)x;
+    return make_float2(h, (float)(x - (double)h));
+  }
+};
+
+// cos, sin of 2 pi n k / K, k = 0..K/2
+template <typename T>
+static int upload_trig(int N, T** out) {
+  using PV = PairOf<T>;
+  const int K = 3 * N - 2, KH = K / 2, n1 = N * (KH + 1);
+  const double pi = 3.14159265358979323846;
+  std::vector<typename PV::V> t(2 * n1);
+  for (int n = 0; n < N; ++n)
+    for (int k = 0; k <= KH; ++k) {
+      const double th = 2.0 * pi * ((n * k) % K) / K;
+      t[n * (KH + 1) + k] = PV::of(std::cos(th));
+      t[n1 + n * (KH + 1) + k] = PV::of(std::sin(th));
+    }
+  TS_TRY(dalloc(out, t.size()));
+  TS_CUDA(cudaMemcpy(*out, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice));
+  return 0;
+}
+
+// the state's operands (uc, us) from y
+template <typename T, int N>
+static int prepare_state(ts_problem* pr, LinState<T>& l, const T* y, cudaStream_t st) {
+  using V = typename PairOf<T>::V;
+  static_assert(sizeof(V) == sizeof(T), "pairs are stored in place of FP64 values");
+  const ts_mesh* m = pr->mesh;
+  if (!l.trig) TS_TRY(upload_trig<T>(N, &l.trig));
+  if (!l.uc) TS_TRY(dalloc(&l.uc, (size_t)field_len(pr)));
+  if (!l.us) TS_TRY(dalloc(&l.us, (size_t)m->V * 3 * pr->K));
+  if (launch_node_prepass<V, N>(y, nullptr, (V*)l.uc, (V*)l.us, (const V*)l.trig, m->V, st))
+    return fail(TS_ERR_CUDA, "node pre-pass launch failed");
+  l.prepared = true;
+  return 0;
+}
+
+// out = the element operator on v (the state itself for the residual)
+template <typename T, int N>
+static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T* out, bool with_mass,
+                         cudaStream_t st, T* l0 = nullptr) {
+  using PV = PairOf<T>;
+  using V = typename PV::V;
+  const ts_mesh* m = pr->mesh;
+  if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
+  const bool res = mode == MODE_RESIDUAL;
+  if (!res) {
+    if (!l.vc) TS_TRY(dalloc(&l.vc, (size_t)field_len(pr)));
+    if (!l.vs) TS_TRY(dalloc(&l.vs, (size_t)m->V * 3 * pr->K));
+    if (launch_node_prepass<V, N>(v, pr->d_dmask, (V*)l.vc, (V*)l.vs, (const V*)l.trig, m->V, st))
+      return fail(TS_ERR_CUDA, "node pre-pass launch failed");
+  }
+  if (!l.rows) TS_TRY(dalloc(&l.rows, (size_t)m->E * 16 * pr->C));
+  const Phys<double> ph = phys_of<double>(pr, with_mass);
+  ElementArgs<V> a;
+  a.tets = m->d_tets;
+  a.geo = geo_of<T>(m);
+  a.u0t = (const V*)l.us;
+  a.vt = (const V*)(res ? l.us : l.vs);
+  a.ud = (const V*)l.uc;
+  a.vd = (const V*)(res ? l.uc : l.vc);
+  a.tau = l.tau;
+  a.t0 = l.t0;
+  a.l0 = l0;
+  a.trig = (const V*)l.trig;
+  a.rows = (V*)l.rows;
+  a.rho = PV::of(ph.rho);
+  a.irho = PV::of(1.0 / ph.rho);
+  a.mu4 = PV::of(4.0 * ph.mu);
+  a.mass5 = PV::of(0.2 * ph.mass_coef);
+  a.omega = PV::of(ph.omega);
+  a.n_elem = m->E;
+  if (launch_element<V, N>(mode, a, st)) return fail(TS_ERR_CUDA, "element kernel launch failed");
+  if (launch_gather<V>(m->d_node_off, m->d_node_elem, (const V*)l.rows, pr->d_dmask, out, m->V, pr->C, st))
+    return fail(TS_ERR_CUDA, "gather kernel launch failed");
+  return outlet_terms<T>(pr, v, res ? 0 : 1, out, st);
+}
+
 // dispatch on the compiled mode counts
 template <typename T, int N>
 static int apply_colours(ts_problem* pr, int mode, const T* v, const T* u0, LinState<T>& l,
@@ -289,29 +403,11 @@ static int apply_colours(ts_problem* pr, int mode, const T* v, const T* u0, LinS
   const ts_mesh* m = pr->mesh;
   Phys<T> ph = phys_of<T>(pr, with_mass);
   for (size_t c = 0; c + 1 < m->colour_off.size(); ++c) {
-    int rc;
-    if constexpr (sizeof(T) == 8) {
-      if (pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT)
-        rc = launch_apply_dd<N>(mode, m->d_tets, m->d_geo64, (const double*)v, (const double*)u0,
-                                (const double*)l.tau, (double*)l.t0, pr->d_dmask, (double*)out,
-                                (const double*)l.dft, phys_of<double>(pr, with_mass), m->colour_off[c],
-                                m->colour_off[c + 1], st, (double*)l0);
-      else
-        rc = launch_apply<T, N>(mode, m->d_tets, geo_of<T>(m), v, u0, l.tau, l.t0, pr->d_dmask,
-                                out, l.dft, ph, m->colour_off[c], m->colour_off[c + 1], st, l0);
-    } else {
-      rc = launch_apply<T, N>(mode, m->d_tets, geo_of<T>(m), v, u0, l.tau, l.t0, pr->d_dmask,
-                              out, l.dft, ph, m->colour_off[c], m->colour_off[c + 1], st, l0);
-    }
+    const int rc = launch_apply<T, N>(mode, m->d_tets, geo_of<T>(m), v, u0, l.tau, l.t0, pr->d_dmask, out, l.dft, ph,
+                                      m->colour_off[c], m->colour_off[c + 1], st, l0);
     if (rc) return fail(rc == -6 ? TS_ERR_UNSUPPORTED : TS_ERR_CUDA, "element kernel launch failed");
   }
-  const bool mask_input = mode != MODE_RESIDUAL;
-  for (auto& o : pr->outlets) {
-    int rc = launch_outlet<T>(o.d_nodes, outlet_w<T>(o), (int)o.nodes.size(), (T)o.R, v,
-                              pr->d_dmask, mask_input ? 1 : 0, out, pr->C, st);
-    if (rc) return fail(TS_ERR_CUDA, "outlet kernel launch failed");
-  }
-  return 0;
+  return outlet_terms<T>(pr, v, mode != MODE_RESIDUAL ? 1 : 0, out, st);
 }
 
 template <typename T>
@@ -368,17 +464,19 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
     if (!l.l0) TS_TRY(dalloc(&l.l0, (size_t)m->E * 12 * pr->C));
     eig = pr->d_eig;
   }
+  l.prepared = false;
+  // FP32, and FP64 in double-float: one element launch; native FP64: colours
+  const bool one_launch = sizeof(T) == 4 || pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT;
+  if (one_launch || (sizeof(T) == 8 && pr->tau64 == TS_TAU64_DOUBLEFLOAT)) TS_TRY((prepare_state<T, N>(pr, l, y, st)));
   TS_CUDA(cudaEventRecord(pr->sev[0], st));
   int rc;
   if constexpr (sizeof(T) == 8) {
     if (pr->tau64 == TS_TAU64_JACOBI)
       rc = launch_tau<T, N>(m->d_tets, geo_of<T>(m), y, m->E, l.tau, (T)(pr->p.mu / pr->p.rho),
                             (T)pr->p.C_I, pr->d_counter, st, eig);
-    else if (pr->tau64 == TS_TAU64_DOUBLEFLOAT) {
-      if (launch_split_dd((const double*)y, l.udd, n, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
-      rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, l.udd, m->E, (double*)l.tau, pr->p.mu / pr->p.rho, pr->p.C_I,
-                            pr->d_counter, st, eig);
-    }
+    else if (pr->tau64 == TS_TAU64_DOUBLEFLOAT)
+      rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, (const float2*)l.uc, m->E, (double*)l.tau, pr->p.mu / pr->p.rho,
+                            pr->p.C_I, pr->d_counter, st, eig);
     else
       rc = launch_tau_polish<N>(m->d_tets, m->d_geo64, (const double*)y, m->E, (double*)l.tau,
                                 pr->p.mu / pr->p.rho, pr->p.C_I, pr->d_counter, st, eig);
@@ -388,8 +486,12 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
   }
   if (rc) return fail(TS_ERR_CUDA, "tau kernel launch failed");
   TS_CUDA(cudaEventRecord(pr->sev[1], st));
-  TS_CUDA(cudaMemsetAsync(r, 0, n * sizeof(T), st));
-  TS_TRY(apply_colours<T, N>(pr, MODE_RESIDUAL, y, y, l, r, false, st, exact ? l.l0 : nullptr));
+  if (one_launch) {
+    TS_TRY((element_apply<T, N>(pr, MODE_RESIDUAL, l, y, r, false, st, exact ? l.l0 : nullptr)));
+  } else {
+    TS_CUDA(cudaMemsetAsync(r, 0, n * sizeof(T), st));
+    TS_TRY(apply_colours<T, N>(pr, MODE_RESIDUAL, y, y, l, r, false, st, exact ? l.l0 : nullptr));
+  }
   TS_CUDA(cudaEventRecord(pr->sev[2], st));
   pr->sev_res = true;
   TS_TRY(bneg_alloc(pr, l));
@@ -411,6 +513,7 @@ template <typename D, typename S, int N>
 static int convert_lin(ts_problem* pr, LinState<D>& dst, LinState<S>& src, cudaStream_t st) {
   TS_TRY(lin_alloc(pr, dst));
   const ts_mesh* m = pr->mesh;
+  dst.prepared = false;
   const int64_t n_u = field_len(pr), n_tau = m->E * 4 * pr->NTP, n_t0 = m->E * 12 * pr->C;
   int rc = 0;
   dst.exact_valid = src.exact_valid && src.l0;
@@ -486,10 +589,11 @@ static int jvp_impl(ts_problem* pr, const T* v, T* hv, cudaStream_t st) {
     int rc = launch_jvp32<N>(mode, I, st, pr->sev[3], pr->sev[4]);
     if (rc) return fail(TS_ERR_CUDA, "FP32 tangent kernel launch failed");
     pr->sev_jvp = true;
-    for (auto& o : pr->outlets)
-      if (launch_outlet<T>(o.d_nodes, outlet_w<T>(o), (int)o.nodes.size(), (T)o.R, v, pr->d_dmask, 1,
-                           hv, pr->C, st))
-        return fail(TS_ERR_CUDA, "outlet kernel launch failed");
+    TS_TRY(outlet_terms<T>(pr, v, 1, hv, st));
+    return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
+  }
+  if (sizeof(T) == 4 ? pr->fast32 : pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) {
+    TS_TRY((element_apply<T, N>(pr, mode, l, v, hv, true, st)));
     return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
   }
   TS_CUDA(cudaMemsetAsync(hv, 0, field_len(pr) * sizeof(T), st));
@@ -549,10 +653,7 @@ static int j32_inst_impl(ts_problem* pr, J32Inst* I, cudaStream_t st) {
 
 template <int N>
 static int j32_boundary_impl(ts_problem* pr, const float* v, float* hv, cudaStream_t st) {
-  for (auto& o : pr->outlets)
-    if (launch_outlet<float>(o.d_nodes, outlet_w<float>(o), (int)o.nodes.size(), (float)o.R, v,
-                             pr->d_dmask, 1, hv, pr->C, st))
-      return fail(TS_ERR_CUDA, "outlet kernel launch failed");
+  TS_TRY(outlet_terms<float>(pr, v, 1, hv, st));
   return backflow_terms<float, N>(pr, pr->l32, v, false, 1, hv, st);
 }
 
@@ -665,11 +766,7 @@ static int spmv_impl(ts_problem* pr, const float* v, float* hv, cudaStream_t st)
   const ts_mesh* m = pr->mesh;
   int rc = launch_spmv_paper<N>(m->d_row_off, m->d_cols, pr->d_hasm, pr->d_dmask, v, hv, m->V, st);
   if (rc) return fail(rc == -6 ? TS_ERR_UNSUPPORTED : TS_ERR_CUDA, "assembled product kernel launch failed");
-  for (auto& o : pr->outlets)
-    if (launch_outlet<float>(o.d_nodes, outlet_w<float>(o), (int)o.nodes.size(), (float)o.R, v, pr->d_dmask, 1,
-                             hv, pr->C, st))
-      return fail(TS_ERR_CUDA, "outlet kernel launch failed");
-  return 0;
+  return outlet_terms<float>(pr, v, 1, hv, st);
 }
 
 static int spmv_any(ts_problem* pr, const float* v, float* hv, cudaStream_t st) {

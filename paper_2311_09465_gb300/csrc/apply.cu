@@ -382,9 +382,6 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// warps (elements in flight) per block of the double-float element operator
-constexpr int APPLY_DD_WARPS = 4;
-
 template <typename T, int N, int MODE, typename S = T>
 static int launch_mode(const int4* tets, const S* geo, const S* v, const S* u0, const S* tau,
                        S* t0cache, const uint8_t* dmask, S* out, const S* dft, Phys<T> ph,
@@ -392,7 +389,7 @@ static int launch_mode(const int4* tets, const S* geo, const S* v, const S* u0, 
   using L = ApplyLayout<N, MODE>;
   static_assert(sizeof(T) == sizeof(S) || sizeof(T) == 8, "workspace sized by T");
   if (e1 <= e0) return 0;
-  int warps = std::is_same<T, ddv>::value ? APPLY_DD_WARPS : 4;
+  int warps = 4;
   while (warps > 1 && (size_t)(L::TABLES + warps * L::WARP) * sizeof(T) > 200 * 1024) --warps;
   const size_t smem = (size_t)(L::TABLES + warps * L::WARP) * sizeof(T);
   if (smem > 227 * 1024) return -6;
@@ -439,29 +436,6 @@ int launch_apply(int mode, const int4* tets, const T* geo, const T* v, const T* 
     case MODE_JVP_LIN_A:
       return launch_mode<T, N, MODE_JVP_LIN_A>(tets, geo, v, u0, tau, t0cache, dmask, out, dft,
                                                ph, e0, e1, st);
-  }
-  return -1;
-}
-
-// The FP64 operator with its arithmetic in double-float (FP64 storage)
-template <int N>
-int launch_apply_dd(int mode, const int4* tets, const double* geo, const double* v, const double* u0,
-                    const double* tau, double* t0cache, const uint8_t* dmask, double* out, const double* dft,
-                    Phys<double> p, int64_t e0, int64_t e1, cudaStream_t st, double* l0cache) {
-  Phys<ddv> ph{ddv(p.rho), ddv(p.mu), ddv(p.omega), ddv(p.nu), ddv(p.C_I), ddv(p.mass_coef)};
-  switch (mode) {
-    case MODE_RESIDUAL:
-      return launch_mode<ddv, N, MODE_RESIDUAL, double>(tets, geo, v, u0, tau, t0cache, dmask, out, dft,
-                                                        ph, e0, e1, st, l0cache);
-    case MODE_JVP_PAPER:
-      return launch_mode<ddv, N, MODE_JVP_PAPER, double>(tets, geo, v, u0, tau, t0cache, dmask, out, dft,
-                                                         ph, e0, e1, st);
-    case MODE_JVP_FROZEN:
-      return launch_mode<ddv, N, MODE_JVP_FROZEN, double>(tets, geo, v, u0, tau, t0cache, dmask, out, dft,
-                                                          ph, e0, e1, st);
-    case MODE_JVP_LIN_A:
-      return launch_mode<ddv, N, MODE_JVP_LIN_A, double>(tets, geo, v, u0, tau, t0cache, dmask, out, dft,
-                                                         ph, e0, e1, st);
   }
   return -1;
 }
@@ -813,11 +787,6 @@ TS_FOR_EACH_N(TS_INST_APPLY, float)
 #define TS_INST_PRELOAD_APPLY(T, N) template int preload_apply_residual<T, N>();
 TS_FOR_EACH_N(TS_INST_PRELOAD_APPLY, float)
 TS_FOR_EACH_N(TS_INST_APPLY, double)
-#define TS_INST_APPLY_DD(T, N)                                                                         \
-  template int launch_apply_dd<N>(int, const int4*, const double*, const double*, const double*,      \
-                                  const double*, double*, const uint8_t*, double*, const double*,     \
-                                  Phys<double>, int64_t, int64_t, cudaStream_t, double*);
-TS_FOR_EACH_N(TS_INST_APPLY_DD, double)
 #define TS_INST_TRACER(T, N)                                                                        \
   template int launch_tracer<T, N>(const int4*, const T*, const T*, const T*, const T*, const uint8_t*, \
                                    T*, const T*, double, double, int64_t, int64_t, cudaStream_t, int);

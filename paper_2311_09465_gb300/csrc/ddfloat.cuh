@@ -23,6 +23,24 @@ __device__ __forceinline__ dd dd_from_double(double x) {
   return {h, (float)(x - (double)h)};
 }
 
+// The same without the FP64 pipe (each of its instructions costs as much issue
+// time as dozens of integer ones): hi is x rounded to 24 bits (ties away from
+// zero), lo the signed remainder of 28 bits rounded to FP32.  |x| below 2^-126
+// gives 0; infinities and NaN pass through.
+__device__ __forceinline__ dd dd_split(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  const int e = (int)(b >> 52) & 0x7ff;                       // biased exponent
+  if (e < 897) return {0.f, 0.f};
+  if (e > 1149)                                               // FP32 overflow, infinity, NaN
+    return {e == 0x7ff && (b << 12) ? __int_as_float(0x7fffffff) : __int_as_float((int)(sign | 0x7f800000u)), 0.f};
+  // exponent e - 896, 23 bits of the mantissa; a carry moves into the exponent
+  const unsigned h = (unsigned)((b + 0x10000000ull) >> 29) - 0xc0000000u;
+  const int rem = (int)((unsigned)b << 3) >> 3;               // x - hi in units of 2^(e - 1075)
+  const float unit = __int_as_float((int)(sign | ((unsigned)(e - 896) << 23)));   // 2^(e - 1023)
+  return {__int_as_float((int)(h | sign)), ((float)rem * 2.220446049250313e-16f) * unit};
+}
+
 __device__ __forceinline__ double dd_to_double(dd a) { return (double)a.hi + (double)a.lo; }
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {

@@ -61,12 +61,47 @@ int launch_apply(int mode, const int4* tets, const T* geo, const T* v, const T* 
 template <typename T>
 int launch_inlet_fill(const int32_t* nodes, const double* vals, int64_t n, int C, T* y, cudaStream_t st);
 
-// The same element operator on FP64 data with double-float arithmetic
-// (FP32-pipe pairs, ~48 significant bits; see ddfloat.cuh)
-template <int N>
-int launch_apply_dd(int mode, const int4* tets, const double* geo, const double* v, const double* u0,
-                    const double* tau, double* t0cache, const uint8_t* dmask, double* out, const double* dft,
-                    Phys<double> ph, int64_t e0, int64_t e1, cudaStream_t st, double* l0cache = nullptr);
+// The same element operator in one launch (element.cuh).  V: the arithmetic's
+// value type, float or float2 = double-float pair; S: the caller's type
+template <typename V>
+struct StoreOf;
+template <>
+struct StoreOf<float> {
+  using S = float;
+};
+template <>
+struct StoreOf<float2> {
+  using S = double;
+};
+
+template <typename V>
+struct ElementArgs {
+  using S = typename StoreOf<V>::S;
+  const int4* tets;
+  const S* geo;
+  const V* u0t;      // [V][3][K] linearisation velocity on samples
+  const V* vt;       // [V][3][K] the operand's
+  const V* ud;       // [V][4][C] linearisation state
+  const V* vd;       // [V][4][C] the operand without fixed entries
+  const S* tau;
+  S* t0;             // [E][4][3][C] tau L (written by the residual, read by LIN_A)
+  S* l0;             // [E][4][3][C] L (residual, exact tangent only) or null
+  const V* trig;     // cos, sin of 2 pi n k / K: [2][N][KH + 1]
+  V* rows;           // [E][4][4][C]
+  V rho, irho, mu4, mass5, omega;   // rho, 1/rho, 4 mu, mass coefficient / 5, omega
+  int64_t n_elem;
+};
+
+template <typename V, int N>
+int launch_element(int mode, const ElementArgs<V>& P, cudaStream_t st);
+// clean = y without fixed entries (dmask null: all velocities kept), samples of its velocity
+template <typename V, int N>
+int launch_node_prepass(const typename StoreOf<V>::S* y, const uint8_t* dmask, V* clean, V* samples, const V* trig,
+                        int64_t n_nodes, cudaStream_t st);
+// out = per node the sum of its element rows
+template <typename V>
+int launch_gather(const int32_t* node_off, const int32_t* node_elem, const V* rows, const uint8_t* dmask,
+                  typename StoreOf<V>::S* out, int64_t n_nodes, int C, cudaStream_t st);
 
 // Tracer residual of eq. (3D-weak) on one colour range [e0, e1) (apply.cu):
 // phi [V][C], a4 the advecting velocity in the flow layout [V][4][C], tau the
