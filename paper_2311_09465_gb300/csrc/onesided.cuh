@@ -52,35 +52,88 @@ __device__ __forceinline__ void rotation_of(float ax, float ay, float g, float& 
   ta = s * rcp_ftz(1.f + c);
 }
 
-// Cholesky factor of the group's matrix in place: on entry x, y hold the full
-// columns 2p-1 and 2p, on return the columns of L (zeros above the diagonal).
-// base: the group's first lane.  floor: a lower bound of the eigenvalues, hence
-// of the exact pivots; rounding may take a computed pivot below it.
-template <int N>
-__device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, int base,
-                                                 float floor) {
+// Cholesky factor of the group's matrix: on entry x, y hold the full columns 2p-1
+// and 2p, on return the columns of L (zeros above the diagonal).  rows: scratch
+// of NM rows of LD floats (16-byte aligned, LD a multiple of 4 and >= NM), of
+// which a lane uses its own two.  base: the group's first lane; own: whether the
+// lane belongs to a group.  floor: a lower bound of the eigenvalues, hence of the
+// exact pivots; rounding may take a computed pivot below it.
+// ROLLED: a loop over pivots in which the registers move up one row a step, so
+// that the pivot is always at index 0, and finished columns go through shared
+// memory.  Unrolled it needs no memory and half the shuffles, but is up to a
+// quarter of a kernel's code: rolled where that no longer fits the instruction
+// cache (fixed-point tau, N = 10: 34.5 ms unrolled, 8.0 rolled; N = 7: 10.8 and
+// 10.7; N = 5: 3.6 and 3.7; FP32 tau, N = 10: 2.42 and 2.16, N = 7: 2.60 and 2.99).
+template <int N, int LD, bool ROLLED>
+__device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, bool own, int base,
+                                                 float floor, float* rows) {
   constexpr int NM = 2 * N - 1;
+  if constexpr (!ROLLED) {
+    // a lane outside a group must stay zero: no column of it is a pivot
+    const int jx = own ? 2 * p - 1 : 4 * N, jy = own ? 2 * p : 4 * N;
 #pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      const int src = base + (k + 1) / 2;
+      float l[NM];
+#pragma unroll
+      for (int i = k; i < NM; ++i) l[i] = __shfl_sync(0xffffffffu, (k & 1) ? x[i] : y[i], src);
+      const float piv = fmaxf(l[k], floor), rd = rsqrt_newton(piv);
+      const float mx = jx > k ? x[k] * rd * rd : 0.f, my = jy > k ? y[k] * rd * rd : 0.f;
+#pragma unroll
+      for (int i = k + 1; i < NM; ++i) {
+        const float sx = fmaf(-l[i], mx, x[i]), sy = fmaf(-l[i], my, y[i]);
+        x[i] = jx == k ? l[i] * rd : sx;
+        y[i] = jy == k ? l[i] * rd : sy;
+      }
+      if (jx >= k) x[k] = jx == k ? piv * rd : 0.f;
+      if (jy >= k) y[k] = jy == k ? piv * rd : 0.f;
+    }
+    return;
+  }
+  float* rx = rows + (own && p > 0 ? 2 * p - 1 : 0) * LD;
+  float* ry = rows + 2 * p * LD;
+  if (own) {
+#pragma unroll
+    for (int i = 0; i < (NM + 3) / 4; ++i) {
+      if (p > 0) reinterpret_cast<float4*>(rx)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      reinterpret_cast<float4*>(ry)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+#pragma unroll 1
   for (int k = 0; k < NM; ++k) {
     const int src = base + (k + 1) / 2;
+    const bool odd = k & 1;
     float l[NM];
 #pragma unroll
-    for (int i = k; i < NM; ++i) l[i] = __shfl_sync(0xffffffffu, (k & 1) ? x[i] : y[i], src);
-    const float rd = rsqrt_newton(fmaxf(l[k], floor));
-    // the pivot column itself becomes l; a column j > k loses l l_j, l_j = rd A_jk
-    const int jx = 2 * p - 1, jy = 2 * p;
-    const float mx = jx > k ? x[k] * rd * rd : 0.f;
-    const float my = jy > k ? y[k] * rd * rd : 0.f;
-    const bool ox = jx == k, oy = jy == k;
+    for (int i = 0; i < NM; ++i) l[i] = __shfl_sync(0xffffffffu, odd ? x[i] : y[i], src);
+    const float rd = rsqrt_newton(fmaxf(l[0], floor));
+    l[0] = fmaxf(l[0], floor);
+    if (own && p == (k + 1) / 2) {
+      float* dst = (odd ? rx : ry) + k;
 #pragma unroll
-    for (int i = k + 1; i < NM; ++i) {
-      const float sx = fmaf(-l[i], mx, x[i]), sy = fmaf(-l[i], my, y[i]);
-      x[i] = ox ? l[i] * rd : sx;
-      y[i] = oy ? l[i] * rd : sy;
+      for (int i = 0; i < NM; ++i)
+        if (i < NM - k) dst[i] = l[i] * rd;
     }
-    const float dk = fmaxf(l[k], floor) * rd;
-    if (jx >= k) x[k] = ox ? dk : 0.f;
-    if (jy >= k) y[k] = oy ? dk : 0.f;
+    // a column j > k loses l l_j, l_j = rd A_jk
+    const float mx = 2 * p - 1 > k ? x[0] * rd * rd : 0.f;
+    const float my = 2 * p > k ? y[0] * rd * rd : 0.f;
+#pragma unroll
+    for (int i = 0; i + 1 < NM; ++i) {
+      x[i] = fmaf(-l[i + 1], mx, x[i + 1]);
+      y[i] = fmaf(-l[i + 1], my, y[i + 1]);
+    }
+    x[NM - 1] = y[NM - 1] = 0.f;
+  }
+#pragma unroll
+  for (int j = 0; j < (NM + 3) / 4; ++j) {
+    const float4 a = reinterpret_cast<const float4*>(rx)[j], b = reinterpret_cast<const float4*>(ry)[j];
+    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (4 * j + t < NM) {
+        x[4 * j + t] = own && p > 0 ? av[t] : 0.f;
+        y[4 * j + t] = own ? bv[t] : 0.f;
+      }
   }
 }
 

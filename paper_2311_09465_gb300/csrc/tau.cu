@@ -335,7 +335,9 @@ __global__ void __launch_bounds__(128) tau32_kernel(const int4* __restrict__ tet
       if (p == 0 || !in_group) x[i] = 0.f;
       if (!in_group) yy[i] = 0.f;
     }
-    cholesky_columns<N>(x, yy, in_group ? p : 64, g * N, fmaxf(cd, 1e-30f));
+    __syncwarp();                       // all lanes have read C_m
+    cholesky_columns<N, LDC, (N > 7)>(x, yy, p, in_group, in_group ? g * N : 0, fmaxf(cd, 1e-30f), cm);
+    __syncwarp();
     const bool conv = onesided_jacobi<N>(x, yy, p, lane, 1e-8f);
     {
       const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);

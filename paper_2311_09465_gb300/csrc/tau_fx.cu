@@ -13,14 +13,15 @@
 // number) take more corrections, up to FX_MAX_IT.
 //
 // Fixed point: a value v, |v| <= 1, is the integer V = v 2^58, split into two
-// 29-bit signed limbs V = 2^29 h + l, |l| <= 2^28.  A dot product of length
-// n <= 29 sums h h' in one 64-bit accumulator and h l' + l h' in another (no
-// overflow: 29 * 2^58 and 58 * 2^57 stay below 2^63), exactly; l l' (below
-// 2^-58 of the largest term) is left out.  That is three 32 x 32 -> 64 bit
-// multiply-adds a term against 12 to 15 FP32 instructions for a double-float
-// term, and GB300 issues them at half the FP32 rate: 6 issue slots against 12
-// to 15, with an absolute error near 2^-57 instead of 2^-47.  In R the scale of
-// X enters twice, so R is known to about cond(M) 2^-57.
+// signed limbs V = 2^29 h + l, |h| <= 2^29, |l| <= 2^28, l kept as FP32 (24 bits:
+// v is then good to 2^-54).  A dot product of length n <= 29 sums h h' exactly in
+// a 64-bit integer (29 * 2^58 < 2^63) and the mixed products h l' + l h', 2^29
+// smaller, in FP32; l l' is left out.  A term is one 32 x 32 -> 64 bit multiply-add
+// (4.8 issue cycles of an SM sub-partition, measured with all operands in vector
+// registers) and two FP32 ones, about 7 cycles against 12 to 15 for a double-float
+// term, with an absolute error near 2^-53 instead of 2^-47.  With the mixed
+// products in a second 64-bit accumulator it was 14 cycles.  In R the scale of X
+// enters twice, so R is known to about cond(M) 2^-53.
 //
 // Mapping: as tau32_kernel (tau.cu), a group of N lanes owns a point and lane p
 // the columns 2p-1 and 2p of every matrix.  A product reads the left matrix
@@ -51,13 +52,26 @@ __device__ __forceinline__ void fx_mad(i64& acc, int a, int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 }
 
-struct Limbs {
-  int h, l;
+struct __align__(8) Limbs {
+  int h;
+  float l;
 };
 
 __device__ __forceinline__ Limbs fx_split(i64 v) {
   const int l = (int)((unsigned)v << 3) >> 3;   // the low 29 bits, signed
-  return {(int)((v - l) >> 29), l};
+  return {(int)((v - l) >> 29), (float)l};
+}
+__device__ __forceinline__ i64 fx_join(int h, float l) { return ((i64)h << 29) + (int)l; }
+
+// Conversions between FP32 and 64-bit integers by way of 32 bits: the direct
+// instructions run on the FP64 pipe, at 1/64 of the FP32 rate.
+// |x| < 2^58, rounded to the nearest integer
+__device__ __forceinline__ i64 fx_int(float x) {
+  const int hi = __float2int_rn(x * 3.7252902984619140625e-9f);           // 2^-28
+  return ((i64)hi << 28) + __float2int_rn(fmaf((float)hi, -268435456.f, x));
+}
+__device__ __forceinline__ float fx_float(i64 v) {
+  return fmaf((float)(int)(v >> 32), 4294967296.f, (float)(unsigned)v);
 }
 
 // v sqrt(2) for |v| <= 2^58 (rounded to the last place)
@@ -68,7 +82,7 @@ __device__ __forceinline__ i64 fx_sqrt2(i64 v) {
 
 __device__ __forceinline__ i64 fx_from_dd(dd a) {   // |a| <= 1
   constexpr float B = 288230376151711744.f;         // 2^58
-  return __float2ll_rn(a.hi * B) + __float2ll_rn(a.lo * B);
+  return fx_int(a.hi * B) + fx_int(a.lo * B);
 }
 
 // V 2^e as a double, rounded to nearest (ties away from zero)
@@ -82,25 +96,31 @@ __device__ __forceinline__ double fx_to_double(i64 v, int e) {
   return __longlong_as_double((i64)(b | (v < 0 ? 1ull << 63 : 0ull)));
 }
 
-// sums over j of row[j] a[j] and row[j] b[j]; row: limb pairs stored one place
-// off (entry j at j + 1), so that a lane's columns 2p-1 and 2p are one int4
+// Sums over j of row[j] a[j] and row[j] b[j], as integers times 2^-58; row: limb
+// pairs stored one place off (entry j at j + 1), so that a lane's columns 2p-1
+// and 2p are one 16-byte unit.
 template <int NM>
 __device__ __forceinline__ void fx_dot2(const int4* __restrict__ row, const Limbs (&a)[NM], const Limbs (&b)[NM],
-                                        i64& h0, i64& x0, i64& h1, i64& x1) {
-  i64 y0 = 0, y1 = 0;
+                                        const float (&ah)[NM], const float (&bh)[NM], i64& va, i64& vb) {
+  i64 h0 = 0, h1 = 0;
+  float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f;
 #pragma unroll
   for (int j = 0; j < NM; ++j) {
     const int4 r = row[(j + 1) / 2];
-    const int rh = (j & 1) ? r.x : r.z, rl = (j & 1) ? r.y : r.w;
+    const int rh = (j & 1) ? r.x : r.z;
+    const float rl = __int_as_float((j & 1) ? r.y : r.w), rf = (float)rh;
     fx_mad(h0, rh, a[j].h);
-    fx_mad(x0, rh, a[j].l);
-    fx_mad(y0, rl, a[j].h);
     fx_mad(h1, rh, b[j].h);
-    fx_mad(x1, rh, b[j].l);
-    fx_mad(y1, rl, b[j].h);
+    x0 = fmaf(rf, a[j].l, x0);
+    x1 = fmaf(rf, b[j].l, x1);
+    y0 = fmaf(rl, ah[j], y0);
+    y1 = fmaf(rl, bh[j], y1);
   }
-  x0 += y0;
-  x1 += y1;
+  // mixed products times 2^-29: below 2^31.4 (rows and columns have 2-norms of at
+  // most 1), converted as half of it
+  constexpr float U = 1.f / 1073741824.f;   // 2^-30
+  va = h0 + ((i64)__float2int_rn((x0 + y0) * U) << 1);
+  vb = h1 + ((i64)__float2int_rn((x1 + y1) * U) << 1);
 }
 
 template <int W>
@@ -131,11 +151,12 @@ __device__ __forceinline__ void store_floats(float* dst, const float (&v)[NM], f
   }
 }
 template <int NM>
-__device__ __forceinline__ void store_limbs(Limbs* dst, const Limbs (&v)[NM]) {
+__device__ __forceinline__ void load_limbs(const Limbs* src, Limbs (&v)[NM]) {
 #pragma unroll
   for (int j = 0; j <= NM; j += 2) {
-    const Limbs lo = j == 0 ? Limbs{0, 0} : v[j == 0 ? 0 : j - 1], hi = j < NM ? v[j < NM ? j : 0] : Limbs{0, 0};
-    *reinterpret_cast<int4*>(dst + j) = make_int4(lo.h, lo.l, hi.h, hi.l);
+    const int4 t = *reinterpret_cast<const int4*>(src + j);
+    if (j > 0) v[j == 0 ? 0 : j - 1] = Limbs{t.x, __int_as_float(t.y)};
+    if (j < NM) v[j < NM ? j : 0] = Limbs{t.z, __int_as_float(t.w)};
   }
 }
 
@@ -144,19 +165,19 @@ __device__ __forceinline__ void store_limbs(Limbs* dst, const Limbs (&v)[NM]) {
 template <int N>
 struct FxLayout {
   static constexpr int NM = 2 * N - 1, C = 2 * N, L = N - 1, GPW = 32 / N;
-  // entry i of a row is stored at i + 1; a row is an odd number of 16-byte units,
-  // so that 16-byte reads of different rows by the lanes of a group spread over the banks
+  // entry i of a row is stored at i + 1; a row of limbs is an odd number of 16-byte
+  // units, so that 16-byte reads of different rows by the lanes of a group spread over
+  // the banks (rows of floats are mostly read by the whole group at once: kept short,
+  // which makes it 12 warps an SM at N = 7 instead of 10)
   static constexpr int LDQ = (N & 1) ? 2 * N : 2 * N + 2;            // limb pairs a row
-  static constexpr int LDF0 = (2 * N + 3) & ~3;
-  static constexpr int LDF = (LDF0 / 4) & 1 ? LDF0 : LDF0 + 4;       // floats a row
+  static constexpr int LDF = (2 * N + 3) & ~3;                       // floats a row
   static constexpr int TW = 3 * N;
   // in 4-byte words
   static constexpr int M = 0;                           // [NM][LDQ] limbs
   static constexpr int X = M + 2 * NM * LDQ;            // [NM][LDQ] limbs: C_m, then X
   static constexpr int F = X + 2 * NM * LDQ;            // [NM][LDF]: h_a, R, U^T R, E
-  static constexpr int U = F + NM * LDF;                // [NM][LDF]: row a = eigenvector a
-  static constexpr int S = U + NM * LDF;                // [2N] sqrt of the eigenvalues
-  static constexpr int END = S + ((2 * N + 3) & ~3);
+  static constexpr int U = F + NM * LDF;                // [NM][LDF]: row a = sqrt(eigenvalue a), eigenvector a
+  static constexpr int END = U + NM * LDF;
   static constexpr int T = F;                           // [3][2][TW] 64-bit modes, [3][2][N] times sqrt2: over F, U
   static constexpr int TEND = T + 2 * (3 * 2 * TW + 3 * 2 * N);
   static constexpr int OUTP = M;                        // packed tau (doubles) over M
@@ -169,7 +190,7 @@ struct FxLayout {
 
 // y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2
 template <int N>
-__global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
+__global__ void __launch_bounds__(128, N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
                                                      const float2* __restrict__ y, int64_t n_qp,
                                                      double* __restrict__ tau_out, dd nu2,
                                                      unsigned* __restrict__ n_unconverged,
@@ -187,7 +208,6 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
   Limbs* Xs = reinterpret_cast<Limbs*>(base + Lt::X);
   float* F = reinterpret_cast<float*>(base + Lt::F);
   float* U = reinterpret_cast<float*>(base + Lt::U);
-  float* sv = reinterpret_cast<float*>(base + Lt::S);
   i64* T = reinterpret_cast<i64*>(base + Lt::T);
   i64* T2 = T + 3 * 2 * TW;
   // the lane's columns, and whether it has a first one
@@ -207,11 +227,13 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
     const int64_t e = gq >> 2;
     const int q = (int)(gq & 3);
     // ---- w_m = sum_i L_im u_i for mode p, G = L L^T (double-float)
-    dd w[3][2], diff;
+    dd diff;
+    float bound = 0.f;
+    __syncwarp();
     {
       const double* gg = geo + e * GEO_STRIDE + GEO_G;
-      const dd gxx = dd_from_double(gg[0]), gxy = dd_from_double(gg[1]), gxz = dd_from_double(gg[2]),
-               gyy = dd_from_double(gg[3]), gyz = dd_from_double(gg[4]), gzz = dd_from_double(gg[5]);
+      const dd gxx = dd_split(gg[0]), gxy = dd_split(gg[1]), gxz = dd_split(gg[2]), gyy = dd_split(gg[3]),
+               gyz = dd_split(gg[4]), gzz = dd_split(gg[5]);
       const dd off = dd_fma(gxy, gxy, dd_fma(gxz, gxz, dd_mul(gyz, gyz)));
       const dd dia = dd_fma(gxx, gxx, dd_fma(gyy, gyy, dd_mul(gzz, gzz)));
       diff = dd_mul(nu2, dd_add(dia, dd_scale(off, 2.f)));
@@ -225,7 +247,7 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
       // lambda_a(q) = b + (a - b) delta_aq: u = b sum_a y_a + (a - b) y_q
       constexpr double BQ = qp_bary(0, 1), DQ = qp_bary(0, 0) - qp_bary(0, 1);
       constexpr float BH = (float)BQ, BL = (float)(BQ - (double)BH), DH = (float)DQ, DL = (float)(DQ - (double)DH);
-#pragma unroll
+#pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         dd u[3];
 #pragma unroll
@@ -241,16 +263,21 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
           u[i] = dd_fma(dd{DH, DL}, vq, dd_mul(dd{BH, BL}, sum));
           if (p == 0 && h == 1) u[i] = dd{0.f, 0.f};
         }
-        w[0][h] = dd_fma(l00, u[0], dd_fma(l10, u[1], dd_mul(l20, u[2])));
-        w[1][h] = dd_fma(l11, u[1], dd_mul(l21, u[2]));
-        w[2][h] = dd_mul(l22, u[2]);
+        const dd w0 = dd_fma(l00, u[0], dd_fma(l10, u[1], dd_mul(l20, u[2])));
+        const dd w1 = dd_fma(l11, u[1], dd_mul(l21, u[2]));
+        const dd w2 = dd_mul(l22, u[2]);
+        // parked as pairs in the table's places until the scale is known
+        float2* park = reinterpret_cast<float2*>(T + h * TW + L + p);
+        if (in_group) {
+          park[0] = make_float2(w0.hi, w0.lo);
+          park[2 * TW] = make_float2(w1.hi, w1.lo);
+          park[4 * TW] = make_float2(w2.hi, w2.lo);
+        }
+        // |C_m| <= beta_m = |w_0| + 2 sum |w_n|: with sum_m beta_m + sqrt(c) <= 1 after
+        // the scale 2^-ex, M's eigenvalues (and so its entries) are at most 1
+        bound += (fabsf(w0.hi) + fabsf(w1.hi) + fabsf(w2.hi)) * (p == 0 ? 1.f : 2.f);
       }
     }
-    // |C_m| <= beta_m = |w_0| + 2 sum |w_n|: with sum_m beta_m + sqrt(c) <= 1 after
-    // the scale 2^-ex, M's eigenvalues (and so its entries) are at most 1
-    float bound = 0.f;
-#pragma unroll
-    for (int m = 0; m < 3; ++m) bound += (fabsf(w[m][0].hi) + fabsf(w[m][1].hi)) * (p == 0 ? 1.f : 2.f);
     {
       float sum = 0.f;
 #pragma unroll
@@ -262,11 +289,12 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
     if (finite) frexpf(bound, &ex);
     const float sc = ldexpf(1.f, -ex);
     const i64 cfix = finite ? fx_from_dd(dd_scale(diff, sc * sc)) : (1ll << 57);
-    __syncwarp();
-#pragma unroll
+#pragma unroll 1
     for (int m = 0; m < 3; ++m) {
       i64* tr = T + m * 2 * TW + L;                     // mode k at tr[k], its imaginary part at tr[TW + k]
-      const i64 re = finite ? fx_from_dd(dd_scale(w[m][0], sc)) : 0, im = finite ? fx_from_dd(dd_scale(w[m][1], sc)) : 0;
+      const float2 wr = *reinterpret_cast<const float2*>(tr + p), wi = *reinterpret_cast<const float2*>(tr + TW + p);
+      const i64 re = finite ? fx_from_dd(dd{wr.x * sc, wr.y * sc}) : 0, im = finite ? fx_from_dd(dd{wi.x * sc, wi.y * sc}) : 0;
+      __syncwarp();
       if (in_group) {
         tr[p] = re;
         tr[TW + p] = im;
@@ -290,29 +318,40 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
         const i64* tr = T + m * 2 * TW + L;
         const i64* ti = tr + TW;
         const i64* t2 = T2 + m * 2 * N;
-        Limbs a[NM], b[NM];
-        a[0] = fx_split(t2[p]);
-        b[0] = fx_split(p == 0 ? tr[0] : t2[N + p]);
-#pragma unroll
+        // C_m's columns as rows (symmetric): entry i at i + 1
+        Limbs* rx = Xs + (hx ? cx : 0) * LDQ + 1;
+        Limbs* ry = Xs + cy * LDQ + 1;
+        __syncwarp();                                   // all lanes have read the previous C_m
+        if (hx) rx[0] = fx_split(t2[p]);
+        if (hy) ry[0] = fx_split(p == 0 ? tr[0] : t2[N + p]);
+#pragma unroll 1
         for (int k = 1; k < N; ++k) {
           const i64 pl = tr[k - p], ph = tr[k + p], ql = ti[k - p], qh = ti[k + p];
-          a[2 * k - 1] = fx_split(pl + ph);
-          a[2 * k] = fx_split(ql + qh);
-          b[2 * k - 1] = fx_split(p == 0 ? t2[k] : qh - ql);
-          b[2 * k] = fx_split(p == 0 ? t2[N + k] : pl - ph);
+          if (hx) {
+            rx[2 * k - 1] = fx_split(pl + ph);
+            rx[2 * k] = fx_split(ql + qh);
+          }
+          if (hy) {
+            ry[2 * k - 1] = fx_split(p == 0 ? t2[k] : qh - ql);
+            ry[2 * k] = fx_split(p == 0 ? t2[N + k] : pl - ph);
+          }
         }
-        __syncwarp();                                   // all lanes have read the previous C_m
-        // C_m's columns as rows (symmetric)
-        if (hx) store_limbs<NM>(Xs + cx * LDQ, a);
-        if (hy) store_limbs<NM>(Xs + cy * LDQ, b);
         __syncwarp();
+        Limbs a[NM], b[NM];
+        load_limbs<NM>(Xs + (hx ? cx : 0) * LDQ, a);
+        load_limbs<NM>(Xs + cy * LDQ, b);
+        float ah[NM], bh[NM];
+#pragma unroll
+        for (int j = 0; j < NM; ++j) {
+          ah[j] = (float)a[j].h;
+          bh[j] = (float)b[j].h;
+        }
 #pragma unroll 1
         for (int o = 0; o <= N; ++o) {
           const int r = half_row(o);
           const int4* row = reinterpret_cast<const int4*>(Xs + r * LDQ);
-          i64 h0 = 0, x0 = 0, h1 = 0, x1 = 0;
-          fx_dot2<NM>(row, a, b, h0, x0, h1, x1);
-          const i64 v0 = h0 + ((x0 + (1ll << 28)) >> 29), v1 = h1 + ((x1 + (1ll << 28)) >> 29);
+          i64 v0, v1;
+          fx_dot2<NM>(row, a, b, ah, bh, v0, v1);
           if (hx && o < N) acc[r * LDQ + cx] = m == 0 ? v0 : acc[r * LDQ + cx] + v0;
           if (hy && o > 0) acc[r * LDQ + cy] = m == 0 ? v1 : acc[r * LDQ + cy] + v1;
         }
@@ -342,11 +381,12 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
         const int4 mm = *reinterpret_cast<const int4*>(Ms + i * LDQ + 2 * p);   // (i, 2p-1) and (i, 2p)
-        x[i] = hx ? fmaf((float)mm.y, HL, (float)mm.x * H) : 0.f;
-        yv[i] = hy ? fmaf((float)mm.w, HL, (float)mm.z * H) : 0.f;
+        x[i] = hx ? fmaf(__int_as_float(mm.y), HL, (float)mm.x * H) : 0.f;
+        yv[i] = hy ? fmaf(__int_as_float(mm.w), HL, (float)mm.z * H) : 0.f;
       }
-      const float cd = (float)cfix * HL;
-      cholesky_columns<N>(x, yv, in_group ? p : 64, first, fmaxf(cd, 1e-30f));
+      const float cd = fx_float(cfix) * HL;
+      cholesky_columns<N, LDF, (N > 5)>(x, yv, p, in_group, first, fmaxf(cd, 1e-30f), F);
+      __syncwarp();
       const bool conv = onesided_jacobi<N>(x, yv, p, lane, FX_ORTHO2);
       {
         const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);
@@ -381,13 +421,13 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
       }
       // U, s, and h_a = f_a / |f_a|^{3/2}
       if (hx) {
-        sv[cx] = ax * ix;
         store_floats<NM, LDF>(U + cx * LDF, x, ix);
+        U[cx * LDF] = ax * ix;
         store_floats<NM, LDF>(F + cx * LDF, x, jx);
       }
       if (hy) {
-        sv[cy] = ay * iy;
         store_floats<NM, LDF>(U + cy * LDF, yv, iy);
+        U[cy * LDF] = ay * iy;
         store_floats<NM, LDF>(F + cy * LDF, yv, jy);
       }
     }
@@ -425,54 +465,50 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
       float rmax = 0.f;
       {
         Limbs pa[NM], pb[NM];
+        float pah[NM], pbh[NM];
         {
           // M X: M is symmetric, so row j of M times X_j,col adds to all rows of the column
-          i64 ha[NM], xa[NM], hb[NM], xb[NM];
+          i64 ha[NM], hb[NM];
+          float xa[NM], xb[NM];
 #pragma unroll
-          for (int r = 0; r < NM; ++r) ha[r] = xa[r] = hb[r] = xb[r] = 0;
+          for (int r = 0; r < NM; ++r) {
+            ha[r] = hb[r] = 0;
+            xa[r] = xb[r] = 0.f;
+          }
 #pragma unroll 1
           for (int j = 0; j < NM; ++j) {
             const int4* row = reinterpret_cast<const int4*>(Ms + j * LDQ);
             const int4 v = *reinterpret_cast<const int4*>(Xs + j * LDQ + 2 * p);
-            int mh[NM], ml[NM];
+            const float v0l = __int_as_float(v.y), v1l = __int_as_float(v.w), v0h = (float)v.x, v1h = (float)v.z;
 #pragma unroll
             for (int r = 0; r < NM; ++r) {
               const int4 w4 = row[(r + 1) / 2];
-              mh[r] = (r & 1) ? w4.x : w4.z;
-              ml[r] = (r & 1) ? w4.y : w4.w;
-            }
-            // in this order no multiply-add waits for the one before it
-#pragma unroll
-            for (int r = 0; r < NM; ++r) {
-              fx_mad(ha[r], mh[r], v.x);
-              fx_mad(hb[r], mh[r], v.z);
-            }
-#pragma unroll
-            for (int r = 0; r < NM; ++r) {
-              fx_mad(xa[r], mh[r], v.y);
-              fx_mad(xb[r], mh[r], v.w);
-            }
-#pragma unroll
-            for (int r = 0; r < NM; ++r) {
-              fx_mad(xa[r], ml[r], v.x);
-              fx_mad(xb[r], ml[r], v.z);
+              const int mh = (r & 1) ? w4.x : w4.z;
+              const float ml = __int_as_float((r & 1) ? w4.y : w4.w), mf = (float)mh;
+              fx_mad(ha[r], mh, v.x);
+              fx_mad(hb[r], mh, v.z);
+              xa[r] = fmaf(ml, v0h, fmaf(mf, v0l, xa[r]));
+              xb[r] = fmaf(ml, v1h, fmaf(mf, v1l, xb[r]));
             }
           }
           // to 2^-58 (|M X| <= 1)
+          const float to = ldexpf(1.f, xe - 29);
 #pragma unroll
           for (int r = 0; r < NM; ++r) {
-            pa[r] = fx_split((ha[r] << xe) + (xa[r] >> (29 - xe)));
-            pb[r] = fx_split((hb[r] << xe) + (xb[r] >> (29 - xe)));
+            pa[r] = fx_split((ha[r] << xe) + fx_int(xa[r] * to));
+            pb[r] = fx_split((hb[r] << xe) + fx_int(xb[r] * to));
+            pah[r] = (float)pa[r].h;
+            pbh[r] = (float)pb[r].h;
           }
         }
         const i64 one = (1ll << 58) >> xe;
 #pragma unroll 1
         for (int o = 0; o <= N; ++o) {
           const int r = half_row(o);
-          i64 h0 = 0, x0 = 0, h1 = 0, x1 = 0;
-          fx_dot2<NM>(reinterpret_cast<const int4*>(Xs + r * LDQ), pa, pb, h0, x0, h1, x1);
-          const float r0 = (float)((r == cx ? one : 0) - h0 - ((x0 + (1ll << 28)) >> 29)) * rscale;
-          const float r1 = (float)((r == cy ? one : 0) - h1 - ((x1 + (1ll << 28)) >> 29)) * rscale;
+          i64 v0, v1;
+          fx_dot2<NM>(reinterpret_cast<const int4*>(Xs + r * LDQ), pa, pb, pah, pbh, v0, v1);
+          const float r0 = fx_float((r == cx ? one : 0) - v0) * rscale;
+          const float r1 = fx_float((r == cy ? one : 0) - v1) * rscale;
           if (hx && o < N) {
             rmax = fmaxf(rmax, fabsf(r0));
             F[r * LDF + cx + 1] = r0;
@@ -507,7 +543,7 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
       load_floats<LDF>(U + (hx ? cx : 0) * LDF, rx);
       load_floats<LDF>(U + cy * LDF, ry);
       {
-        const float s0 = sv[hx ? cx : 0], s1 = sv[cy];
+        const float s0 = rx[0], s1 = ry[0];
 #pragma unroll 1
         for (int a = 0; a < NM; ++a) {                  // times U, divided, in place
           float row[LDF], sx = 0.f, sy = 0.f;
@@ -517,7 +553,7 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
             sx = fmaf(row[i], rx[i], sx);
             sy = fmaf(row[i], ry[i], sy);
           }
-          const float sa = sv[a];
+          const float sa = U[a * LDF];
           __syncwarp();
           if (hy)
             *reinterpret_cast<float2*>(F + a * LDF + 2 * p) = make_float2(sx * rcp_ftz(sa + s0), sy * rcp_ftz(sa + s1));
@@ -563,8 +599,8 @@ __global__ void __launch_bounds__(128, N <= 7 ? 3 : 1) tau_fx_kernel(const int4*
         const int r = half_row(o);
         const int4 v = *reinterpret_cast<const int4*>(Xs + r * LDQ + 2 * p);
         const float2 ev = *reinterpret_cast<const float2*>(F + r * LDF + 2 * p);
-        const i64 n0 = ((i64)v.x << 29) + v.y + __float2ll_rn(ev.x * escale);
-        const i64 n1 = ((i64)v.z << 29) + v.w + __float2ll_rn(ev.y * escale);
+        const i64 n0 = fx_join(v.x, __int_as_float(v.y)) + fx_int(ev.x * escale);
+        const i64 n1 = fx_join(v.z, __int_as_float(v.w)) + fx_int(ev.y * escale);
         if (more) {
           if (hx && o < N) Xs[r * LDQ + cx + 1] = Xs[cx * LDQ + r + 1] = fx_split(n0);
           if (hy && o > 0) Xs[r * LDQ + cy + 1] = Xs[cy * LDQ + r + 1] = fx_split(n1);
