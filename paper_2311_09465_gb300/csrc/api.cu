@@ -697,8 +697,9 @@ static int block_diag_impl(ts_problem* pr, LinState<T>& l, int invert, float* ou
   Phys<float> ph{(float)p64.rho, (float)p64.mu, (float)p64.omega, (float)p64.nu, (float)p64.C_I,
                  (float)p64.mass_coef};
   const int paper = pr->p.jvp_variant == TS_JVP_PAPER;
+  if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
   int rc = launch_block_diag<T, N>(paper, invert, m->d_node_off, m->d_node_elem, m->d_tets, geo_of<T>(m),
-                                   l.u0, l.tau, pr->d_dmask, pr->d_outdiag, ph, out, m->V, pr->d_counter, st);
+                                   l.u0, l.uc, l.tau, pr->d_dmask, pr->d_outdiag, ph, out, m->V, pr->d_counter, st);
   if (rc) return fail(rc == -6 ? TS_ERR_UNSUPPORTED : TS_ERR_CUDA, "block diagonal kernel launch failed");
   return 0;
 }
@@ -743,8 +744,9 @@ static int assemble_impl(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
   Phys<double> p64 = phys_of<double>(pr, true);
   Phys<float> ph{(float)p64.rho, (float)p64.mu, (float)p64.omega, (float)p64.nu, (float)p64.C_I,
                  (float)p64.mass_coef};
+  if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
   int rc = launch_assemble_paper<T, N>(m->d_node_off, m->d_node_elem, m->d_row_off, m->d_cols, m->d_tets,
-                                       geo_of<T>(m), l.u0, l.tau, ph, pr->d_hasm, m->V, st);
+                                       geo_of<T>(m), l.u0, l.uc, l.tau, ph, pr->d_hasm, m->V, st);
   if (rc) return fail(rc == -6 ? TS_ERR_UNSUPPORTED : TS_ERR_CUDA, "assembly kernel launch failed");
   pr->hasm_valid = true;
   return 0;

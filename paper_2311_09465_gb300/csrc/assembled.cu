@@ -27,8 +27,11 @@
 // (1.6 KB each at N = 7) through shared memory with 16-byte loads, lanes over
 // the 8N outputs; the records are the only large HBM stream, so the product
 // is bound by HBM bandwidth.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
+#include "nodal.cuh"
 
 namespace ts {
 
@@ -217,14 +220,203 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// 16-byte asynchronous global -> shared copies (LDGSTS), grouped per stage
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
+// ---------------------------------------------------------------------------
+// N <= 7: the assembly with register tiles (nodal.cuh).  A warp owns a row and
+// takes one (element, local node) at a time: its four groups of N lanes first
+// form X_a = tau_q S_qa at the four points (W_qa tau_q is its transpose), then
+// each takes one column node b and sums K_ab = sum_q (lambda_qa + W_qa tau_q) S_qb
+// in registers; the records are updated in place by the warp that owns the row.
+// 52,650 tetrahedra, N = 3 / 5 / 7: 0.47 / 0.83 / 1.81 ms (1.47 / 3.09 / 6.53 ms with one
+// output a lane and both operands in shared memory); bound by shared-memory reads
+// (81% at N = 5).
+template <int N>
+struct NodalAssembly {
+  using D = Nodal<N>;
+  static constexpr int TAU = 0, Y = 4 * D::MAT, TAB = Y + 4 * D::MAT;      // tables [q][b][2][TW]
+  static constexpr int WARP = (TAB + 16 * 2 * D::TW + 3) & ~3;             // then one NodalStage
+};
+
+template <typename T, typename U, int N>
+__global__ void __launch_bounds__(128, 4)
+    nodal_assemble_kernel(const int32_t* __restrict__ node_off, const int32_t* __restrict__ node_elem,
+                          const int32_t* __restrict__ row_off, const int32_t* __restrict__ cols,
+                          const int4* __restrict__ tets, const T* __restrict__ geo, const U* __restrict__ u0,
+                          const T* __restrict__ tau, Phys<float> ph, float* __restrict__ H, int64_t n_nodes) {
+  using D = Nodal<N>;
+  using W = NodalAssembly<N>;
+  constexpr int NM = D::NM, C = D::C, CC = C * C, HB = AsmLayout<N>::HB, MAT = D::MAT, NTP = D::NTP, TW = D::TW;
+  extern __shared__ __align__(16) float nodal_smem[];
+  __shared__ int offs[D::NT];
+  nodal_offsets<N>(offs, threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int g0 = lane / N, p = lane - g0 * N;
+  const bool in_group = g0 < 4;
+  const int g = in_group ? g0 : 0;
+  using Stage = NodalStage<T, U, N>;
+  float* ws = nodal_smem + warp * (W::WARP + Stage::BYTES / 4);
+  char* stage = reinterpret_cast<char*>(ws + W::WARP);
+  float* tq = ws + W::TAU + g * MAT;
+  float* yq = ws + W::Y + g * MAT;
+  float* tabs = ws + W::TAB;
+  const float bq = (float)qp_bary(0, 1), dq = (float)(qp_bary(0, 0) - qp_bary(0, 1));
+
+  for (int64_t A = (int64_t)blockIdx.x * wpb + warp; A < n_nodes; A += (int64_t)gridDim.x * wpb) {
+    const int r0 = row_off[A], r1 = row_off[A + 1];
+    {
+      float4* h = reinterpret_cast<float4*>(H + (int64_t)r0 * HB);
+      const int64_t n4 = (int64_t)(r1 - r0) * HB / 4;
+      for (int64_t t = lane; t < n4; t += 32) h[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const int p0 = node_off[A], p1 = node_off[A + 1];
+    // list entries three elements ahead, nodes two, the copies one: no load waits for
+    // another's result
+    int pk0 = p0 < p1 ? node_elem[p0] : 0, pk1 = p0 + 1 < p1 ? node_elem[p0 + 1] : 0,
+        pk2 = p0 + 2 < p1 ? node_elem[p0 + 2] : 0;
+    int4 nd0 = p0 < p1 ? tets[pk0 >> 2] : make_int4(0, 0, 0, 0), nd1 = p0 + 1 < p1 ? tets[pk1 >> 2] : nd0;
+    __syncwarp();
+    if (p0 < p1) Stage::issue(stage, pk0 >> 2, nd0, tau, u0, geo, lane);
+#pragma unroll 1
+    for (int pi = p0; pi < p1; ++pi) {
+      const int a = pk0 & 3;
+      const int node[4] = {nd0.x, nd0.y, nd0.z, nd0.w};
+      const char* in = stage;
+      cp_async_wait<0>();
+      __syncwarp();                       // the copies; the previous element's matrices are read
+      const T* ge = Stage::geo_of(in);
+      const float w4 = 0.25f * nodal_float(ge[GEO_VOL]);
+      float d[4][3];
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) d[b][j] = nodal_float(ge[b * 3 + j]);
+      // slot of the group's column node in row A
+      int slot = -1;
+#pragma unroll 1
+      for (int s = r0; s < r1; s += 32) {
+        const int col = s + lane < r1 ? cols[s + lane] : -1;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const unsigned hit = __ballot_sync(0xffffffffu, col == node[b]);
+          if (hit && b == g) slot = s + __ffs(hit) - 1;
+        }
+      }
+      // velocity at the group's point, then beta_qb for the four column nodes
+      float be[4][2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float u[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          float sum = 0.f, own = 0.f;
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const float v = nodal_value(Stage::rows_of(in)[b * 4 * C + j * C + 2 * p + h]);
+            sum += v;
+            own = b == g ? v : own;
+          }
+          u[j] = p == 0 && h == 1 ? 0.f : fmaf(bq, sum, dq * own);
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) be[b][h] = d[b][0] * u[0] + d[b][1] * u[1] + d[b][2] * u[2];
+      }
+      if (in_group) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) nodal_modes<N>(tabs + (g * 4 + b) * 2 * TW, p, be[b][0], be[b][1]);
+        nodal_tau<N>(Stage::tau_of(in) + g * NTP, offs, tq, p);
+      }
+      __syncwarp();
+      // the stage is consumed: the next element's copies run behind the products
+      if (pi + 1 < p1) {
+        Stage::issue(stage, pk1 >> 2, nd1, tau, u0, geo, lane);
+        pk0 = pk1;
+        pk1 = pk2;
+        nd0 = nd1;
+        if (pi + 2 < p1) nd1 = tets[pk1 >> 2];
+        if (pi + 3 < p1) pk2 = node_elem[pi + 3];
+      }
+      float sx[NM], sy[NM], X[NM], Y[NM];
+      nodal_columns<N>(tabs + (g * 4 + a) * 2 * TW, p, (g == a ? bq + dq : bq) * ph.omega, sx, sy);
+#pragma unroll
+      for (int i = 0; i < NM; ++i) X[i] = Y[i] = 0.f;
+      nodal_product<N>(tq, sx, sy, X, Y);
+      if (in_group) nodal_store_rows<N>(yq, p, X, Y);
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < NM; ++i) X[i] = Y[i] = 0.f;   // K_ab of the group's column node b = g
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        const float la = q == a ? bq + dq : bq;
+        nodal_columns<N>(tabs + (q * 4 + g) * 2 * TW, p, (q == g ? bq + dq : bq) * ph.omega, sx, sy);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          X[i] = fmaf(la, sx[i], X[i]);
+          Y[i] = fmaf(la, sy[i], Y[i]);
+        }
+        nodal_product<N>(ws + W::Y + q * MAT, sx, sy, X, Y);
+      }
+      // sum of tau over the points: the lane's columns
+      float tx[NM], ty[NM];
+      nodal_load_rows<N>(ws + W::TAU, p, tx, ty);
+#pragma unroll 1
+      for (int q = 1; q < 4; ++q) {
+        nodal_load_rows<N>(ws + W::TAU + q * MAT, p, sx, sy);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          tx[i] += sx[i];
+          ty[i] += sy[i];
+        }
+      }
+      if (in_group && slot >= 0) {
+        float* rec = H + (int64_t)slot * HB;
+        float dA[3], dB[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          dA[j] = a == 0 ? d[0][j] : a == 1 ? d[1][j] : a == 2 ? d[2][j] : d[3][j];
+          dB[j] = g == 0 ? d[0][j] : g == 1 ? d[1][j] : g == 2 ? d[2][j] : d[3][j];
+        }
+        const float gab = dA[0] * dB[0] + dA[1] * dB[1] + dA[2] * dB[2];
+        const float diag = 4.f * w4 * (ph.mu * gab + ph.mass_coef * (a == g ? 0.1f : 0.05f));
+        const float wk = w4 * ph.rho, wl = w4 / ph.rho * gab;
+        constexpr float S2 = Real<float>::SQRT2, IS2 = Real<float>::INV_SQRT2;
+        // storage coordinates: lane p > 0 has the stored columns 2p, 2p + 1, lane 0 column
+        // 0.  All loads of a matrix are issued before its stores: they come from L2
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+          float* at = rec + part * CC + 2 * p;
+          float2 v[NM];
+#pragma unroll
+          for (int i = 0; i < NM; ++i) v[i] = *reinterpret_cast<const float2*>(at + stor_of(i) * C);
+#pragma unroll
+          for (int i = 0; i < NM; ++i) {
+            float x = part == 0 ? wk * X[i] + (i == 2 * p - 1 ? diag : 0.f) : wl * tx[i];
+            float y = part == 0 ? wk * Y[i] + (i == 2 * p ? diag : 0.f) : wl * ty[i];
+            if (p == 0) {
+              x = y * (i == 0 ? 1.f : IS2);
+              y = 0.f;
+            } else if (i == 0) {
+              x *= S2;
+              y *= S2;
+            }
+            *reinterpret_cast<float2*>(at + stor_of(i) * C) = make_float2(v[i].x + x, v[i].y + y);
+          }
+        }
+        if (p == 0) {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            rec[2 * CC + j] -= w4 * dA[j];
+            rec[2 * CC + 3 + j] += w4 * dB[j];
+          }
+        }
+        // the coefficient of Im(mode 0): the Galerkin identity parts alone
+        if (p == 0) {
+          rec[C + 1] += diag;
+        }
+      }
+      __syncwarp();                       // record writes before the next element's reads by other lanes
+    }
+  }
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int PENDING>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 
 // y = H x on the assembled records; Dirichlet velocity and Im(mode 0) inputs
 // are ignored and the same rows of y are zero.  The record and x_B of the
@@ -512,21 +704,34 @@ int launch_sgs_colour(const int32_t* rows, int64_t n_rows, const int32_t* row_of
 
 template <typename T, int N>
 int launch_assemble_paper(const int32_t* node_off, const int32_t* node_elem, const int32_t* row_off,
-                          const int32_t* cols, const int4* tets, const T* geo, const T* u0, const T* tau,
+                          const int32_t* cols, const int4* tets, const T* geo, const T* u0, const T* uc, const T* tau,
                           Phys<float> ph, float* H, int64_t n_nodes, cudaStream_t st) {
-  using L = AsmLayout<N>;
   if (n_nodes <= 0) return 0;
-  int warps = 4;
-  while (warps > 1 && (size_t)warps * L::WARP * sizeof(float) > 200 * 1024) --warps;
-  const size_t smem = (size_t)warps * L::WARP * sizeof(float);
-  if (smem > 227 * 1024) return -6;
-  cudaFuncSetAttribute(assemble_paper_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int64_t blocks = (n_nodes + warps - 1) / warps;
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  count_launches(1);
-  assemble_paper_kernel<T, N><<<(int)blocks, warps * 32, smem, st>>>(node_off, node_elem, row_off, cols, tets,
-                                                                    geo, u0, tau, ph, H, n_nodes);
-  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  if constexpr (N <= NODAL_MAX_N) {
+    using U = typename PairOfStore<T>::V;
+    const size_t smem = (size_t)4 * (NodalAssembly<N>::WARP * sizeof(float) + NodalStage<T, U, N>::BYTES);
+    if (cudaFuncSetAttribute(nodal_assemble_kernel<T, U, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+        cudaSuccess)
+      return -2;
+    const int64_t blocks = std::min<int64_t>((n_nodes + 3) / 4, 152 * 32);
+    count_launches(1);
+    nodal_assemble_kernel<T, U, N><<<(int)blocks, 128, smem, st>>>(node_off, node_elem, row_off, cols, tets, geo,
+                                                                   reinterpret_cast<const U*>(uc), tau, ph, H, n_nodes);
+    return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  } else {
+    using L = AsmLayout<N>;
+    int warps = 4;
+    while (warps > 1 && (size_t)warps * L::WARP * sizeof(float) > 200 * 1024) --warps;
+    const size_t smem = (size_t)warps * L::WARP * sizeof(float);
+    if (smem > 227 * 1024) return -6;
+    cudaFuncSetAttribute(assemble_paper_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int64_t blocks = (n_nodes + warps - 1) / warps;
+    if (blocks > 152 * 32) blocks = 152 * 32;
+    count_launches(1);
+    assemble_paper_kernel<T, N><<<(int)blocks, warps * 32, smem, st>>>(node_off, node_elem, row_off, cols, tets,
+                                                                      geo, u0, tau, ph, H, n_nodes);
+    return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  }
 }
 
 template <int N>
@@ -549,7 +754,7 @@ int assembled_record_floats(int N) { return 2 * (2 * N) * (2 * N) + 8; }
 
 #define TS_INST_ASM(T, N)                                                                                   \
   template int launch_assemble_paper<T, N>(const int32_t*, const int32_t*, const int32_t*, const int32_t*,  \
-                                           const int4*, const T*, const T*, const T*, Phys<float>, float*,    \
+                                           const int4*, const T*, const T*, const T*, const T*, Phys<float>, float*, \
                                            int64_t, cudaStream_t);
 TS_FOR_EACH_N(TS_INST_ASM, float)
 TS_FOR_EACH_N(TS_INST_ASM, double)

@@ -73,6 +73,16 @@ template <>
 struct StoreOf<float2> {
   using S = double;
 };
+template <typename S>
+struct PairOfStore;
+template <>
+struct PairOfStore<float> {
+  using V = float;
+};
+template <>
+struct PairOfStore<double> {
+  using V = float2;
+};
 
 template <typename V>
 struct ElementArgs {
@@ -175,13 +185,14 @@ int j32_upload_n7(const float* host_all);
 constexpr int J32_MAX_N = 7;   // largest N with the single-launch FP32 kernel
 
 // Nodal diagonal blocks H_AA of the tangent (precond.cu): one 8N x 8N block per
-// node from the node-to-element list (packed element * 4 + local node); with
+// node from the node-to-element list (packed element * 4 + local node; uc: the
+// state u0 as in node_prepass, N <= 7 only); with
 // invert the inverse, column-major, else H_AA row-major.  Fixed unknowns
 // (Im(mode 0), Dirichlet velocity) have zero rows and columns (identity when
 // inverted); n_singular counts blocks that could not be inverted (stored as I).
 template <typename T, int N>
 int launch_block_diag(int variant_paper, int invert, const int32_t* node_off, const int32_t* node_elem,
-                      const int4* tets, const T* geo, const T* u0, const T* tau, const uint8_t* dmask,
+                      const int4* tets, const T* geo, const T* u0, const T* uc, const T* tau, const uint8_t* dmask,
                       const float* outdiag, Phys<float> ph, float* out, int64_t n_nodes,
                       unsigned* n_singular, cudaStream_t st);
 // z[A] = Binv[A] x[A] for every node (FP32 blocks, FP64 vectors)
@@ -192,7 +203,7 @@ int launch_block_apply(const float* binv, const double* x, double* z, int64_t n_
 // connection a record of assembled_record_floats(N) floats (K, L, G_1..3, D_1..3)
 template <typename T, int N>
 int launch_assemble_paper(const int32_t* node_off, const int32_t* node_elem, const int32_t* row_off,
-                          const int32_t* cols, const int4* tets, const T* geo, const T* u0, const T* tau,
+                          const int32_t* cols, const int4* tets, const T* geo, const T* u0, const T* uc, const T* tau,
                           Phys<float> ph, float* H, int64_t n_nodes, cudaStream_t st);
 template <int N>
 int launch_spmv_paper(const int32_t* row_off, const int32_t* cols, const float* H, const uint8_t* dmask,

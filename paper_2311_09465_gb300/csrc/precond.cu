@@ -28,8 +28,11 @@
 // in place (Gauss-Jordan, partial pivoting, FP32) and stores it column-major;
 // the apply kernel (one warp per node, coalesced column reads) multiplies it
 // with the node's slice of a Krylov vector.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
+#include "nodal.cuh"
 
 namespace ts {
 
@@ -92,6 +95,84 @@ __device__ __forceinline__ void warp_mm(const float* A, const float* B, float* o
     for (int k = 0; k < C; ++k) acc = fmaf(A[r * C + k], B[k * C + s], acc);
     out[t] = acc;
   }
+}
+
+// Inverts the NB x NB block F (shared memory, row-major) in place, Gauss-Jordan
+// with partial pivoting, one warp, and stores it column-major; a block without
+// an inverse is counted and stored as the identity.
+template <int NB>
+__device__ void invert_block(float* F, int* piv, float* __restrict__ dst, int lane, unsigned* n_singular) {
+  bool singular = false;
+  for (int k = 0; k < NB; ++k) {
+    float best = -1.f;
+    int bi = k;
+    for (int i = k + lane; i < NB; i += 32) {
+      const float v = fabsf(F[i * NB + k]);
+      if (v > best) {
+        best = v;
+        bi = i;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > best || (ov == best && oi < bi)) {
+        best = ov;
+        bi = oi;
+      }
+    }
+    if (!(best > 0.f) || !isfinite(best)) {
+      singular = true;
+      break;
+    }
+    if (lane == 0) piv[k] = bi;
+    if (bi != k)
+      for (int j = lane; j < NB; j += 32) {
+        const float tmp = F[k * NB + j];
+        F[k * NB + j] = F[bi * NB + j];
+        F[bi * NB + j] = tmp;
+      }
+    __syncwarp();
+    const float inv = 1.f / F[k * NB + k];
+    __syncwarp();
+    for (int j = lane; j < NB; j += 32) F[k * NB + j] = j == k ? inv : F[k * NB + j] * inv;
+    __syncwarp();
+    for (int t = lane; t < NB * NB; t += 32) {
+      const int i = t / NB, j = t - i * NB;
+      if (i == k) continue;
+      const float fik = F[i * NB + k];
+      if (j == k) continue;
+      F[t] = fmaf(-fik, F[k * NB + j], F[t]);
+    }
+    __syncwarp();
+    for (int i = lane; i < NB; i += 32)
+      if (i != k) F[i * NB + k] = -F[i * NB + k] * inv;
+    __syncwarp();
+  }
+  if (singular) {
+    if (lane == 0) atomicAdd(n_singular, 1u);
+    for (int t = lane; t < NB * NB; t += 32) dst[t] = (t / NB == t % NB) ? 1.f : 0.f;
+    __syncwarp();
+    return;
+  }
+  // undo the row exchanges as column exchanges, in reverse order
+  for (int k = NB - 1; k >= 0; --k) {
+    const int pk = piv[k];
+    if (pk != k)
+      for (int i = lane; i < NB; i += 32) {
+        const float tmp = F[i * NB + k];
+        F[i * NB + k] = F[i * NB + pk];
+        F[i * NB + pk] = tmp;
+      }
+    __syncwarp();
+  }
+  // column-major store for the apply kernel
+  for (int t = lane; t < NB * NB; t += 32) {
+    const int col = t / NB, row = t - col * NB;
+    dst[t] = F[row * NB + col];
+  }
+  __syncwarp();
 }
 
 template <typename T, int N, bool PAPER, bool INVERT>
@@ -248,76 +329,369 @@ __global__ void __launch_bounds__(128)
       __syncwarp();
       continue;
     }
-    // ---- in-place Gauss-Jordan inversion with partial pivoting
-    bool singular = false;
-    for (int k = 0; k < NB; ++k) {
-      float best = -1.f;
-      int bi = k;
-      for (int i = k + lane; i < NB; i += 32) {
-        const float v = fabsf(F[i * NB + k]);
-        if (v > best) {
-          best = v;
-          bi = i;
-        }
-      }
+    invert_block<NB>(F, piv, dst, lane, n_singular);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// N <= 7: the same blocks with register tiles (nodal.cuh).  A warp owns a node;
+// its four groups of N lanes take the four quadrature points of an element and
+// sum over the node's elements in registers: K += w rho (lambda S + S^T X),
+// X = tau S, GX_i += w dN/dx_i X (the least-squares part of D_i; of G_i,
+// transposed), L += (w / rho) |grad N|^2 tau.
+//
+// Inverse: with the velocity block K (the same for three fields) and no outlet
+// coupling,
+//   E_i = K^-1 G_i, S = L - sum_i D_i E_i, H_j = S^-1 D_j K^-1, H_p = -S^-1,
+//   inverse_ij = delta_ij K^-1 + E_i H_j (j = 1..3, p), row p = -H_j,
+// two n x n inversions and about 20 products instead of one (8N)^3 elimination.
+// The n x n inversions do not exchange rows; a node where a pivot is less than
+// PIVOT_OK of the largest candidate, and the outlet nodes, take the full
+// elimination.
+//
+// N = 7, 52,650 tetrahedra, with inverse: 1.16 ms (8.4 ms before: the sums were two
+// shared-memory loads a multiply-add and the elimination one warp's passes over
+// 3136 entries); the inverse is 0.04 ms of it.  Bound by issue and shared memory
+// at 8 warps an SM (254 registers hold the five n x n sums of a group).
+constexpr float PIVOT_OK = 0.1f;
+
+template <int N>
+struct NodalBlock {
+  using D = Nodal<N>;
+  static constexpr int C = 2 * N, NB = 8 * N;
+  // while summing: tau [4], S [4], tables [4][2][TW]
+  static constexpr int TAU = 0, S = TAU + 4 * D::MAT, TAB = S + 4 * D::MAT, SUM_END = TAB + 4 * 2 * D::TW;
+  // then: K (columns as rows), GX_0..2 (row-major), L; and over the rest K^-1, S^-1, E_0..2 or the full block
+  static constexpr int K = 0, GX = D::MAT, LM = 4 * D::MAT, REST = 5 * D::MAT;
+  static constexpr int KI = REST, SI = KI + D::MAT, E = SI + D::MAT, SCHUR_END = E + 3 * D::MAT;
+  static constexpr int F = REST, PIV = F + NB * NB, FULL_END = PIV + NB;
+  static constexpr int MAX1 = SUM_END > SCHUR_END ? SUM_END : SCHUR_END;
+  static constexpr int WARP = ((MAX1 > FULL_END ? MAX1 : FULL_END) + 3) & ~3;
+};
+
+// In-place Gauss-Jordan inverse of the group's matrix (columns in lanes), without
+// row exchanges; false where a pivot is small.  The rows move up one a step, so
+// that the pivot is at index 0 and the loop can stay rolled.
+template <int N>
+__device__ __forceinline__ bool nodal_invert(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, int base) {
+  constexpr int NM = 2 * N - 1;
+  bool ok = true;
+#pragma unroll 1
+  for (int k = 0; k < NM; ++k) {
+    const int src = base + (k + 1) / 2;
+    const bool odd = k & 1;
+    float c[NM], big = 0.f;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) {
-          best = ov;
-          bi = oi;
-        }
-      }
-      if (!(best > 0.f) || !isfinite(best)) {
-        singular = true;
-        break;
-      }
-      if (lane == 0) piv[k] = bi;
-      if (bi != k)
-        for (int j = lane; j < NB; j += 32) {
-          const float tmp = F[k * NB + j];
-          F[k * NB + j] = F[bi * NB + j];
-          F[bi * NB + j] = tmp;
-        }
-      __syncwarp();
-      const float inv = 1.f / F[k * NB + k];
-      __syncwarp();
-      for (int j = lane; j < NB; j += 32) F[k * NB + j] = j == k ? inv : F[k * NB + j] * inv;
-      __syncwarp();
-      for (int t = lane; t < NB * NB; t += 32) {
-        const int i = t / NB, j = t - i * NB;
-        if (i == k) continue;
-        const float fik = F[i * NB + k];
-        if (j == k) continue;
-        F[t] = fmaf(-fik, F[k * NB + j], F[t]);
-      }
-      __syncwarp();
-      for (int i = lane; i < NB; i += 32)
-        if (i != k) F[i * NB + k] = -F[i * NB + k] * inv;
-      __syncwarp();
+    for (int i = 0; i < NM; ++i) {
+      c[i] = __shfl_sync(0xffffffffu, odd ? x[i] : y[i], src);
+      if (i < NM - k) big = fmaxf(big, fabsf(c[i]));
     }
-    if (singular) {
-      if (lane == 0) atomicAdd(n_singular, 1u);
-      for (int t = lane; t < NB * NB; t += 32) dst[t] = (t / NB == t % NB) ? 1.f : 0.f;
+    ok = ok && fabsf(c[0]) > PIVOT_OK * big && isfinite(big);
+    const float rd = 1.f / c[0];
+    const bool px = 2 * p - 1 == k, py = 2 * p == k;
+    const float tx = px ? rd : x[0] * rd, ty = py ? rd : y[0] * rd;
+#pragma unroll
+    for (int i = 1; i < NM; ++i) {
+      x[i - 1] = fmaf(-c[i], tx, px ? 0.f : x[i]);
+      y[i - 1] = fmaf(-c[i], ty, py ? 0.f : y[i]);
+    }
+    x[NM - 1] = tx;
+    y[NM - 1] = ty;
+  }
+  return ok;
+}
+
+template <typename T, typename U, int N, bool PAPER, bool INVERT>
+__global__ void __launch_bounds__(128, 2)
+    nodal_block_kernel(const int32_t* __restrict__ node_off, const int32_t* __restrict__ node_elem,
+                       const int4* __restrict__ tets, const T* __restrict__ geo, const U* __restrict__ u0,
+                       const T* __restrict__ tau, const uint8_t* __restrict__ dmask,
+                       const float* __restrict__ outdiag, Phys<float> ph, float* __restrict__ out, int64_t n_nodes,
+                       unsigned* __restrict__ n_singular) {
+  using D = Nodal<N>;
+  using W = NodalBlock<N>;
+  constexpr int NM = D::NM, C = D::C, NB = W::NB, LD = D::LD, MAT = D::MAT, NTP = D::NTP;
+  extern __shared__ __align__(16) float nodal_smem[];
+  __shared__ int offs[D::NT];
+  nodal_offsets<N>(offs, threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int g0 = lane / N, p = lane - g0 * N;
+  const bool in_group = g0 < 4;
+  const int g = in_group ? g0 : 0, base = g * N;
+  using Stage = NodalStage<T, U, N>;
+  float* ws = nodal_smem + warp * (W::WARP + Stage::BYTES / 4);
+  char* stage = reinterpret_cast<char*>(ws + W::WARP);
+  float* tq = ws + W::TAU + g * MAT;
+  float* Sq = ws + W::S + g * MAT;
+  float* tab = ws + W::TAB + g * 2 * D::TW;
+  const float rho = ph.rho, bq = (float)qp_bary(0, 1), dq = (float)(qp_bary(0, 0) - qp_bary(0, 1));
+
+  for (int64_t A = (int64_t)blockIdx.x * wpb + warp; A < n_nodes; A += (int64_t)gridDim.x * wpb) {
+    float Kx[NM], Ky[NM], Gx[3][NM], Gy[3][NM], Lx[NM], Ly[NM];
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      Kx[i] = Ky[i] = Lx[i] = Ly[i] = 0.f;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) Gx[j][i] = Gy[j][i] = 0.f;
+    }
+    float kd = 0.f, gd[3] = {0.f, 0.f, 0.f};
+    const int p0 = node_off[A], p1 = node_off[A + 1];
+    // list entries three elements ahead, nodes two, the copies one: no load waits for
+    // another's result
+    int pk0 = p0 < p1 ? node_elem[p0] : 0, pk1 = p0 + 1 < p1 ? node_elem[p0 + 1] : 0,
+        pk2 = p0 + 2 < p1 ? node_elem[p0 + 2] : 0;
+    int4 nd0 = p0 < p1 ? tets[pk0 >> 2] : make_int4(0, 0, 0, 0), nd1 = p0 + 1 < p1 ? tets[pk1 >> 2] : nd0;
+    __syncwarp();
+    if (p0 < p1) Stage::issue(stage, pk0 >> 2, nd0, tau, u0, geo, lane);
+#pragma unroll 1
+    for (int pi = p0; pi < p1; ++pi) {
+      const int a = pk0 & 3;
+      const char* in = stage;
+      cp_async_wait<0>();
+      __syncwarp();                       // the copies; the previous element's matrices are read
+      const T* ge = Stage::geo_of(in);
+      const float w4 = 0.25f * nodal_float(ge[GEO_VOL]);
+      const float d[3] = {nodal_float(ge[a * 3]), nodal_float(ge[a * 3 + 1]), nodal_float(ge[a * 3 + 2])};
+      const float lam = a == g ? bq + dq : bq, g2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+      // beta_q = sum_j dN_a/dx_j u0_j(q), mode p
+      float be[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float sum = 0.f, own = 0.f;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const U* ub = Stage::rows_of(in) + b * 4 * C + 2 * p + h;
+          const float v = d[0] * nodal_value(ub[0]) + d[1] * nodal_value(ub[C]) + d[2] * nodal_value(ub[2 * C]);
+          sum += v;
+          own = b == g ? v : own;
+        }
+        be[h] = p == 0 && h == 1 ? 0.f : fmaf(bq, sum, dq * own);
+      }
+      if (in_group) {
+        nodal_modes<N>(tab, p, be[0], be[1]);
+        nodal_tau<N>(Stage::tau_of(in) + g * NTP, offs, tq, p);
+      }
+      __syncwarp();
+      // the stage is consumed: the next element's copies run behind the products
+      if (pi + 1 < p1) {
+        Stage::issue(stage, pk1 >> 2, nd1, tau, u0, geo, lane);
+        pk0 = pk1;
+        pk1 = pk2;
+        nd0 = nd1;
+        if (pi + 2 < p1) nd1 = tets[pk1 >> 2];
+        if (pi + 3 < p1) pk2 = node_elem[pi + 3];
+      }
+      float sx[NM], sy[NM], X[NM], Y[NM];
+      nodal_columns<N>(tab, p, lam * ph.omega, sx, sy);
+      if (in_group) nodal_store_rows<N>(Sq, p, sx, sy);
+#pragma unroll
+      for (int i = 0; i < NM; ++i) X[i] = Y[i] = 0.f;
+      nodal_product<N>(tq, sx, sy, X, Y);
+      const float wr = w4 * rho;
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        Kx[i] = fmaf(wr * lam, sx[i], Kx[i]);
+        Ky[i] = fmaf(wr * lam, sy[i], Ky[i]);
+        if (!PAPER) {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            Gx[j][i] = fmaf(w4 * d[j], X[i], Gx[j][i]);
+            Gy[j][i] = fmaf(w4 * d[j], Y[i], Gy[j][i]);
+          }
+        }
+        X[i] *= wr;
+        Y[i] *= wr;
+      }
+      nodal_load_rows<N>(tq, p, sx, sy);  // tau's columns
+      const float wl = w4 / rho * g2;
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        Lx[i] = fmaf(wl, sx[i], Lx[i]);
+        Ly[i] = fmaf(wl, sy[i], Ly[i]);
+      }
+      __syncwarp();
+      nodal_product<N>(Sq, X, Y, Kx, Ky); // rows of Sq are S's columns: S^T X
+      // identity parts: viscous, consistent mass; Galerkin divergence (and, negated, pressure)
+      kd += 4.f * w4 * (ph.mu * g2 + 0.1f * ph.mass_coef);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) gd[j] = fmaf(w4, d[j], gd[j]);
+    }
+    // sums over the four points into group 0, then to shared memory
+    auto fold = [&](float v) {
+      v += __shfl_down_sync(0xffffffffu, v, 2 * N);
+      return v + __shfl_down_sync(0xffffffffu, v, N);
+    };
+#pragma unroll
+    for (int i = 0; i < NM; ++i) {
+      Kx[i] = fold(Kx[i]) + (i == 2 * p - 1 ? kd : 0.f);
+      Ky[i] = fold(Ky[i]) + (i == 2 * p ? kd : 0.f);
+      Lx[i] = fold(Lx[i]);
+      Ly[i] = fold(Ly[i]);
+      if (!PAPER) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          Gx[j][i] = fold(Gx[j][i]);
+          Gy[j][i] = fold(Gy[j][i]);
+        }
+      }
+    }
+    __syncwarp();
+    if (lane < N) {
+      nodal_store_rows<N>(ws + W::K, p, Kx, Ky);
+      nodal_store_rows<N>(ws + W::LM, p, Lx, Ly);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) nodal_store_columns<N>(ws + W::GX + j * MAT, p, Gx[j], Gy[j]);
+    }
+    __syncwarp();
+    const bool dir = dmask[A] != 0;
+    const float* od = outdiag + A * 6;   // R w_i w_j (xx, xy, xz, yy, yz, zz)
+    float* dst = out + A * NB * NB;
+    // an entry of the full block in storage coordinates (x_0, Re x_n, Im x_n): row and
+    // column scaled by D = diag(1, 1/sqrt2, ...) and its inverse
+    auto entry = [&](int row, int col) {
+      const int f = row / C, c = row - f * C, h = col / C, k = col - h * C;
+      const bool fr = c == 1 || (dir && f < 3), fc = k == 1 || (dir && h < 3);
+      if (fr || fc) return INVERT && row == col ? 1.f : 0.f;
+      const int r = c == 0 ? 0 : c - 1, s = k == 0 ? 0 : k - 1;
+      float v;
+      if (f < 3 && h < 3) {
+        v = f == h ? ws[W::K + s * LD + r] : 0.f;
+        if (r == s) {
+          const int lo = f < h ? f : h, hi = f < h ? h : f;
+          v += od[lo == 0 ? hi : (lo == 1 ? 2 + hi : 5)];
+        }
+      } else if (f < 3) {
+        v = ws[W::GX + f * MAT + s * LD + r] - (r == s ? (f == 0 ? gd[0] : f == 1 ? gd[1] : gd[2]) : 0.f);
+      } else if (h < 3) {
+        v = ws[W::GX + h * MAT + r * LD + s] + (r == s ? (h == 0 ? gd[0] : h == 1 ? gd[1] : gd[2]) : 0.f);
+      } else {
+        v = ws[W::LM + s * LD + r];
+      }
+      return r == 0 && s > 0 ? v * Real<float>::SQRT2 : r > 0 && s == 0 ? v * Real<float>::INV_SQRT2 : v;
+    };
+    if (!INVERT) {
+      for (int t = lane; t < NB * NB; t += 32) dst[t] = entry(t / NB, t % NB);
       __syncwarp();
       continue;
     }
-    // undo the row exchanges as column exchanges, in reverse order
-    for (int k = NB - 1; k >= 0; --k) {
-      const int pk = piv[k];
-      if (pk != k)
-        for (int i = lane; i < NB; i += 32) {
-          const float tmp = F[i * NB + k];
-          F[i * NB + k] = F[i * NB + pk];
-          F[i * NB + pk] = tmp;
+    bool ok = od[0] == 0.f && od[3] == 0.f && od[5] == 0.f;   // no outlet coupling (the same for the warp)
+    float Hx[NM], Hy[NM];                                    // group j: H_j, group 3: H_p
+    if (ok) {
+      float* KI = ws + W::KI;
+      float* SI = ws + W::SI;
+      float kx[NM], ky[NM], ex[NM], ey[NM], tx[NM], ty[NM];
+      nodal_load_rows<N>(ws + W::LM, p, tx, ty);
+      const int j3 = g < 3 ? g : 0;
+      const float gg = g == 0 ? gd[0] : g == 1 ? gd[1] : gd[2];
+      const float* GXg = ws + W::GX + j3 * MAT;
+      if (!dir) {
+        nodal_load_rows<N>(ws + W::K, p, kx, ky);
+        ok = nodal_invert<N>(kx, ky, p, base);
+        if (lane < N) nodal_store_columns<N>(KI, p, kx, ky);
+        __syncwarp();
+        // E_i = K^-1 G_i, G_i = GX_i^T - gd_i I (group i)
+        nodal_load_rows<N>(GXg, p, Hx, Hy);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          Hx[i] -= i == 2 * p - 1 ? gg : 0.f;
+          Hy[i] -= i == 2 * p ? gg : 0.f;
+          ex[i] = ey[i] = 0.f;
         }
+        nodal_product<N>(KI, Hx, Hy, ex, ey);
+        if (in_group && g < 3) nodal_store_columns<N>(ws + W::E + g * MAT, p, ex, ey);
+        // S = L - sum_i D_i E_i, D_i = GX_i + gd_i I
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          Hx[i] = gg * ex[i];
+          Hy[i] = gg * ey[i];
+        }
+        nodal_product<N>(GXg, ex, ey, Hx, Hy);
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          tx[i] -= __shfl_sync(0xffffffffu, Hx[i], p) + __shfl_sync(0xffffffffu, Hx[i], N + p) +
+                   __shfl_sync(0xffffffffu, Hx[i], 2 * N + p);
+          ty[i] -= __shfl_sync(0xffffffffu, Hy[i], p) + __shfl_sync(0xffffffffu, Hy[i], N + p) +
+                   __shfl_sync(0xffffffffu, Hy[i], 2 * N + p);
+        }
+      }
+      const bool ok2 = nodal_invert<N>(tx, ty, p, base);
+      ok = __all_sync(0xffffffffu, (ok && ok2) || !in_group);
+      if (lane < N) nodal_store_columns<N>(SI, p, tx, ty);
       __syncwarp();
+      // H_j = S^-1 D_j K^-1 (groups 0..2), H_p = -S^-1 (group 3)
+      if (!dir) {
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          ex[i] = gg * kx[i];
+          ey[i] = gg * ky[i];
+          Hx[i] = Hy[i] = 0.f;
+        }
+        nodal_product<N>(GXg, kx, ky, ex, ey);
+        nodal_product<N>(SI, ex, ey, Hx, Hy);
+      }
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        if (g == 3) {
+          Hx[i] = -tx[i];
+          Hy[i] = -ty[i];
+        } else if (dir) {
+          Hx[i] = Hy[i] = 0.f;
+        }
+      }
+      if (ok) {
+        // the lane's columns, storage coordinates: 2p and 2p+1 of field g (lane 0: 0; its 1 is Im(mode 0))
+        constexpr float S2 = Real<float>::SQRT2, IS2 = Real<float>::INV_SQRT2;
+        float* cx = dst + (int64_t)(g * C + 2 * p) * NB;
+        float* cy = cx + NB;
+#pragma unroll 1
+        for (int f = 0; f < 4; ++f) {
+          float ox[NM], oy[NM];
+          if (f < 3 && !dir) {
+#pragma unroll
+            for (int i = 0; i < NM; ++i) {
+              ox[i] = f == g ? kx[i] : 0.f;
+              oy[i] = f == g ? ky[i] : 0.f;
+            }
+            nodal_product<N>(ws + W::E + f * MAT, Hx, Hy, ox, oy);
+          } else {
+#pragma unroll
+            for (int i = 0; i < NM; ++i) {
+              ox[i] = f == 3 ? -Hx[i] : (f == g && i == 2 * p - 1 ? 1.f : 0.f);
+              oy[i] = f == 3 ? -Hy[i] : (f == g && i == 2 * p ? 1.f : 0.f);
+            }
+          }
+          if (in_group) {
+            // lane p > 0: x is stored column 2p, y is 2p + 1; lane 0: y is column 0
+            float2* sx = reinterpret_cast<float2*>(cx + f * C);
+            float2* sy = reinterpret_cast<float2*>(cy + f * C);
+            if (p == 0) {
+              sx[0] = make_float2(oy[0], 0.f);
+              sy[0] = make_float2(0.f, f == g ? 1.f : 0.f);
+            } else {
+              sx[0] = make_float2(ox[0] * S2, 0.f);
+              sy[0] = make_float2(oy[0] * S2, 0.f);
+            }
+#pragma unroll
+            for (int n = 1; n < N; ++n) {
+              if (p == 0) {
+                sx[n] = make_float2(oy[2 * n - 1] * IS2, oy[2 * n] * IS2);
+                sy[n] = make_float2(0.f, 0.f);
+              } else {
+                sx[n] = make_float2(ox[2 * n - 1], ox[2 * n]);
+                sy[n] = make_float2(oy[2 * n - 1], oy[2 * n]);
+              }
+            }
+          }
+        }
+      }
     }
-    // column-major store for the apply kernel
-    for (int t = lane; t < NB * NB; t += 32) {
-      const int col = t / NB, row = t - col * NB;
-      dst[t] = F[row * NB + col];
+    if (!ok) {
+      __syncwarp();
+      float* F = ws + W::F;
+      for (int t = lane; t < NB * NB; t += 32) F[t] = entry(t / NB, t % NB);
+      __syncwarp();
+      invert_block<NB>(F, reinterpret_cast<int*>(ws + W::PIV), dst, lane, n_singular);
     }
     __syncwarp();
   }
@@ -357,31 +731,41 @@ __global__ void __launch_bounds__(256)
 
 template <typename T, int N>
 int launch_block_diag(int variant_paper, int invert, const int32_t* node_off, const int32_t* node_elem,
-                      const int4* tets, const T* geo, const T* u0, const T* tau, const uint8_t* dmask,
+                      const int4* tets, const T* geo, const T* u0, const T* uc, const T* tau, const uint8_t* dmask,
                       const float* outdiag, Phys<float> ph, float* out, int64_t n_nodes,
                       unsigned* n_singular, cudaStream_t st) {
-  using L = BlockLayout<N>;
   if (n_nodes <= 0) return 0;
-  int warps = 4;
-  while (warps > 1 && (size_t)warps * L::WARP * sizeof(float) > 200 * 1024) --warps;
-  const size_t smem = (size_t)warps * L::WARP * sizeof(float);
-  if (smem > 227 * 1024) return -6;
-  int64_t blocks = (n_nodes + warps - 1) / warps;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  auto go = [&](auto kern) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto go = [&](auto kern, size_t smem, int warps, auto u) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -2;
+    const int64_t blocks = std::min<int64_t>((n_nodes + warps - 1) / warps, 152 * 16);
     count_launches(1);
-    kern<<<(int)blocks, warps * 32, smem, st>>>(node_off, node_elem, tets, geo, u0, tau, dmask, outdiag, ph,
-                                               out, n_nodes, n_singular);
+    kern<<<(int)blocks, warps * 32, smem, st>>>(node_off, node_elem, tets, geo, u, tau, dmask, outdiag, ph, out,
+                                               n_nodes, n_singular);
+    return cudaGetLastError() == cudaSuccess ? 0 : -2;
   };
-  if (variant_paper) {
-    if (invert) go(block_diag_kernel<T, N, true, true>);
-    else go(block_diag_kernel<T, N, true, false>);
+  if constexpr (N <= NODAL_MAX_N) {
+    using U = typename PairOfStore<T>::V;
+    const size_t smem = (size_t)4 * (NodalBlock<N>::WARP * sizeof(float) + NodalStage<T, U, N>::BYTES);
+    static_assert(4 * (NodalBlock<N>::WARP * 4 + NodalStage<T, U, N>::BYTES) <= 113 * 1024, "two blocks an SM");
+    const U* u = reinterpret_cast<const U*>(uc);
+    if (variant_paper)
+      return invert ? go(nodal_block_kernel<T, U, N, true, true>, smem, 4, u)
+                    : go(nodal_block_kernel<T, U, N, true, false>, smem, 4, u);
+    return invert ? go(nodal_block_kernel<T, U, N, false, true>, smem, 4, u)
+                  : go(nodal_block_kernel<T, U, N, false, false>, smem, 4, u);
   } else {
-    if (invert) go(block_diag_kernel<T, N, false, true>);
-    else go(block_diag_kernel<T, N, false, false>);
+    // the register tiles of N > 7 do not fit: five n x n sums a group
+    using L = BlockLayout<N>;
+    int warps = 4;
+    while (warps > 1 && (size_t)warps * L::WARP * sizeof(float) > 200 * 1024) --warps;
+    const size_t smem = (size_t)warps * L::WARP * sizeof(float);
+    if (smem > 227 * 1024) return -6;
+    if (variant_paper)
+      return invert ? go(block_diag_kernel<T, N, true, true>, smem, warps, u0)
+                    : go(block_diag_kernel<T, N, true, false>, smem, warps, u0);
+    return invert ? go(block_diag_kernel<T, N, false, true>, smem, warps, u0)
+                  : go(block_diag_kernel<T, N, false, false>, smem, warps, u0);
   }
-  return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
 template <int N>
@@ -397,7 +781,7 @@ int launch_block_apply(const float* binv, const double* x, double* z, int64_t n_
 
 #define TS_INST_BLOCK(T, N)                                                                          \
   template int launch_block_diag<T, N>(int, int, const int32_t*, const int32_t*, const int4*, const T*, \
-                                       const T*, const T*, const uint8_t*, const float*, Phys<float>,  \
+                                       const T*, const T*, const T*, const uint8_t*, const float*, Phys<float>,  \
                                        float*, int64_t, unsigned*, cudaStream_t);
 TS_FOR_EACH_N(TS_INST_BLOCK, float)
 TS_FOR_EACH_N(TS_INST_BLOCK, double)
