@@ -139,6 +139,7 @@ struct ts_problem {
   double *d_w = nullptr, *d_r = nullptr, *d_dy = nullptr, *d_partial = nullptr, *d_h = nullptr;
   float *d_v32 = nullptr, *d_w32 = nullptr;
   double *d_D = nullptr, *d_t = nullptr;      // preconditioner diagonal (inverted), temp
+  double* d_dpart = nullptr;                  // [E][4][3] element parts of that diagonal
   float* d_binv = nullptr;                    // inverted nodal blocks [V][8N][8N] (block Jacobi)
   bool binv_valid = false;                    // d_binv built at the current linearisation state
   float* d_eig = nullptr;                     // eigenpairs of M per point [E*4][EIG] (exact tangent)
@@ -391,7 +392,7 @@ static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T
   a.omega = PV::of(ph.omega);
   a.n_elem = m->E;
   if (launch_element<V, N>(mode, a, st)) return fail(TS_ERR_CUDA, "element kernel launch failed");
-  if (launch_gather<V>(m->d_node_off, m->d_node_elem, (const V*)l.rows, pr->d_dmask, out, m->V, pr->C, st))
+  if (launch_gather<V>(m->d_node_off, m->d_node_elem, (const V*)l.rows, pr->d_dmask, out, m->V, pr->C, 4, 3, st))
     return fail(TS_ERR_CUDA, "gather kernel launch failed");
   return outlet_terms<T>(pr, v, res ? 0 : 1, out, st);
 }
@@ -659,13 +660,11 @@ static int j32_boundary_impl(ts_problem* pr, const float* v, float* hv, cudaStre
 
 static int precond_diag(ts_problem* pr, const double* y, double* D, cudaStream_t st) {
   TS_TRY(sync_dmask(pr));
-  TS_CUDA(cudaMemsetAsync(D, 0, field_len(pr) * sizeof(double), st));
-  const ts_mesh* msh = pr->mesh;
-  Phys<double> ph = phys_of<double>(pr, true);
-  for (size_t c = 0; c + 1 < msh->colour_off.size(); ++c)
-    if (launch_diag(msh->d_tets, msh->d_geo64, y, pr->p.N, ph, D, msh->colour_off[c], msh->colour_off[c + 1], st))
-      return fail(TS_ERR_CUDA, "diag kernel");
-  if (launch_diag_invert(D, pr->d_dmask, msh->V, pr->C, st)) return fail(TS_ERR_CUDA, "diag invert");
+  const ts_mesh* m = pr->mesh;
+  if (!pr->d_dpart) TS_TRY(dalloc(&pr->d_dpart, (size_t)m->E * 12));
+  if (launch_diag(m->d_tets, m->d_geo64, y, pr->p.N, phys_of<double>(pr, true), m->d_node_off, m->d_node_elem,
+                  pr->d_dmask, pr->d_dpart, D, m->E, m->V, st))
+    return fail(TS_ERR_CUDA, "diagonal kernel launch failed");
   return 0;
 }
 
@@ -1166,6 +1165,7 @@ void ts_problem_free(ts_problem* pr) {
   dfree(pr->d_v32);
   dfree(pr->d_w32);
   dfree(pr->d_D);
+  dfree(pr->d_dpart);
   dfree(pr->d_t);
   dfree(pr->d_binv);
   dfree(pr->d_eig);
@@ -1582,9 +1582,15 @@ struct ts_tracer {
   std::vector<uint8_t> dmask;
   uint8_t* d_dmask = nullptr;
   bool dirty = true;
-  double *a4_64 = nullptr, *tau64 = nullptr, *dft64 = nullptr;
-  float *a4_32 = nullptr, *tau32 = nullptr, *dft32 = nullptr;
-  float2* add = nullptr;             // a4_64 as double-float pairs
+  // per precision: velocity in the flow layout [V][4][C], tau, trigonometric table,
+  // velocity on samples [V][3][K], phi without Im(mode 0), element rows [E][4][C]
+  template <typename T>
+  struct Work {
+    T *a4 = nullptr, *tau = nullptr, *trig = nullptr, *at = nullptr, *phi = nullptr, *rows = nullptr;
+  };
+  Work<double> w64;
+  Work<float> w32;
+  float2* add = nullptr;             // the FP64 velocity as double-float pairs
   unsigned* d_counter = nullptr;
   int gls = 1;                       // 0: Galerkin terms only (no least-squares term)
   // solve workspace (FP64)
@@ -1595,53 +1601,55 @@ struct ts_tracer {
 namespace {
 
 template <typename T>
-T*& tr_a4(ts_tracer* t);
+ts_tracer::Work<T>& tr_work(ts_tracer* t);
 template <>
-double*& tr_a4<double>(ts_tracer* t) { return t->a4_64; }
+ts_tracer::Work<double>& tr_work<double>(ts_tracer* t) { return t->w64; }
 template <>
-float*& tr_a4<float>(ts_tracer* t) { return t->a4_32; }
-template <typename T>
-T*& tr_tau(ts_tracer* t);
-template <>
-double*& tr_tau<double>(ts_tracer* t) { return t->tau64; }
-template <>
-float*& tr_tau<float>(ts_tracer* t) { return t->tau32; }
-template <typename T>
-T*& tr_dft(ts_tracer* t);
-template <>
-double*& tr_dft<double>(ts_tracer* t) { return t->dft64; }
-template <>
-float*& tr_dft<float>(ts_tracer* t) { return t->dft32; }
+ts_tracer::Work<float>& tr_work<float>(ts_tracer* t) { return t->w32; }
 
-// advecting velocity and tau of the tracer (once per velocity)
+// cos, sin of 2 pi n k / K, k = 0..K/2, in the tracer's own types
+template <typename T>
+int upload_trig_plain(int N, T** out) {
+  const int K = 3 * N - 2, KH = K / 2, n1 = N * (KH + 1);
+  const double pi = 3.14159265358979323846;
+  std::vector<T> t(2 * n1);
+  for (int n = 0; n < N; ++n)
+    for (int k = 0; k <= KH; ++k) {
+      const double th = 2.0 * pi * ((n * k) % K) / K;
+      t[n * (KH + 1) + k] = (T)std::cos(th);
+      t[n1 + n * (KH + 1) + k] = (T)std::sin(th);
+    }
+  TS_TRY(dalloc(out, t.size()));
+  TS_CUDA(cudaMemcpy(*out, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice));
+  return 0;
+}
+
+// advecting velocity (flow layout, samples) and tau of the tracer, once per velocity
 template <typename T, int N>
 int tracer_prepare(ts_tracer* tr, const T* a, cudaStream_t st) {
   const ts_mesh* m = tr->mesh;
-  T*& a4 = tr_a4<T>(tr);
-  T*& tau = tr_tau<T>(tr);
-  T*& dft = tr_dft<T>(tr);
-  if (!a4) TS_TRY(dalloc(&a4, (size_t)m->V * 4 * tr->C));
-  if (!tau) TS_TRY(dalloc(&tau, (size_t)m->E * 4 * tr->NTP));
-  if (!dft) {
-    std::vector<double> tab;
-    dft_tables(N, tab);
-    std::vector<T> tt(tab.begin(), tab.end());
-    TS_TRY(dalloc(&dft, tt.size()));
-    TS_CUDA(cudaMemcpy(dft, tt.data(), tt.size() * sizeof(T), cudaMemcpyHostToDevice));
-  }
+  ts_tracer::Work<T>& w = tr_work<T>(tr);
+  const int64_t n = m->V * 4 * (int64_t)tr->C;
+  if (!w.a4) TS_TRY(dalloc(&w.a4, (size_t)n));
+  if (!w.at) TS_TRY(dalloc(&w.at, (size_t)m->V * 3 * (3 * N - 2)));
+  if (!w.phi) TS_TRY(dalloc(&w.phi, (size_t)m->V * tr->C));
+  if (!w.rows) TS_TRY(dalloc(&w.rows, (size_t)m->E * 4 * tr->C));
+  if (!w.tau) TS_TRY(dalloc(&w.tau, (size_t)m->E * 4 * tr->NTP));
+  if (!w.trig) TS_TRY(upload_trig_plain<T>(N, &w.trig));
   if (tr->dirty) {
     TS_CUDA(cudaMemcpy(tr->d_dmask, tr->dmask.data(), tr->dmask.size(), cudaMemcpyHostToDevice));
     tr->dirty = false;
   }
-  if (launch_repack_velocity<T>(a, a4, m->V, tr->C, st)) return fail(TS_ERR_CUDA, "repack kernel launch failed");
+  if (launch_repack_velocity<T>(a, w.a4, m->V, tr->C, st)) return fail(TS_ERR_CUDA, "repack kernel launch failed");
+  if (launch_node_prepass<T, N>(w.a4, nullptr, nullptr, w.at, w.trig, m->V, st))
+    return fail(TS_ERR_CUDA, "node pre-pass launch failed");
   int rc;
   if constexpr (sizeof(T) == 8) {
-    const int64_t n = m->V * 4 * (int64_t)tr->C;
     if (!tr->add) TS_TRY(dalloc(&tr->add, (size_t)n));
-    if (launch_split_dd(a4, tr->add, n, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
-    rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, tr->add, m->E, tau, tr->kappa, tr->C_I, tr->d_counter, st);
+    if (launch_split_dd(w.a4, tr->add, n, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
+    rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, tr->add, m->E, w.tau, tr->kappa, tr->C_I, tr->d_counter, st);
   } else {
-    rc = launch_tau<float, N>(m->d_tets, m->d_geo32, a4, m->E, tau, (float)tr->kappa, (float)tr->C_I,
+    rc = launch_tau<float, N>(m->d_tets, m->d_geo32, w.a4, m->E, w.tau, (float)tr->kappa, (float)tr->C_I,
                               tr->d_counter, st);
   }
   if (rc) return fail(TS_ERR_CUDA, "tau kernel launch failed");
@@ -1652,12 +1660,23 @@ int tracer_prepare(ts_tracer* tr, const T* a, cudaStream_t st) {
 template <typename T, int N>
 int tracer_apply(ts_tracer* tr, const T* phi, T* r, cudaStream_t st) {
   const ts_mesh* m = tr->mesh;
-  TS_CUDA(cudaMemsetAsync(r, 0, (size_t)m->V * tr->C * sizeof(T), st));
-  for (size_t c = 0; c + 1 < m->colour_off.size(); ++c)
-    if (launch_tracer<T, N>(m->d_tets, geo_of<T>(m), tr_a4<T>(tr), phi, tr_tau<T>(tr), tr->d_dmask, r,
-                            tr_dft<T>(tr), tr->kappa, tr->omega, m->colour_off[c], m->colour_off[c + 1], st,
-                            tr->gls))
-      return fail(TS_ERR_CUDA, "tracer kernel launch failed");
+  ts_tracer::Work<T>& w = tr_work<T>(tr);
+  if (launch_clean<T>(phi, w.phi, m->V * (int64_t)tr->C, tr->C, st)) return fail(TS_ERR_CUDA, "tracer kernel launch failed");
+  TracerArgs<T> a;
+  a.tets = m->d_tets;
+  a.geo = geo_of<T>(m);
+  a.at = w.at;
+  a.phi = w.phi;
+  a.tau = w.tau;
+  a.trig = w.trig;
+  a.rows = w.rows;
+  a.omega = (T)tr->omega;
+  a.kappa4 = (T)(4.0 * tr->kappa);
+  a.n_elem = m->E;
+  a.gls = tr->gls;
+  if (launch_tracer<T, N>(a, st)) return fail(TS_ERR_CUDA, "tracer kernel launch failed");
+  if (launch_gather<T>(m->d_node_off, m->d_node_elem, w.rows, tr->d_dmask, r, m->V, tr->C, 1, 1, st))
+    return fail(TS_ERR_CUDA, "gather kernel launch failed");
   return 0;
 }
 
@@ -1810,13 +1829,19 @@ void ts_tracer_free(ts_tracer* t) {
   dfree(t->h);
   dfree(t->d_dmask);
   dfree(t->d_counter);
-  dfree(t->a4_64);
   dfree(t->add);
-  dfree(t->tau64);
-  dfree(t->dft64);
-  dfree(t->a4_32);
-  dfree(t->tau32);
-  dfree(t->dft32);
+  dfree(t->w64.a4);
+  dfree(t->w64.tau);
+  dfree(t->w64.trig);
+  dfree(t->w64.at);
+  dfree(t->w64.phi);
+  dfree(t->w64.rows);
+  dfree(t->w32.a4);
+  dfree(t->w32.tau);
+  dfree(t->w32.trig);
+  dfree(t->w32.at);
+  dfree(t->w32.phi);
+  dfree(t->w32.rows);
   delete t;
 }
 
@@ -2130,7 +2155,7 @@ int ts_solve(ts_problem* pr, void* y_inout, const ts_solve_opts* opts, ts_solve_
         const double tj = now_s();
         TS_CUDA(cudaEventRecord(pr->ev_a, st));
         double* vk = V + (int64_t)k * n;
-        if (o.precond == 1) {
+        if (o.precond == 1 && o.precision != 32) {
           if (vec_mul(pr->d_t, pr->d_D, vk, n, st)) return fail(TS_ERR_CUDA, "mul");
           vk = pr->d_t;
         } else if (o.precond == 2) {
@@ -2141,7 +2166,8 @@ int ts_solve(ts_problem* pr, void* y_inout, const ts_solve_opts* opts, ts_solve_
           vk = pr->d_t;
         }
         if (o.precision == 32) {
-          if (vec_cast_d2f(pr->d_v32, vk, n, st)) return fail(TS_ERR_CUDA, "cast");
+          if (o.precond == 1 ? vec_mul_d2f(pr->d_v32, pr->d_D, vk, n, st) : vec_cast_d2f(pr->d_v32, vk, n, st))
+            return fail(TS_ERR_CUDA, "cast");
           TS_TRY(ts_jvp(pr, pr->d_v32, pr->d_w32, 32, st));
           if (vec_cast_f2d(pr->d_w, pr->d_w32, n, st)) return fail(TS_ERR_CUDA, "cast");
         } else {

@@ -440,231 +440,6 @@ int launch_apply(int mode, const int4* tets, const T* geo, const T* v, const T* 
   return -1;
 }
 
-// ---------------------------------------------------------------- tracer
-// Time-spectral GLS convection-diffusion of a scalar phi (eq. 3D-weak with
-// eq. 3D-weak-def, section 2.2) advected by a given velocity a: per element
-// and quadrature point (weights V/4)
-//   res  = Omega phi + A_j dphi/dx_j          (A_j = A(a_j), eq. phi-def)
-//   T    = tau res                            (tau of eq. 3D-tau with kappa)
-//   r_a += w [N_a res - N_a Omega T + dN_a/dx_j A_j T] + kappa V dN_a/dx_j dphi/dx_j
-// The products A_j x are formed on K = 3N - 2 time samples, as in the flow
-// operator; the SUPG sum sum_q w A_j T is transformed once per element.
-template <int N>
-struct TracerLayout {
-  using D = Dims<N>;
-  static constexpr int C = D::C, K = D::K, NM = D::NM;
-  static constexpr int LDF = C | 1, LDI = K | 1;
-  static constexpr int TABLES = K * LDF + C * LDI;
-  static constexpr int SG = 0;              // geometry 20 (+4)
-  static constexpr int PH = 24;             // phi at nodes [4][C]
-  static constexpr int AN = PH + 4 * C;     // a at nodes [4][3][C]
-  static constexpr int GP = AN + 12 * C;    // grad phi [3][C]
-  static constexpr int PQ = GP + 3 * C;     // phi at points [4][C]
-  static constexpr int AQ = PQ + 4 * C;     // a at points [4][3][C]
-  static constexpr int AQT = AQ + 12 * C;   // a samples [4][3][K]
-  static constexpr int GPT = AQT + 12 * K;  // grad phi samples [3][K], later W samples
-  static constexpr int CT = GPT + 3 * K;    // c samples [4][K], later T samples
-  static constexpr int RES = CT + 4 * K;    // res modes [4][C]
-  static constexpr int TQ = RES + 4 * C;    // T modes [4][C]
-  static constexpr int WM = TQ + 4 * C;     // W modes [3][C]
-  static constexpr int TAU = WM + 3 * C;    // tau [4][NM][NM] (storage scaling)
-  static constexpr int OUT = TAU + 4 * NM * NM;   // [4][C]
-  static constexpr int WARP = (OUT + 4 * C + 3) & ~3;
-};
-
-template <typename T, int N, typename S = T>
-__global__ void __launch_bounds__(128)
-    tracer_kernel(const int4* __restrict__ tets, const S* __restrict__ geo, const S* __restrict__ a4,
-                  const S* __restrict__ phi, const S* __restrict__ tau, const uint8_t* __restrict__ dmask,
-                  S* __restrict__ out, const S* __restrict__ dft, T kappa, T omega, int64_t e0, int64_t e1,
-                  int gls) {
-  using D = Dims<N>;
-  using L = TracerLayout<N>;
-  constexpr int C = D::C, K = D::K, NM = D::NM, NT = D::NT, NTP = D::NT_PAD;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sF = reinterpret_cast<T*>(smem_raw);
-  T* sI = sF + K * L::LDF;
-  for (int t = threadIdx.x; t < K * C; t += blockDim.x) {
-    const int kk = t / C, c = t - kk * C;
-    sF[kk * L::LDF + c] = T(dft[t]);
-  }
-  for (int t = threadIdx.x; t < C * K; t += blockDim.x) {
-    const int c = t / K, kk = t - c * K;
-    sI[c * L::LDI + kk] = T(dft[K * C + t]);
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* ws = sF + L::TABLES + warp * L::WARP;
-  T* sg = ws + L::SG;
-  T* ph = ws + L::PH;
-  T* an = ws + L::AN;
-  T* gp = ws + L::GP;
-  T* pq = ws + L::PQ;
-  T* aq = ws + L::AQ;
-  T* aqt = ws + L::AQT;
-  T* gpt = ws + L::GPT;
-  T* ct = ws + L::CT;
-  T* res = ws + L::RES;
-  T* tq = ws + L::TQ;
-  T* wm = ws + L::WM;
-  T* st = ws + L::TAU;
-  T* so = ws + L::OUT;
-  const int wpb = blockDim.x >> 5;
-  for (int64_t e = e0 + (int64_t)blockIdx.x * wpb + warp; e < e1; e += (int64_t)gridDim.x * wpb) {
-    const int4 nd = tets[e];
-    const int node[4] = {nd.x, nd.y, nd.z, nd.w};
-    if (lane < GEO_STRIDE) sg[lane] = T(geo[e * GEO_STRIDE + lane]);
-    for (int t = lane; t < 4 * C; t += 32) {
-      const int a = t / C, c = t - a * C;
-      ph[t] = c == 1 ? T(0) : T(phi[(int64_t)node[a] * C + c]);
-    }
-    for (int t = lane; t < 12 * C; t += 32) {
-      const int a = t / (3 * C), r = t - a * 3 * C;
-      const int c = r % C;
-      an[t] = c == 1 ? T(0) : T(a4[(int64_t)node[a] * 4 * C + r]);
-    }
-    {
-      const S* tp = tau + e * 4 * NTP;
-      for (int t = lane; t < 4 * NTP; t += 32) {
-        const int q = t / NTP, p = t - q * NTP;
-        if (p >= NT) continue;
-        int r = 0, rem = p;
-        while (rem >= NM - r) {
-          rem -= NM - r;
-          ++r;
-        }
-        const int s2 = r + rem;
-        const T val = T(tp[t]);
-        const T drs = (r == 0 && s2 > 0) ? sqrt2_of<T>() : T(1);
-        const T dsr = (r == 0 && s2 > 0) ? inv_sqrt2_of<T>() : T(1);
-        st[q * NM * NM + r * NM + s2] = val * drs;
-        st[q * NM * NM + s2 * NM + r] = val * dsr;
-      }
-    }
-    __syncwarp();
-    const T vol = sg[GEO_VOL], w4 = T(0.25) * vol;
-    for (int t = lane; t < 3 * C; t += 32) {
-      const int j = t / C, c = t - j * C;
-      T acc = 0;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) acc += sg[a * 3 + j] * ph[a * C + c];
-      gp[t] = acc;
-    }
-    for (int t = lane; t < 4 * C; t += 32) {
-      const int q = t / C, c = t - q * C;
-      T acc = 0;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) acc += T(qp_bary(q, a)) * ph[a * C + c];
-      pq[t] = acc;
-    }
-    for (int t = lane; t < 12 * C; t += 32) {
-      const int q = t / (3 * C), r = t - q * 3 * C;
-      T acc = 0;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) acc += T(qp_bary(q, a)) * an[a * 3 * C + r];
-      aq[t] = acc;
-    }
-    __syncwarp();
-    warp_bmv<T, K, C>(sF, L::LDF, aq, C, aqt, K, 12, lane);
-    warp_bmv<T, K, C>(sF, L::LDF, gp, C, gpt, K, 3, lane);
-    __syncwarp();
-    // convective product on samples c(q, t) = sum_j a_j(q, t) dphi/dx_j(t)
-    for (int t = lane; t < 4 * K; t += 32) {
-      const int q = t / K, kk = t - q * K;
-      T acc = 0;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) acc += aqt[(q * 3 + j) * K + kk] * gpt[j * K + kk];
-      ct[t] = acc;
-    }
-    __syncwarp();
-    warp_bmv<T, C, K>(sI, L::LDI, ct, K, res, C, 4, lane);
-    __syncwarp();
-    for (int t = lane; t < 4 * C; t += 32) {
-      const int c = t % C;
-      res[t] = c == 1 ? T(0) : omega_apply(pq + (t - c), c, omega) + res[t];
-    }
-    __syncwarp();
-    // T = tau res (storage coordinates)
-    for (int t = lane; t < 4 * NM; t += 32) {
-      const int q = t / NM, r = t - q * NM;
-      const T* tr = st + q * NM * NM + r * NM;
-      const T* rq = res + q * C;
-      T acc = 0;
-#pragma unroll
-      for (int kk = 0; kk < NM; ++kk) acc = mad(tr[kk], rq[stor_of(kk)], acc);
-      tq[q * C + stor_of(r)] = gls ? acc : T(0);   // Galerkin only: no least-squares term
-    }
-    for (int q = lane; q < 4; q += 32) tq[q * C + 1] = T(0);
-    __syncwarp();
-    warp_bmv<T, K, C>(sF, L::LDF, tq, C, ct, K, 4, lane);
-    __syncwarp();
-    // SUPG sums on samples W_j(t) = sum_q a_j(q, t) T(q, t)
-    for (int t = lane; t < 3 * K; t += 32) {
-      const int j = t / K, kk = t - j * K;
-      T acc = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc += aqt[(q * 3 + j) * K + kk] * ct[q * K + kk];
-      gpt[t] = acc;
-    }
-    __syncwarp();
-    warp_bmv<T, C, K>(sI, L::LDI, gpt, K, wm, C, 3, lane);
-    __syncwarp();
-    for (int t = lane; t < 4 * C; t += 32) {
-      const int a = t / C, c = t - a * C;
-      T acc = 0;
-      if (c != 1) {
-        T gal = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const T lam = T(qp_bary(q, a));
-          gal += lam * (res[q * C + c] - omega_apply(tq + q * C, c, omega));
-        }
-        T supg = 0, diff = 0;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          supg += sg[a * 3 + j] * wm[j * C + c];
-          diff += sg[a * 3 + j] * gp[j * C + c];
-        }
-        acc = w4 * (gal + supg) + kappa * vol * diff;
-      }
-      so[t] = acc;
-    }
-    __syncwarp();
-    for (int t = lane; t < 4 * C; t += 32) {
-      const int a = t / C, c = t - a * C;
-      if (c == 1 || dmask[node[a]]) continue;
-      out[(int64_t)node[a] * C + c] += static_cast<S>(so[t]);
-    }
-    __syncwarp();
-  }
-}
-
-template <typename T, int N, typename S>
-static int launch_tracer_t(const int4* tets, const S* geo, const S* a4, const S* phi, const S* tau,
-                           const uint8_t* dmask, S* out, const S* dft, double kappa, double omega,
-                           int64_t e0, int64_t e1, cudaStream_t st, int gls) {
-  using L = TracerLayout<N>;
-  if (e1 <= e0) return 0;
-  int warps = 4;
-  while (warps > 1 && (size_t)(L::TABLES + warps * L::WARP) * sizeof(T) > 200 * 1024) --warps;
-  const size_t smem = (size_t)(L::TABLES + warps * L::WARP) * sizeof(T);
-  if (smem > 227 * 1024) return -6;
-  cudaFuncSetAttribute(tracer_kernel<T, N, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int64_t blocks = (e1 - e0 + warps - 1) / warps;
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  count_launches(1);
-  tracer_kernel<T, N, S><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, a4, phi, tau, dmask, out, dft,
-                                                                T(kappa), T(omega), e0, e1, gls);
-  return cudaGetLastError() == cudaSuccess ? 0 : -2;
-}
-
-template <typename T, int N>
-int launch_tracer(const int4* tets, const T* geo, const T* a4, const T* phi, const T* tau,
-                  const uint8_t* dmask, T* out, const T* dft, double kappa, double omega, int64_t e0,
-                  int64_t e1, cudaStream_t st, int gls) {
-  return launch_tracer_t<T, N, T>(tets, geo, a4, phi, tau, dmask, out, dft, kappa, omega, e0, e1, st, gls);
-}
-
 // a [V][3][C] -> a4 [V][4][C] (the flow layout the tau kernels read; pressure zero)
 template <typename T>
 __global__ void repack_velocity_kernel(const T* __restrict__ a, T* __restrict__ a4, int64_t V, int C) {
@@ -688,50 +463,39 @@ template int launch_repack_velocity<float>(const float*, float*, int64_t, int, c
 template int launch_repack_velocity<double>(const double*, double*, int64_t, int, cudaStream_t);
 
 // ---------------------------------------------------------------- outlets
-// One block per call: Q_c = sum_A sum_i w_Ai v[A][i][c]; out[A][i][c] += R w_Ai Q_c.
-// Thread t owns the outlet nodes t, t + blockDim, ... and keeps its partial
-// flow rates of all C coefficients in its own column of part[C][blockDim]
-// (the loads of a node are independent, so one node costs one memory round
-// trip, not one per coefficient); warp w then sums the columns of the
-// coefficients c = w, w + nw, ... in a fixed order (deterministic), and the
-// threads scatter to their own nodes.
+// Q_c = sum_A sum_i w_Ai v[A][i][c]; out[A][i][c] += R w_Ai Q_c.  One block a
+// stored coordinate c: the coordinates do not depend on each other, so a block
+// sums its flow rate (fixed order: threads over nodes, then a tree) and adds it to
+// its own entries in the same launch.  Latency-bound: 81 nodes, C = 6 and 529
+// nodes, C = 14 took 10 and 31 us with all coordinates in one block.
 template <typename T>
-__global__ void __launch_bounds__(256) outlet_kernel(const int32_t* __restrict__ nodes,
+__global__ void __launch_bounds__(128) outlet_kernel(const int32_t* __restrict__ nodes,
                                                      const T* __restrict__ w, int n, T R,
                                                      const T* __restrict__ v,
                                                      const uint8_t* __restrict__ dmask, int mask_input,
                                                      T* __restrict__ out, int C) {
-  extern __shared__ __align__(16) unsigned char outlet_smem[];
-  T* part = reinterpret_cast<T*>(outlet_smem);   // [C][blockDim.x]
-  T* Q = part + (int64_t)C * blockDim.x;         // [C]
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-  for (int c = 0; c < C; ++c) part[c * nt + tid] = T(0);
+  __shared__ T part[4];
+  const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31;
+  const int c = blockIdx.x == 0 ? 0 : blockIdx.x + 1;   // Im(mode 0) is left out
+  T acc = 0;
   for (int b = tid; b < n; b += nt) {
     const int A = nodes[b];
     if (mask_input && dmask[A]) continue;
-    const T w0 = w[b * 3 + 0], w1 = w[b * 3 + 1], w2 = w[b * 3 + 2];
-    const T* va = v + (int64_t)A * 4 * C;
-    for (int c = 0; c < C; ++c) part[c * nt + tid] += w0 * va[c] + w1 * va[C + c] + w2 * va[2 * C + c];
+    const T* va = v + (int64_t)A * 4 * C + c;
+    acc += w[b * 3 + 0] * va[0] + w[b * 3 + 1] * va[C] + w[b * 3 + 2] * va[2 * C];
   }
-  __syncthreads();
-  for (int c = warp; c < C; c += nw) {
-    T acc = 0;
-    for (int k = lane; k < nt; k += 32) acc += part[c * nt + k];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) Q[c] = (c == 1) ? T(0) : acc;
-  }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) part[warp] = acc;
   __syncthreads();
+  const T q = R * ((part[0] + part[1]) + (part[2] + part[3]));
   for (int b = tid; b < n; b += nt) {
     const int A = nodes[b];
     if (dmask[A]) continue;
-    T* oa = out + (int64_t)A * 4 * C;
-    for (int i = 0; i < 3; ++i) {
-      const T s = R * w[b * 3 + i];
-      for (int c = 0; c < C; ++c)
-        if (c != 1) oa[i * C + c] += s * Q[c];
-    }
+    T* oa = out + (int64_t)A * 4 * C + c;
+    oa[0] += q * w[b * 3 + 0];
+    oa[C] += q * w[b * 3 + 1];
+    oa[2 * C] += q * w[b * 3 + 2];
   }
 }
 
@@ -739,15 +503,8 @@ template <typename T>
 int launch_outlet(const int32_t* nodes, const T* w, int n_nodes, T R, const T* v,
                   const uint8_t* dmask, int mask_input, T* out, int C, cudaStream_t st) {
   if (n_nodes <= 0) return 0;
-  if (C > 128) return -1;
-  const int threads = 256;
-  const size_t smem = ((size_t)C * threads + C) * sizeof(T);
-  if (smem > 227 * 1024) return -1;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(outlet_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return -2;
   count_launches(1);
-  outlet_kernel<T><<<1, threads, smem, st>>>(nodes, w, n_nodes, R, v, dmask, mask_input, out, C);
+  outlet_kernel<T><<<C - 1, 128, 0, st>>>(nodes, w, n_nodes, R, v, dmask, mask_input, out, C);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
@@ -787,10 +544,5 @@ TS_FOR_EACH_N(TS_INST_APPLY, float)
 #define TS_INST_PRELOAD_APPLY(T, N) template int preload_apply_residual<T, N>();
 TS_FOR_EACH_N(TS_INST_PRELOAD_APPLY, float)
 TS_FOR_EACH_N(TS_INST_APPLY, double)
-#define TS_INST_TRACER(T, N)                                                                        \
-  template int launch_tracer<T, N>(const int4*, const T*, const T*, const T*, const T*, const uint8_t*, \
-                                   T*, const T*, double, double, int64_t, int64_t, cudaStream_t, int);
-TS_FOR_EACH_N(TS_INST_TRACER, float)
-TS_FOR_EACH_N(TS_INST_TRACER, double)
 
 }  // namespace ts

@@ -66,6 +66,27 @@ struct Ar<float> {
   static __device__ __forceinline__ float to(float x) { return x; }
 };
 
+// FP64 as it is (the tracer: its residual has always been native FP64)
+template <>
+struct Ar<double> {
+  struct Acc {
+    double s;
+    __device__ __forceinline__ Acc(double v) : s(v) {}
+    __device__ __forceinline__ void add(double a, double b) { s = ::fma(a, b, s); }
+    __device__ __forceinline__ double get() const { return s; }
+  };
+  static __device__ __forceinline__ double zero() { return 0.0; }
+  static __device__ __forceinline__ double of(double x) { return x; }
+  static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+  static __device__ __forceinline__ double sub(double a, double b) { return a - b; }
+  static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+  static __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
+  static __device__ __forceinline__ double neg(double a) { return -a; }
+  static __device__ __forceinline__ double twice(double a) { return a + a; }
+  static __device__ __forceinline__ double from(double x) { return x; }
+  static __device__ __forceinline__ double to(double x) { return x; }
+};
+
 template <>
 struct Ar<float2> {
   static __device__ __forceinline__ dd d(float2 a) { return dd{a.x, a.y}; }
@@ -179,14 +200,15 @@ __device__ __forceinline__ void forward_row(const V (&x)[2 * N], V* out, const V
   }
 }
 
-// out[j * CS] = d/dx_j of entry fc of the field x
+// out[j * CS] = d/dx_j of entry fc of the field x (`stride` entries a node)
 template <typename V, int C, int CS>
-__device__ __forceinline__ void gradient_of(const V* __restrict__ x, const int* nd, int fc, const V* dN, V* out) {
+__device__ __forceinline__ void gradient_of(const V* __restrict__ x, const int* nd, int fc, int stride, const V* dN,
+                                            V* out) {
   using R = Ar<V>;
-  const V x0 = x[(int64_t)nd[0] * 4 * C + fc];
+  const V x0 = x[(int64_t)nd[0] * stride + fc];
   V d[3];
 #pragma unroll
-  for (int a = 1; a < 4; ++a) d[a - 1] = R::sub(x[(int64_t)nd[a] * 4 * C + fc], x0);
+  for (int a = 1; a < 4; ++a) d[a - 1] = R::sub(x[(int64_t)nd[a] * stride + fc], x0);
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     typename R::Acc s(R::zero());
@@ -237,13 +259,13 @@ __global__ void __launch_bounds__(EL_THREADS) element_kernel(ElementArgs<V> P) {
     for (int t = tid; t < nel * 4 * C; t += EL_THREADS) {
       const int el = t / (4 * C), fc = t - el * 4 * C, f = fc / C, c = fc - f * C;
       V* E = es + el * L::ELEM;
-      gradient_of<V, C, CS>(P.vd, nodes + 4 * el, fc, E + L::GEO, E + L::GM + f * 3 * CS + c);
+      gradient_of<V, C, CS>(P.vd, nodes + 4 * el, fc, 4 * C, E + L::GEO, E + L::GM + f * 3 * CS + c);
     }
     if constexpr (LINA) {
       for (int t = tid; t < nel * 3 * C; t += EL_THREADS) {
         const int el = t / (3 * C), fc = t - el * 3 * C, f = fc / C, c = fc - f * C;
         V* E = es + el * L::ELEM;
-        gradient_of<V, C, CS>(P.ud, nodes + 4 * el, fc, E + L::GEO, E + L::M1 + f * 3 * CS + c);
+        gradient_of<V, C, CS>(P.ud, nodes + 4 * el, fc, 4 * C, E + L::GEO, E + L::M1 + f * 3 * CS + c);
       }
     }
 #pragma unroll 1
@@ -547,28 +569,31 @@ __global__ void __launch_bounds__(128) node_prepass_kernel(const typename StoreO
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       x[c] = c == 1 || fixed ? R::zero() : R::from(y[t * C + c]);
-      clean[t * C + c] = x[c];
+      if (clean) clean[t * C + c] = x[c];
       if (c > 1) x[c] = R::twice(x[c]);
     }
     if (f < 3) forward_row<V, N, 1>(x, samples + (node * 3 + f) * K, table, table + N * (KH + 1), 0);
   }
 }
 
-// out[node][f][c] = sum of the node's element rows; fixed rows are zero
+// out[node][f][c] = sum of the node's element rows; Im(mode 0) and, on Dirichlet
+// nodes, the first `masked` of the fields are zero
 template <typename V>
 __global__ void __launch_bounds__(256) gather_kernel(const int32_t* __restrict__ node_off,
                                                      const int32_t* __restrict__ node_elem,
                                                      const V* __restrict__ rows, const uint8_t* __restrict__ dmask,
-                                                     typename StoreOf<V>::S* __restrict__ out, int64_t n_nodes, int C) {
+                                                     typename StoreOf<V>::S* __restrict__ out, int64_t n_nodes, int C,
+                                                     int fields, int masked) {
   using R = Ar<V>;
-  const int64_t total = n_nodes * 4 * C;
+  const int FC = fields * C;
+  const int64_t total = n_nodes * FC;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t node = t / (4 * C);
-    const int fc = (int)(t - node * 4 * C), f = fc / C, c = fc - f * C;
+    const int64_t node = t / FC;
+    const int fc = (int)(t - node * FC), f = fc / C, c = fc - f * C;
     V s = R::zero();
-    if (c != 1 && !(f < 3 && dmask[node])) {
+    if (c != 1 && !(f < masked && dmask[node])) {
       const int p1 = node_off[node + 1];
-      for (int p = node_off[node]; p < p1; ++p) s = R::add(s, rows[(int64_t)node_elem[p] * 4 * C + fc]);
+      for (int p = node_off[node]; p < p1; ++p) s = R::add(s, rows[(int64_t)node_elem[p] * FC + fc]);
     }
     out[t] = R::to(s);
   }
@@ -611,11 +636,236 @@ int launch_node_prepass(const typename StoreOf<V>::S* y, const uint8_t* dmask, V
 
 template <typename V>
 int launch_gather(const int32_t* node_off, const int32_t* node_elem, const V* rows, const uint8_t* dmask,
-                  typename StoreOf<V>::S* out, int64_t n_nodes, int C, cudaStream_t st) {
+                  typename StoreOf<V>::S* out, int64_t n_nodes, int C, int fields, int masked, cudaStream_t st) {
   if (n_nodes <= 0) return 0;
-  const int64_t blocks = std::min<int64_t>((n_nodes * 4 * C + 255) / 256, 152 * 64);
+  const int64_t blocks = std::min<int64_t>((n_nodes * fields * C + 255) / 256, 152 * 64);
   count_launches(1);
-  gather_kernel<V><<<(int)blocks, 256, 0, st>>>(node_off, node_elem, rows, dmask, out, n_nodes, C);
+  gather_kernel<V><<<(int)blocks, 256, 0, st>>>(node_off, node_elem, rows, dmask, out, n_nodes, C, fields, masked);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}
+
+// ---------------------------------------------------------------- tracer
+// Time-spectral GLS convection-diffusion of a scalar phi (eq. 3D-weak with
+// eq. 3D-weak-def, section 2.2) advected by a given velocity a: per element and
+// quadrature point (weights V/4)
+//   res  = Omega phi + A_j dphi/dx_j          (A_j = A(a_j), eq. phi-def)
+//   T    = tau res                            (tau of eq. 3D-tau with kappa)
+//   r_a += w [N_a res - N_a Omega T + dN_a/dx_j A_j T] + kappa V dN_a/dx_j dphi/dx_j
+// The flow operator's structure with one field: an element takes 3 forward
+// transforms of grad phi, 4 inverse ones of the products at the nodes, 4 forward
+// ones of T and 3 inverse ones of the SUPG sums.  N = 7, 26,784 tetrahedra, FP64:
+// 1.33 ms with one warp an element in 30 coloured launches; bound by the FP64
+// pipe, about 3 k multiply-adds an element.
+template <typename V, int N>
+struct TracerLayout {
+  static constexpr int C = 2 * N, K = 3 * N - 2, KH = K / 2, KS = K | 1, CS = C | 1;
+  static constexpr int EB = N <= 7 ? 8 : 4, PARTS = EL_THREADS / (4 * EB);   // lanes a row
+  static constexpr int GEO = 0, A = 13, B = A + 4 * KS, GM = B + 3 * KS, M1 = GM + 3 * CS, M2 = M1 + 4 * CS,
+                       M3 = M2 + 4 * CS, ELEM = (M3 + 4 * CS) | 1;
+  static constexpr int TABLE = 2 * N * (KH + 1) + N;
+  static constexpr size_t BYTES = sizeof(V) * (TABLE + (size_t)EB * ELEM) + EB * 4 * sizeof(int);
+};
+
+template <typename V, int N>
+__global__ void __launch_bounds__(EL_THREADS) tracer_kernel(TracerArgs<V> P) {
+  using R = Ar<V>;
+  using L = TracerLayout<V, N>;
+  constexpr int C = L::C, K = L::K, NM = 2 * N - 1, NTP = Dims<N>::NT_PAD, KH = L::KH, KS = L::KS, CS = L::CS;
+  constexpr int EB = L::EB, PARTS = L::PARTS;
+  extern __shared__ __align__(16) unsigned char el_smem[];
+  V* cosv = reinterpret_cast<V*>(el_smem);
+  V* sinv = cosv + N * (KH + 1);
+  V* om = sinv + N * (KH + 1);
+  V* es = om + N;
+  int* nodes = reinterpret_cast<int*>(es + EB * L::ELEM);
+  const int tid = threadIdx.x;
+  for (int t = tid; t < 2 * N * (KH + 1); t += EL_THREADS) cosv[t] = P.trig[t];
+  for (int t = tid; t < N; t += EL_THREADS) om[t] = R::mul(P.omega, R::of((double)t));
+  const V bq = R::of(qp_bary(0, 1)), dq = R::of(qp_bary(0, 0) - qp_bary(0, 1));
+  const V bqK = R::of(qp_bary(0, 1) / K), dqK = R::of((qp_bary(0, 0) - qp_bary(0, 1)) / K), iK = R::of(1.0 / K);
+
+  for (int64_t e0 = (int64_t)blockIdx.x * EB; e0 < P.n_elem; e0 += (int64_t)gridDim.x * EB) {
+    const int nel = (int)(P.n_elem - e0 < EB ? P.n_elem - e0 : EB);
+    __syncthreads();
+    for (int t = tid; t < nel * 16; t += EL_THREADS) {
+      const int el = t / 16, x = t & 15;
+      if (x < 13) {
+        const V val = R::from(P.geo[(e0 + el) * GEO_STRIDE + (x < 12 ? x : GEO_VOL)]);
+        es[el * L::ELEM + L::GEO + x] = x < 12 ? val : R::mul(val, R::of(0.25));
+      }
+    }
+    for (int t = tid; t < nel * 4; t += EL_THREADS) nodes[t] = reinterpret_cast<const int*>(P.tets + e0)[t];
+    __syncthreads();
+    // ---- gradient: modes, samples; products at the nodes c(a) = a_j(a) dphi/dx_j, times K
+    for (int t = tid; t < nel * C; t += EL_THREADS) {
+      const int el = t / C, c = t - el * C;
+      V* E = es + el * L::ELEM;
+      gradient_of<V, C, CS>(P.phi, nodes + 4 * el, c, C, E + L::GEO, E + L::GM + c);
+    }
+    __syncthreads();
+    for (int t = tid; t < nel * 3 * PARTS; t += EL_THREADS) {
+      const int part = t % PARTS, row = (t / PARTS) % 3, el = t / (3 * PARTS);
+      V* E = es + el * L::ELEM;
+      V x[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        const V v = E[L::GM + row * CS + c];
+        x[c] = c > 1 ? R::twice(v) : v;
+      }
+      forward_row<V, N, PARTS>(x, E + L::B + row * KS, cosv, sinv, part);
+    }
+    __syncthreads();
+    for (int t = tid; t < nel * 4 * K; t += EL_THREADS) {
+      const int el = t / (4 * K), ak = t - el * 4 * K, a = ak / K, k = ak - a * K;
+      V* E = es + el * L::ELEM;
+      typename R::Acc s(R::zero());
+#pragma unroll
+      for (int j = 0; j < 3; ++j) s.add(P.at[((int64_t)nodes[4 * el + a] * 3 + j) * K + k], E[L::B + j * KS + k]);
+      E[L::A + a * KS + k] = s.get();
+    }
+    __syncthreads();
+    for (int t = tid; t < nel * 4 * PARTS; t += EL_THREADS) {
+      const int part = t % PARTS, row = (t / PARTS) & 3, el = t / (4 * PARTS);
+      V* E = es + el * L::ELEM;
+      inverse_row<V, N, PARTS>(E + L::A + row * KS, E + L::M1 + row * CS, cosv, sinv, part);
+    }
+    __syncthreads();
+    // ---- res at the points (M2 for tau, M3 for the rows)
+    for (int t = tid; t < nel * 4 * N; t += EL_THREADS) {
+      const int n = t % N, q = (t / N) & 3, el = t / (4 * N);
+      V* E = es + el * L::ELEM;
+      V pq[2], cq[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = 2 * n + h;
+        V v[4], m[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          v[a] = P.phi[(int64_t)nodes[4 * el + a] * C + c];
+          m[a] = E[L::M1 + a * CS + c];
+        }
+        const V va = q == 0 ? v[0] : q == 1 ? v[1] : q == 2 ? v[2] : v[3];
+        const V ma = q == 0 ? m[0] : q == 1 ? m[1] : q == 2 ? m[2] : m[3];
+        pq[h] = R::fma(bq, R::add(R::add(v[0], v[1]), R::add(v[2], v[3])), R::mul(dq, va));
+        cq[h] = R::fma(bqK, R::add(R::add(m[0], m[1]), R::add(m[2], m[3])), R::mul(dqK, ma));
+      }
+      const V w = om[n];
+      V* x2 = E + L::M2 + q * CS + 2 * n;
+      V* x3 = E + L::M3 + q * CS + 2 * n;
+      x2[0] = x3[0] = R::fma(R::neg(w), pq[1], cq[0]);
+      x2[1] = x3[1] = n == 0 ? R::zero() : R::fma(w, pq[0], cq[1]);
+    }
+    __syncthreads();
+    // ---- T = tau res (orthonormal basis: see element_kernel), zero without the least-squares terms
+    for (int t = tid; t < nel * 4 * PARTS; t += EL_THREADS) {
+      const int part = t % PARTS, q = (t / PARTS) & 3, el = t / (4 * PARTS);
+      V* E = es + el * L::ELEM;
+      const typename TracerArgs<V>::S* tg = P.tau + ((e0 + el) * 4 + q) * NTP;
+      const V* l = E + L::M2 + q * CS;
+      V* o = E + L::M1 + q * CS;
+      const V l0 = R::mul(l[0], R::of(0.70710678118654752440));
+#pragma unroll 1
+      for (int r = part; r < NM; r += PARTS) {
+        typename R::Acc a(R::mul(R::from(tg[r]), l0));                 // packed (0, r)
+#pragma unroll 4
+        for (int s = 1; s < NM; ++s)
+          a.add(R::from(tg[r <= s ? packed_index(r, s, NM) : packed_index(s, r, NM)]), l[s + 1]);
+        const V v = r == 0 ? R::mul(a.get(), R::of(1.41421356237309504880)) : a.get();
+        o[stor_of(r)] = P.gls ? v : R::zero();
+      }
+      if (part == 0) o[1] = R::zero();
+    }
+    __syncthreads();
+    for (int t = tid; t < nel * 4 * N; t += EL_THREADS) {
+      const int n = t % N, q = (t / N) & 3, el = t / (4 * N);
+      V* E = es + el * L::ELEM;
+      V* g = E + L::M3 + q * CS + 2 * n;
+      const V* tm = E + L::M1 + q * CS + 2 * n;
+      const V w = om[n], tr = tm[0], ti = tm[1];
+      g[0] = R::fma(w, ti, g[0]);
+      g[1] = R::fma(R::neg(w), tr, g[1]);
+    }
+    for (int t = tid; t < nel * 4 * PARTS; t += EL_THREADS) {
+      const int part = t % PARTS, q = (t / PARTS) & 3, el = t / (4 * PARTS);
+      V* E = es + el * L::ELEM;
+      V x[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        const V v = E[L::M1 + q * CS + c];
+        x[c] = c > 1 ? R::twice(v) : v;
+      }
+      forward_row<V, N, PARTS>(x, E + L::A + q * KS, cosv, sinv, part);
+    }
+    __syncthreads();
+    // ---- SUPG sums W_j = sum_a a_j(a) (b sum_q T_q + d T_a)
+    for (int t = tid; t < nel * 3 * K; t += EL_THREADS) {
+      const int el = t / (3 * K), jk = t - el * 3 * K, j = jk / K, k = jk - j * K;
+      V* E = es + el * L::ELEM;
+      V tq[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) tq[q] = E[L::A + q * KS + k];
+      const V ts = R::mul(bq, R::add(R::add(tq[0], tq[1]), R::add(tq[2], tq[3])));
+      typename R::Acc s(R::zero());
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        s.add(P.at[((int64_t)nodes[4 * el + a] * 3 + j) * K + k], R::fma(dq, tq[a], ts));
+      E[L::B + j * KS + k] = s.get();
+    }
+    __syncthreads();
+    for (int t = tid; t < nel * 3 * PARTS; t += EL_THREADS) {
+      const int part = t % PARTS, row = (t / PARTS) % 3, el = t / (3 * PARTS);
+      V* E = es + el * L::ELEM;
+      inverse_row<V, N, PARTS>(E + L::B + row * KS, E + L::M2 + row * CS, cosv, sinv, part);
+    }
+    __syncthreads();
+    // ---- the element's rows
+    for (int t = tid; t < nel * C; t += EL_THREADS) {
+      const int el = t / C, c = t - el * C;
+      const V* E = es + el * L::ELEM;
+      const V* dN = E + L::GEO;
+      V* out = P.rows + (e0 + el) * 4 * C + c;
+      V G[4], X[3];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) G[q] = E[L::M3 + q * CS + c];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) X[j] = R::fma(P.kappa4, E[L::GM + j * CS + c], R::mul(E[L::M2 + j * CS + c], iK));
+      const V base = R::mul(bq, R::add(R::add(G[0], G[1]), R::add(G[2], G[3])));
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        typename R::Acc s(base);
+        s.add(dq, G[a]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) s.add(dN[a * 3 + j], X[j]);
+        out[a * C] = c == 1 ? R::zero() : R::mul(dN[12], s.get());
+      }
+    }
+  }
+}
+
+template <typename V, int N>
+int launch_tracer(const TracerArgs<V>& P, cudaStream_t st) {
+  using L = TracerLayout<V, N>;
+  static_assert(L::BYTES <= 227 * 1024, "shared memory of a block");
+  if (P.n_elem <= 0) return 0;
+  if (cudaFuncSetAttribute(tracer_kernel<V, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES) != cudaSuccess)
+    return -2;
+  const int64_t blocks = std::min<int64_t>((P.n_elem + L::EB - 1) / L::EB, 152 * 256);
+  count_launches(1);
+  tracer_kernel<V, N><<<(int)blocks, EL_THREADS, L::BYTES, st>>>(P);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}
+
+// out = in without Im(mode 0), [V][C]
+template <typename V>
+__global__ void clean_kernel(const V* __restrict__ in, V* __restrict__ out, int64_t n, int C) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
+    out[t] = t % C == 1 ? V(0) : in[t];
+}
+template <typename V>
+int launch_clean(const V* in, V* out, int64_t n, int C, cudaStream_t st) {
+  if (n <= 0) return 0;
+  count_launches(1);
+  clean_kernel<V><<<(int)std::min<int64_t>((n + 255) / 256, 152 * 16), 256, 0, st>>>(in, out, n, C);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 

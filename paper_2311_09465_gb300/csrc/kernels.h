@@ -73,6 +73,10 @@ template <>
 struct StoreOf<float2> {
   using S = double;
 };
+template <>
+struct StoreOf<double> {
+  using S = double;
+};
 template <typename S>
 struct PairOfStore;
 template <>
@@ -104,22 +108,37 @@ struct ElementArgs {
 
 template <typename V, int N>
 int launch_element(int mode, const ElementArgs<V>& P, cudaStream_t st);
-// clean = y without fixed entries (dmask null: all velocities kept), samples of its velocity
+// clean (may be null) = y without fixed entries (dmask null: all velocities kept),
+// samples of its velocity
 template <typename V, int N>
 int launch_node_prepass(const typename StoreOf<V>::S* y, const uint8_t* dmask, V* clean, V* samples, const V* trig,
                         int64_t n_nodes, cudaStream_t st);
-// out = per node the sum of its element rows
+// out = per node the sum of its element rows [4][fields][C]; on Dirichlet nodes the
+// first `masked` fields are zero
 template <typename V>
 int launch_gather(const int32_t* node_off, const int32_t* node_elem, const V* rows, const uint8_t* dmask,
-                  typename StoreOf<V>::S* out, int64_t n_nodes, int C, cudaStream_t st);
+                  typename StoreOf<V>::S* out, int64_t n_nodes, int C, int fields, int masked, cudaStream_t st);
 
-// Tracer residual of eq. (3D-weak) on one colour range [e0, e1) (apply.cu):
-// phi [V][C], a4 the advecting velocity in the flow layout [V][4][C], tau the
-// tracer's tau cache; out += element rows (Dirichlet rows and Im(mode 0) skipped)
-template <typename T, int N>
-int launch_tracer(const int4* tets, const T* geo, const T* a4, const T* phi, const T* tau,
-                  const uint8_t* dmask, T* out, const T* dft, double kappa, double omega, int64_t e0,
-                  int64_t e1, cudaStream_t st, int gls = 1);
+// Tracer residual of eq. (3D-weak) in one launch (element.cuh), V = float or double
+template <typename V>
+struct TracerArgs {
+  using S = V;
+  const int4* tets;
+  const V* geo;
+  const V* at;       // [V][3][K] advecting velocity on samples
+  const V* phi;      // [V][C] without Im(mode 0)
+  const V* tau;
+  const V* trig;
+  V* rows;           // [E][4][C]
+  V omega, kappa4;   // kappa4: 4 kappa
+  int64_t n_elem;
+  int gls;
+};
+template <typename V, int N>
+int launch_tracer(const TracerArgs<V>& P, cudaStream_t st);
+// out = in [V][C] without Im(mode 0)
+template <typename V>
+int launch_clean(const V* in, V* out, int64_t n, int C, cudaStream_t st);
 template <typename T>
 int launch_repack_velocity(const T* a, T* a4, int64_t V, int C, cudaStream_t st);
 
@@ -236,10 +255,12 @@ int krylov_partial_blocks();
 int vec_mul(double* out, const double* a, const double* b, int64_t n, cudaStream_t st);
 // out = in / sqrt(*n2) with the squared norm read on the device
 int vec_normalise(double* out, const double* in, const double* n2, int64_t n, cudaStream_t st);
-// approximate diagonal of the tangent for right preconditioning (one colour range)
-int launch_diag(const int4* tets, const double* geo, const double* y, int N, Phys<double> ph,
-                double* D, int64_t e0, int64_t e1, cudaStream_t st);
-// D <- 1/D on free unknowns, 1 on fixed ones
-int launch_diag_invert(double* D, const uint8_t* dmask, int64_t V, int C, cudaStream_t st);
+// out = (float)(a b)
+int vec_mul_d2f(float* out, const double* a, const double* b, int64_t n, cudaStream_t st);
+// D = approximate inverse diagonal of the tangent for right preconditioning, 1 on
+// fixed unknowns; part: scratch of 12 values an element
+int launch_diag(const int4* tets, const double* geo, const double* y, int N, Phys<double> ph, const int32_t* node_off,
+                const int32_t* node_elem, const uint8_t* dmask, double* part, double* D, int64_t n_elem,
+                int64_t n_nodes, cudaStream_t st);
 
 }  // namespace ts
