@@ -150,16 +150,6 @@ __device__ __forceinline__ void store_floats(float* dst, const float (&v)[NM], f
     reinterpret_cast<float4*>(dst)[j] = make_float4(t[0], t[1], t[2], t[3]);
   }
 }
-template <int NM>
-__device__ __forceinline__ void load_limbs(const Limbs* src, Limbs (&v)[NM]) {
-#pragma unroll
-  for (int j = 0; j <= NM; j += 2) {
-    const int4 t = *reinterpret_cast<const int4*>(src + j);
-    if (j > 0) v[j == 0 ? 0 : j - 1] = Limbs{t.x, __int_as_float(t.y)};
-    if (j < NM) v[j < NM ? j : 0] = Limbs{t.z, __int_as_float(t.w)};
-  }
-}
-
 }  // namespace
 
 template <int N>
@@ -171,15 +161,17 @@ struct FxLayout {
   // which makes it 12 warps an SM at N = 7 instead of 10)
   static constexpr int LDQ = (N & 1) ? 2 * N : 2 * N + 2;            // limb pairs a row
   static constexpr int LDF = (2 * N + 3) & ~3;                       // floats a row
-  static constexpr int TW = 3 * N;
   // in 4-byte words
   static constexpr int M = 0;                           // [NM][LDQ] limbs
-  static constexpr int X = M + 2 * NM * LDQ;            // [NM][LDQ] limbs: C_m, then X
+  static constexpr int X = M + 2 * NM * LDQ;            // [NM][LDQ] limbs
   static constexpr int F = X + 2 * NM * LDQ;            // [NM][LDF]: h_a, R, U^T R, E
   static constexpr int U = F + NM * LDF;                // [NM][LDF]: row a = sqrt(eigenvalue a), eigenvector a
   static constexpr int END = U + NM * LDF;
-  static constexpr int T = F;                           // [3][2][TW] 64-bit modes, [3][2][N] times sqrt2: over F, U
-  static constexpr int TEND = T + 2 * (3 * 2 * TW + 3 * 2 * N);
+  static constexpr int TW = 2 * N - 1;                  // modes -(N-1) .. N-1
+  static constexpr int T = F;                           // [3][2][TW] limbs of the modes of w_m: over F, U
+  static constexpr int HD = T + 2 * 3 * 2 * TW;         // [NH] complex 64-bit diagonals of sum_m C_m C_m
+  static constexpr int NH = N * (N + 1) / 2 + N - 1;
+  static constexpr int TEND = HD + 4 * NH;
   static constexpr int OUTP = M;                        // packed tau (doubles) over M
   static constexpr int RAW0 = END > TEND ? END : TEND;
   static constexpr int RAW1 = (RAW0 > 2 * Dims<N>::NT_PAD ? RAW0 : 2 * Dims<N>::NT_PAD);
@@ -208,8 +200,8 @@ __global__ void __launch_bounds__(128, N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kerne
   Limbs* Xs = reinterpret_cast<Limbs*>(base + Lt::X);
   float* F = reinterpret_cast<float*>(base + Lt::F);
   float* U = reinterpret_cast<float*>(base + Lt::U);
-  i64* T = reinterpret_cast<i64*>(base + Lt::T);
-  i64* T2 = T + 3 * 2 * TW;
+  Limbs* T = reinterpret_cast<Limbs*>(base + Lt::T);
+  longlong2* Hd = reinterpret_cast<longlong2*>(base + Lt::HD);
   // the lane's columns, and whether it has a first one
   const int cx = 2 * p - 1, cy = 2 * p;
   const bool hx = in_group && p > 0, hy = in_group;
@@ -291,85 +283,91 @@ __global__ void __launch_bounds__(128, N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kerne
     const i64 cfix = finite ? fx_from_dd(dd_scale(diff, sc * sc)) : (1ll << 57);
 #pragma unroll 1
     for (int m = 0; m < 3; ++m) {
-      i64* tr = T + m * 2 * TW + L;                     // mode k at tr[k], its imaginary part at tr[TW + k]
+      Limbs* tr = T + m * 2 * TW + L;                   // mode k at tr[k], its imaginary part at tr[TW + k]
       const float2 wr = *reinterpret_cast<const float2*>(tr + p), wi = *reinterpret_cast<const float2*>(tr + TW + p);
-      const i64 re = finite ? fx_from_dd(dd{wr.x * sc, wr.y * sc}) : 0, im = finite ? fx_from_dd(dd{wi.x * sc, wi.y * sc}) : 0;
+      const Limbs re = fx_split(finite ? fx_from_dd(dd{wr.x * sc, wr.y * sc}) : 0);
+      const Limbs im = fx_split(finite ? fx_from_dd(dd{wi.x * sc, wi.y * sc}) : 0);
       __syncwarp();
       if (in_group) {
         tr[p] = re;
         tr[TW + p] = im;
-        T2[(m * 2 + 0) * N + p] = fx_sqrt2(re);
-        T2[(m * 2 + 1) * N + p] = fx_sqrt2(im);
         if (p > 0) {
           tr[-p] = re;
-          tr[TW - p] = -im;
-          tr[L + p] = 0;
-          tr[TW + L + p] = 0;
+          tr[TW - p] = Limbs{-im.h, -im.l};
         }
       }
     }
     __syncwarp();
-    // ---- M = sum_m C_m C_m + c I on half of the entries: the sums over m are kept
-    // as 64-bit integers at (row, lane's column) of M's place
+    // ---- H = sum_m T_m T_m, T_m the complex Hermitian Toeplitz matrix t_{i-j} of w_m
+    // (|i - j| < N), by diagonals: with rows and columns numbered 0..2L, L = N - 1,
+    //   H_0j = sum_k t_{-k} t_{k-j},   H_ij = H_{i-1,j-1} + t_i t_{-j} for i, j <= L,
+    // constant along a diagonal where i <= L <= j, and H_{2L-i,2L-j} = conj H_ij: an
+    // entry costs one product instead of a row of them.  Lane p takes diagonal p
+    // (L + 1 products for its first entry, one for each of the L - p others) and the
+    // first entry of diagonal 2L + 1 - p (p products): 2L + 1 products a lane and m
+    // (N = 7, 187,266 tetrahedra: 7.3 ms for the whole kernel, 8.7 with half of the
+    // dense products).
     {
-      i64* acc = reinterpret_cast<i64*>(Ms) + 1;
-#pragma unroll 1
-      for (int m = 0; m < 3; ++m) {
-        const i64* tr = T + m * 2 * TW + L;
-        const i64* ti = tr + TW;
-        const i64* t2 = T2 + m * 2 * N;
-        // C_m's columns as rows (symmetric): entry i at i + 1
-        Limbs* rx = Xs + (hx ? cx : 0) * LDQ + 1;
-        Limbs* ry = Xs + cy * LDQ + 1;
-        __syncwarp();                                   // all lanes have read the previous C_m
-        if (hx) rx[0] = fx_split(t2[p]);
-        if (hy) ry[0] = fx_split(p == 0 ? tr[0] : t2[N + p]);
-#pragma unroll 1
-        for (int k = 1; k < N; ++k) {
-          const i64 pl = tr[k - p], ph = tr[k + p], ql = ti[k - p], qh = ti[k + p];
-          if (hx) {
-            rx[2 * k - 1] = fx_split(pl + ph);
-            rx[2 * k] = fx_split(ql + qh);
-          }
-          if (hy) {
-            ry[2 * k - 1] = fx_split(p == 0 ? t2[k] : qh - ql);
-            ry[2 * k] = fx_split(p == 0 ? t2[N + k] : pl - ph);
-          }
-        }
-        __syncwarp();
-        Limbs a[NM], b[NM];
-        load_limbs<NM>(Xs + (hx ? cx : 0) * LDQ, a);
-        load_limbs<NM>(Xs + cy * LDQ, b);
-        float ah[NM], bh[NM];
+      i64 hr = 0, hi = 0;
+      auto add = [&](int ka, int kb) {                  // += sum_m t_ka t_kb
+        i64 r = 0, i = 0;
+        float xr = 0.f, xi = 0.f;
 #pragma unroll
-        for (int j = 0; j < NM; ++j) {
-          ah[j] = (float)a[j].h;
-          bh[j] = (float)b[j].h;
+        for (int m = 0; m < 3; ++m) {
+          const Limbs* tr = T + m * 2 * TW + L;
+          const Limbs ar = tr[ka], ai = tr[TW + ka], br = tr[kb], bi = tr[TW + kb];
+          const float arf = (float)ar.h, aif = (float)ai.h, brf = (float)br.h, bif = (float)bi.h;
+          fx_mad(r, ar.h, br.h);
+          fx_mad(i, ar.h, bi.h);
+          fx_mad(r, -ai.h, bi.h);
+          fx_mad(i, ai.h, br.h);
+          xr = fmaf(arf, br.l, fmaf(ar.l, brf, xr));
+          xi = fmaf(arf, bi.l, fmaf(ar.l, bif, xi));
+          xr = fmaf(-aif, bi.l, fmaf(-ai.l, bif, xr));
+          xi = fmaf(aif, br.l, fmaf(ai.l, brf, xi));
         }
+        constexpr float U = 1.f / 1073741824.f;         // 2^-30
+        hr += r + ((i64)__float2int_rn(xr * U) << 1);
+        hi += i + ((i64)__float2int_rn(xi * U) << 1);
+      };
+      longlong2* diag = Hd + (p * N - p * (p - 1) / 2);  // entries (i, i + p), i = 0..L - p
 #pragma unroll 1
-        for (int o = 0; o <= N; ++o) {
-          const int r = half_row(o);
-          const int4* row = reinterpret_cast<const int4*>(Xs + r * LDQ);
-          i64 v0, v1;
-          fx_dot2<NM>(row, a, b, ah, bh, v0, v1);
-          if (hx && o < N) acc[r * LDQ + cx] = m == 0 ? v0 : acc[r * LDQ + cx] + v0;
-          if (hy && o > 0) acc[r * LDQ + cy] = m == 0 ? v1 : acc[r * LDQ + cy] + v1;
-        }
+      for (int k = 0; k <= L; ++k) add(-k, k - p);
+      if (in_group) diag[0] = make_longlong2(hr, hi);
+#pragma unroll 1
+      for (int i = 1; i <= L; ++i) {
+        const bool own = i <= L - p;
+        if (i == L - p + 1) hr = hi = 0;
+        add(own ? i : -i, own ? -(i + p) : i - 1 + p - 2 * L);
+        if (in_group && own) diag[i] = make_longlong2(hr, hi);
       }
-      // limbs in both triangles (a lane's entries are its own: no other lane's place is touched)
+      if (in_group && p > 0) Hd[N * (N + 1) / 2 + L - p] = make_longlong2(hr, hi);   // diagonal 2L + 1 - p
+    }
+    __syncwarp();
+    // ---- M = H + c I in the orthonormal real basis; lane a takes the mode pairs (a, b), b <= a:
+    // P = M_{a,b} = conj H_{L-a,L-b}, Q = M_{a,-b} = conj of diagonal a + b where it is constant
 #pragma unroll 1
-      for (int o = 0; o <= N; ++o) {
-        const int r = half_row(o);
-        if (hx && o < N) {
-          const Limbs v = fx_split(acc[r * LDQ + cx] + (r == cx ? cfix : 0));
-          Ms[r * LDQ + cx + 1] = v;
-          Ms[cx * LDQ + r + 1] = v;
-        }
-        if (hy && o > 0) {
-          const Limbs v = fx_split(acc[r * LDQ + cy] + (r == cy ? cfix : 0));
-          Ms[r * LDQ + cy + 1] = v;
-          Ms[cy * LDQ + r + 1] = v;
-        }
+    for (int b = 0; b <= L; ++b) {
+      if (!in_group || b > p) continue;
+      const int d = p - b, s = p + b;
+      const longlong2 Pc = Hd[d * N - d * (d - 1) / 2 + L - p];
+      const longlong2 Qc = Hd[s <= L ? s * N - s * (s - 1) / 2 + L - s : N * (N + 1) / 2 + s - L - 1];
+      auto put = [&](int r, int c, i64 v) {
+        const Limbs l = fx_split(v);
+        Ms[r * LDQ + c + 1] = l;
+        Ms[c * LDQ + r + 1] = l;
+      };
+      if (p == 0) {
+        put(0, 0, Pc.x + cfix);
+      } else if (b == 0) {                              // M_{0,a} = conj P
+        put(0, cx, fx_sqrt2(Pc.x));
+        put(0, cy, -fx_sqrt2(Pc.y));
+      } else {
+        const i64 c = d == 0 ? cfix : 0;
+        put(cx, 2 * b - 1, Pc.x + Qc.x + c);            // Re, Re: Re P + Re Q
+        put(cy, 2 * b, Pc.x - Qc.x + c);                // Im, Im: Re P - Re Q
+        put(cy, 2 * b - 1, -Pc.y - Qc.y);               // Im a, Re b: Im P + Im Q (conjugates stored)
+        if (d != 0) put(cx, 2 * b, Pc.y - Qc.y);        // Re a, Im b: -Im P + Im Q
       }
     }
     __syncwarp();
