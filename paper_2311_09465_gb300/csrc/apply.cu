@@ -469,12 +469,12 @@ template int launch_repack_velocity<double>(const double*, double*, int64_t, int
 // its own entries in the same launch.  Latency-bound: 81 nodes, C = 6 and 529
 // nodes, C = 14 took 10 and 31 us with all coordinates in one block.
 template <typename T>
-__global__ void __launch_bounds__(128) outlet_kernel(const int32_t* __restrict__ nodes,
+__global__ void __launch_bounds__(1024) outlet_kernel(const int32_t* __restrict__ nodes,
                                                      const T* __restrict__ w, int n, T R,
                                                      const T* __restrict__ v,
                                                      const uint8_t* __restrict__ dmask, int mask_input,
                                                      T* __restrict__ out, int C) {
-  __shared__ T part[4];
+  __shared__ T part[32];
   const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x == 0 ? 0 : blockIdx.x + 1;   // Im(mode 0) is left out
   T acc = 0;
@@ -488,7 +488,9 @@ __global__ void __launch_bounds__(128) outlet_kernel(const int32_t* __restrict__
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) part[warp] = acc;
   __syncthreads();
-  const T q = R * ((part[0] + part[1]) + (part[2] + part[3]));
+  T q = 0;
+  for (int k = 0; k < nt / 32; ++k) q += part[k];
+  q *= R;
   for (int b = tid; b < n; b += nt) {
     const int A = nodes[b];
     if (dmask[A]) continue;
@@ -504,7 +506,9 @@ int launch_outlet(const int32_t* nodes, const T* w, int n_nodes, T R, const T* v
                   const uint8_t* dmask, int mask_input, T* out, int C, cudaStream_t st) {
   if (n_nodes <= 0) return 0;
   count_launches(1);
-  outlet_kernel<T><<<C - 1, 128, 0, st>>>(nodes, w, n_nodes, R, v, dmask, mask_input, out, C);
+  // about one node a thread: the two dependent loads of a node are the kernel's time
+  const int threads = n_nodes >= 1024 ? 1024 : (n_nodes + 31) & ~31;
+  outlet_kernel<T><<<C - 1, threads, 0, st>>>(nodes, w, n_nodes, R, v, dmask, mask_input, out, C);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
