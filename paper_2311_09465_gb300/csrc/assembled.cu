@@ -23,10 +23,9 @@
 // GB300 mapping.  Assembly: one warp per row gathers the row's (element,
 // local node) pairs from the node-to-element list and adds every element
 // contribution to the row's records (the warp owns the row: no atomics,
-// deterministic).  Product: one warp per row streams the row's records
-// (1.6 KB each at N = 7) through shared memory with 16-byte loads, lanes over
-// the 8N outputs; the records are the only large HBM stream, so the product
-// is bound by HBM bandwidth.
+// deterministic).  Product: a warp streams the records of a few rows
+// (1.6 KB each at N = 7); the records are the only large HBM stream, so the
+// product is bound by HBM bandwidth.
 #include <algorithm>
 
 #include "common.cuh"
@@ -419,95 +418,215 @@ __global__ void __launch_bounds__(128, 4)
 }
 
 // y = H x on the assembled records; Dirichlet velocity and Im(mode 0) inputs
-// are ignored and the same rows of y are zero.  The record and x_B of the
-// next connection are copied into shared memory (double buffer) while the
-// current one is multiplied, so a warp keeps one record in flight.
-constexpr int SPMV_WARPS = 8;   // warps (rows in flight) per block
+// are ignored and the same rows of y are zero.
+//
+// Bound by the record stream once enough of it is in flight.  A warp takes a few
+// consecutive rows, whose records lie one behind the other, and copies them with
+// their x_B through a ring of shared-memory slots that runs on across the ends
+// of rows; columns and Dirichlet marks come 32 at a time, a window ahead.  A lane
+// owns fixed pairs of adjacent columns of K and L (position t = row t / N, pair
+// t % N) and keeps its partial sums in registers over the whole row: each
+// coefficient of K is read once and feeds the three velocity components, and
+// the N partial sums of an output meet once per row.  K of a Dirichlet row is not
+// copied (its products are not used).
+// 9,996 rows, 138 k records: N = 5 (118 MB) 35 us, N = 7 (227 MB) 52 us, N = 15
+// (1.0 GB) 176 us, 5.8 TB/s; with one lane per output and one record in flight a
+// warp, each coefficient of K read three times from shared memory, 48, 65 and
+// 237 us.
+constexpr int SPMV_WARPS = 4;   // warps (groups of rows in flight) per block
+constexpr int SPMV_ROWS = 31;   // most rows a warp takes at a time (row_off in one warp load)
 
 template <int N>
-__global__ void __launch_bounds__(256)
+struct SpmvShape {
+  // slots a warp and blocks an SM: enough records in flight at 4 to 16 warps and more an SM
+  static constexpr int S = N <= 10 ? 4 : 3;
+  static constexpr int SLOT = AsmLayout<N>::PWARP;
+  static constexpr int BYTES = SPMV_WARPS * S * SLOT * (int)sizeof(float);
+  static constexpr int FIT = (220 * 1024) / (BYTES + 1024);
+  static constexpr int BLOCKS = FIT > 9 ? 9 : FIT;
+};
+
+template <int N>
+__global__ void __launch_bounds__(32 * SPMV_WARPS, SpmvShape<N>::BLOCKS)
     spmv_paper_kernel(const int32_t* __restrict__ row_off, const int32_t* __restrict__ cols,
                       const float* __restrict__ H, const uint8_t* __restrict__ dmask,
-                      const float* __restrict__ x, float* __restrict__ y, int64_t n_nodes) {
+                      const float* __restrict__ x, float* __restrict__ y, int64_t n_nodes, int rows) {
   using L = AsmLayout<N>;
-  constexpr int C = L::C, CC = L::CC, HB = L::HB, NB = 4 * C;
-  constexpr int R = (NB + 31) / 32;
+  using K = SpmvShape<N>;
+  constexpr int C = L::C, CC = L::CC, HB = L::HB, NB = 4 * C, NPOS = CC / 2, S = K::S;
+  constexpr int P = (NPOS + 31) / 32;
+  static_assert(C <= 32 && NB / 4 <= 32, "lane r adds the identity parts of row r");
   extern __shared__ __align__(16) float smem_f[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wpb = blockDim.x >> 5;
-  float* buf0 = smem_f + warp * 2 * L::PWARP;   // [2][HB + NB]
-  auto stage = [&](int p, float* dst) {
-    const float4* src = reinterpret_cast<const float4*>(H + (int64_t)p * HB);
-    for (int t = lane; t < HB / 4; t += 32) cp_async16(dst + 4 * t, src + t);
-    const float4* xb = reinterpret_cast<const float4*>(x + (int64_t)cols[p] * NB);
-    for (int t = lane; t < NB / 4; t += 32) cp_async16(dst + HB + 4 * t, xb + t);
-    cp_async_commit();
-  };
-  for (int64_t A = (int64_t)blockIdx.x * wpb + warp; A < n_nodes; A += (int64_t)gridDim.x * wpb) {
-    float acc[R];
+  float* ring = smem_f + warp * S * K::SLOT;
+  const int64_t n_groups = (n_nodes + rows - 1) / rows;
+  for (int64_t grp = (int64_t)blockIdx.x * SPMV_WARPS + warp; grp < n_groups;
+       grp += (int64_t)gridDim.x * SPMV_WARPS) {
+    const int64_t A0 = grp * rows;
+    const int nr = n_nodes - A0 < rows ? (int)(n_nodes - A0) : rows;
+    const int off = lane <= nr ? row_off[A0 + lane] : 0;
+    const unsigned dir_rows = __ballot_sync(0xffffffffu, lane < nr && dmask[A0 + lane] != 0);
+    const int p0 = __shfl_sync(0xffffffffu, off, 0), p1 = __shfl_sync(0xffffffffu, off, nr);
+    // windows of 32 columns: [base, base + 32) and the one behind it
+    auto window = [&](int base) { return base + lane < p1 ? cols[base + lane] : 0; };
+    int base = p0, c_cur = window(p0), c_next = window(p0 + 32);
+    int row_s = 0, end_s = __shfl_sync(0xffffffffu, off, 1);   // row of the record staged next
+    float* at_s = ring;
+    float* const last = ring + (S - 1) * K::SLOT;
+    auto stage = [&](int p) {
+      if (p < p1) {
+        while (p >= end_s) end_s = __shfl_sync(0xffffffffu, off, ++row_s + 1);
+        if (p - base == 32) {
+          base += 32;
+          c_cur = c_next;
+          c_next = window(base + 32);
+        }
+        const float4* src = reinterpret_cast<const float4*>(H + (int64_t)p * HB) + lane;
+        const int first = (dir_rows >> row_s) & 1 ? CC / 4 : 0;
 #pragma unroll
-    for (int k = 0; k < R; ++k) acc[k] = 0.f;
-    const int r0 = row_off[A], r1 = row_off[A + 1];
-    if (r0 < r1) stage(r0, buf0);
-    for (int p = r0; p < r1; ++p) {
-      float* rec = buf0 + ((p - r0) & 1) * L::PWARP;
-      float* xs = rec + HB;
-      if (p + 1 < r1) {
-        stage(p + 1, buf0 + ((p + 1 - r0) & 1) * L::PWARP);
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
+        for (int j = 0; j < (HB / 4 + 31) / 32; ++j)
+          if (lane + 32 * j >= first && lane + 32 * j < HB / 4) cp_async16(at_s + 4 * (lane + 32 * j), src + 32 * j);
+        const float4* xb =
+            reinterpret_cast<const float4*>(x + (int64_t)__shfl_sync(0xffffffffu, c_cur, p - base) * NB);
+        if (lane < NB / 4) cp_async16(at_s + HB + 4 * lane, xb + lane);
       }
-      __syncwarp();
-      const bool dirB = dmask[cols[p]] != 0;
-      for (int t = lane; t < NB; t += 32) {
-        const int f = t / C, c = t - f * C;
-        if (c == 1 || (dirB && f < 3)) xs[t] = 0.f;
-      }
-      __syncwarp();
+      cp_async_commit();
+      at_s = at_s == last ? ring : at_s + K::SLOT;
+    };
 #pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const int o = lane + 32 * k;
-        if (o < NB) {
-          const int f = o / C, r = o - f * C;
-          float s = acc[k];
-          // rows and x slices start at multiples of 2 floats: 8-byte shared loads
-          if (f < 3) {
-            const float2* Kr = reinterpret_cast<const float2*>(rec + r * C);
-            const float2* xi = reinterpret_cast<const float2*>(xs + f * C);
+    for (int i = 0; i < S - 1; ++i) stage(p0 + i);
+    unsigned dir_cols = 0;                       // Dirichlet marks of 32 columns from p on
+    int p = p0;
+    float* rec = ring;
+    for (int a = 0; a < nr; ++a) {
+      const int64_t A = A0 + a;
+      const bool dirA = (dir_rows >> a) & 1;
+      const int r1 = __shfl_sync(0xffffffffu, off, a + 1);
+      float k0[P], k1[P], k2[P], kl[P], g[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int c = 0; c < C / 2; ++c) {
-              const float2 a = Kr[c], b = xi[c];
-              s = fmaf(a.x, b.x, fmaf(a.y, b.y, s));
+      for (int j = 0; j < P; ++j) k0[j] = k1[j] = k2[j] = kl[j] = 0.f;
+      for (; p < r1; ++p) {
+        stage(p + S - 1);
+        if (((p - p0) & 31) == 0)
+          dir_cols = __ballot_sync(0xffffffffu, p + lane < p1 && dmask[cols[p + lane]] != 0);
+        const bool dirB = (dir_cols >> ((p - p0) & 31)) & 1;
+        cp_async_wait<S - 1>();
+        __syncwarp();
+        const float* xs = rec + HB;
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+          const int t = lane + 32 * j;
+          if (t < NPOS) {
+            const int c = 2 * (t % N);
+            const float2 l = *reinterpret_cast<const float2*>(rec + CC + 2 * t);
+            float2 v = *reinterpret_cast<const float2*>(xs + 3 * C + c);
+            if (c == 0) v.y = 0.f;
+            kl[j] = fmaf(l.x, v.x, fmaf(l.y, v.y, kl[j]));
+            if (!dirA && !dirB) {
+              const float2 k = *reinterpret_cast<const float2*>(rec + 2 * t);
+              float2 v0 = *reinterpret_cast<const float2*>(xs + c);
+              float2 v1 = *reinterpret_cast<const float2*>(xs + C + c);
+              float2 v2 = *reinterpret_cast<const float2*>(xs + 2 * C + c);
+              if (c == 0) v0.y = v1.y = v2.y = 0.f;
+              k0[j] = fmaf(k.x, v0.x, fmaf(k.y, v0.y, k0[j]));
+              k1[j] = fmaf(k.x, v1.x, fmaf(k.y, v1.y, k1[j]));
+              k2[j] = fmaf(k.x, v2.x, fmaf(k.y, v2.y, k2[j]));
             }
-            s = fmaf(rec[2 * CC + f], xs[3 * C + r], s);
-          } else {
-            const float2* Lr = reinterpret_cast<const float2*>(rec + CC + r * C);
-            const float2* xp = reinterpret_cast<const float2*>(xs + 3 * C);
-#pragma unroll
-            for (int c = 0; c < C / 2; ++c) {
-              const float2 a = Lr[c], b = xp[c];
-              s = fmaf(a.x, b.x, fmaf(a.y, b.y, s));
-            }
-            s = fmaf(rec[2 * CC + 3], xs[r], s);
-            s = fmaf(rec[2 * CC + 4], xs[C + r], s);
-            s = fmaf(rec[2 * CC + 5], xs[2 * C + r], s);
           }
-          acc[k] = s;
+        }
+        if (lane < C) {
+          const float4 q0 = *reinterpret_cast<const float4*>(rec + 2 * CC);
+          const float2 q1 = *reinterpret_cast<const float2*>(rec + 2 * CC + 4);
+          const float xp = xs[3 * C + lane];
+          g[0] = fmaf(q0.x, xp, g[0]);
+          g[1] = fmaf(q0.y, xp, g[1]);
+          g[2] = fmaf(q0.z, xp, g[2]);
+          if (!dirB)
+            g[3] = fmaf(q0.w, xs[lane], fmaf(q1.x, xs[C + lane], fmaf(q1.y, xs[2 * C + lane], g[3])));
+        }
+        rec = rec == last ? ring : rec + K::SLOT;
+        __syncwarp();
+      }
+      // the slot before the next record's is free: the partial sums of the row meet there
+      float* part = rec == ring ? last : rec - K::SLOT;
+#pragma unroll
+      for (int j = 0; j < P; ++j) {
+        const int t = lane + 32 * j;
+        if (t < NPOS) {
+          part[t] = k0[j];
+          part[NPOS + t] = k1[j];
+          part[2 * NPOS + t] = k2[j];
+          part[3 * NPOS + t] = kl[j];
+        }
+      }
+      __syncwarp();
+      if (lane < C) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          float s = g[f];
+#pragma unroll
+          for (int k = 0; k < N; ++k) s += part[f * NPOS + lane * N + k];
+          y[A * NB + f * C + lane] = (lane == 1 || (dirA && f < 3)) ? 0.f : s;
         }
       }
       __syncwarp();
     }
-    const bool dirA = dmask[A] != 0;
+    cp_async_wait<0>();                  // the groups still open are empty
+    __syncwarp();
+  }
+}
+
+// The same product for records of a few rows (N <= 3), where a record is less
+// work than its staging: a lane owns one output (field, row) and reads the row
+// of K or L and x_B directly; 32 / 8N records (N = 1, 2) share a warp.  9,996
+// rows: N = 2 15.6 us, N = 3 22.5 us (22.5 and 26.3 with one record at a time staged
+// in shared memory).
+template <int N>
+__global__ void __launch_bounds__(128)
+    spmv_small_kernel(const int32_t* __restrict__ row_off, const int32_t* __restrict__ cols,
+                      const float* __restrict__ H, const uint8_t* __restrict__ dmask,
+                      const float* __restrict__ x, float* __restrict__ y, int64_t n_nodes) {
+  using L = AsmLayout<N>;
+  constexpr int C = L::C, CC = L::CC, HB = L::HB, NB = 4 * C, SUB = 32 / NB;
+  static_assert(SUB >= 1, "one lane an output");
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / NB, o = lane - sub * NB, f = o / C, r = o - f * C;
+  const int64_t A = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (A >= n_nodes) return;
+  float s = 0.f, g = 0.f;
+  if (sub < SUB) {
+    const int r1 = row_off[A + 1];
+    const int mat = (f < 3 ? 0 : CC) + r * C;
+#pragma unroll 4
+    for (int p = row_off[A] + sub; p < r1; p += SUB) {
+      const float* rec = H + (int64_t)p * HB;
+      const int B = cols[p];
+      const float* xb = x + (int64_t)B * NB;
+      const bool dirB = dmask[B] != 0;
+      const bool drop = dirB && f < 3;
+      float t = 0.f;
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int o = lane + 32 * k;
-      if (o < NB) {
-        const int f = o / C, r = o - f * C;
-        y[A * NB + o] = (r == 1 || (dirA && f < 3)) ? 0.f : acc[k];
+      for (int c = 0; c < N; ++c) {
+        const float2 a = *reinterpret_cast<const float2*>(rec + mat + 2 * c);
+        float2 v = *reinterpret_cast<const float2*>(xb + f * C + 2 * c);
+        if (drop) v.x = 0.f;
+        if (drop || c == 0) v.y = 0.f;
+        t = fmaf(a.x, v.x, fmaf(a.y, v.y, t));
+      }
+      s += t;
+      if (f < 3) {
+        g = fmaf(rec[2 * CC + f], xb[3 * C + r], g);
+      } else if (!dirB) {
+        g = fmaf(rec[2 * CC + 3], xb[r], g);
+        g = fmaf(rec[2 * CC + 4], xb[C + r], g);
+        g = fmaf(rec[2 * CC + 5], xb[2 * C + r], g);
       }
     }
   }
+  s += g;
+#pragma unroll
+  for (int d = NB; SUB > 1 && d < 32; d *= 2) s += __shfl_down_sync(0xffffffffu, s, d);
+  if (lane < NB) y[A * NB + lane] = (r == 1 || (dmask[A] != 0 && f < 3)) ? 0.f : s;
 }
 
 // One colour of a symmetric block Gauss-Seidel sweep with the assembled
@@ -737,17 +856,24 @@ int launch_assemble_paper(const int32_t* node_off, const int32_t* node_elem, con
 template <int N>
 int launch_spmv_paper(const int32_t* row_off, const int32_t* cols, const float* H, const uint8_t* dmask,
                       const float* x, float* y, int64_t n_nodes, cudaStream_t st) {
-  using L = AsmLayout<N>;
   if (n_nodes <= 0) return 0;
-  const int warps = SPMV_WARPS;
-  const size_t smem = (size_t)warps * 2 * L::PWARP * sizeof(float);
-  if (smem > 227 * 1024) return -6;
-  cudaFuncSetAttribute(spmv_paper_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int64_t blocks = (n_nodes + warps - 1) / warps;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  count_launches(1);
-  spmv_paper_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(row_off, cols, H, dmask, x, y, n_nodes);
-  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  // 9,996 rows: N = 3 22.5 us (25.8 with the ring), N = 4 32.5 (27.1)
+  if constexpr (N <= 3) {
+    count_launches(1);
+    spmv_small_kernel<N><<<(unsigned)((n_nodes + 3) / 4), 128, 0, st>>>(row_off, cols, H, dmask, x, y, n_nodes);
+    return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  } else {
+    using K = SpmvShape<N>;
+    if (cudaFuncSetAttribute(spmv_paper_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, K::BYTES) != cudaSuccess)
+      return -2;
+    const int64_t warps = (int64_t)152 * K::BLOCKS * SPMV_WARPS;   // one wave
+    const int rows = (int)std::min<int64_t>((n_nodes + warps - 1) / warps, SPMV_ROWS);
+    const int64_t groups = (n_nodes + rows - 1) / rows;
+    const int64_t blocks = std::min<int64_t>((groups + SPMV_WARPS - 1) / SPMV_WARPS, 152 * 64);
+    count_launches(1);
+    spmv_paper_kernel<N><<<(int)blocks, 32 * SPMV_WARPS, K::BYTES, st>>>(row_off, cols, H, dmask, x, y, n_nodes, rows);
+    return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  }
 }
 
 int assembled_record_floats(int N) { return 2 * (2 * N) * (2 * N) + 8; }
