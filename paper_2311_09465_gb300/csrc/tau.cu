@@ -264,12 +264,14 @@ __global__ void __launch_bounds__(128) tau32_kernel(const int4* __restrict__ tet
     int ex = 0;
     if (finite) frexpf(bound, &ex);
     const float sc = ldexpf(1.f, -ex);
-    const float cd = diff * sc * sc;
+    // a point that is not finite takes a harmless matrix here and NaN at the end: the
+    // rotations mix in neighbouring lanes' values times zero
+    const float cd = finite ? diff * sc * sc : 0.5f;
     __syncwarp();
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       float* tr = tw + m * 2 * TW + L;        // mode k at tr[k], im at tr[TW + k]
-      const float re = w[m][0] * sc, im = w[m][1] * sc;
+      const float re = finite ? w[m][0] * sc : 0.f, im = finite ? w[m][1] * sc : 0.f;
       if (in_group) {
         tr[p] = re;
         tr[TW + p] = im;
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(128) tau32_kernel(const int4* __restrict__ tet
     // lane's two vectors are columns 2p-1 and 2p of the cache
     if (live && eig_out) {
       float* eo = eig_out + gq * D::EIG;
-      const float back = ldexpf(1.f, 2 * ex);
+      const float back = finite ? ldexpf(1.f, 2 * ex) : __int_as_float(0x7fc00000);
       const float ix = rsqrt_newton(ax), iy = rsqrt_newton(ay);
       if (p > 0) {
 #pragma unroll

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(128, N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kerne
       for (int j = 0; j < N; ++j) sum += __shfl_sync(0xffffffffu, bound, first + j);
       bound = 1.0001f * (sum + sqrtf(diff.hi));
     }
-    const bool finite = bound < 1e18f && bound > 1e-18f;
+    const bool finite = bound < 4e18f && bound > 2e-19f;   // 2^-ex squared stays in range
     int ex = 0;
     if (finite) frexpf(bound, &ex);
     const float sc = ldexpf(1.f, -ex);
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(128, N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kerne
       // eigenpairs for the derivative of tau (exact tangent), when asked
       if (live && eig_out) {
         float* eo = eig_out + gq * Dims<N>::EIG;
-        const float back = ldexpf(1.f, 2 * ex);
+        const float back = finite ? ldexpf(1.f, 2 * ex) : __int_as_float(0x7fc00000);
         if (hx) {
 #pragma unroll
           for (int i = 0; i < NM; ++i) eo[i * NM + cx] = x[i] * ix;
