@@ -18,15 +18,14 @@
 // derivative of A_j: rho A(v_j) du0_i/dx_j in c_i and dN_a/dx_j A(v_j) T0_i).
 // Pseudo-time adds mass_coef * M v on momentum rows (section 2.5.3).
 //
-// GB300 mapping: one warp per element, all per-element arrays in a per-warp
-// shared-memory workspace, lanes over output entries of each batched small
-// contraction (DFT tables shared per CTA).  Elements of one colour share no
-// node, so each warp adds its 4x4xC results to the nodes without atomics;
-// the host launches the colours in order (deterministic).
-#include <type_traits>
-
+// This file is the colour-ordered form, for native FP64 arithmetic, on request in
+// FP32, and where no scratch may be allocated; element.cuh is the default.  One
+// warp per element, all per-element arrays in a per-warp shared-memory
+// workspace, lanes over output entries of each batched small contraction (DFT
+// tables shared per CTA).  Elements of one colour share no node, so each warp
+// adds its 4x4xC results to the nodes without atomics; the host launches the
+// colours in order (deterministic).
 #include "common.cuh"
-#include "ddfloat.cuh"
 #include "kernels.h"
 
 namespace ts {
@@ -68,7 +67,6 @@ struct ApplyLayout {
 
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return ::fma(a, b, c); }
-__device__ __forceinline__ ddv mad(ddv a, ddv b, ddv c) { return ddv(dd_fma(a.v, b.v, c.v)); }
 
 // out[b*os + r] = sum_c M[r*ld + c] in[b*is + c]
 template <typename T, int R, int CN>
@@ -92,28 +90,12 @@ __device__ __forceinline__ T omega_apply(const T* x, int c, T omega) {
   return (c & 1) ? T(n) * omega * x[c - 1] : -T(n) * omega * x[c + 1];
 }
 
-template <>
-struct Real<ddv> {
-  static __device__ __forceinline__ ddv sqrt2() { return ddv(dd{1.41421353816986083984375f, 2.4203234101944225e-08f}); }
-  static __device__ __forceinline__ ddv inv_sqrt2() { return ddv(dd{0.707106769084930419921875f, 1.2101617050972112e-08f}); }
-};
-template <typename T>
-__device__ __forceinline__ T sqrt2_of() { return Real<T>::SQRT2; }
-template <>
-__device__ __forceinline__ ddv sqrt2_of<ddv>() { return Real<ddv>::sqrt2(); }
-template <typename T>
-__device__ __forceinline__ T inv_sqrt2_of() { return Real<T>::INV_SQRT2; }
-template <>
-__device__ __forceinline__ ddv inv_sqrt2_of<ddv>() { return Real<ddv>::inv_sqrt2(); }
-
-// T: arithmetic type (float, double, or the double-float ddv); S: storage type
-// of every global array (T, or double for ddv)
-template <typename T, int N, int MODE, typename S = T>
+template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(128)
-    apply_kernel(const int4* __restrict__ tets, const S* __restrict__ geo,
-                 const S* __restrict__ v, const S* __restrict__ u0, const S* __restrict__ tau,
-                 S* __restrict__ t0cache, const uint8_t* __restrict__ dmask, S* __restrict__ out,
-                 const S* __restrict__ dft, Phys<T> ph, int64_t e0, int64_t e1, S* __restrict__ l0cache) {
+    apply_kernel(const int4* __restrict__ tets, const T* __restrict__ geo,
+                 const T* __restrict__ v, const T* __restrict__ u0, const T* __restrict__ tau,
+                 T* __restrict__ t0cache, const uint8_t* __restrict__ dmask, T* __restrict__ out,
+                 const T* __restrict__ dft, Phys<T> ph, int64_t e0, int64_t e1, T* __restrict__ l0cache) {
   using D = Dims<N>;
   using L = ApplyLayout<N, MODE>;
   constexpr int C = D::C, K = D::K, NM = D::NM, NT = D::NT, NTP = D::NT_PAD;
@@ -179,7 +161,7 @@ __global__ void __launch_bounds__(128)
     }
     // tau: packed symmetric (orthonormal basis) -> full matrix in storage scaling
     {
-      const S* tp = tau + e * 4 * NTP;
+      const T* tp = tau + e * 4 * NTP;
       for (int t = lane; t < 4 * NTP; t += 32) {
         const int q = t / NTP, p = t - q * NTP;
         if (p >= NT) continue;
@@ -191,14 +173,14 @@ __global__ void __launch_bounds__(128)
         const int s = r + rem;
         const T val = T(tp[t]);
         // T_s[r] = (1/d_r) sum_k tau[r][k] d_k L_s[k], d_0 = 1, d_k = sqrt2
-        const T drs = (r == 0 && s > 0) ? sqrt2_of<T>() : T(1);
-        const T dsr = (r == 0 && s > 0) ? inv_sqrt2_of<T>() : T(1);
+        const T drs = (r == 0 && s > 0) ? Real<T>::SQRT2 : T(1);
+        const T dsr = (r == 0 && s > 0) ? Real<T>::INV_SQRT2 : T(1);
         st[q * NM * NM + r * NM + s] = val * drs;
         st[q * NM * NM + s * NM + r] = val * dsr;
       }
     }
     if (LINA) {
-      const S* tp = t0cache + e * 12 * C;
+      const T* tp = t0cache + e * 12 * C;
       for (int t = lane; t < 12 * C; t += 32) t0[t] = T(tp[t]);
     }
     __syncwarp();
@@ -292,18 +274,18 @@ __global__ void __launch_bounds__(128)
       // the strong residual itself (the exact tangent's tau derivative acts on it)
       if (RES && l0cache) {
         const int cs = stor_of(r);
-        l0cache[(e * 12 + qi) * C + cs] = static_cast<S>(lu[cs] + lp[cs]);
+        l0cache[(e * 12 + qi) * C + cs] = lu[cs] + lp[cs];
       }
     }
     for (int qi = lane; qi < 12; qi += 32) {
       tq[qi * C + 1] = T(0);
       if (PAPER) tc[qi * C + 1] = T(0);
-      if (RES && l0cache) l0cache[(e * 12 + qi) * C + 1] = S(0);
+      if (RES && l0cache) l0cache[(e * 12 + qi) * C + 1] = T(0);
     }
     __syncwarp();
     if (RES) {
-      S* tp = t0cache + e * 12 * C;
-      for (int t = lane; t < 12 * C; t += 32) tp[t] = static_cast<S>(tq[t]);
+      T* tp = t0cache + e * 12 * C;
+      for (int t = lane; t < 12 * C; t += 32) tp[t] = tq[t];
     }
     // ---- phase 7: T (and T0) to samples
     warp_bmv<T, K, C>(sF, L::LDF, tq, C, ct, K, 12, lane);
@@ -375,31 +357,30 @@ __global__ void __launch_bounds__(128)
       const int f = r / C, c = r - f * C;
       if (c == 1) continue;
       if (f < 3 && dmask[node[a]]) continue;
-      S* dst = out + (int64_t)node[a] * 4 * C + r;
-      *dst += static_cast<S>(so[t]);
+      T* dst = out + (int64_t)node[a] * 4 * C + r;
+      *dst += so[t];
     }
     __syncwarp();
   }
 }
 
-template <typename T, int N, int MODE, typename S = T>
-static int launch_mode(const int4* tets, const S* geo, const S* v, const S* u0, const S* tau,
-                       S* t0cache, const uint8_t* dmask, S* out, const S* dft, Phys<T> ph,
-                       int64_t e0, int64_t e1, cudaStream_t st, S* l0cache = nullptr) {
+template <typename T, int N, int MODE>
+static int launch_mode(const int4* tets, const T* geo, const T* v, const T* u0, const T* tau,
+                       T* t0cache, const uint8_t* dmask, T* out, const T* dft, Phys<T> ph,
+                       int64_t e0, int64_t e1, cudaStream_t st, T* l0cache = nullptr) {
   using L = ApplyLayout<N, MODE>;
-  static_assert(sizeof(T) == sizeof(S) || sizeof(T) == 8, "workspace sized by T");
   if (e1 <= e0) return 0;
   int warps = 4;
   while (warps > 1 && (size_t)(L::TABLES + warps * L::WARP) * sizeof(T) > 200 * 1024) --warps;
   const size_t smem = (size_t)(L::TABLES + warps * L::WARP) * sizeof(T);
   if (smem > 227 * 1024) return -6;
-  cudaFuncSetAttribute(apply_kernel<T, N, MODE, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(apply_kernel<T, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)smem);
   int64_t blocks = (e1 - e0 + warps - 1) / warps;
   if (blocks > 152 * 32) blocks = 152 * 32;
   count_launches(1);
-  apply_kernel<T, N, MODE, S><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, v, u0, tau, t0cache,
-                                                                     dmask, out, dft, ph, e0, e1, l0cache);
+  apply_kernel<T, N, MODE><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, v, u0, tau, t0cache,
+                                                                  dmask, out, dft, ph, e0, e1, l0cache);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 

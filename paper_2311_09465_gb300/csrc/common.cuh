@@ -69,8 +69,6 @@ struct Real<double> {
   static constexpr double INV_SQRT2 = 0.70710678118654752;
 };
 
-struct ddv;   // double-float value type (ddfloat.cuh)
-
 // kernel-side view of the problem constants
 template <typename T>
 struct Phys {

@@ -6,8 +6,8 @@
 //   TwoProd with a fused multiply-add: p + e = a * b exactly.
 // sqrt and the reciprocal take one Newton correction from the FP32 value.
 // Sums carry an absolute error of about 2^-46 of the largest operand, which
-// is what the FP64 tau refinement needs; the exponent range is FP32's, so the
-// caller scales its data to magnitudes near 1 first.
+// is what the element operator and the entries of tau's matrix need; the
+// exponent range is FP32's.
 #pragma once
 
 namespace ts {
@@ -15,8 +15,6 @@ namespace ts {
 struct dd {
   float hi, lo;
 };
-
-__device__ __forceinline__ dd dd_make(float h) { return {h, 0.f}; }
 
 __device__ __forceinline__ dd dd_from_double(double x) {
   const float h = (float)x;
@@ -41,8 +39,6 @@ __device__ __forceinline__ dd dd_split(double x) {
   return {__int_as_float((int)(h | sign)), ((float)rem * 2.220446049250313e-16f) * unit};
 }
 
-__device__ __forceinline__ double dd_to_double(dd a) { return (double)a.hi + (double)a.lo; }
-
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;
   const float bb = s - a;
@@ -65,46 +61,12 @@ __device__ __forceinline__ dd dd_add(dd a, dd b) {
   return r;
 }
 
-__device__ __forceinline__ dd dd_add_f(dd a, float b) {
-  float s, e;
-  two_sum(a.hi, b, s, e);
-  e += a.lo;
-  dd r;
-  fast_two_sum(s, e, r.hi, r.lo);
-  return r;
-}
-
 // a * b + c
 __device__ __forceinline__ dd dd_fma(dd a, dd b, dd c) {
   const float p = a.hi * b.hi;
   float e = fmaf(a.hi, b.hi, -p);
   e = fmaf(a.hi, b.lo, e);
   e = fmaf(a.lo, b.hi, e);
-  float s, t;
-  two_sum(p, c.hi, s, t);
-  t += e + c.lo;
-  dd r;
-  fast_two_sum(s, t, r.hi, r.lo);
-  return r;
-}
-
-// a * b + c for FP32 a, b (the product is exact as p + e)
-__device__ __forceinline__ dd dd_fma_ff(float a, float b, dd c) {
-  const float p = a * b;
-  const float e = fmaf(a, b, -p);
-  float s, t;
-  two_sum(p, c.hi, s, t);
-  t += e + c.lo;
-  dd r;
-  fast_two_sum(s, t, r.hi, r.lo);
-  return r;
-}
-
-// a * b + c for an FP32 a
-__device__ __forceinline__ dd dd_fma_fd(float a, dd b, dd c) {
-  const float p = a * b.hi;
-  float e = fmaf(a, b.hi, -p);
-  e = fmaf(a, b.lo, e);
   float s, t;
   two_sum(p, c.hi, s, t);
   t += e + c.lo;
@@ -146,28 +108,5 @@ __device__ __forceinline__ dd dd_rcp(dd a) {
   fast_two_sum(y0, y0 * rem, r.hi, r.lo);
   return r;
 }
-
-// A double-float value type with arithmetic operators, so that kernels
-// templated on their arithmetic type can run in double-float: storage stays
-// FP64 (converted on load and store), every operation runs on the FP32 pipe.
-struct ddv {
-  dd v;
-  __host__ __device__ ddv() : v{0.f, 0.f} {}
-  __host__ __device__ ddv(double x) {
-    const float h = (float)x;
-    v = {h, (float)(x - (double)h)};
-  }
-  __host__ __device__ ddv(float x) : v{x, 0.f} {}
-  __host__ __device__ ddv(int x) : v{(float)x, 0.f} {}   // exact for |x| < 2^24
-  __device__ ddv(dd x) : v(x) {}
-  __host__ __device__ explicit operator double() const { return (double)v.hi + (double)v.lo; }
-};
-__device__ __forceinline__ ddv operator+(ddv a, ddv b) { return ddv(dd_add(a.v, b.v)); }
-__device__ __forceinline__ ddv operator-(ddv a) { return ddv(dd_neg(a.v)); }
-__device__ __forceinline__ ddv operator-(ddv a, ddv b) { return ddv(dd_add(a.v, dd_neg(b.v))); }
-__device__ __forceinline__ ddv operator*(ddv a, ddv b) { return ddv(dd_mul(a.v, b.v)); }
-__device__ __forceinline__ ddv operator/(ddv a, ddv b) { return ddv(dd_mul(a.v, dd_rcp(b.v))); }
-__device__ __forceinline__ ddv& operator+=(ddv& a, ddv b) { a.v = dd_add(a.v, b.v); return a; }
-__device__ __forceinline__ bool operator!=(ddv a, ddv b) { return a.v.hi != b.v.hi || a.v.lo != b.v.lo; }
 
 }  // namespace ts

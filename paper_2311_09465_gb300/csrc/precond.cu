@@ -24,8 +24,10 @@
 //
 // GB300 mapping: one warp per node gathers its (element, local node) pairs
 // from a node-to-element list, so each block is summed in shared memory and
-// written once (no atomics, deterministic).  The warp then inverts the block
-// in place (Gauss-Jordan, partial pivoting, FP32) and stores it column-major;
+// written once (no atomics, deterministic), and inverted before it leaves the
+// chip: for N <= 7 register tiles and the Schur complement of the velocity
+// fields (nodal_block_kernel), above that in place by Gauss-Jordan with partial
+// pivoting (block_diag_kernel).  Stored column-major;
 // the apply kernel (one warp per node, coalesced column reads) multiplies it
 // with the node's slice of a Krylov vector.
 #include <algorithm>

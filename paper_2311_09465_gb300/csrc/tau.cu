@@ -7,10 +7,12 @@
 // GB300 mapping: a group of N lanes owns one quadrature point; a warp holds
 // floor(32/N) points.  With G = L L^T (3x3 Cholesky) the argument becomes
 // M = sum_m C_m C_m + C_I nu^2 (G:G) I, C_m = A(w_m), w_m = sum_i L_im u_i,
-// because the convolution matrix is linear in the velocity modes.  The
-// symmetric eigenproblem of the real (2N-1)x(2N-1) form of M is solved by
-// parallel cyclic Jacobi (round-robin ordering, N disjoint rotations per
-// round, one per lane), padded with a decoupled dummy row to size 2N.
+// because the convolution matrix is linear in the velocity modes.  In FP32
+// (tau32_kernel) the eigenpairs of the real (2N-1)x(2N-1) form of M come from a
+// one-sided Jacobi iteration in registers (onesided.cuh); in FP64 by default from
+// tau_fx.cu.  tau_kernel is the FP64 form on request: parallel cyclic Jacobi on M in
+// shared memory (round-robin ordering, N disjoint rotations per round, one per
+// lane), padded with a decoupled dummy row to size 2N.
 // tau = V diag(lambda^{-1/2}) V^T is written as a packed upper triangle.
 #include <algorithm>
 
