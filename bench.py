@@ -193,7 +193,8 @@ def _tau_flops(case):
 
 
 def _tau_dd_instr(case):
-    """FP32 instructions of the double-float refinement in one tau_dd launch.
+    """FP32 instructions of tau by a double-float Newton-Schulz refinement, the
+    yardstick for the fixed-point form that replaced it.
 
     Per quadrature point (n = 2N - 1, t = n(n+1)/2): M (3 t n), the second
     Newton-Schulz Gram matrix, B and tau (t n each, symmetric) and the four
@@ -294,10 +295,10 @@ def run_gpu(args):
     value = _job_rate(ws, E, N, ops, t_total)
     ms_step = t_total / args.steps * 1e3
 
-    # ---- kernel timings.  The dominant kernel of the step (largest share of
-    # device time in the ncu launch list) is tau_dd_kernel, the tau of the FP64
-    # residual; its time and the tangent product's element kernel come from the
-    # library's own CUDA events on the launching stream (ts_stage_times).
+    # ---- kernel timings.  The two largest kernels of the step are jvp32_kernel
+    # (the FP32 tangent product) and tau_fx_kernel (tau of the FP64 residual, the
+    # longest launch); their times come from the library's own CUDA events on the
+    # launching stream (ts_stage_times).
     R = 20
     r64 = torch.empty_like(y)
     t_tau, t_res64 = [], []
@@ -306,12 +307,11 @@ def run_gpu(args):
         st_ = ts.ts_stage_times(g.prob)
         t_tau.append(st_["tau_ms"] / 1e3)
         t_res64.append(st_["residual_element_ms"] / 1e3)
-    t_tau_cold = float(np.mean(t_tau))
+    t_tau_alone = float(np.mean(t_tau))
     t_res64 = float(np.mean(t_res64))
     # the roofline's launch time: the tau launches of the timed solve (CUDA
-    # events around each one, summed by ts_solve; all but the first start
-    # their eigensolve from the previous step's eigenvectors)
-    t_tau = rep["t_tau"] / max(rep["n_residual"], 1) if rep.get("n_residual") else t_tau_cold
+    # events around each one, summed by ts_solve)
+    t_tau = rep["t_tau"] / max(rep["n_residual"], 1) if rep.get("n_residual") else t_tau_alone
     y32 = y.float().contiguous()
     ts.ts_residual(g.prob, y32, torch.empty_like(y32))
     v32 = torch.tensor(np.random.default_rng(0).standard_normal(y.shape), dtype=torch.float32, device="cuda")
@@ -363,14 +363,12 @@ def run_gpu(args):
     achieved = alg / t_jel / 1e9
     csrc = os.path.join(ROOT, "paper_2311_09465_gb300", "csrc")
     traffic = _profile_traffic(os.path.join(csrc, "jvp32.cuh"))
-    # FP32 peaks: SMs x 128 FP32 lanes x the maximum SM clock (instructions), x 2 (FMA flops)
+    # FP32 peak: SMs x 128 FP32 lanes x 2 (FMA flops) x the maximum SM clock
     sms = torch.cuda.get_device_properties(local).multi_processor_count
-    alu_peak = sms * 128 * _sm_max_mhz() * 1e6 / 1e12
-    fma_peak = 2 * alu_peak
-    tau_work = _tau_dd_instr(case)
+    fma_peak = 2 * sms * 128 * _sm_max_mhz() * 1e6 / 1e12
     tau_flops = _tau_flops(case)
     jvp_flops = _jvp_flops(case)
-    tau_traffic = _profile_traffic(os.path.join(csrc, "tau_dd.cu"), "tau_dd_traffic.json", "dram_bytes_per_launch")
+    tau_traffic = _profile_traffic(os.path.join(csrc, "tau_fx.cu"), "tau_fx_traffic.json", "dram_bytes_per_launch")
 
     # ---- end-to-end through the public API with host buffers
     y_host = y0.cpu().pin_memory()
@@ -402,15 +400,12 @@ def run_gpu(args):
         "roofline": {"bound": "alu", "achieved": tau_flops / t_tau / 1e12, "peak": fma_peak,
                      "unit": "TFLOP/s", "frac": tau_flops / t_tau / 1e12 / fma_peak,
                      "traffic": tau_traffic,
-                     "kernel": "tau_dd_kernel<7> (tau of the FP64 residual, double-float refinement)",
+                     "kernel": "tau_fx_kernel<7> (tau of the FP64 residual, fixed-point refinement)",
                      "algorithmic_flops": tau_flops, "flop_model": "45 n_m^3 per quadrature point",
                      "launch_ms": t_tau * 1e3, "launches_timed": int(rep.get("n_residual", 0)),
-                     "launch_ms_cold": t_tau_cold * 1e3,
+                     "launch_ms_outside_solve": t_tau_alone * 1e3,
                      "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 x {_sm_max_mhz():.0f} MHz "
-                                    "(an FMA probe measured 78.4 TFLOP/s FP32, 1.25 FP64)",
-                     "issue": {"achieved": tau_work / t_tau / 1e12, "peak": alu_peak,
-                               "unit": "T FP32 instructions/s", "frac": tau_work / t_tau / 1e12 / alu_peak,
-                               "instructions": tau_work}},
+                                    "(an FMA probe measured 78.4 TFLOP/s FP32, 1.25 FP64)"},
         "roofline_tangent": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                              "frac": achieved / peak, "traffic": traffic,
                              "kernel": "jvp32_kernel<7, LIN_A> (FP32 tangent product, element pass)",
@@ -434,7 +429,7 @@ def run_gpu(args):
         "cpu_baseline": cpu,
         "clocks": clk,
         "breakdown": {"jvp_fp32_ms": t_jvp * 1e3, "jvp_element_kernel_ms": t_jel * 1e3,
-                      "tau_dd_ms": t_tau * 1e3, "residual_fp64_element_pass_ms": t_res64 * 1e3,
+                      "tau_ms": t_tau * 1e3, "residual_fp64_element_pass_ms": t_res64 * 1e3,
                       "residual_fp32_ms": t_res32 * 1e3,
                       "solve_report": {k: rep[k] for k in ("steps", "matvecs", "t_residual", "t_jvp", "t_krylov")}},
         "time_to_residual_1e-8": ttr or None,
@@ -449,7 +444,7 @@ def run_gpu(args):
 def _elem64(tau64):
     """The plain FP64 legs run every FP64 operation as FP64 instructions
     (tau by the FP64 refinement, the native FP64 element operator); the mixed
-    legs use the library defaults (double-float tau and element pass)."""
+    legs use the library defaults (fixed-point tau, double-float element pass)."""
     return "native" if tau64 == "refine" else None
 
 

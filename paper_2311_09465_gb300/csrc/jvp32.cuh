@@ -255,7 +255,9 @@ constexpr unsigned FULL = 0xffffffffu;
 template <int N, int MODE>
 struct J32Layout {
   static constexpr int C = 2 * N, K = 3 * N - 2, NTP = Dims<N>::NT_PAD;
-  static constexpr int KP = (K + 3) & ~3;   // sample rows padded to 16 bytes
+  // sample rows: an odd number of 16-byte units, so that the rows of a 16-byte access
+  // by 8 lanes fall into different banks (point phase: rows [i][q], lanes (i, q))
+  static constexpr int KP = ((K + 3) & ~3) | 4;
   static constexpr bool LINA = MODE == MODE_JVP_LIN_A || MODE == MODE_JVP_EXACT;
   static constexpr int STG_TAU = 0;                               // [2][4][NTP]
   static constexpr int STG_T0 = STG_TAU + EPW * 4 * NTP;          // [2][4][3][C] (LIN_A)
@@ -265,14 +267,21 @@ struct J32Layout {
   static constexpr int GM = VM + 16 * C;               // gradients [4 f][3 j][C]
   static constexpr int VS = GM + 12 * C;               // sum over nodes [4 f][C]
   static constexpr int GE = VS + 4 * C;                // dN_a/dx_j [12], volume, pad, node ids [4]
-  static constexpr int CT = GE + 20;                    // c, later T samples [4 q][3 i][KP]
-  static constexpr int TS = CT + 12 * KP;               // T0 samples [4 q][3 i][KP] (LIN_A)
-  // SUPG sums [3 j][3 i][KP], then Z modes; they take the place of v at the nodes
+  static constexpr int CT = GE + 20;                    // c, later T samples [3 i][4 q][KP]
+  static constexpr int TS = CT + 12 * KP;               // T0 samples [3 i][4 q][KP] (LIN_A)
+  // SUPG sums [3 j][3 i][WP], then Z modes; they take the place of v at the nodes
   // (dead after the point phase) when that is large enough
-  static constexpr bool WS_IN_VM = 9 * KP <= 16 * C;
+  static constexpr int WP = 9 * KP <= 16 * C ? KP : (K + 3) & ~3;
+  static constexpr bool WS_IN_VM = 9 * WP <= 16 * C;
   static constexpr int END = TS + (LINA ? 12 * KP : 0);
   static constexpr int WS = WS_IN_VM ? VM : END;
-  static constexpr int ELEM = WS_IN_VM ? END : END + 9 * KP;
+  static constexpr int RAW = WS_IN_VM ? END : END + 9 * WP;
+  // In the per-sample phases lanes 0..K-1 take the samples of the first element and
+  // lanes S1.. those of the second, whose rows start S1 banks further: every access
+  // of a full warp is one wavefront.  With both and the rows above, N = 5 runs
+  // 326 -> 267 us (lin_a, 187,266 tetrahedra), N = 7 412 -> 390 us.
+  static constexpr int S1 = (K + 3) & ~3;
+  static constexpr int ELEM = RAW + ((S1 - RAW) % 32 + 32) % 32;
   static constexpr int WORK = EPW * ELEM;
   static constexpr int WARP = STG + WORK;
 };
@@ -367,8 +376,9 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
   const float4* __restrict__ u0t = reinterpret_cast<const float4*>(I.u0t);
   const float4* __restrict__ vt = reinterpret_cast<const float4*>(I.vt);
 #pragma unroll 1
-  for (int t = lane; t < EPW * K; t += 32) {
-    const int s = t >= K ? 1 : 0, k = t - s * K;
+  for (int t = lane; t < L::S1 + K; t += 32) {
+    const int s = t >= L::S1 ? 1 : 0, k = t - s * L::S1;
+    if (k >= K) continue;
     const float* g = work + s * L::ELEM + L::GE;
     const int4 nd = *reinterpret_cast<const int4*>(g + 16);
     float dN[12];
@@ -412,7 +422,7 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
           acc = fmaf(fmaf(QD, ua[qq][j], su[j]), gv[i][j], acc);
           if (LINA) acc = fmaf(fmaf(QD, va[qq][j], sv[j]), gu[i][j], acc);
         }
-        ct[(qq * 3 + i) * L::KP] = acc;
+        ct[(i * 4 + qq) * L::KP] = acc;
       }
   }
   __syncwarp();
@@ -433,7 +443,7 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
     float cm[C];
     {
       float ctv[K];
-      ld4<K>(es + L::CT + (q * 3 + i) * L::KP, ctv);
+      ld4<K>(es + L::CT + (i * 4 + q) * L::KP, ctv);
       inv<N>(ctv, cm);
     }
     float G[C], Lm[C], dp[C];
@@ -474,13 +484,13 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
     {
       float Tt[K];
       fwd<N>(T, Tt);
-      st4<K>(es + L::CT + (q * 3 + i) * L::KP, Tt);
+      st4<K>(es + L::CT + (i * 4 + q) * L::KP, Tt);
     }
     if (LINA) {
       float T0m[C], T0t[K];
       ld2<C>(stg + L::STG_T0 + ((slot * 4 + q) * 3 + i) * C, T0m);
       fwd<N>(T0m, T0t);
-      st4<K>(es + L::TS + (q * 3 + i) * L::KP, T0t);
+      st4<K>(es + L::TS + (i * 4 + q) * L::KP, T0t);
     }
     {
       // row (a = q, i): mass_coef V/20 (sum_b v_ib + v_ia) - dN_a/dx_i V pbar
@@ -523,8 +533,9 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
   }
   // ---- C: one lane per (element, sample): SUPG products W_ji = sum_q u0_j T_i (+ v_j T0_i)
 #pragma unroll 1
-  for (int t = lane; t < EPW * K; t += 32) {
-    const int s = t >= K ? 1 : 0, k = t - s * K;
+  for (int t = lane; t < L::S1 + K; t += 32) {
+    const int s = t >= L::S1 ? 1 : 0, k = t - s * L::S1;
+    if (k >= K) continue;
     const float* ew = work + s * L::ELEM;
     const int4 nd = *reinterpret_cast<const int4*>(ew + L::GE + 16);
     const int na[4] = {nd.x, nd.y, nd.z, nd.w};
@@ -563,8 +574,8 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
       }
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const float Ti = ew[L::CT + (qq * 3 + i) * L::KP + k];
-        const float T0i = LINA ? ew[L::TS + (qq * 3 + i) * L::KP + k] : 0.f;
+        const float Ti = ew[L::CT + (i * 4 + qq) * L::KP + k];
+        const float T0i = LINA ? ew[L::TS + (i * 4 + qq) * L::KP + k] : 0.f;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
           W[j][i] = fmaf(uq[j], Ti, W[j][i]);
@@ -576,7 +587,7 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) ws[(j * 3 + i) * L::KP] = W[j][i];
+      for (int i = 0; i < 3; ++i) ws[(j * 3 + i) * L::WP] = W[j][i];
   }
   __syncwarp();
   // ---- D: SUPG sums to modes, one lane per (element, j, i), in place, with the
@@ -585,7 +596,7 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
     const int s = lane >= 9 ? 1 : 0, ji = lane - 9 * s;
     const int j = ji / 3, i = ji - 3 * j;
     const float* ew = work + s * L::ELEM;
-    float* p = work + s * L::ELEM + L::WS + ji * L::KP;
+    float* p = work + s * L::ELEM + L::WS + ji * L::WP;
     float wt[K], wm[C], gm[C];
     ld4<K>(p, wt);
     inv<N>(wt, wm);
@@ -610,7 +621,7 @@ __device__ __forceinline__ bool j32_pass(const J32Inst I, int64_t base, const fl
       const int i = f;
 #pragma unroll
       for (int j = 0; j < 3; ++j) {   // SUPG + viscous
-        ld2<C>(es + L::WS + (j * 3 + i) * L::KP, x);
+        ld2<C>(es + L::WS + (j * 3 + i) * L::WP, x);
 #pragma unroll
         for (int c = 0; c < C; ++c) row[c] = fmaf(da[j], x[c], row[c]);
       }
@@ -637,8 +648,11 @@ __device__ __forceinline__ void j32_abort(float* out, uint32_t bar, uint32_t par
   mbar_wait(bar, parity);
 }
 
+// blocks an SM: what the register file holds without spills
+constexpr int j32_blocks(int N) { return N == 1 ? 7 : N == 2 ? 8 : N == 3 ? 7 : N == 4 ? 6 : N == 5 ? 5 : 4; }
+
 template <int N, int MODE>
-__global__ void __launch_bounds__(128) jvp32_kernel(J32Inst I) {
+__global__ void __launch_bounds__(128, j32_blocks(N)) jvp32_kernel(J32Inst I) {
   using L = J32Layout<N, MODE>;
   extern __shared__ __align__(128) float smem[];
   __shared__ __align__(8) uint64_t s_bar[4];
