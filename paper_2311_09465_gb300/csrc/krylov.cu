@@ -5,15 +5,17 @@
 //
 // Reductions are two-stage and deterministic: a fixed grid of blocks writes
 // per-block partial sums, one warp per vector adds them in block order.
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace ts {
 
-// at most 4 blocks per SM (11% less Gram-Schmidt time than 2 or 6 per SM on a
-// 2.1M-unknown field); small fields take one block per 2048 entries, so that
+// at most 2 blocks per SM: dots_kernel keeps 3 values a thread of five streams in
+// registers (120 of them); small fields take one block per 2048 entries, so that
 // launch and reduction overheads do not grow with the grid
-constexpr int RED_BLOCKS = 608;
+constexpr int RED_BLOCKS = 304;
 static int dots_blocks(int64_t n) {
   const int64_t b = (n + 2047) / 2048;
   return (int)(b < 1 ? 1 : (b > RED_BLOCKS ? RED_BLOCKS : b));
@@ -48,64 +50,83 @@ __device__ __forceinline__ double warp_sum4(const double (&a)[4], int lane) {
 // partial[j * gridDim.x + b] = sum over block b's chunk of basis_j . w for
 // j < nvec (nvec >= 1), and with self != 0 also row nvec = w . w.  With *skip != 0 the
 // block writes zeros and reads nothing (a second Gram-Schmidt pass that is not
-// needed).  On GB300 the multiply-adds run on the FP64 pipe (two a clock and SM),
-// where the warp reductions were 20 additions to 48 multiply-adds a lane: over a
-// Krylov space of 30 vectors of 2.1M values a call averages 48 us (72 with them).
-__global__ void __launch_bounds__(RED_THREADS) dots_kernel(const double* __restrict__ basis,
-                                                           int64_t ld, int nvec,
-                                                           const double* __restrict__ w,
-                                                           int64_t n, double* __restrict__ partial,
-                                                           int self, const double* __restrict__ skip) {
+// needed).  On GB300 the multiply-adds run on the FP64 pipe (two a clock and SM:
+// 13.7 us for a group of four vectors of 2.1M values).  To keep it busy, loads are issued
+// DOT_BATCH values of a thread ahead, and warps run through DOT_STASH groups without a
+// barrier (their sums wait in shared memory).  Two Newton steps of 30 products with 2.1M
+// unknowns, all Krylov kernels: 18.5 ms; 21.1 with one or two values ahead and a barrier a
+// group, 19.2 with 2 ahead and 4 blocks an SM, 18.8 with 4 ahead and 2.
+constexpr int DOT_BATCH = 3, DOT_STASH = 16;
+
+__global__ void __launch_bounds__(RED_THREADS, 2)
+    dots_kernel(const double* __restrict__ basis, int64_t ld, int nvec, const double* __restrict__ w, int64_t n,
+                double* __restrict__ partial, int self, const double* __restrict__ skip) {
   const int nout = nvec + (self ? 1 : 0);
   if (skip != nullptr && *skip != 0.0) {
     for (int j = threadIdx.x; j < nout; j += blockDim.x) partial[(int64_t)j * gridDim.x + blockIdx.x] = 0.0;
     return;
   }
-  __shared__ double red[2][RED_THREADS / 32][DOT_GROUP];
+  __shared__ double red[DOT_STASH][RED_THREADS / 32][DOT_GROUP];
+  __shared__ double red_self[RED_THREADS / 32];
   const int64_t chunk = ((n + gridDim.x - 1) / gridDim.x + 1) & ~(int64_t)1;
   const int64_t i0 = (int64_t)blockIdx.x * chunk;
   const int64_t i1 = i0 + chunk < n ? i0 + chunk : n;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double self_acc = 0;
-  int flip = 0;
-  for (int j0 = 0; j0 < nvec; j0 += DOT_GROUP, flip ^= 1) {
-    const int nj = nvec - j0 < DOT_GROUP ? nvec - j0 : DOT_GROUP;
-    double acc[DOT_GROUP] = {0, 0, 0, 0};
-    const double* bj = basis + (int64_t)j0 * ld;
-    if (nj == DOT_GROUP) {
-#pragma unroll 2
-      for (int64_t i = i0 + threadIdx.x; i < i1; i += RED_THREADS) {
-        const double wi = w[i];
+  double self_acc = 0, acc[DOT_GROUP];
+  auto pass = [&](auto count, const double* bj, bool with_self) {   // acc = the sums of COUNT vectors
+    constexpr int COUNT = decltype(count)::value;
 #pragma unroll
-        for (int jj = 0; jj < DOT_GROUP; ++jj) acc[jj] = fma(bj[(int64_t)jj * ld + i], wi, acc[jj]);
-        if (self && j0 == 0) self_acc = fma(wi, wi, self_acc);
-      }
-    } else {
-      for (int64_t i = i0 + threadIdx.x; i < i1; i += RED_THREADS) {
-        const double wi = w[i];
+    for (int jj = 0; jj < DOT_GROUP; ++jj) acc[jj] = 0;
+    const double* wp = w + i0 + threadIdx.x;
+    const double* bp = bj + i0 + threadIdx.x;
+    int left = (int)(i1 - i0) - (int)threadIdx.x;       // values from this one to the chunk's end
+#pragma unroll 1
+    for (; left > 0; left -= DOT_BATCH * RED_THREADS, wp += DOT_BATCH * RED_THREADS, bp += DOT_BATCH * RED_THREADS) {
+      double x[DOT_BATCH], b[DOT_BATCH][COUNT];
 #pragma unroll
-        for (int jj = 0; jj < DOT_GROUP; ++jj)
-          if (jj < nj) acc[jj] = fma(bj[(int64_t)jj * ld + i], wi, acc[jj]);
-        if (self && j0 == 0) self_acc = fma(wi, wi, self_acc);
+      for (int u = 0; u < DOT_BATCH; ++u)
+        if (u * RED_THREADS < left) {
+          x[u] = wp[u * RED_THREADS];
+#pragma unroll
+          for (int jj = 0; jj < COUNT; ++jj) b[u][jj] = bp[(int64_t)jj * ld + u * RED_THREADS];
+        }
+#pragma unroll
+      for (int u = 0; u < DOT_BATCH; ++u)
+        if (u * RED_THREADS < left) {
+#pragma unroll
+          for (int jj = 0; jj < COUNT; ++jj) acc[jj] = fma(b[u][jj], x[u], acc[jj]);
+          if (with_self) self_acc = fma(x[u], x[u], self_acc);
+        }
+    }
+  };
+  for (int base = 0; base < nvec; base += DOT_GROUP * DOT_STASH) {
+    const int end = nvec - base < DOT_GROUP * DOT_STASH ? nvec : base + DOT_GROUP * DOT_STASH;
+    if (base > 0) __syncthreads();                       // the sums before this batch are read
+    for (int j0 = base; j0 < end; j0 += DOT_GROUP) {
+      const double* bj = basis + (int64_t)j0 * ld;
+      const bool with_self = self && j0 == 0;
+      switch (end - j0) {
+        case 1: pass(std::integral_constant<int, 1>{}, bj, with_self); break;
+        case 2: pass(std::integral_constant<int, 2>{}, bj, with_self); break;
+        case 3: pass(std::integral_constant<int, 3>{}, bj, with_self); break;
+        default: pass(std::integral_constant<int, DOT_GROUP>{}, bj, with_self);
       }
+      const double s = warp_sum4(acc, lane);
+      if ((lane & 7) == 0) red[(j0 - base) / DOT_GROUP][warp][lane >> 3] = s;
     }
-    const double s = warp_sum4(acc, lane);
-    if ((lane & 7) == 0) red[flip][warp][lane >> 3] = s;
-    __syncthreads();                     // the other buffer's readers are past it: one barrier a group
-    if ((int)threadIdx.x < nj) {
-      double t = 0;
-      for (int k = 0; k < RED_THREADS / 32; ++k) t += red[flip][k][threadIdx.x];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+    if (self && base == 0) {
+      const double s = warp_sum(self_acc);
+      if (lane == 0) red_self[warp] = s;
     }
-  }
-  if (self) {   // row nvec: w . w (accumulated with the first group)
     __syncthreads();
-    const double s = warp_sum(self_acc);
-    if (lane == 0) red[0][warp][0] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    for (int j = base + threadIdx.x; j < end; j += RED_THREADS) {
       double t = 0;
-      for (int k = 0; k < RED_THREADS / 32; ++k) t += red[0][k][0];
+      for (int k = 0; k < RED_THREADS / 32; ++k) t += red[(j - base) / DOT_GROUP][k][(j - base) % DOT_GROUP];
+      partial[(int64_t)j * gridDim.x + blockIdx.x] = t;
+    }
+    if (self && base == 0 && threadIdx.x == RED_THREADS - 1) {   // row nvec: w . w
+      double t = 0;
+      for (int k = 0; k < RED_THREADS / 32; ++k) t += red_self[k];
       partial[(int64_t)nvec * gridDim.x + blockIdx.x] = t;
     }
   }
