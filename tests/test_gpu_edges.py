@@ -89,6 +89,25 @@ def test_a_bad_node_stays_in_its_elements(N, bits):
     g.close()
 
 
+@pytest.mark.parametrize("N,bits", [(3, 64), (7, 64), (10, 64), (10, 32)])
+def test_the_first_product_can_be_captured(N, bits):
+    # a product after a residual of its own precision allocates nothing
+    import torch
+    import paper_2311_09465_gb300 as ts
+    case = _case(N, "tiny")
+    g = ts.GLSProblem(case, variant="frozen", dt_pseudo=0.6)
+    g.residual(to_dev(_state(case, seed=41), _dtype(bits)))
+    v = to_dev(cases.random_state(case.mesh, N, seed=42, smooth=False), _dtype(bits))
+    hv = torch.empty_like(v)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g.jvp(v, hv)
+    hv.zero_()
+    graph.replay()
+    np.testing.assert_array_equal(to_np(hv), to_np(g.jvp(v)))
+    g.close()
+
+
 @pytest.mark.parametrize("bits", [64, 32])
 def test_outlet_with_more_nodes_than_threads(bits):
     import paper_2311_09465_gb300 as ts
@@ -188,3 +207,20 @@ def test_tracer_with_ragged_counts(N, mesh, bits):
     assert rel_l2(got, tr.tracer_residual(tp, a, phi)) <= TOL[bits]
     t.close()
     ts.ts_mesh_free(h)
+
+
+@pytest.mark.parametrize("krylov", [1, 3, 5, 66])
+def test_gram_schmidt_group_remainders(krylov):
+    # dot products run four basis vectors at a time and 64 between barriers: with every
+    # remainder the solve reaches the root
+    import torch
+    import paper_2311_09465_gb300 as ts
+    case = _case(3, "pipe")
+    g = ts.GLSProblem(case, variant="lin_a", dt_pseudo=0.3)
+    y = to_dev(case.y0, torch.float64)
+    rep = g.solve(y, precision=64, tol=1e-6, max_steps=400, krylov=krylov, eps_ls=0.05, max_matvec=4000, precond=1)
+    r = to_np(g.residual(y))
+    assert rep["status"] == 0
+    assert np.linalg.norm(r) <= 1.0001 * rep["r_final"] * rep["r_ref"]
+    assert rel_l2(r, op.residual(op.problem_from_case(case), to_np(y))) <= 1e-5   # small against r itself
+    g.close()
