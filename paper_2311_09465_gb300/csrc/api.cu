@@ -356,7 +356,27 @@ static int prepare_state(ts_problem* pr, LinState<T>& l, const T* y, cudaStream_
   return 0;
 }
 
-// out = the element operator on v (the state itself for the residual)
+// Scratch of the one-launch element operator, taken at a state's first residual so
+// that products allocate nothing.  Without room for it, or inside a capture, the
+// colour-ordered kernel runs, which needs none.
+template <typename T>
+static bool element_scratch(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
+  if (l.rows) return true;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return false;
+  const ts_mesh* m = pr->mesh;
+  if (cudaMalloc(&l.vc, (size_t)field_len(pr) * sizeof(T)) == cudaSuccess &&
+      cudaMalloc(&l.vs, (size_t)m->V * 3 * pr->K * sizeof(T)) == cudaSuccess &&
+      cudaMalloc(&l.rows, (size_t)m->E * 16 * pr->C * sizeof(T)) == cudaSuccess)
+    return true;
+  cudaGetLastError();                     // the failed allocation is not this call's error
+  dfree(l.vc);
+  dfree(l.vs);
+  l.rows = nullptr;
+  return false;
+}
+
+// out = the element operator on v (the state itself for the residual), after element_scratch
 template <typename T, int N>
 static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T* out, bool with_mass,
                          cudaStream_t st, T* l0 = nullptr) {
@@ -366,12 +386,9 @@ static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T
   if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
   const bool res = mode == MODE_RESIDUAL;
   if (!res) {
-    if (!l.vc) TS_TRY(dalloc(&l.vc, (size_t)field_len(pr)));
-    if (!l.vs) TS_TRY(dalloc(&l.vs, (size_t)m->V * 3 * pr->K));
     if (launch_node_prepass<V, N>(v, pr->d_dmask, (V*)l.vc, (V*)l.vs, (const V*)l.trig, m->V, st))
       return fail(TS_ERR_CUDA, "node pre-pass launch failed");
   }
-  if (!l.rows) TS_TRY(dalloc(&l.rows, (size_t)m->E * 16 * pr->C));
   const Phys<double> ph = phys_of<double>(pr, with_mass);
   ElementArgs<V> a;
   a.tets = m->d_tets;
@@ -467,7 +484,8 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
   }
   l.prepared = false;
   // FP32, and FP64 in double-float: one element launch; native FP64: colours
-  const bool one_launch = sizeof(T) == 4 || pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT;
+  const bool one_launch =
+      (sizeof(T) == 4 || pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) && element_scratch(pr, l, st);
   if (one_launch || (sizeof(T) == 8 && pr->tau64 == TS_TAU64_DOUBLEFLOAT)) TS_TRY((prepare_state<T, N>(pr, l, y, st)));
   TS_CUDA(cudaEventRecord(pr->sev[0], st));
   int rc;
@@ -593,7 +611,7 @@ static int jvp_impl(ts_problem* pr, const T* v, T* hv, cudaStream_t st) {
     TS_TRY(outlet_terms<T>(pr, v, 1, hv, st));
     return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
   }
-  if (sizeof(T) == 4 ? pr->fast32 : pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) {
+  if ((sizeof(T) == 4 ? pr->fast32 : pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) && element_scratch(pr, l, st)) {
     TS_TRY((element_apply<T, N>(pr, mode, l, v, hv, true, st)));
     return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
   }
