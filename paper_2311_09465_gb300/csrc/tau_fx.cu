@@ -180,9 +180,11 @@ struct FxLayout {
   static constexpr int WARP = GPW * GROUP;
 };
 
-// y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2
+// y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2.  Blocks of 128 threads an SM:
+// N <= 3 6 (85 registers; N = 3, 187,266 tetrahedra: 735 us, 751 with 4), N = 4, 5 4 (2.63 ms at N = 5,
+// 2.74 with 2, 2.81 with 5), N = 7 3, above that the compiler's choice (N = 10 with 3: 6.1 ms, 5.6 so).
 template <int N>
-__global__ void __launch_bounds__(128, N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
+__global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
                                                      const float2* __restrict__ y, int64_t n_qp,
                                                      double* __restrict__ tau_out, dd nu2,
                                                      unsigned* __restrict__ n_unconverged,
