@@ -451,7 +451,7 @@ int  ts_tracer_set_dirichlet(ts_tracer* tracer, int tag);
 /* r(phi) for the advecting velocity a: caller-owned device arrays of the
  * given precision, a [V][3][N][2] (the velocity part of a modal field), phi and
  * r [V][N][2] (one field of the modal layout).  Computes tau at every point
- * (FP64: the double-float refinement; FP32: FP32 Jacobi) into library-owned
+ * (FP64: the fixed-point refinement; FP32: FP32 Jacobi) into library-owned
  * buffers allocated at the first call.  r may not alias a or phi. */
 int  ts_tracer_residual(ts_tracer* tracer, const void* a, const void* phi, void* r, int precision,
                         void* stream);
