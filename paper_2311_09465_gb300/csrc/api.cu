@@ -79,6 +79,7 @@ struct LinState {
   T* vs = nullptr;
   T* rows = nullptr;    // [E][4][4][C] element rows
   bool prepared = false;   // uc, us belong to u0
+  unsigned* hard = nullptr;   // T = double: points that tau_fx leaves to FP64 (HARD_LIST + 4E)
   T* u0t = nullptr;     // [V][K][4] u0 velocity sampled in time (FP32 fast path)
   T* vt = nullptr;      // [V][K][4] scratch of the FP32 fast path: the product's input sampled
   T* bneg = nullptr;    // [backflow points][NT_PAD] |A_n|_- (section 2.6)
@@ -216,6 +217,7 @@ static int lin_alloc(ts_problem* pr, LinState<T>& l) {
   std::vector<T> tt(tab.begin(), tab.end());
   TS_TRY(dalloc(&l.dft, tt.size()));
   TS_CUDA(cudaMemcpy(l.dft, tt.data(), tt.size() * sizeof(T), cudaMemcpyHostToDevice));
+  if (sizeof(T) == 8) TS_TRY(dalloc(&l.hard, (size_t)(HARD_LIST + 4 * m->E)));
   if (sizeof(T) == 4) {
     TS_TRY(dalloc(&l.u0t, (size_t)m->V * 4 * pr->K));
     TS_TRY(dalloc(&l.vt, (size_t)m->V * 4 * pr->K));
@@ -247,6 +249,7 @@ static void lin_free(LinState<T>& l) {
   dfree(l.vc);
   dfree(l.vs);
   dfree(l.rows);
+  dfree(l.hard);
   l.prepared = false;
   dfree(l.vt);
   dfree(l.bneg);
@@ -341,7 +344,7 @@ static int upload_trig(int N, T** out) {
   return 0;
 }
 
-// the state's operands (uc, us) from y
+// the state's operands (uc, us) from y, and its copy u0 where y is the caller's
 template <typename T, int N>
 static int prepare_state(ts_problem* pr, LinState<T>& l, const T* y, cudaStream_t st) {
   using V = typename PairOf<T>::V;
@@ -350,7 +353,8 @@ static int prepare_state(ts_problem* pr, LinState<T>& l, const T* y, cudaStream_
   if (!l.trig) TS_TRY(upload_trig<T>(N, &l.trig));
   if (!l.uc) TS_TRY(dalloc(&l.uc, (size_t)field_len(pr)));
   if (!l.us) TS_TRY(dalloc(&l.us, (size_t)m->V * 3 * pr->K));
-  if (launch_node_prepass<V, N>(y, nullptr, (V*)l.uc, (V*)l.us, (const V*)l.trig, m->V, st))
+  if (launch_node_prepass<V, N>(y, nullptr, (V*)l.uc, (V*)l.us, (const V*)l.trig, m->V, st, l.hard,
+                                y == l.u0 ? nullptr : l.u0))
     return fail(TS_ERR_CUDA, "node pre-pass launch failed");
   l.prepared = true;
   return 0;
@@ -473,7 +477,6 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
   LinState<T>& l = lin_of<T>(pr);
   TS_TRY(lin_alloc(pr, l));
   const int64_t n = field_len(pr);
-  TS_CUDA(cudaMemcpyAsync(l.u0, y, n * sizeof(T), cudaMemcpyDeviceToDevice, st));
   // the exact tangent also needs the eigenpairs of M and the strong residual
   const bool exact = pr->p.jvp_variant == TS_JVP_EXACT;
   float* eig = nullptr;
@@ -486,17 +489,23 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
   // FP32, and FP64 in double-float: one element launch; native FP64: colours
   const bool one_launch =
       (sizeof(T) == 4 || pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) && element_scratch(pr, l, st);
-  if (one_launch || (sizeof(T) == 8 && pr->tau64 == TS_TAU64_DOUBLEFLOAT)) TS_TRY((prepare_state<T, N>(pr, l, y, st)));
+  if (one_launch || (sizeof(T) == 8 && pr->tau64 == TS_TAU64_DOUBLEFLOAT))
+    TS_TRY((prepare_state<T, N>(pr, l, y, st)));
+  else
+    TS_CUDA(cudaMemcpyAsync(l.u0, y, n * sizeof(T), cudaMemcpyDeviceToDevice, st));
   TS_CUDA(cudaEventRecord(pr->sev[0], st));
   int rc;
   if constexpr (sizeof(T) == 8) {
     if (pr->tau64 == TS_TAU64_JACOBI)
       rc = launch_tau<T, N>(m->d_tets, geo_of<T>(m), y, m->E, l.tau, (T)(pr->p.mu / pr->p.rho),
                             (T)pr->p.C_I, pr->d_counter, st, eig);
-    else if (pr->tau64 == TS_TAU64_DOUBLEFLOAT)
-      rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, (const float2*)l.uc, m->E, (double*)l.tau, pr->p.mu / pr->p.rho,
-                            pr->p.C_I, pr->d_counter, st, eig);
-    else
+    else if (pr->tau64 == TS_TAU64_DOUBLEFLOAT) {
+      const double nu = pr->p.mu / pr->p.rho;
+      rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, (const float2*)l.uc, m->E, (double*)l.tau, nu, pr->p.C_I, l.hard, st,
+                            eig);
+      rc |= launch_tau_hard<N>(m->d_tets, m->d_geo64, (const double*)y, l.hard, (double*)l.tau, nu, pr->p.C_I,
+                               pr->d_counter, st);
+    } else
       rc = launch_tau_polish<N>(m->d_tets, m->d_geo64, (const double*)y, m->E, (double*)l.tau,
                                 pr->p.mu / pr->p.rho, pr->p.C_I, pr->d_counter, st, eig);
   } else {
@@ -1605,6 +1614,7 @@ struct ts_tracer {
   template <typename T>
   struct Work {
     T *a4 = nullptr, *tau = nullptr, *trig = nullptr, *at = nullptr, *phi = nullptr, *rows = nullptr;
+    unsigned* hard = nullptr;   // points that tau_fx leaves to FP64
   };
   Work<double> w64;
   Work<float> w32;
@@ -1664,8 +1674,10 @@ int tracer_prepare(ts_tracer* tr, const T* a, cudaStream_t st) {
   int rc;
   if constexpr (sizeof(T) == 8) {
     if (!tr->add) TS_TRY(dalloc(&tr->add, (size_t)n));
-    if (launch_split_dd(w.a4, tr->add, n, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
-    rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, tr->add, m->E, w.tau, tr->kappa, tr->C_I, tr->d_counter, st);
+    if (!w.hard) TS_TRY(dalloc(&w.hard, (size_t)(HARD_LIST + 4 * m->E)));
+    if (launch_split_dd(w.a4, tr->add, n, w.hard, st)) return fail(TS_ERR_CUDA, "split kernel launch failed");
+    rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, tr->add, m->E, w.tau, tr->kappa, tr->C_I, w.hard, st);
+    rc |= launch_tau_hard<N>(m->d_tets, m->d_geo64, w.a4, w.hard, w.tau, tr->kappa, tr->C_I, tr->d_counter, st);
   } else {
     rc = launch_tau<float, N>(m->d_tets, m->d_geo32, w.a4, m->E, w.tau, (float)tr->kappa, (float)tr->C_I,
                               tr->d_counter, st);
@@ -1854,6 +1866,7 @@ void ts_tracer_free(ts_tracer* t) {
   dfree(t->w64.at);
   dfree(t->w64.phi);
   dfree(t->w64.rows);
+  dfree(t->w64.hard);
   dfree(t->w32.a4);
   dfree(t->w32.tau);
   dfree(t->w32.trig);

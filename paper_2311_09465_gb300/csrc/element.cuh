@@ -558,10 +558,12 @@ template <typename V, int N>
 __global__ void __launch_bounds__(128) node_prepass_kernel(const typename StoreOf<V>::S* __restrict__ y,
                                                            const uint8_t* __restrict__ dmask, V* __restrict__ clean,
                                                            V* __restrict__ samples, const V* __restrict__ trig,
-                                                           int64_t n_nodes) {
+                                                           int64_t n_nodes, unsigned* __restrict__ zero,
+                                                           typename StoreOf<V>::S* __restrict__ copy) {
   using R = Ar<V>;
   constexpr int C = 2 * N, K = 3 * N - 2, KH = K / 2;
   __shared__ V table[2 * N * (KH + 1)];
+  if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
   for (int t = threadIdx.x; t < 2 * N * (KH + 1); t += blockDim.x) table[t] = trig[t];
   __syncthreads();
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_nodes * 4; t += (int64_t)gridDim.x * blockDim.x) {
@@ -571,7 +573,9 @@ __global__ void __launch_bounds__(128) node_prepass_kernel(const typename StoreO
     V x[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      x[c] = c == 1 || fixed ? R::zero() : R::from(y[t * C + c]);
+      const typename StoreOf<V>::S value = y[t * C + c];
+      if (copy) copy[t * C + c] = value;
+      x[c] = c == 1 || fixed ? R::zero() : R::from(value);
       if (clean) clean[t * C + c] = x[c];
       if (c > 1) x[c] = R::twice(x[c]);
     }
@@ -629,11 +633,12 @@ int launch_element(int mode, const ElementArgs<V>& P, cudaStream_t st) {
 
 template <typename V, int N>
 int launch_node_prepass(const typename StoreOf<V>::S* y, const uint8_t* dmask, V* clean, V* samples, const V* trig,
-                        int64_t n_nodes, cudaStream_t st) {
+                        int64_t n_nodes, cudaStream_t st, unsigned* zero,
+                        typename StoreOf<V>::S* copy) {
   if (n_nodes <= 0) return 0;
   const int64_t blocks = std::min<int64_t>((n_nodes * 4 + 127) / 128, 152 * 32);
   count_launches(1);
-  node_prepass_kernel<V, N><<<(int)blocks, 128, 0, st>>>(y, dmask, clean, samples, trig, n_nodes);
+  node_prepass_kernel<V, N><<<(int)blocks, 128, 0, st>>>(y, dmask, clean, samples, trig, n_nodes, zero, copy);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 

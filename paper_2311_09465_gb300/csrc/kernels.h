@@ -35,12 +35,21 @@ int launch_tau_polish(const int4* tets, const double* geo, const double* y, int6
                       cudaStream_t st, float* eig_out = nullptr);
 
 // FP64 tau from FP32 eigenpairs and Newton corrections with residuals in 58-bit
-// fixed point (tau_fx.cu); y: the state as double-float pairs [V][4][C]
+// fixed point (tau_fx.cu); y: the state as double-float pairs [V][4][C].  Points it
+// does not take (tau_fx.cu) are listed in hard, to be redone by launch_tau_hard:
+// hard[0] their number (zero before the launch), hard[HARD_LIST..] element * 4 + point
+constexpr int HARD_LIST = 4;
 template <int N>
 int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t n_elem, double* tau_out, double nu,
-                  double C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out = nullptr);
-// n doubles as (hi, lo) FP32 pairs
-int launch_split_dd(const double* in, float2* out, int64_t n, cudaStream_t st);
+                  double C_I, unsigned* hard, cudaStream_t st, float* eig_out = nullptr);
+// FP64 tau of the listed points, for any condition number: the FP64 refinement with
+// Jacobi sweeps in FP64 on its nearly diagonal matrix (tau.cu); y: [V][4][C].
+// n_unconverged counts points whose smallest eigenvalues FP64 does not resolve
+template <int N>
+int launch_tau_hard(const int4* tets, const double* geo, const double* y, const unsigned* hard, double* tau_out,
+                    double nu, double C_I, unsigned* n_unconverged, cudaStream_t st);
+// n doubles as (hi, lo) FP32 pairs; hard[0] = 0
+int launch_split_dd(const double* in, float2* out, int64_t n, unsigned* hard, cudaStream_t st);
 
 // Backflow stabilisation on one Neumann face set (tau.cu): when y_for_matrix
 // is given, first |A_n|_- at the 3 points of every face into bneg; then
@@ -109,10 +118,11 @@ struct ElementArgs {
 template <typename V, int N>
 int launch_element(int mode, const ElementArgs<V>& P, cudaStream_t st);
 // clean (may be null) = y without fixed entries (dmask null: all velocities kept),
-// samples of its velocity
+// samples of its velocity; *zero = 0, copy = y as it is (both may be null)
 template <typename V, int N>
 int launch_node_prepass(const typename StoreOf<V>::S* y, const uint8_t* dmask, V* clean, V* samples, const V* trig,
-                        int64_t n_nodes, cudaStream_t st);
+                        int64_t n_nodes, cudaStream_t st, unsigned* zero = nullptr,
+                        typename StoreOf<V>::S* copy = nullptr);
 // out = per node the sum of its element rows [4][fields][C]; on Dirichlet nodes the
 // first `masked` fields are zero
 template <typename V>

@@ -57,7 +57,8 @@ __device__ __forceinline__ void rotation_of(float ax, float ay, float g, float& 
 // of NM rows of LD floats (16-byte aligned, LD a multiple of 4 and >= NM), of
 // which a lane uses its own two.  base: the group's first lane; own: whether the
 // lane belongs to a group.  floor: a lower bound of the eigenvalues, hence of the
-// exact pivots; rounding may take a computed pivot below it.
+// exact pivots; rounding may take a computed pivot below it.  Returns the smallest
+// pivot as computed, the same in the whole group (lanes outside: of the first group).
 // ROLLED: a loop over pivots in which the registers move up one row a step, so
 // that the pivot is always at index 0, and finished columns go through shared
 // memory.  Unrolled it needs no memory and half the shuffles, but is up to a
@@ -65,9 +66,10 @@ __device__ __forceinline__ void rotation_of(float ax, float ay, float g, float& 
 // cache (fixed-point tau, N = 10: 34.5 ms unrolled, 8.0 rolled; N = 7: 10.8 and
 // 10.7; N = 5: 3.6 and 3.7; FP32 tau, N = 10: 2.42 and 2.16, N = 7: 2.60 and 2.99).
 template <int N, int LD, bool ROLLED>
-__device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, bool own, int base,
-                                                 float floor, float* rows) {
+__device__ __forceinline__ float cholesky_columns(float (&x)[2 * N - 1], float (&y)[2 * N - 1], int p, bool own, int base,
+                                                  float floor, float* rows) {
   constexpr int NM = 2 * N - 1;
+  float least = 3e38f;
   if constexpr (!ROLLED) {
     // a lane outside a group must stay zero: no column of it is a pivot
     const int jx = own ? 2 * p - 1 : 4 * N, jy = own ? 2 * p : 4 * N;
@@ -78,6 +80,7 @@ __device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&
 #pragma unroll
       for (int i = k; i < NM; ++i) l[i] = __shfl_sync(0xffffffffu, (k & 1) ? x[i] : y[i], src);
       const float piv = fmaxf(l[k], floor), rd = rsqrt_newton(piv);
+      least = fminf(least, l[k]);
       const float mx = jx > k ? x[k] * rd * rd : 0.f, my = jy > k ? y[k] * rd * rd : 0.f;
 #pragma unroll
       for (int i = k + 1; i < NM; ++i) {
@@ -88,7 +91,7 @@ __device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&
       if (jx >= k) x[k] = jx == k ? piv * rd : 0.f;
       if (jy >= k) y[k] = jy == k ? piv * rd : 0.f;
     }
-    return;
+    return least;
   }
   float* rx = rows + (own && p > 0 ? 2 * p - 1 : 0) * LD;
   float* ry = rows + 2 * p * LD;
@@ -107,6 +110,7 @@ __device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&
 #pragma unroll
     for (int i = 0; i < NM; ++i) l[i] = __shfl_sync(0xffffffffu, odd ? x[i] : y[i], src);
     const float rd = rsqrt_newton(fmaxf(l[0], floor));
+    least = fminf(least, l[0]);
     l[0] = fmaxf(l[0], floor);
     if (own && p == (k + 1) / 2) {
       float* dst = (odd ? rx : ry) + k;
@@ -135,6 +139,7 @@ __device__ __forceinline__ void cholesky_columns(float (&x)[2 * N - 1], float (&
         y[4 * j + t] = own ? bv[t] : 0.f;
       }
   }
+  return least;
 }
 
 // One-sided Jacobi on the group's columns.  Sweeps until every pair of the warp

@@ -485,7 +485,14 @@ int preload_tau() {
 //   f[a,b,c] = (s_a + s_b + s_c) / (s_a s_b s_c (s_a+s_b)(s_b+s_c)(s_a+s_c)),
 // which gives, with X_ik = E_ik / (s_i s_k (s_i + s_k)) and E = offdiag(B),
 //   Z = diag(1/s) - X + X D_s X + (X D_{s^2} X) ./ (s_i + s_j),
-// tau = V Z V^T, error third order in E.
+// tau = V Z V^T, error third order in E / (s_i s_j).
+//
+// LISTED: the points that the fixed-point form leaves out (tau_fx.cu), mostly with large
+// condition numbers.  E, 1e-7 of the largest eigenvalue, is not small there against the
+// smallest ones, so Jacobi sweeps in FP64 on B (two or three: it starts nearly diagonal)
+// reduce it first; M is scaled to FP32's range by a power of four, and eigenvalues are at
+// least c = C_I nu^2 G:G, their lower bound.  The sweeps stop early or late with equal
+// eigenvalues, where the expansion needs no more.  Bound by the FP64 pipe.
 template <int N>
 struct PolishLayout {
   static constexpr int NP = 2 * N, NM = 2 * N - 1, C = 2 * N, LD = NP + 1;
@@ -500,14 +507,15 @@ struct PolishLayout {
   static constexpr int WARP = GPW * GROUP + 64 + 32; // + double and float reduction scratch
 };
 
-template <int N>
-__global__ void __launch_bounds__(128) tau_polish_kernel(const int4* __restrict__ tets,
+template <int N, bool LISTED>
+__global__ void __launch_bounds__(LISTED ? 256 : 128) tau_polish_kernel(const int4* __restrict__ tets,
                                                          const double* __restrict__ geo,
                                                          const double* __restrict__ y,
                                                          int64_t n_qp, double* __restrict__ tau_out,
                                                          double nu, double C_I,
                                                          unsigned* __restrict__ n_unconverged,
-                                                         float* __restrict__ eig_out) {
+                                                         float* __restrict__ eig_out,
+                                                         const unsigned* __restrict__ hard) {
   using L = PolishLayout<N>;
   constexpr int NP = L::NP, NM = L::NM, C = L::C, LD = L::LD, GPW = L::GPW;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -526,11 +534,12 @@ __global__ void __launch_bounds__(128) tau_polish_kernel(const int4* __restrict_
   double* red_d = wbase + GPW * L::GROUP;
   float* red_f = reinterpret_cast<float*>(red_d + 64);
 
+  if (LISTED) n_qp = hard[0];
   const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
   for (int64_t qb = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * GPW; qb < n_qp;
        qb += warps_total * GPW) {
-    const int64_t gq = qb + g;
-    const bool live = in_group && gq < n_qp;
+    const bool live = in_group && qb + g < n_qp;
+    const int64_t gq = LISTED ? (live ? hard[HARD_LIST + qb + g] : 0) : qb + g;
     const int64_t e = live ? gq >> 2 : 0;
     const int q = (int)(gq & 3);
     double diff = 0;
@@ -585,14 +594,30 @@ __global__ void __launch_bounds__(128) tau_polish_kernel(const int4* __restrict_
         }
         M[r * LD + s] = acc;
         M[s * LD + r] = acc;
-        Mf[r * LD + s] = (float)acc;
-        Mf[s * LD + r] = (float)acc;
+        if (!LISTED) {
+          Mf[r * LD + s] = (float)acc;
+          Mf[s * LD + r] = (float)acc;
+        }
         Vf[r * LD + s] = (r == s) ? 1.f : 0.f;
         Vf[s * LD + r] = (r == s) ? 1.f : 0.f;
       }
     __syncwarp();
+    if (LISTED) {
+      if (live) {
+        double top = 0;
+        for (int i = 0; i < NM; ++i) top = fmax(top, M[i * LD + i]);
+        int ex;
+        frexp(top, &ex);
+        const double sc = ldexp(1.0, -ex);
+        for (int t = k; t < NP * NP; t += N) {
+          const int r = t / NP, s = t - r * NP;
+          Mf[r * LD + s] = r < NM && s < NM ? (float)(M[r * LD + s] * sc) : r == s ? 1.f : 0.f;
+        }
+      }
+      __syncwarp();
+    }
     const bool conv32 = jacobi_group<float, N>(Mf, Vf, k, g, lane, live, red_f, 12, 1e-12f);
-    if (live && k == 0 && !conv32) atomicAdd(n_unconverged, 1u);
+    if (!LISTED && live && k == 0 && !conv32) atomicAdd(n_unconverged, 1u);
     // V in FP64, re-orthonormalised by two Newton-Schulz steps V <- V (3I - V^T V) / 2
     // (the FP32 eigenvectors are orthonormal only to FP32 rounding)
     if (live)
@@ -638,6 +663,16 @@ __global__ void __launch_bounds__(128) tau_polish_kernel(const int4* __restrict_
         M[s * LD + r] = acc;
       }
     __syncwarp();
+    if (LISTED) {
+      jacobi_group<double, N>(M, Vd, k, g, lane, live, red_d, 8, 1e-36);
+      if (live)
+        for (int i = k; i < NM; i += N) {
+          // below half of its bound: FP64 does not resolve it
+          if (!(M[i * LD + i] > 0.5 * diff)) atomicAdd(n_unconverged, 1u);
+          M[i * LD + i] = fmax(M[i * LD + i], diff);
+        }
+      __syncwarp();
+    }
     if (live && eig_out) {
       float* eo = eig_out + gq * Dims<N>::EIG;
       for (int t = k; t < NM * NM; t += N) eo[t] = (float)Vd[(t / NM) * LD + t % NM];
@@ -705,15 +740,34 @@ int launch_tau_polish(const int4* tets, const double* geo, const double* y, int6
   while (warps > 1 && (size_t)warps * L::WARP * sizeof(double) > 200 * 1024) --warps;
   const size_t smem = (size_t)warps * L::WARP * sizeof(double);
   if (smem > 227 * 1024) return -6;
-  cudaFuncSetAttribute(tau_polish_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(tau_polish_kernel<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const int64_t n_qp = n_elem * 4;
   const int64_t groups = (n_qp + L::GPW - 1) / L::GPW;
   int64_t blocks = (groups + warps - 1) / warps;
   if (blocks > 152 * 64) blocks = 152 * 64;
   if (blocks < 1) blocks = 1;
   count_launches(1);
-  tau_polish_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, nu, C_I,
-                                                              n_unconverged, eig_out);
+  tau_polish_kernel<N, false><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, nu, C_I,
+                                                                     n_unconverged, eig_out, nullptr);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
+}
+
+// One block an SM: the list is empty for most flows, and a full one keeps the FP64 pipe
+// busy with the 5 warps (N = 7) that fit.
+template <int N>
+int launch_tau_hard(const int4* tets, const double* geo, const double* y, const unsigned* hard, double* tau_out,
+                    double nu, double C_I, unsigned* n_unconverged, cudaStream_t st) {
+  using L = PolishLayout<N>;
+  int warps = 8;
+  while (warps > 1 && (size_t)warps * L::WARP * sizeof(double) > 200 * 1024) --warps;
+  const size_t smem = (size_t)warps * L::WARP * sizeof(double);
+  static_assert(L::WARP * sizeof(double) <= 227 * 1024, "a warp's shared memory");
+  if (cudaFuncSetAttribute(tau_polish_kernel<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+      cudaSuccess)
+    return -2;
+  count_launches(1);
+  tau_polish_kernel<N, true><<<152, warps * 32, smem, st>>>(tets, geo, y, 0, tau_out, nu, C_I, n_unconverged, nullptr,
+                                                            hard);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
@@ -721,6 +775,10 @@ int launch_tau_polish(const int4* tets, const double* geo, const double* y, int6
   template int launch_tau_polish<N>(const int4*, const double*, const double*, int64_t,      \
                                     double*, double, double, unsigned*, cudaStream_t, float*);
 TS_FOR_EACH_N(TS_INST_POLISH, double)
+#define TS_INST_HARD(T, N)                                                                     \
+  template int launch_tau_hard<N>(const int4*, const double*, const double*, const unsigned*, double*, double, double, \
+                                  unsigned*, cudaStream_t);
+TS_FOR_EACH_N(TS_INST_HARD, double)
 
 
 // ---------------------------------------------------------------------------

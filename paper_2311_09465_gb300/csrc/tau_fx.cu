@@ -9,8 +9,13 @@
 // Sylvester equation is solved in the FP32 eigenbasis, E_ab = R_ab / (s_a + s_b).
 // The start X0 = U diag(1/s) U^T rounded to 29 bits leaves |R| near 1e-6; the
 // first correction leaves |R| near 1e-11 and the second is below the output's
-// rounding.  Matrices whose FP32 eigenpairs are poor (very large condition
-// number) take more corrections, up to FX_MAX_IT.
+// rounding.  With the eigenbasis held fixed the corrections converge only from FP32
+// eigenpairs that resolve the smallest eigenvalue, and the integers hold R only while
+// |M X| stays near 1; a point whose smallest eigenvalue is below FX_LAMBDA of its
+// scale, or whose last R is not small, is therefore put on a list, and
+// tau_polish_kernel redoes it in FP64 (tau.cu; the point's result here is overwritten).
+// Without the list such points came out wrong by up to a factor of 1000 (one harmonic
+// without a mean, u h / nu = 3e4 and above).
 //
 // Fixed point: a value v, |v| <= 1, is the integer V = v 2^58, split into two
 // signed limbs V = 2^29 h + l, |h| <= 2^29, |l| <= 2^28, l kept as FP32 (24 bits:
@@ -44,6 +49,13 @@ namespace {
 
 constexpr int FX_MAX_IT = 10;
 constexpr float FX_ORTHO2 = 1e-6f;   // leaves cosines near 1e-6: the corrections absorb them
+// Smallest eigenvalue, of a point's scale of 1, that this form takes.  tau's error there
+// is about 2^-54 / lambda: near 1e-12 at 2^-14, where FP64 takes over with its
+// 2^-53 / lambda or less.  The flows with a mean of tests and bench stay above 2^-12.
+constexpr float FX_LAMBDA = 6.103515625e-5f;
+// Pivots of the FP32 factor below this (a pivot is no smaller than the smallest
+// eigenvalue, and FP32 rounding stays below 1e-5) mean a point for the list
+constexpr float FX_PIVOT = 0.25f * FX_LAMBDA;
 
 using i64 = long long;
 
@@ -180,14 +192,15 @@ struct FxLayout {
   static constexpr int WARP = GPW * GROUP;
 };
 
-// y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2.  Blocks of 128 threads an SM:
+// y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2; hard: the list
+// (HARD_LIST in kernels.h).  Blocks of 128 threads an SM:
 // N <= 3 6 (85 registers; N = 3, 187,266 tetrahedra: 735 us, 751 with 4), N = 4, 5 4 (2.63 ms at N = 5,
 // 2.74 with 2, 2.81 with 5), N = 7 3, above that the compiler's choice (N = 10 with 3: 6.1 ms, 5.6 so).
 template <int N>
 __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
                                                      const float2* __restrict__ y, int64_t n_qp,
                                                      double* __restrict__ tau_out, dd nu2,
-                                                     unsigned* __restrict__ n_unconverged,
+                                                     unsigned* __restrict__ hard,
                                                      float* __restrict__ eig_out) {
   using Lt = FxLayout<N>;
   constexpr int NM = Lt::NM, C = Lt::C, L = Lt::L, LDQ = Lt::LDQ, LDF = Lt::LDF, GPW = Lt::GPW, TW = Lt::TW;
@@ -375,6 +388,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
     __syncwarp();
     // ---- FP32 eigenpairs: f_a with M = sum f_a f_a^T
     int xe;                                             // |X| <= 2^xe
+    bool on_list;
     {
       float x[NM], yv[NM];
       constexpr float H = 1.f / 536870912.f, HL = H * H;   // 2^-29, 2^-58
@@ -384,15 +398,18 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
         x[i] = hx ? fmaf(__int_as_float(mm.y), HL, (float)mm.x * H) : 0.f;
         yv[i] = hy ? fmaf(__int_as_float(mm.w), HL, (float)mm.z * H) : 0.f;
       }
-      const float cd = fx_float(cfix) * HL;
-      cholesky_columns<N, LDF, (N > 5)>(x, yv, p, in_group, first, fmaxf(cd, 1e-30f), F);
-      __syncwarp();
-      const bool conv = onesided_jacobi<N>(x, yv, p, lane, FX_ORTHO2);
-      {
-        const unsigned bad = __ballot_sync(0xffffffffu, live && !conv);
-        const unsigned mine = ((1u << N) - 1u) << first;
-        if (live && p == 0 && (bad & mine)) atomicAdd(n_unconverged, 1u);
+      const float least = cholesky_columns<N, LDF, (N > 5)>(x, yv, p, in_group, first, FX_PIVOT, F);
+      on_list = !(least > FX_PIVOT);
+      if (__any_sync(0xffffffffu, on_list)) {
+        // the factor of such a point means nothing: I takes its place
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          x[i] = !on_list ? x[i] : hx && i == cx ? 1.f : 0.f;
+          yv[i] = !on_list ? yv[i] : hy && i == cy ? 1.f : 0.f;
+        }
       }
+      __syncwarp();
+      onesided_jacobi<N>(x, yv, p, lane, FX_ORTHO2);
       float ax = 0.f, ay = 0.f;
 #pragma unroll
       for (int i = 0; i < NM; ++i) {
@@ -404,6 +421,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
       float big = fmaxf(ix, iy), all = 0.f;
 #pragma unroll
       for (int j = 0; j < N; ++j) all = fmaxf(all, __shfl_sync(0xffffffffu, big, first + j));
+      on_list = on_list || !(all * all * FX_LAMBDA <= 1.f);
       frexpf(1.01f * all, &xe);
       xe = min(max(xe, 0), 28);
       // eigenpairs for the derivative of tau (exact tangent), when asked
@@ -456,7 +474,8 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
       }
     }
     const float rscale = ldexpf(1.f, xe - 58), escale = ldexpf(1.f, 58 - xe);
-    const float small = fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
+    // what is left to correct; negative, so never reached, at a point for the list
+    const float small = on_list ? -1.f : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
     // ---- corrections
 #pragma unroll 1
     for (int it = 0;; ++it) {
@@ -521,7 +540,12 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
           }
         }
       }
-      const bool more = __any_sync(0xffffffffu, live && rmax > small) && it + 1 < FX_MAX_IT;
+      const unsigned left = __ballot_sync(0xffffffffu, live && rmax > small);
+      const bool more = __any_sync(0xffffffffu, live && rmax > small && small > 0.f) && it + 1 < FX_MAX_IT;
+      if (left && !more) {
+        const unsigned mine = ((1u << N) - 1u) << first;
+        if (live && p == 0 && finite && (left & mine)) hard[HARD_LIST + atomicAdd(hard, 1u)] = (unsigned)gq;
+      }
       __syncwarp();
       // E = U [(U^T R U)_ab / (s_a + s_b)] U^T, row by row; R is symmetric (column = row)
       float rx[LDF], ry[LDF];
@@ -629,7 +653,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
 
 template <int N>
 int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t n_elem, double* tau_out, double nu,
-                  double C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out) {
+                  double C_I, unsigned* hard, cudaStream_t st, float* eig_out) {
   using Lt = FxLayout<N>;
   // warps a block (1..4) that keep the most warps resident in 227 KB of shared memory
   int warps = 1, best = 0;
@@ -651,7 +675,7 @@ int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t 
   const float kh = (float)k;
   count_launches(1);
   tau_fx_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, dd{kh, (float)(k - (double)kh)},
-                                                          n_unconverged, eig_out);
+                                                          hard, eig_out);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
@@ -660,19 +684,21 @@ int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t 
                                 unsigned*, cudaStream_t, float*);
 TS_FOR_EACH_N(TS_INST_TAU_FX, double)
 
-// double -> (hi, lo) pairs of FP32 numbers
-__global__ void split_dd_kernel(const double* __restrict__ in, float2* __restrict__ out, int64_t n) {
+// double -> (hi, lo) pairs of FP32 numbers; empties tau's list
+__global__ void split_dd_kernel(const double* __restrict__ in, float2* __restrict__ out, int64_t n,
+                                unsigned* __restrict__ hard) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *hard = 0;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const dd v = dd_from_double(in[t]);
     out[t] = make_float2(v.hi, v.lo);
   }
 }
 
-int launch_split_dd(const double* in, float2* out, int64_t n, cudaStream_t st) {
+int launch_split_dd(const double* in, float2* out, int64_t n, unsigned* hard, cudaStream_t st) {
   if (n <= 0) return 0;
   const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 16);
   count_launches(1);
-  split_dd_kernel<<<(int)blocks, 256, 0, st>>>(in, out, n);
+  split_dd_kernel<<<(int)blocks, 256, 0, st>>>(in, out, n, hard);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
