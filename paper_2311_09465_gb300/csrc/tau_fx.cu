@@ -56,6 +56,11 @@ constexpr float FX_LAMBDA = 6.103515625e-5f;
 // Pivots of the FP32 factor below this (a pivot is no smaller than the smallest
 // eigenvalue, and FP32 rounding stays below 1e-5) mean a point for the list
 constexpr float FX_PIVOT = 0.25f * FX_LAMBDA;
+// Smallest diagonal entry that this form takes.  Where a mode hardly couples to the
+// others (a cosine without a mean, N = 2: its sine) the entry is an eigenvalue, which
+// floating point has to a relative 2^-53 and fixed point to 2^-54 of the scale: 1e-14
+// of it at 2^-8.  Tests and bench: above 2^-6.
+constexpr float FX_DIAGONAL = 3.90625e-3f;
 
 using i64 = long long;
 
@@ -235,7 +240,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
     const int q = (int)(gq & 3);
     // ---- w_m = sum_i L_im u_i for mode p, G = L L^T (double-float)
     dd diff;
-    float bound = 0.f;
+    float n2 = 0.f;
     __syncwarp();
     {
       const double* gg = geo + e * GEO_STRIDE + GEO_G;
@@ -280,16 +285,19 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
           park[2 * TW] = make_float2(w1.hi, w1.lo);
           park[4 * TW] = make_float2(w2.hi, w2.lo);
         }
-        // |C_m| <= beta_m = |w_0| + 2 sum |w_n|: with sum_m beta_m + sqrt(c) <= 1 after
-        // the scale 2^-ex, M's eigenvalues (and so its entries) are at most 1
-        bound += (fabsf(w0.hi) + fabsf(w1.hi) + fabsf(w2.hi)) * (p == 0 ? 1.f : 2.f);
+        n2 = fmaf(w0.hi, w0.hi, fmaf(w1.hi, w1.hi, fmaf(w2.hi, w2.hi, n2)));
       }
     }
+    // |C_m| <= beta_m = |w_m0| + 2 sum_n |w_mn|, so |sum_m C_m^2| <= sum_m beta_m^2 <=
+    // (|w_0| + 2 sum_n |w_n|)^2, |w_n| over the three m: with that plus c at most 1 after
+    // the scale 2^-ex, M's eigenvalues (and so its entries) are at most 1
+    float bound;
     {
+      const float mag = sqrtf(n2) * (p == 0 ? 1.f : 2.f);
       float sum = 0.f;
 #pragma unroll
-      for (int j = 0; j < N; ++j) sum += __shfl_sync(0xffffffffu, bound, first + j);
-      bound = 1.0001f * (sum + sqrtf(diff.hi));
+      for (int j = 0; j < N; ++j) sum += __shfl_sync(0xffffffffu, mag, first + j);
+      bound = 1.0001f * sqrtf(fmaf(sum, sum, diff.hi));
     }
     const bool finite = bound < 4e18f && bound > 2e-19f;   // 2^-ex squared stays in range
     int ex = 0;
@@ -399,7 +407,11 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
         yv[i] = hy ? fmaf(__int_as_float(mm.w), HL, (float)mm.z * H) : 0.f;
       }
       const float least = cholesky_columns<N, LDF, (N > 5)>(x, yv, p, in_group, first, FX_PIVOT, F);
-      on_list = !(least > FX_PIVOT);
+      {
+        const float dx = hx ? (float)Ms[cx * LDQ + cx + 1].h : 1e9f, dy = hy ? (float)Ms[cy * LDQ + cy + 1].h : 1e9f;
+        const unsigned small = __ballot_sync(0xffffffffu, fminf(dx, dy) < FX_DIAGONAL * 536870912.f);   // 2^29
+        on_list = !(least > FX_PIVOT) || (small & (((1u << N) - 1u) << first));
+      }
       if (__any_sync(0xffffffffu, on_list)) {
         // the factor of such a point means nothing: I takes its place
 #pragma unroll

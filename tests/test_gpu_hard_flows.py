@@ -86,3 +86,44 @@ def test_fp64_residuals_of_ill_conditioned_flows(N, flow, peclet):
     assert np.linalg.norm(got - ref) <= bar * np.linalg.norm(ref)
     t.close()
     ts.ts_mesh_free(h)
+
+
+def _cosine_rows(tp, a, h, phi):
+    """Tracer rows in closed form: velocity a cos(h t) along z, h = N - 1, and phi uniform
+    with harmonic h alone.  The sine is in the null space of the convolution and the
+    cosine and the mean have its square 2 a^2, so tau is 1 / sqrt(c) and
+    1 / sqrt(2 a^2 G_zz + c)."""
+    s = tp.omega * h
+    c = tp.C_I * tp.kappa ** 2 * np.einsum("eij,eij->e", tp.G, tp.G)
+    res = np.array([-s * phi[1], s * phi[0]])
+    T = np.stack([res[0] / np.sqrt(2 * a * a * tp.G[:, 2, 2] + c), res[1] / np.sqrt(c)])
+    r = np.zeros((tp.xyz.shape[0], tp.N, 2))
+    for k in range(4):
+        np.add.at(r[:, h, 0], tp.tets[:, k], tp.vol / 4 * (res[0] + s * T[1]))
+        np.add.at(r[:, h, 1], tp.tets[:, k], tp.vol / 4 * (res[1] - s * T[0]))
+        np.add.at(r[:, 0, 0], tp.tets[:, k], tp.vol * tp.dN[:, k, 2] * 2 * a * T[0])
+    return r
+
+
+@pytest.mark.parametrize("peclet", [1e2, 3e2, 1e4])
+@pytest.mark.parametrize("N", [2, 3, 5])
+def test_fp64_tau_of_a_cosine_without_a_mean(N, peclet):
+    # an eigenvalue alone in its row keeps its relative accuracy: 2^-46 holds the 2^-53 of
+    # sums of some 30 terms and tau's 2^-54 over a diagonal entry of at least 2^-8
+    import torch
+    import paper_2311_09465_gb300 as ts
+    mesh = mg.pipe(nc=1, nr=1, nz=1)
+    h = N - 1
+    size = float(np.mean(op.problem_from_case(cases.pipe_case(N=N, Re=100.0, Wo=5.0, mesh=mesh)).vol) ** (1 / 3))
+    tp = tr.make_tracer_problem(mesh.xyz, mesh.tets, N, size / peclet, 1.0, np.zeros(mesh.n_nodes, dtype=bool), 3.0)
+    vel = np.zeros((mesh.n_nodes, 3, N, 2))
+    vel[:, 2, h, 0] = 0.5
+    phi = np.zeros((mesh.n_nodes, N, 2))
+    phi[:, h] = 1.0, 1.0
+    ref = _cosine_rows(tp, 0.5, h, (1.0, 1.0))
+    hm = ts.ts_mesh_load(mesh.xyz, mesh.tets, mesh.bfaces, mesh.btag)
+    t = ts.Tracer(hm, mesh.n_nodes, N, tp.kappa, 1.0, 3.0)
+    got = to_np(t.residual(to_dev(vel, torch.float64), to_dev(phi, torch.float64)))
+    assert np.linalg.norm(got - ref) <= 2.0 ** -46 * np.linalg.norm(ref)
+    t.close()
+    ts.ts_mesh_free(hm)
