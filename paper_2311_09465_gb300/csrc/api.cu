@@ -503,8 +503,9 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
       const double nu = pr->p.mu / pr->p.rho;
       rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, (const float2*)l.uc, m->E, (double*)l.tau, nu, pr->p.C_I, l.hard, st,
                             eig);
+      if (eig) rc |= launch_tau_pairs<N>((const double*)l.tau, m->E, eig, st);
       rc |= launch_tau_hard<N>(m->d_tets, m->d_geo64, (const double*)y, l.hard, (double*)l.tau, nu, pr->p.C_I,
-                               pr->d_counter, st);
+                               pr->d_counter, st, eig);
     } else
       rc = launch_tau_polish<N>(m->d_tets, m->d_geo64, (const double*)y, m->E, (double*)l.tau,
                                 pr->p.mu / pr->p.rho, pr->p.C_I, pr->d_counter, st, eig);

@@ -17,6 +17,8 @@
 //
 // GB300 mapping: one warp per quadrature point, the point's n x n matrices
 // (n = 2N - 1) in shared memory, lanes over matrix entries.
+#include <algorithm>
+
 #include "common.cuh"
 #include "jacobi.cuh"
 #include "kernels.h"
@@ -204,6 +206,206 @@ int launch_dtau(const int4* tets, const float* geo, const float* u0, const float
   dtau_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, u0, v, dmask, eig, l0, dT, n_qp);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
+
+// Eigenpairs after an FP64 residual.  The fixed-point tau leaves FP32 ones whose
+// eigenvalues are good to 1e-7 of the largest eigenvalue; tau itself is good to FP64, so
+// they are refined on it: V^T tau V in FP64 is nearly diagonal and has the small
+// eigenvalues of M as its large ones, and FP32 Jacobi sweeps on it keep every eigenvalue
+// to a few 1e-7 of itself.  V's own error R = I - V^T V, near 1e-6, enters to first order:
+//   B = V^T tau V + (R D + D R) / 2, D its diagonal;   B = W diag(mu) W^T;
+//   V <- V (I + R / 2) W,   lambda = mu^-2.
+//
+// Mapping: a group of N lanes a point, columns 2p-1 and 2p in lane p, as in tau.cu.  The
+// two FP64 products (4 NM^3 flops a point) are the whole arithmetic on the FP64 pipe.
+// N = 7, 187,266 tetrahedra: 13 ms, about half of it the FP64 pipe, the rest
+// mostly Jacobi sweeps in shared memory (45 ms with M, its products and an orthonormalisation in
+// FP64, tau_polish_kernel's way).
+template <int N>
+struct PairsLayout {
+  static constexpr int NM = 2 * N - 1, NP = 2 * N, LD = NP + 1, LDD = 2 * N, GPW = 32 / N;
+  // in 4-byte words
+  static constexpr int T = 0;                      // tau [NM][LDD] doubles, later R [NM][LDD] floats
+  static constexpr int VD = T + 2 * NM * LDD;      // row a: vector a, doubles
+  static constexpr int VS = VD + 2 * NM * LDD;     // the same, floats
+  static constexpr int B = VS + NM * LDD;          // [NP][LD]
+  static constexpr int W = B + NP * LD;            // [NP][LD]
+  static constexpr int D = W + NP * LD;            // diagonal [NM]
+  static constexpr int GROUP = (D + NM + 3) & ~3;
+  static constexpr int WARP = GPW * GROUP + 64;    // + reduction scratch
+};
+
+template <int N>
+__global__ void __launch_bounds__(128) pairs_kernel(const double* __restrict__ tau, float* __restrict__ eig, int64_t n_qp) {
+  using Lt = PairsLayout<N>;
+  constexpr int NM = Lt::NM, NP = Lt::NP, LD = Lt::LD, LDD = Lt::LDD, GPW = Lt::GPW;
+  extern __shared__ __align__(16) float smem_f[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane / N, p = lane - (lane / N) * N;
+  const bool in_group = g < GPW;
+  float* wbase = smem_f + warp * Lt::WARP;
+  float* base = wbase + (in_group ? g : 0) * Lt::GROUP;
+  double* T = reinterpret_cast<double*>(base + Lt::T);
+  float* R = base + Lt::T;
+  double* VD = reinterpret_cast<double*>(base + Lt::VD);
+  float* VS = base + Lt::VS;
+  float* B = base + Lt::B;
+  float* W = base + Lt::W;
+  float* D = base + Lt::D;
+  float* red = wbase + GPW * Lt::GROUP;
+  const int cy = 2 * p, cx = p > 0 ? cy - 1 : 0;   // lane 0 has no first column
+  const int64_t warps_total = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t qb = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * GPW; qb < n_qp; qb += warps_total * GPW) {
+    const bool live = in_group && qb + g < n_qp, lx = live && p > 0;
+    const int64_t gq = live ? qb + g : qb;
+    float* eo = eig + gq * Dims<N>::EIG;
+    if (live) {
+      const double* tp = tau + gq * Dims<N>::NT_PAD;
+      for (int r = 0; r < NM; ++r)
+        for (int s = r + p; s < NM; s += N) T[r * LDD + s] = T[s * LDD + r] = tp[packed_index(r, s, NM)];
+      for (int t = p; t < NM * NM; t += N) {
+        const float v = eo[t];
+        VS[(t % NM) * LDD + t / NM] = v;
+        VD[(t % NM) * LDD + t / NM] = (double)v;
+      }
+      for (int t = p; t < NP * LD; t += N) {
+        const int r = t / LD, s = t - r * LD;
+        W[t] = r == s ? 1.f : 0.f;
+        if (r == NM || s == NM) B[t] = W[t];       // decoupled dummy
+      }
+    }
+    __syncwarp();
+    // P = tau V, the lane's columns; tau is symmetric: its row j times V_jc adds to all rows
+    double pa[NM], pb[NM], top = 0;
+#pragma unroll
+    for (int r = 0; r < NM; ++r) pa[r] = pb[r] = 0;
+#pragma unroll 1
+    for (int j = 0; j < NM; ++j) {
+      const double va = VD[cx * LDD + j], vb = VD[cy * LDD + j];
+      top = fmax(top, T[j * LDD + j]);
+#pragma unroll
+      for (int r = 0; r < NM; ++r) {
+        const double t = T[j * LDD + r];
+        pa[r] = fma(t, va, pa[r]);
+        pb[r] = fma(t, vb, pb[r]);
+      }
+    }
+    int ex;
+    frexp(top, &ex);
+    const double sc = ldexp(1.0, -ex);
+    __syncwarp();
+    // B = V^T P (scaled) and R = I - V^T V, row by row
+    {
+      float xa[NM], xb[NM];
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        xa[i] = VS[cx * LDD + i];
+        xb[i] = VS[cy * LDD + i];
+      }
+#pragma unroll 1
+      for (int r = 0; r < NM; ++r) {
+        double ba = 0, bb = 0;
+        float ra = r == cx ? 1.f : 0.f, rb = r == cy ? 1.f : 0.f;
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          const double v = VD[r * LDD + i];
+          const float f = VS[r * LDD + i];
+          ba = fma(v, pa[i], ba);
+          bb = fma(v, pb[i], bb);
+          ra = fmaf(-f, xa[i], ra);
+          rb = fmaf(-f, xb[i], rb);
+        }
+        if (lx) {
+          B[r * LD + cx] = (float)(ba * sc);
+          R[r * LDD + cx] = ra;
+          if (r == cx) D[r] = (float)(ba * sc);
+        }
+        if (live) {
+          B[r * LD + cy] = (float)(bb * sc);
+          R[r * LDD + cy] = rb;
+          if (r == cy) D[r] = (float)(bb * sc);
+        }
+      }
+    }
+    __syncwarp();
+    auto column = [&](int c) {                     // the upper triangle's, copied to the lower one
+      for (int r = 0; r <= c; ++r)
+        B[r * LD + c] = B[c * LD + r] = fmaf(0.5f * R[r * LDD + c], D[r] + D[c], B[r * LD + c]);
+    };
+    if (lx) column(cx);
+    if (live) column(cy);
+    __syncwarp();
+    jacobi_group<float, N>(B, W, p, g, lane, live, red, 3, 1e-24f);
+    if (live) {
+      const float ma = B[cx * LD + cx], mb = B[cy * LD + cy];
+      if (lx) eo[NM * NM + cx] = ldexpf(1.f / (ma * ma), -2 * ex);
+      eo[NM * NM + cy] = ldexpf(1.f / (mb * mb), -2 * ex);
+    }
+    __syncwarp();
+    // (I + R / 2) W over B, then V times it
+    {
+      float wa[NM], wb[NM];
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        wa[i] = W[i * LD + cx];
+        wb[i] = W[i * LD + cy];
+      }
+#pragma unroll 1
+      for (int r = 0; r < NM; ++r) {
+        float sa = 0.f, sb = 0.f;
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          const float f = R[r * LDD + i];
+          sa = fmaf(f, wa[i], sa);
+          sb = fmaf(f, wb[i], sb);
+        }
+        if (lx) B[r * LD + cx] = fmaf(0.5f, sa, W[r * LD + cx]);
+        if (live) B[r * LD + cy] = fmaf(0.5f, sb, W[r * LD + cy]);
+      }
+#pragma unroll
+      for (int i = 0; i < NM; ++i) wa[i] = wb[i] = 0.f;
+#pragma unroll 1
+      for (int a = 0; a < NM; ++a) {
+        const float ya = B[a * LD + cx], yb = B[a * LD + cy];   // own columns
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          const float f = VS[a * LDD + i];
+          wa[i] = fmaf(f, ya, wa[i]);
+          wb[i] = fmaf(f, yb, wb[i]);
+        }
+      }
+      if (live) {
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          if (p > 0) eo[i * NM + cx] = wa[i];
+          eo[i * NM + cy] = wb[i];
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
+template <int N>
+int launch_tau_pairs(const double* tau, int64_t n_elem, float* eig, cudaStream_t st) {
+  if constexpr (N > J32_MAX_N) return 0;
+  else {
+    using L = PairsLayout<N>;
+    if (n_elem <= 0) return 0;
+    const int warps = 4;
+    const size_t smem = (size_t)warps * L::WARP * sizeof(float);
+    static_assert(warps * L::WARP * sizeof(float) <= 227 * 1024, "shared memory of a block");
+    if (cudaFuncSetAttribute(pairs_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return -2;
+    const int64_t n_qp = 4 * n_elem, groups = (n_qp + L::GPW - 1) / L::GPW;
+    const int64_t blocks = std::min<int64_t>((groups + warps - 1) / warps, 152 * 64);
+    count_launches(1);
+    pairs_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tau, eig, n_qp);
+    return cudaGetLastError() == cudaSuccess ? 0 : -2;
+  }
+}
+
+#define TS_INST_PAIRS(T, N) template int launch_tau_pairs<N>(const double*, int64_t, float*, cudaStream_t);
+TS_FOR_EACH_N(TS_INST_PAIRS, double)
 
 #define TS_INST_DTAU(T, N)                                                                                   \
   template int launch_dtau<N>(const int4*, const float*, const float*, const float*, const uint8_t*,         \

@@ -44,10 +44,11 @@ int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t 
                   double C_I, unsigned* hard, cudaStream_t st, float* eig_out = nullptr);
 // FP64 tau of the listed points, for any condition number: the FP64 refinement with
 // Jacobi sweeps in FP64 on its nearly diagonal matrix (tau.cu); y: [V][4][C].
-// n_unconverged counts points whose smallest eigenvalues FP64 does not resolve
+// n_unconverged counts points whose smallest eigenvalues FP64 does not resolve.  eig_out
+// (may be null): their eigenpairs
 template <int N>
 int launch_tau_hard(const int4* tets, const double* geo, const double* y, const unsigned* hard, double* tau_out,
-                    double nu, double C_I, unsigned* n_unconverged, cudaStream_t st);
+                    double nu, double C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out = nullptr);
 // n doubles as (hi, lo) FP32 pairs; hard[0] = 0
 int launch_split_dd(const double* in, float2* out, int64_t n, unsigned* hard, cudaStream_t st);
 
@@ -193,6 +194,11 @@ int j32_upload_batch(const float* host_all);
 template <int N>
 int launch_jvp32(int mode, const J32Inst& I, cudaStream_t st, cudaEvent_t e_before = nullptr,
                  cudaEvent_t e_after = nullptr);
+// FP32 eigenpairs of M by launch_tau_fx, refined in place on its tau (dtau.cu; N <=
+// J32_MAX_N, above which nothing reads them).  Listed points: meaningless until
+// launch_tau_hard writes them
+template <int N>
+int launch_tau_pairs(const double* tau, int64_t n_elem, float* eig, cudaStream_t st);
 // d tau[v] L_i(u0) at every quadrature point (dtau.cu): the Frechet derivative of
 // tau = M^{-1/2} (eq. 3D-tau) in the direction of v, from the cached eigenpairs
 // of M (eig [E*4][EIG]) and strong residual L(u0) (l0 [E][4][3][C]);

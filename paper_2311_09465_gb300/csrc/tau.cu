@@ -756,7 +756,7 @@ int launch_tau_polish(const int4* tets, const double* geo, const double* y, int6
 // busy with the 5 warps (N = 7) that fit.
 template <int N>
 int launch_tau_hard(const int4* tets, const double* geo, const double* y, const unsigned* hard, double* tau_out,
-                    double nu, double C_I, unsigned* n_unconverged, cudaStream_t st) {
+                    double nu, double C_I, unsigned* n_unconverged, cudaStream_t st, float* eig_out) {
   using L = PolishLayout<N>;
   int warps = 8;
   while (warps > 1 && (size_t)warps * L::WARP * sizeof(double) > 200 * 1024) --warps;
@@ -766,7 +766,7 @@ int launch_tau_hard(const int4* tets, const double* geo, const double* y, const 
       cudaSuccess)
     return -2;
   count_launches(1);
-  tau_polish_kernel<N, true><<<152, warps * 32, smem, st>>>(tets, geo, y, 0, tau_out, nu, C_I, n_unconverged, nullptr,
+  tau_polish_kernel<N, true><<<152, warps * 32, smem, st>>>(tets, geo, y, 0, tau_out, nu, C_I, n_unconverged, eig_out,
                                                             hard);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
@@ -777,7 +777,7 @@ int launch_tau_hard(const int4* tets, const double* geo, const double* y, const 
 TS_FOR_EACH_N(TS_INST_POLISH, double)
 #define TS_INST_HARD(T, N)                                                                     \
   template int launch_tau_hard<N>(const int4*, const double*, const double*, const unsigned*, double*, double, double, \
-                                  unsigned*, cudaStream_t);
+                                  unsigned*, cudaStream_t, float*);
 TS_FOR_EACH_N(TS_INST_HARD, double)
 
 

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
       on_list = on_list || !(all * all * FX_LAMBDA <= 1.f);
       frexpf(1.01f * all, &xe);
       xe = min(max(xe, 0), 28);
-      // eigenpairs for the derivative of tau (exact tangent), when asked
+      // FP32 eigenpairs for the derivative of tau (exact tangent), when asked; launch_tau_pairs refines them
       if (live && eig_out) {
         float* eo = eig_out + gq * Dims<N>::EIG;
         const float back = finite ? ldexpf(1.f, 2 * ex) : __int_as_float(0x7fc00000);
