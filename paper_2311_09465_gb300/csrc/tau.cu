@@ -345,7 +345,18 @@ __global__ void __launch_bounds__(128, tau32_blocks(N)) tau32_kernel(const int4*
       if (!in_group) yy[i] = 0.f;
     }
     __syncwarp();                       // all lanes have read C_m
-    cholesky_columns<N, LDC, (N > 7)>(x, yy, p, in_group, in_group ? g * N : 0, fmaxf(cd, 1e-30f), cm);
+    const float least =
+        cholesky_columns<N, LDC, (N > 7)>(x, yy, p, in_group, in_group ? g * N : 0, fmaxf(cd, 1e-30f), cm);
+    // a pivot that rounding took to zero or below: FP32 does not resolve the smallest
+    // eigenvalue, the factor means nothing (its columns may overflow) and the point is NaN
+    const bool resolved = least > 0.f;
+    if (__any_sync(0xffffffffu, !resolved)) {
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        x[i] = resolved ? x[i] : in_group && i == 2 * p - 1 ? 1.f : 0.f;
+        yy[i] = resolved ? yy[i] : in_group && i == 2 * p ? 1.f : 0.f;
+      }
+    }
     __syncwarp();
     const bool conv = onesided_jacobi<N>(x, yy, p, lane, 1e-8f);
     {
@@ -363,7 +374,7 @@ __global__ void __launch_bounds__(128, tau32_blocks(N)) tau32_kernel(const int4*
     // lane's two vectors are columns 2p-1 and 2p of the cache
     if (live && eig_out) {
       float* eo = eig_out + gq * D::EIG;
-      const float back = finite ? ldexpf(1.f, 2 * ex) : __int_as_float(0x7fc00000);
+      const float back = finite && resolved ? ldexpf(1.f, 2 * ex) : __int_as_float(0x7fc00000);
       const float ix = rsqrt_newton(ax), iy = rsqrt_newton(ay);
       if (p > 0) {
 #pragma unroll
@@ -407,7 +418,7 @@ __global__ void __launch_bounds__(128, tau32_blocks(N)) tau32_kernel(const int4*
     }
     // packed upper triangle through shared memory
     float* op = base + Lt::OUTP;
-    const float un = finite ? sc : __int_as_float(0x7fc00000);
+    const float un = finite && resolved ? sc : __int_as_float(0x7fc00000);
     __syncwarp();
     if (in_group) {
 #pragma unroll
