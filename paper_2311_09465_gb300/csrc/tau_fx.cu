@@ -37,6 +37,7 @@
 // both triangles are written.  The loops over rows stay rolled: a correction is
 // one instruction stream of a few hundred instructions, not of several thousand.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "ddfloat.cuh"
@@ -197,14 +198,14 @@ struct FxLayout {
   static constexpr int WARP = GPW * GROUP;
 };
 
-// y: the velocity field as double-float pairs [V][4][C]; nu2 = C_I nu^2; hard: the list
+// y: the velocity field as double-float pairs [V][4][C]; nu2 2^nu2_exp = C_I nu^2; hard: the list
 // (HARD_LIST in kernels.h).  Blocks of 128 threads an SM:
 // N <= 3 6 (85 registers; N = 3, 187,266 tetrahedra: 735 us, 751 with 4), N = 4, 5 4 (2.63 ms at N = 5,
 // 2.74 with 2, 2.81 with 5), N = 7 3, above that the compiler's choice (N = 10 with 3: 6.1 ms, 5.6 so).
 template <int N>
 __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1) tau_fx_kernel(const int4* __restrict__ tets, const double* __restrict__ geo,
                                                      const float2* __restrict__ y, int64_t n_qp,
-                                                     double* __restrict__ tau_out, dd nu2,
+                                                     double* __restrict__ tau_out, dd nu2, int nu2_exp,
                                                      unsigned* __restrict__ hard,
                                                      float* __restrict__ eig_out) {
   using Lt = FxLayout<N>;
@@ -240,15 +241,23 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
     const int q = (int)(gq & 3);
     // ---- w_m = sum_i L_im u_i for mode p, G = L L^T (double-float)
     dd diff;
+    int ed;
     float n2 = 0.f;
     __syncwarp();
     {
       const double* gg = geo + e * GEO_STRIDE + GEO_G;
       const dd gxx = dd_split(gg[0]), gxy = dd_split(gg[1]), gxz = dd_split(gg[2]), gyy = dd_split(gg[3]),
                gyz = dd_split(gg[4]), gzz = dd_split(gg[5]);
-      const dd off = dd_fma(gxy, gxy, dd_fma(gxz, gxz, dd_mul(gyz, gyz)));
-      const dd dia = dd_fma(gxx, gxx, dd_fma(gyy, gyy, dd_mul(gzz, gzz)));
+      // C_I nu^2 G:G = diff 2^ed, from G 2^-eg: squares of 1 / h^2 leave FP32's range (and
+      // from h = 1e8 on their low parts) long before anything else does
+      const int eg = min((int)((__float_as_uint(gxx.hi) >> 23) & 0xff) - 127, 126);
+      const float f = __uint_as_float((unsigned)(127 - eg) << 23);
+      const dd sxx = dd_scale(gxx, f), sxy = dd_scale(gxy, f), sxz = dd_scale(gxz, f), syy = dd_scale(gyy, f),
+               syz = dd_scale(gyz, f), szz = dd_scale(gzz, f);
+      const dd off = dd_fma(sxy, sxy, dd_fma(sxz, sxz, dd_mul(syz, syz)));
+      const dd dia = dd_fma(sxx, sxx, dd_fma(syy, syy, dd_mul(szz, szz)));
       diff = dd_mul(nu2, dd_add(dia, dd_scale(off, 2.f)));
+      ed = nu2_exp + 2 * eg;
       const dd l00 = dd_sqrt(gxx), r00 = dd_rcp(l00);
       const dd l10 = dd_mul(gxy, r00), l20 = dd_mul(gxz, r00);
       const dd l11 = dd_sqrt(dd_fma(dd_neg(l10), l10, gyy)), r11 = dd_rcp(l11);
@@ -297,13 +306,13 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
       float sum = 0.f;
 #pragma unroll
       for (int j = 0; j < N; ++j) sum += __shfl_sync(0xffffffffu, mag, first + j);
-      bound = 1.0001f * sqrtf(fmaf(sum, sum, diff.hi));
+      bound = 1.0001f * sqrtf(fmaf(sum, sum, ldexpf(diff.hi, ed)));
     }
     const bool finite = bound < 4e18f && bound > 2e-19f;   // 2^-ex squared stays in range
     int ex = 0;
     if (finite) frexpf(bound, &ex);
     const float sc = ldexpf(1.f, -ex);
-    const i64 cfix = finite ? fx_from_dd(dd_scale(diff, sc * sc)) : (1ll << 57);
+    const i64 cfix = finite ? fx_from_dd(dd_scale(diff, ldexpf(1.f, ed - 2 * ex))) : (1ll << 57);
 #pragma unroll 1
     for (int m = 0; m < 3; ++m) {
       Limbs* tr = T + m * 2 * TW + L;                   // mode k at tr[k], its imaginary part at tr[TW + k]
@@ -683,10 +692,11 @@ int launch_tau_fx(const int4* tets, const double* geo, const float2* y, int64_t 
     return -2;
   const int64_t n_qp = n_elem * 4, groups = (n_qp + Lt::GPW - 1) / Lt::GPW;
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, 152 * 128));
-  const double k = C_I * nu * nu;
+  int ke;
+  const double k = std::frexp(C_I * nu * nu, &ke);
   const float kh = (float)k;
   count_launches(1);
-  tau_fx_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, dd{kh, (float)(k - (double)kh)},
+  tau_fx_kernel<N><<<(int)blocks, warps * 32, smem, st>>>(tets, geo, y, n_qp, tau_out, dd{kh, (float)(k - (double)kh)}, ke,
                                                           hard, eig_out);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }

@@ -127,3 +127,22 @@ def test_fp64_tau_of_a_cosine_without_a_mean(N, peclet):
     assert np.linalg.norm(got - ref) <= 2.0 ** -46 * np.linalg.norm(ref)
     t.close()
     ts.ts_mesh_free(hm)
+
+
+@pytest.mark.parametrize("size", [1e-10, 1e-9, 1e9, 1e10])
+@pytest.mark.parametrize("N", [3, 7])
+def test_fp64_tau_at_small_and_large_lengths(N, size):
+    # G:G leaves FP32's range below h = 1e-9 and its low part from h = 1e8 on; the continuity
+    # rows (velocity gradients and tau) stay inside it at both ends
+    import torch
+    import paper_2311_09465_gb300 as ts
+    case = cases.pipe_case(N=N, Re=100.0, Wo=5.0, mesh=mg.pipe(nc=1, nr=1, nz=1))
+    case.mesh.xyz = case.mesh.xyz * size
+    case.mu, case.omega = 0.3 * case.rho * size, 1.0 / size
+    y = cases.random_state(case.mesh, N, seed=54)
+    y[:, :, 0, 1] = 0.0
+    ref = op.residual(op.problem_from_case(case), y)[:, 3]
+    g = ts.GLSProblem(case)
+    got = to_np(g.residual(to_dev(y, torch.float64)))[:, 3]
+    assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
+    g.close()
