@@ -343,7 +343,11 @@ int  ts_precond_apply(ts_problem* prob, int kind, const double* x, double* z, vo
  * (section 2.5.3) when dt_pseudo is finite.  Dirichlet velocity entries and
  * Im(mode 0) of v are ignored; the same rows of Hv are zero.  If the last
  * residual was computed in the other precision its state is converted.
- * TS_ERR_ARG if no residual was computed yet.  v and Hv may not alias. */
+ * TS_ERR_ARG if no residual was computed yet.  v and Hv may not alias.
+ * Products of one problem on several streams need no ordering among themselves
+ * in FP64 and for N > 7 (they share scratch and wait for each other on the
+ * device; a captured product has its own); FP32 products with N <= 7 do, as does
+ * a ts_residual, which replaces the state, with every product. */
 int  ts_jvp(ts_problem* prob, const void* v, void* Hv, int precision, void* stream);
 
 /* Pseudo-time Newton-GMRES solve (sections 2.4-2.5) in place on y_inout

@@ -78,6 +78,10 @@ struct LinState {
   T* vc = nullptr;      // the same of a product's operand
   T* vs = nullptr;
   T* rows = nullptr;    // [E][4][4][C] element rows
+  // products share vc, vs and rows: one waits for the last one's event, whatever its stream
+  cudaEvent_t scratch_free = nullptr;
+  std::mutex scratch_lock;
+  bool graph_scratch = false;   // a captured product took its own
   bool prepared = false;   // uc, us belong to u0
   unsigned* hard = nullptr;   // T = double: points that tau_fx leaves to FP64 (HARD_LIST + 4E)
   T* u0t = nullptr;     // [V][K][4] u0 velocity sampled in time (FP32 fast path)
@@ -249,6 +253,12 @@ static void lin_free(LinState<T>& l) {
   dfree(l.vc);
   dfree(l.vs);
   dfree(l.rows);
+  if (l.scratch_free) cudaEventDestroy(l.scratch_free);
+  l.scratch_free = nullptr;
+  if (l.graph_scratch) {
+    int dev;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGraphMemTrim(dev);
+  }
   dfree(l.hard);
   l.prepared = false;
   dfree(l.vt);
@@ -363,13 +373,18 @@ static int prepare_state(ts_problem* pr, LinState<T>& l, const T* y, cudaStream_
 // Scratch of the one-launch element operator, taken at a state's first residual so
 // that products allocate nothing.  Without room for it, or inside a capture, the
 // colour-ordered kernel runs, which needs none.
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone;
+}
+
 template <typename T>
 static bool element_scratch(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
   if (l.rows) return true;
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return false;
+  if (capturing(st)) return false;
   const ts_mesh* m = pr->mesh;
-  if (cudaMalloc(&l.vc, (size_t)field_len(pr) * sizeof(T)) == cudaSuccess &&
+  if ((l.scratch_free || cudaEventCreateWithFlags(&l.scratch_free, cudaEventDisableTiming) == cudaSuccess) &&
+      cudaMalloc(&l.vc, (size_t)field_len(pr) * sizeof(T)) == cudaSuccess &&
       cudaMalloc(&l.vs, (size_t)m->V * 3 * pr->K * sizeof(T)) == cudaSuccess &&
       cudaMalloc(&l.rows, (size_t)m->E * 16 * pr->C * sizeof(T)) == cudaSuccess)
     return true;
@@ -380,17 +395,22 @@ static bool element_scratch(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
   return false;
 }
 
-// out = the element operator on v (the state itself for the residual), after element_scratch
+template <typename T>
+struct ElementScratch {
+  T *vc, *vs, *rows;
+};
+
+// out = the element operator on v (the state itself for the residual)
 template <typename T, int N>
-static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T* out, bool with_mass,
-                         cudaStream_t st, T* l0 = nullptr) {
+static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const ElementScratch<T>& w, const T* v, T* out,
+                         bool with_mass, cudaStream_t st, T* l0 = nullptr) {
   using PV = PairOf<T>;
   using V = typename PV::V;
   const ts_mesh* m = pr->mesh;
   if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
   const bool res = mode == MODE_RESIDUAL;
   if (!res) {
-    if (launch_node_prepass<V, N>(v, pr->d_dmask, (V*)l.vc, (V*)l.vs, (const V*)l.trig, m->V, st))
+    if (launch_node_prepass<V, N>(v, pr->d_dmask, (V*)w.vc, (V*)w.vs, (const V*)l.trig, m->V, st))
       return fail(TS_ERR_CUDA, "node pre-pass launch failed");
   }
   const Phys<double> ph = phys_of<double>(pr, with_mass);
@@ -398,14 +418,14 @@ static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T
   a.tets = m->d_tets;
   a.geo = geo_of<T>(m);
   a.u0t = (const V*)l.us;
-  a.vt = (const V*)(res ? l.us : l.vs);
+  a.vt = (const V*)(res ? l.us : w.vs);
   a.ud = (const V*)l.uc;
-  a.vd = (const V*)(res ? l.uc : l.vc);
+  a.vd = (const V*)(res ? l.uc : w.vc);
   a.tau = l.tau;
   a.t0 = l.t0;
   a.l0 = l0;
   a.trig = (const V*)l.trig;
-  a.rows = (V*)l.rows;
+  a.rows = (V*)w.rows;
   a.rho = PV::of(ph.rho);
   a.irho = PV::of(1.0 / ph.rho);
   a.mu4 = PV::of(4.0 * ph.mu);
@@ -413,9 +433,39 @@ static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const T* v, T
   a.omega = PV::of(ph.omega);
   a.n_elem = m->E;
   if (launch_element<V, N>(mode, a, st)) return fail(TS_ERR_CUDA, "element kernel launch failed");
-  if (launch_gather<V>(m->d_node_off, m->d_node_elem, (const V*)l.rows, pr->d_dmask, out, m->V, pr->C, 4, 3, st))
+  if (launch_gather<V>(m->d_node_off, m->d_node_elem, (const V*)w.rows, pr->d_dmask, out, m->V, pr->C, 4, 3, st))
     return fail(TS_ERR_CUDA, "gather kernel launch failed");
   return outlet_terms<T>(pr, v, res ? 0 : 1, out, st);
+}
+
+// A product by the one-launch operator.  Products of one problem may overlap on several
+// streams and with replays of captured ones: a live product waits for the last live one to
+// leave the shared scratch, a captured one has scratch of its own, memory nodes of its
+// graph.  Returns 1 where there is no scratch.
+template <typename T, int N>
+static int element_product(ts_problem* pr, int mode, LinState<T>& l, const T* v, T* out, cudaStream_t st) {
+  std::lock_guard<std::mutex> hold(l.scratch_lock);
+  if (!capturing(st)) {
+    if (!element_scratch(pr, l, st)) return 1;
+    TS_CUDA(cudaStreamWaitEvent(st, l.scratch_free, 0));
+    TS_TRY((element_apply<T, N>(pr, mode, l, ElementScratch<T>{l.vc, l.vs, l.rows}, v, out, true, st)));
+    TS_CUDA(cudaEventRecord(l.scratch_free, st));
+    return 0;
+  }
+  if (!l.rows) return 1;
+  auto padded = [](int64_t n) { return (size_t)(n + 63) & ~(size_t)63; };
+  const size_t n_vc = padded(field_len(pr)), n_vs = padded(pr->mesh->V * 3 * pr->K);
+  T* own = nullptr;
+  if (cudaMallocAsync((void**)&own, (n_vc + n_vs + (size_t)pr->mesh->E * 16 * pr->C) * sizeof(T), st) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  l.graph_scratch = true;
+  const bool prepared = l.prepared;
+  TS_TRY((element_apply<T, N>(pr, mode, l, ElementScratch<T>{own, own + n_vc, own + n_vc + n_vs}, v, out, true, st)));
+  l.prepared = prepared;                  // a captured pre-pass has not run
+  TS_CUDA(cudaFreeAsync(own, st));
+  return 0;
 }
 
 // dispatch on the compiled mode counts
@@ -516,7 +566,8 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
   if (rc) return fail(TS_ERR_CUDA, "tau kernel launch failed");
   TS_CUDA(cudaEventRecord(pr->sev[1], st));
   if (one_launch) {
-    TS_TRY((element_apply<T, N>(pr, MODE_RESIDUAL, l, y, r, false, st, exact ? l.l0 : nullptr)));
+    TS_TRY((element_apply<T, N>(pr, MODE_RESIDUAL, l, ElementScratch<T>{l.vc, l.vs, l.rows}, y, r, false, st,
+                                exact ? l.l0 : nullptr)));
   } else {
     TS_CUDA(cudaMemsetAsync(r, 0, n * sizeof(T), st));
     TS_TRY(apply_colours<T, N>(pr, MODE_RESIDUAL, y, y, l, r, false, st, exact ? l.l0 : nullptr));
@@ -621,9 +672,10 @@ static int jvp_impl(ts_problem* pr, const T* v, T* hv, cudaStream_t st) {
     TS_TRY(outlet_terms<T>(pr, v, 1, hv, st));
     return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
   }
-  if ((sizeof(T) == 4 ? pr->fast32 : pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) && element_scratch(pr, l, st)) {
-    TS_TRY((element_apply<T, N>(pr, mode, l, v, hv, true, st)));
-    return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
+  if (sizeof(T) == 4 ? pr->fast32 : pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) {
+    const int rc = element_product<T, N>(pr, mode, l, v, hv, st);
+    if (rc < 0) return rc;
+    if (rc == 0) return backflow_terms<T, N>(pr, l, v, false, 1, hv, st);
   }
   TS_CUDA(cudaMemsetAsync(hv, 0, field_len(pr) * sizeof(T), st));
   TS_TRY(apply_colours<T, N>(pr, mode, v, l.u0, l, hv, true, st));
