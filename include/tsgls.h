@@ -81,6 +81,16 @@ extern "C" {
                                /* computed from scratch at every residual, faster than a   */
                                /* start from stored eigenvectors was                        */
 
+#define TS_OPT_ELEMENT_SCRATCH 5 /* device scratch of the residual's element pass, of FP64  */
+                               /* products and of FP32 ones with N > 7: 1 (default) taken  */
+                               /* at the residual where there is room (ts_scratch_bytes),  */
+                               /* given back when another allocation of the library needs  */
+                               /* the memory; 0 none, and what there is is given back.     */
+                               /* Without it these run colour by colour, several times     */
+                               /* slower, FP64 ones as TS_ELEMENT64_NATIVE; with 0, or      */
+                               /* without room for the state's copy, tau as                */
+                               /* TS_TAU64_REFINE                                           */
+
 typedef struct ts_mesh ts_mesh;
 typedef struct ts_problem ts_problem;
 
@@ -180,6 +190,9 @@ int  ts_problem_set(ts_problem* prob, double dt_pseudo, int jvp_variant);
 /* Sets an implementation option (TS_OPT_*); TS_ERR_ARG for an unknown key or
  * value.  Takes effect at the next residual evaluation. */
 int  ts_problem_option(ts_problem* prob, int key, int value);
+/* Bytes of element scratch that the problem holds now (TS_OPT_ELEMENT_SCRATCH;
+ * 0: none, its next products run colour by colour), or a negative error. */
+int64_t ts_scratch_bytes(const ts_problem* prob);
 
 /* Assigns a boundary condition to all boundary triangles with this tag.
  * TS_BC_DIRICHLET: nodes of those triangles become Dirichlet velocity nodes;

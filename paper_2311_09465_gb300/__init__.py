@@ -25,7 +25,7 @@ TS_PROFILE_PARABOLIC, TS_PROFILE_WOMERSLEY = 1, 2
 PROFILES = {"parabolic": TS_PROFILE_PARABOLIC, "womersley": TS_PROFILE_WOMERSLEY}
 TS_JVP_PAPER, TS_JVP_FROZEN, TS_JVP_LIN_A, TS_JVP_EXACT = 0, 1, 2, 3
 VARIANTS = {"paper": TS_JVP_PAPER, "frozen": TS_JVP_FROZEN, "lin_a": TS_JVP_LIN_A, "exact": TS_JVP_EXACT}
-TS_OPT_TAU64, TS_OPT_FP32_TANGENT, TS_OPT_ELEMENT64, TS_OPT_TAU_WARM = 1, 2, 3, 4
+TS_OPT_TAU64, TS_OPT_FP32_TANGENT, TS_OPT_ELEMENT64, TS_OPT_TAU_WARM, TS_OPT_ELEMENT_SCRATCH = 1, 2, 3, 4, 5
 TS_ELEMENT64_NATIVE, TS_ELEMENT64_DOUBLEFLOAT = 0, 1
 ELEMENT64 = {"native": TS_ELEMENT64_NATIVE, "doublefloat": TS_ELEMENT64_DOUBLEFLOAT}
 TS_TAU64_REFINE, TS_TAU64_DOUBLEFLOAT, TS_TAU64_JACOBI = 0, 1, 2
@@ -102,6 +102,8 @@ def lib() -> ctypes.CDLL:
     L.ts_spmv.argtypes = [vp, vp, vp, vp]
     L.ts_assembled_bytes.argtypes = [vp]
     L.ts_assembled_bytes.restype = ctypes.c_int64
+    L.ts_scratch_bytes.argtypes = [vp]
+    L.ts_scratch_bytes.restype = ctypes.c_int64
     L.ts_mesh_connections.argtypes = [vp]
     L.ts_mesh_connections.restype = ctypes.c_int64
     L.ts_residual_noalloc.argtypes = [vp, vp, vp, vp]
@@ -251,6 +253,13 @@ def ts_problem_option(prob, key: int, value: int):
     _check(lib().ts_problem_option(prob, key, value))
 
 
+def ts_scratch_bytes(prob) -> int:
+    n = int(lib().ts_scratch_bytes(prob))
+    if n < 0:
+        _check(n)
+    return n
+
+
 def ts_set_bc(prob, tag: int, kind: int, value: float = 0.0):
     _check(lib().ts_set_bc(prob, tag, kind, value))
 
@@ -391,9 +400,12 @@ class GLSProblem:
             ts_set_bc(self.prob, tag, TS_BC_BACKFLOW, beta)
         self.option(tau64=tau64, fp32_tangent=fp32_tangent, element64=element64)
 
-    def option(self, tau64=None, fp32_tangent=None, element64=None, tau_warm=None):
+    def option(self, tau64=None, fp32_tangent=None, element64=None, tau_warm=None, element_scratch=None):
         """tau64: "refine" | "doublefloat" | "jacobi"; fp32_tangent: "single" | "coloured";
-        element64: "native" | "doublefloat"; tau_warm: bool (accepted, without effect)."""
+        element64: "native" | "doublefloat"; tau_warm: bool (accepted, without effect);
+        element_scratch: bool (device scratch of the one-launch element operator)."""
+        if element_scratch is not None:
+            ts_problem_option(self.prob, TS_OPT_ELEMENT_SCRATCH, int(bool(element_scratch)))
         if tau_warm is not None:
             ts_problem_option(self.prob, TS_OPT_TAU_WARM, int(bool(tau_warm)))
         if element64 is not None:

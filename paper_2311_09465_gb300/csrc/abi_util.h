@@ -12,13 +12,22 @@ namespace ts {
 // records msg as the calling thread's ts_last_error and returns code
 int fail(int code, const std::string& msg);
 
+// Gives back device memory that problems on the current device hold only for speed (scratch
+// of the element operator); whether there was any
+bool reclaim_scratch();
+
 template <typename T>
 int dalloc(T** p, size_t count) {
   *p = nullptr;
   if (count == 0) count = 1;
   cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (reclaim_scratch()) e = cudaMalloc((void**)p, count * sizeof(T));
+  }
   if (e != cudaSuccess) {
     *p = nullptr;
+    cudaGetLastError();                   // not the next launch's error
     return fail(e == cudaErrorMemoryAllocation ? TS_ERR_OOM : TS_ERR_CUDA,
                 std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }

@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -75,15 +76,18 @@ struct LinState {
   T* trig = nullptr;    // cos, sin of 2 pi n k / K: [2][N][K/2 + 1]
   T* uc = nullptr;      // [V][4][C] u0 without Im(mode 0)
   T* us = nullptr;      // [V][3][K] its velocity on samples
-  T* vc = nullptr;      // the same of a product's operand
+  unsigned* hard = nullptr;   // T = double: points that tau_fx leaves to FP64 (HARD_LIST + 4E)
+  // scratch, given back when other memory runs out: a product's operand (as uc, us) where
+  // products use this operator, element rows [E][4][4][C]
+  T* vc = nullptr;
   T* vs = nullptr;
-  T* rows = nullptr;    // [E][4][4][C] element rows
+  T* rows = nullptr;
+  bool pinned = false;  // a captured residual holds rows
   // products share vc, vs and rows: one waits for the last one's event, whatever its stream
   cudaEvent_t scratch_free = nullptr;
   std::mutex scratch_lock;
   bool graph_scratch = false;   // a captured product took its own
   bool prepared = false;   // uc, us belong to u0
-  unsigned* hard = nullptr;   // T = double: points that tau_fx leaves to FP64 (HARD_LIST + 4E)
   T* u0t = nullptr;     // [V][K][4] u0 velocity sampled in time (FP32 fast path)
   T* vt = nullptr;      // [V][K][4] scratch of the FP32 fast path: the product's input sampled
   T* bneg = nullptr;    // [backflow points][NT_PAD] |A_n|_- (section 2.6)
@@ -162,6 +166,7 @@ struct ts_problem {
   bool fast32 = true;    // FP32 products with the single-launch kernel (jvp32.cu)
   int tau64 = TS_TAU64_DOUBLEFLOAT;  // how the FP64 residual computes tau
   int elem64 = TS_ELEMENT64_DOUBLEFLOAT;  // arithmetic of the FP64 element operator
+  bool use_scratch = true;   // TS_OPT_ELEMENT_SCRATCH
 };
 
 // ------------------------------------------------------------------ helpers
@@ -221,7 +226,6 @@ static int lin_alloc(ts_problem* pr, LinState<T>& l) {
   std::vector<T> tt(tab.begin(), tab.end());
   TS_TRY(dalloc(&l.dft, tt.size()));
   TS_CUDA(cudaMemcpy(l.dft, tt.data(), tt.size() * sizeof(T), cudaMemcpyHostToDevice));
-  if (sizeof(T) == 8) TS_TRY(dalloc(&l.hard, (size_t)(HARD_LIST + 4 * m->E)));
   if (sizeof(T) == 4) {
     TS_TRY(dalloc(&l.u0t, (size_t)m->V * 4 * pr->K));
     TS_TRY(dalloc(&l.vt, (size_t)m->V * 4 * pr->K));
@@ -336,11 +340,31 @@ struct PairOf<double> {
   }
 };
 
-// cos, sin of 2 pi n k / K, k = 0..K/2
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone;
+}
+
+// cudaMalloc for what can be done without: a failure is no error, and reclaims nothing
 template <typename T>
-static int upload_trig(int N, T** out) {
+static bool optional_alloc(T** p, size_t count) {
+  if (cudaMalloc((void**)p, count * sizeof(T)) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
+// The state's operands of the one-launch operator, the nodal kernels and the fixed-point tau
+// (trig, uc, us, hard), all or none; a few per cent of the state.  They stay once taken.
+template <typename T>
+static bool element_operands(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
   using PV = PairOf<T>;
-  const int K = 3 * N - 2, KH = K / 2, n1 = N * (KH + 1);
+  static_assert(sizeof(typename PV::V) == sizeof(T), "pairs are stored in place of FP64 values");
+  if (l.uc) return true;
+  if (capturing(st)) return false;
+  const ts_mesh* m = pr->mesh;
+  // cos, sin of 2 pi n k / K, k = 0..K/2
+  const int N = pr->p.N, K = pr->K, KH = K / 2, n1 = N * (KH + 1);
   const double pi = 3.14159265358979323846;
   std::vector<typename PV::V> t(2 * n1);
   for (int n = 0; n < N; ++n)
@@ -349,51 +373,83 @@ static int upload_trig(int N, T** out) {
       t[n * (KH + 1) + k] = PV::of(std::cos(th));
       t[n1 + n * (KH + 1) + k] = PV::of(std::sin(th));
     }
-  TS_TRY(dalloc(out, t.size()));
-  TS_CUDA(cudaMemcpy(*out, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice));
-  return 0;
+  if (optional_alloc(&l.trig, t.size()) &&
+      cudaMemcpy(l.trig, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess &&
+      (sizeof(T) == 4 || optional_alloc(&l.hard, (size_t)(HARD_LIST + 4 * m->E))) &&
+      optional_alloc(&l.us, (size_t)m->V * 3 * pr->K) && optional_alloc(&l.uc, (size_t)field_len(pr)))
+    return true;
+  dfree(l.trig);
+  dfree(l.hard);
+  dfree(l.us);
+  return false;
 }
 
 // the state's operands (uc, us) from y, and its copy u0 where y is the caller's
 template <typename T, int N>
 static int prepare_state(ts_problem* pr, LinState<T>& l, const T* y, cudaStream_t st) {
   using V = typename PairOf<T>::V;
-  static_assert(sizeof(V) == sizeof(T), "pairs are stored in place of FP64 values");
-  const ts_mesh* m = pr->mesh;
-  if (!l.trig) TS_TRY(upload_trig<T>(N, &l.trig));
-  if (!l.uc) TS_TRY(dalloc(&l.uc, (size_t)field_len(pr)));
-  if (!l.us) TS_TRY(dalloc(&l.us, (size_t)m->V * 3 * pr->K));
-  if (launch_node_prepass<V, N>(y, nullptr, (V*)l.uc, (V*)l.us, (const V*)l.trig, m->V, st, l.hard,
+  if (!element_operands(pr, l, st)) return fail(TS_ERR_OOM, "no device memory for the state's operands");
+  if (launch_node_prepass<V, N>(y, nullptr, (V*)l.uc, (V*)l.us, (const V*)l.trig, pr->mesh->V, st, l.hard,
                                 y == l.u0 ? nullptr : l.u0))
     return fail(TS_ERR_CUDA, "node pre-pass launch failed");
   l.prepared = true;
   return 0;
 }
 
-// Scratch of the one-launch element operator, taken at a state's first residual so
-// that products allocate nothing.  Without room for it, or inside a capture, the
-// colour-ordered kernel runs, which needs none.
-static bool capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone;
-}
-
+// Scratch of the one-launch element operator, taken (under scratch_lock, after the operands)
+// at a state's residual or conversion, so that products allocate nothing; without it, until
+// the next one, the colour-ordered kernel runs, which needs none.
 template <typename T>
 static bool element_scratch(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
   if (l.rows) return true;
   if (capturing(st)) return false;
   const ts_mesh* m = pr->mesh;
+  const bool products = sizeof(T) == 8 || pr->p.N > J32_MAX_N;   // others are jvp32's
   if ((l.scratch_free || cudaEventCreateWithFlags(&l.scratch_free, cudaEventDisableTiming) == cudaSuccess) &&
-      cudaMalloc(&l.vc, (size_t)field_len(pr) * sizeof(T)) == cudaSuccess &&
-      cudaMalloc(&l.vs, (size_t)m->V * 3 * pr->K * sizeof(T)) == cudaSuccess &&
-      cudaMalloc(&l.rows, (size_t)m->E * 16 * pr->C * sizeof(T)) == cudaSuccess)
+      (!products || (optional_alloc(&l.vc, (size_t)field_len(pr)) && optional_alloc(&l.vs, (size_t)m->V * 3 * pr->K))) &&
+      optional_alloc(&l.rows, (size_t)m->E * 16 * pr->C))
     return true;
-  cudaGetLastError();                     // the failed allocation is not this call's error
   dfree(l.vc);
   dfree(l.vs);
-  l.rows = nullptr;
   return false;
 }
+
+template <typename T>
+static int64_t scratch_bytes(const ts_problem* pr, const LinState<T>& l) {
+  int64_t n = l.rows ? pr->mesh->E * 16 * pr->C : 0;
+  if (l.vc) n += field_len(pr) + pr->mesh->V * 3 * pr->K;
+  return n * (int64_t)sizeof(T);
+}
+
+// gives the scratch back unless a call is using it or a captured residual holds it
+template <typename T>
+static bool scratch_release(LinState<T>& l) {
+  std::unique_lock<std::mutex> hold(l.scratch_lock, std::try_to_lock);
+  if (!hold.owns_lock() || !l.rows || l.pinned) return false;
+  dfree(l.rows);                          // waits for the kernels that use it
+  dfree(l.vc);
+  dfree(l.vs);
+  return true;
+}
+
+// every problem, for reclaim_scratch.  No allocation that reclaims runs under a scratch_lock.
+static std::mutex g_problems_lock;
+static std::set<ts_problem*> g_problems;
+
+namespace ts {
+bool reclaim_scratch() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> hold(g_problems_lock);
+  bool any = false;
+  for (ts_problem* pr : g_problems)
+    if (pr->mesh->device == dev) {
+      any |= scratch_release(pr->l32);
+      any |= scratch_release(pr->l64);
+    }
+  return any;
+}
+}  // namespace ts
 
 template <typename T>
 struct ElementScratch {
@@ -445,14 +501,13 @@ static int element_apply(ts_problem* pr, int mode, LinState<T>& l, const Element
 template <typename T, int N>
 static int element_product(ts_problem* pr, int mode, LinState<T>& l, const T* v, T* out, cudaStream_t st) {
   std::lock_guard<std::mutex> hold(l.scratch_lock);
+  if (!pr->use_scratch || !l.rows) return 1;
   if (!capturing(st)) {
-    if (!element_scratch(pr, l, st)) return 1;
     TS_CUDA(cudaStreamWaitEvent(st, l.scratch_free, 0));
     TS_TRY((element_apply<T, N>(pr, mode, l, ElementScratch<T>{l.vc, l.vs, l.rows}, v, out, true, st)));
     TS_CUDA(cudaEventRecord(l.scratch_free, st));
     return 0;
   }
-  if (!l.rows) return 1;
   auto padded = [](int64_t n) { return (size_t)(n + 63) & ~(size_t)63; };
   const size_t n_vc = padded(field_len(pr)), n_vs = padded(pr->mesh->V * 3 * pr->K);
   T* own = nullptr;
@@ -536,10 +591,15 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
     eig = pr->d_eig;
   }
   l.prepared = false;
-  // FP32, and FP64 in double-float: one element launch; native FP64: colours
+  // FP32, and FP64 in double-float: one element launch; native FP64: colours.  Without
+  // room for the operands tau takes the form that needs none, the FP64 refinement
+  const bool room = pr->use_scratch && element_operands(pr, l, st);
+  std::unique_lock<std::mutex> hold(l.scratch_lock);
   const bool one_launch =
-      (sizeof(T) == 4 || pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) && element_scratch(pr, l, st);
-  if (one_launch || (sizeof(T) == 8 && pr->tau64 == TS_TAU64_DOUBLEFLOAT))
+      room && (sizeof(T) == 4 || pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT) && element_scratch(pr, l, st);
+  const bool fixed_point = sizeof(T) == 8 && room && pr->tau64 == TS_TAU64_DOUBLEFLOAT;
+  if (one_launch && capturing(st)) l.pinned = true;
+  if (one_launch || fixed_point)
     TS_TRY((prepare_state<T, N>(pr, l, y, st)));
   else
     TS_CUDA(cudaMemcpyAsync(l.u0, y, n * sizeof(T), cudaMemcpyDeviceToDevice, st));
@@ -549,7 +609,7 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
     if (pr->tau64 == TS_TAU64_JACOBI)
       rc = launch_tau<T, N>(m->d_tets, geo_of<T>(m), y, m->E, l.tau, (T)(pr->p.mu / pr->p.rho),
                             (T)pr->p.C_I, pr->d_counter, st, eig);
-    else if (pr->tau64 == TS_TAU64_DOUBLEFLOAT) {
+    else if (fixed_point) {
       const double nu = pr->p.mu / pr->p.rho;
       rc = launch_tau_fx<N>(m->d_tets, m->d_geo64, (const float2*)l.uc, m->E, (double*)l.tau, nu, pr->p.C_I, l.hard, st,
                             eig);
@@ -572,6 +632,7 @@ static int residual_impl(ts_problem* pr, const T* y, T* r, cudaStream_t st) {
     TS_CUDA(cudaMemsetAsync(r, 0, n * sizeof(T), st));
     TS_TRY(apply_colours<T, N>(pr, MODE_RESIDUAL, y, y, l, r, false, st, exact ? l.l0 : nullptr));
   }
+  hold.unlock();
   TS_CUDA(cudaEventRecord(pr->sev[2], st));
   pr->sev_res = true;
   TS_TRY(bneg_alloc(pr, l));
@@ -594,6 +655,11 @@ static int convert_lin(ts_problem* pr, LinState<D>& dst, LinState<S>& src, cudaS
   TS_TRY(lin_alloc(pr, dst));
   const ts_mesh* m = pr->mesh;
   dst.prepared = false;
+  if (pr->use_scratch && (sizeof(D) == 8 ? pr->elem64 == TS_ELEMENT64_DOUBLEFLOAT : N > J32_MAX_N && pr->fast32) &&
+      element_operands(pr, dst, st)) {
+    std::lock_guard<std::mutex> hold(dst.scratch_lock);
+    element_scratch(pr, dst, st);
+  }
   const int64_t n_u = field_len(pr), n_tau = m->E * 4 * pr->NTP, n_t0 = m->E * 12 * pr->C;
   int rc = 0;
   dst.exact_valid = src.exact_valid && src.l0;
@@ -776,7 +842,7 @@ static int block_diag_impl(ts_problem* pr, LinState<T>& l, int invert, float* ou
   Phys<float> ph{(float)p64.rho, (float)p64.mu, (float)p64.omega, (float)p64.nu, (float)p64.C_I,
                  (float)p64.mass_coef};
   const int paper = pr->p.jvp_variant == TS_JVP_PAPER;
-  if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
+  if (N <= NODAL_MAX_N && !l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
   int rc = launch_block_diag<T, N>(paper, invert, m->d_node_off, m->d_node_elem, m->d_tets, geo_of<T>(m),
                                    l.u0, l.uc, l.tau, pr->d_dmask, pr->d_outdiag, ph, out, m->V, pr->d_counter, st);
   if (rc) return fail(rc == -6 ? TS_ERR_UNSUPPORTED : TS_ERR_CUDA, "block diagonal kernel launch failed");
@@ -823,7 +889,7 @@ static int assemble_impl(ts_problem* pr, LinState<T>& l, cudaStream_t st) {
   Phys<double> p64 = phys_of<double>(pr, true);
   Phys<float> ph{(float)p64.rho, (float)p64.mu, (float)p64.omega, (float)p64.nu, (float)p64.C_I,
                  (float)p64.mass_coef};
-  if (!l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
+  if (N <= NODAL_MAX_N && !l.prepared) TS_TRY((prepare_state<T, N>(pr, l, l.u0, st)));
   int rc = launch_assemble_paper<T, N>(m->d_node_off, m->d_node_elem, m->d_row_off, m->d_cols, m->d_tets,
                                        geo_of<T>(m), l.u0, l.uc, l.tau, ph, pr->d_hasm, m->V, st);
   if (rc) return fail(rc == -6 ? TS_ERR_UNSUPPORTED : TS_ERR_CUDA, "assembly kernel launch failed");
@@ -1206,12 +1272,20 @@ int ts_problem_create(const ts_mesh* mesh, const ts_params* params, ts_problem**
     ts_problem_free(pr);
     return rc;
   }
+  {
+    std::lock_guard<std::mutex> hold(g_problems_lock);
+    g_problems.insert(pr);
+  }
   *out = pr;
   return 0;
 }
 
 void ts_problem_free(ts_problem* pr) {
   if (!pr) return;
+  {
+    std::lock_guard<std::mutex> hold(g_problems_lock);
+    g_problems.erase(pr);
+  }
   if (pr->ev_a) cudaEventDestroy(pr->ev_a);
   if (pr->ev_b) cudaEventDestroy(pr->ev_b);
   for (auto& e : pr->sev)
@@ -1283,12 +1357,26 @@ int ts_problem_option(ts_problem* pr, int key, int value) {
     if (value != 0 && value != 1) return fail(TS_ERR_ARG, "TS_OPT_TAU_WARM takes 0 or 1");
     return 0;
   }
+  if (key == TS_OPT_ELEMENT_SCRATCH) {
+    if (value != 0 && value != 1) return fail(TS_ERR_ARG, "TS_OPT_ELEMENT_SCRATCH takes 0 or 1");
+    pr->use_scratch = value == 1;
+    if (!pr->use_scratch) {
+      scratch_release(pr->l32);
+      scratch_release(pr->l64);
+    }
+    return 0;
+  }
   if (key == TS_OPT_FP32_TANGENT) {
     if (value != 0 && value != 1) return fail(TS_ERR_ARG, "TS_OPT_FP32_TANGENT takes 0 or 1");
     pr->fast32 = value == 0;
     return 0;
   }
   return fail(TS_ERR_ARG, "unknown option key");
+}
+
+int64_t ts_scratch_bytes(const ts_problem* pr) {
+  if (!pr) return fail(TS_ERR_ARG, "NULL problem");
+  return scratch_bytes(pr, pr->l32) + scratch_bytes(pr, pr->l64);
 }
 
 }  // extern "C"

@@ -218,6 +218,7 @@ int j32_upload_n123(const float* host_all);
 int j32_upload_n45(const float* host_all);
 int j32_upload_n7(const float* host_all);
 constexpr int J32_MAX_N = 7;   // largest N with the single-launch FP32 kernel
+constexpr int NODAL_MAX_N = 7;   // largest N with the register-tiled nodal kernels (nodal.cuh)
 
 // Nodal diagonal blocks H_AA of the tangent (precond.cu): one 8N x 8N block per
 // node from the node-to-element list (packed element * 4 + local node; uc: the

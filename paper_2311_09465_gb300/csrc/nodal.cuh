@@ -19,8 +19,6 @@
 
 namespace ts {
 
-constexpr int NODAL_MAX_N = 7;
-
 template <int N>
 struct Nodal {
   static constexpr int NM = 2 * N - 1, C = 2 * N, L = N - 1, NT = NM * (NM + 1) / 2, NTP = Dims<N>::NT_PAD;
