@@ -215,8 +215,35 @@ static void dft_tables(int N, std::vector<double>& out) {
 }
 
 template <typename T>
-static int lin_alloc(ts_problem* pr, LinState<T>& l) {
-  if (l.u0) return 0;
+static void lin_free(LinState<T>& l) {
+  dfree(l.u0);
+  dfree(l.tau);
+  dfree(l.t0);
+  dfree(l.dft);
+  dfree(l.u0t);
+  dfree(l.trig);
+  dfree(l.uc);
+  dfree(l.us);
+  dfree(l.vc);
+  dfree(l.vs);
+  dfree(l.rows);
+  if (l.scratch_free) cudaEventDestroy(l.scratch_free);
+  l.scratch_free = nullptr;
+  if (l.graph_scratch) {
+    int dev;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGraphMemTrim(dev);
+  }
+  dfree(l.hard);
+  l.prepared = false;
+  dfree(l.vt);
+  dfree(l.bneg);
+  dfree(l.l0);
+  l.bneg_points = 0;
+  l.valid = false;
+}
+
+template <typename T>
+static int lin_alloc_all(ts_problem* pr, LinState<T>& l) {
   const ts_mesh* m = pr->mesh;
   TS_TRY(dalloc(&l.u0, (size_t)field_len(pr)));
   TS_TRY(dalloc(&l.tau, (size_t)m->E * 4 * pr->NTP));
@@ -244,32 +271,13 @@ static int lin_alloc(ts_problem* pr, LinState<T>& l) {
   return 0;
 }
 
+// the state's arrays, all or none
 template <typename T>
-static void lin_free(LinState<T>& l) {
-  dfree(l.u0);
-  dfree(l.tau);
-  dfree(l.t0);
-  dfree(l.dft);
-  dfree(l.u0t);
-  dfree(l.trig);
-  dfree(l.uc);
-  dfree(l.us);
-  dfree(l.vc);
-  dfree(l.vs);
-  dfree(l.rows);
-  if (l.scratch_free) cudaEventDestroy(l.scratch_free);
-  l.scratch_free = nullptr;
-  if (l.graph_scratch) {
-    int dev;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGraphMemTrim(dev);
-  }
-  dfree(l.hard);
-  l.prepared = false;
-  dfree(l.vt);
-  dfree(l.bneg);
-  dfree(l.l0);
-  l.bneg_points = 0;
-  l.valid = false;
+static int lin_alloc(ts_problem* pr, LinState<T>& l) {
+  if (l.u0) return 0;
+  const int rc = lin_alloc_all(pr, l);
+  if (rc) lin_free(l);
+  return rc;
 }
 
 static int sync_dmask(ts_problem* pr) {
@@ -1873,16 +1881,15 @@ int tracer_solve_impl(ts_tracer* tr, const double* a, double* phi, double tol, i
   const int64_t n = tr->mesh->V * (int64_t)tr->C;
   if (tr->basis_m < m + 1) {
     dfree(tr->basis);
+    tr->basis_m = 0;
     TS_TRY(dalloc(&tr->basis, (size_t)(m + 1) * n));
     tr->basis_m = m + 1;
   }
-  if (!tr->w) {
-    TS_TRY(dalloc(&tr->w, n));
-    TS_TRY(dalloc(&tr->r, n));
-    TS_TRY(dalloc(&tr->dphi, n));
-    TS_TRY(dalloc(&tr->partial, (size_t)krylov_partial_blocks() * 130));
-    TS_TRY(dalloc(&tr->h, 512));
-  }
+  if (!tr->w) TS_TRY(dalloc(&tr->w, n));
+  if (!tr->r) TS_TRY(dalloc(&tr->r, n));
+  if (!tr->dphi) TS_TRY(dalloc(&tr->dphi, n));
+  if (!tr->partial) TS_TRY(dalloc(&tr->partial, (size_t)krylov_partial_blocks() * 130));
+  if (!tr->h) TS_TRY(dalloc(&tr->h, 512));
   TS_TRY(tracer_prepare<double, N>(tr, a, st));
   TS_TRY(tracer_apply<double, N>(tr, phi, tr->r, st));
   int rc = 0;
@@ -2216,20 +2223,20 @@ int ts_solve(ts_problem* pr, void* y_inout, const ts_solve_opts* opts, ts_solve_
   const int m = o.krylov;
   if (pr->basis_m < m + 1) {
     dfree(pr->d_basis);
+    pr->basis_m = 0;
     TS_TRY(dalloc(&pr->d_basis, (size_t)(m + 1) * n));
     pr->basis_m = m + 1;
   }
-  if (!pr->d_w) {
-    TS_TRY(dalloc(&pr->d_w, n));
-    TS_TRY(dalloc(&pr->d_r, n));
-    TS_TRY(dalloc(&pr->d_dy, n));
-    TS_TRY(dalloc(&pr->d_partial, (size_t)krylov_partial_blocks() * 130));
-    TS_TRY(dalloc(&pr->d_h, 3 * 130 + 2));
-    TS_TRY(dalloc(&pr->d_v32, n));
-    TS_TRY(dalloc(&pr->d_w32, n));
-    TS_TRY(dalloc(&pr->d_D, n));
-    TS_TRY(dalloc(&pr->d_t, n));
-  }
+  // one by one: an earlier call may have run out of memory among them
+  if (!pr->d_w) TS_TRY(dalloc(&pr->d_w, n));
+  if (!pr->d_r) TS_TRY(dalloc(&pr->d_r, n));
+  if (!pr->d_dy) TS_TRY(dalloc(&pr->d_dy, n));
+  if (!pr->d_partial) TS_TRY(dalloc(&pr->d_partial, (size_t)krylov_partial_blocks() * 130));
+  if (!pr->d_h) TS_TRY(dalloc(&pr->d_h, 3 * 130 + 2));
+  if (!pr->d_v32) TS_TRY(dalloc(&pr->d_v32, n));
+  if (!pr->d_w32) TS_TRY(dalloc(&pr->d_w32, n));
+  if (!pr->d_D) TS_TRY(dalloc(&pr->d_D, n));
+  if (!pr->d_t) TS_TRY(dalloc(&pr->d_t, n));
   if (o.krylov > 128) return fail(TS_ERR_ARG, "ts_solve: krylov must be <= 128");
   double* y = (double*)y_inout;
   double* V = pr->d_basis;

@@ -104,3 +104,32 @@ def test_scratch_makes_room_for_the_krylov_basis():
     g.residual(y0)                                    # there is room again
     assert ts.ts_scratch_bytes(g.prob) == scratch
     g.close()
+
+
+def test_calls_work_again_after_memory_ran_out():
+    import torch
+    import paper_2311_09465_gb300 as ts
+    case = cases.pipe_case(N=7, Re=100.0, Wo=5.0, mesh=mg.pipe(nc=10, nr=10, nz=20))
+    y0 = to_dev(case.y0 + 0.1 * cases.random_state(case.mesh, 7, seed=75), torch.float64)
+    g, h = ts.GLSProblem(case, dt_pseudo=0.5), ts.GLSProblem(case, dt_pseudo=0.5)
+    ref = _solve(g, y0, 4)                            # kernels loaded; a basis of 5 vectors
+    r_ref = g.residual(y0)
+    g.option(element_scratch=False)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    hog = torch.empty(free - (64 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        for call in (lambda: _solve(g, y0, 60),       # 61 vectors of 4.7 MB
+                     lambda: h.residual(y0)):         # tau alone takes 170 MB
+            with pytest.raises(ts.TsError) as ei:
+                call()
+            assert ei.value.code == ts.TS_ERR_OOM
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    g.option(element_scratch=True)
+    assert rel_l2(to_np(_solve(g, y0, 4) - y0), to_np(ref - y0)) <= 1e-6
+    assert rel_l2(to_np(h.residual(y0)), to_np(r_ref)) <= 1e-12
+    g.close()
+    h.close()
