@@ -583,6 +583,28 @@ __global__ void __launch_bounds__(128) node_prepass_kernel(const typename StoreO
   }
 }
 
+// Sum of a node's element rows.  The rows of a nearly converged state are large against
+// their sum, so pairs are added to more than FP64: s, c, d take the rounding errors of the
+// one before.  (As double-float additions the sum was good to 2^-46 of the largest row.)
+template <typename V>
+struct RowSum {
+  V s = V(0);
+  __device__ __forceinline__ void add(V a) { s += a; }
+  __device__ __forceinline__ V get() const { return s; }
+};
+template <>
+struct RowSum<float2> {
+  float s = 0.f, c = 0.f, d = 0.f;
+  __device__ __forceinline__ void add(float2 a) {
+    float e, f, g;
+    two_sum(s, a.x, s, e);
+    two_sum(c, e, c, f);
+    two_sum(c, a.y, c, g);
+    d += f + g;
+  }
+  __device__ __forceinline__ double get() const { return (double)s + ((double)c + (double)d); }
+};
+
 // out[node][f][c] = sum of the node's element rows; Im(mode 0) and, on Dirichlet
 // nodes, the first `masked` of the fields are zero
 template <typename V>
@@ -591,18 +613,25 @@ __global__ void __launch_bounds__(256) gather_kernel(const int32_t* __restrict__
                                                      const V* __restrict__ rows, const uint8_t* __restrict__ dmask,
                                                      typename StoreOf<V>::S* __restrict__ out, int64_t n_nodes, int C,
                                                      int fields, int masked) {
-  using R = Ar<V>;
   const int FC = fields * C;
   const int64_t total = n_nodes * FC;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t node = t / FC;
     const int fc = (int)(t - node * FC), f = fc / C, c = fc - f * C;
-    V s = R::zero();
+    RowSum<V> sum;
     if (c != 1 && !(f < masked && dmask[node])) {
       const int p1 = node_off[node + 1];
-      for (int p = node_off[node]; p < p1; ++p) s = R::add(s, rows[(int64_t)node_elem[p] * FC + fc]);
+      for (int p = node_off[node]; p < p1; p += 4) {     // four loads in flight
+        V v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (p + u < p1) v[u] = rows[(int64_t)node_elem[p + u] * FC + fc];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (p + u < p1) sum.add(v[u]);
+      }
     }
-    out[t] = R::to(s);
+    out[t] = sum.get();
   }
 }
 
