@@ -51,12 +51,18 @@ namespace {
 constexpr int FX_MAX_IT = 10;
 constexpr float FX_ORTHO2 = 1e-6f;   // leaves cosines near 1e-6: the corrections absorb them
 // Smallest eigenvalue, of a point's scale of 1, that this form takes.  tau's error there
-// is about 2^-54 / lambda: near 1e-12 at 2^-14, where FP64 takes over with its
-// 2^-53 / lambda or less.  The flows with a mean of tests and bench stay above 2^-12.
-constexpr float FX_LAMBDA = 6.103515625e-5f;
-// Pivots of the FP32 factor below this (a pivot is no smaller than the smallest
-// eigenvalue, and FP32 rounding stays below 1e-5) mean a point for the list
+// is a few 2^-54 / lambda, up to 6e-11 at 2^-20, below the double-float refinement's and within
+// ten times the FP64 Jacobi form's (five kinds of flow, N = 2 to 15).  FP64 costs 15 times
+// as much a point: with 2^-14 as the line, one harmonic without a mean at u h / nu = 1e3, N = 7,
+// 187,266 tetrahedra, took 128 ms instead of 12, a reversing flow at N = 15 177 instead of 8.5.
+constexpr float FX_LAMBDA = 9.5367431640625e-7f;
+// Pivots of the FP32 factor below this mean a point for the list: a pivot is no smaller
+// than the smallest eigenvalue, and FP32 rounding, n 2^-24, is about as large
 constexpr float FX_PIVOT = 0.25f * FX_LAMBDA;
+// |R| of the start (2-norm, bounded by n times its largest entry) up to which the corrections
+// converge to M^{-1/2}: with a smallest eigenvalue of k times its FP32 value R has 1 - k, and
+// a correction leaves |1 - sqrt k| of the error (k = 4 would end at the negative root)
+constexpr float FX_START = 0.5f;
 // Smallest diagonal entry that this form takes.  Where a mode hardly couples to the
 // others (a cosine without a mean, N = 2: its sine) the entry is an eigenvalue, which
 // floating point has to a relative 2^-53 and fixed point to 2^-54 of the scale: 1e-14
@@ -496,7 +502,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
     }
     const float rscale = ldexpf(1.f, xe - 58), escale = ldexpf(1.f, 58 - xe);
     // what is left to correct; negative, so never reached, at a point for the list
-    const float small = on_list ? -1.f : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
+    float small = on_list ? -1.f : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
     // ---- corrections
 #pragma unroll 1
     for (int it = 0;; ++it) {
@@ -560,6 +566,10 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
             F[cy * LDF + r + 1] = r1;
           }
         }
+      }
+      if (it == 0) {
+        const unsigned off = __ballot_sync(0xffffffffu, rmax > FX_START / NM);
+        if (off & (((1u << N) - 1u) << first)) small = -1.f;
       }
       const unsigned left = __ballot_sync(0xffffffffu, live && rmax > small);
       const bool more = __any_sync(0xffffffffu, live && rmax > small && small > 0.f) && it + 1 < FX_MAX_IT;
