@@ -203,7 +203,7 @@ __device__ __forceinline__ void load_row(const float* src, float (&dst)[W]) {
 // Blocks an SM asked of the compiler: at N = 5 it takes 111 registers by itself, and 96
 // with 5 blocks are faster (187,266 tetrahedra: 0.89 ms against 0.98); its own choice (0) is the
 // fastest elsewhere.
-constexpr int tau32_blocks(int N) { return N == 5 ? 5 : 0; }
+constexpr int tau32_blocks(int N) { return N == 5 || N == 7 ? 5 : 0; }
 
 template <int N>
 __global__ void __launch_bounds__(128, tau32_blocks(N)) tau32_kernel(const int4* __restrict__ tets, const float* __restrict__ geo,

@@ -501,8 +501,10 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
       }
     }
     const float rscale = ldexpf(1.f, xe - 58), escale = ldexpf(1.f, 58 - xe);
-    // what is left to correct; negative, so never reached, at a point for the list
-    float small = on_list ? -1.f : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
+    // what is left to correct; never reached (negative) at a point for the list, always
+    // (infinite) at one that is not finite
+    constexpr float NEVER = -1.f, ALWAYS = 3e38f;
+    float small = !finite ? ALWAYS : on_list ? NEVER : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
     // ---- corrections
 #pragma unroll 1
     for (int it = 0;; ++it) {
@@ -569,13 +571,13 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
       }
       if (it == 0) {
         const unsigned off = __ballot_sync(0xffffffffu, rmax > FX_START / NM);
-        if (off & (((1u << N) - 1u) << first)) small = -1.f;
+        if (off & (((1u << N) - 1u) << first) && small != ALWAYS) small = NEVER;
       }
       const unsigned left = __ballot_sync(0xffffffffu, live && rmax > small);
       const bool more = __any_sync(0xffffffffu, live && rmax > small && small > 0.f) && it + 1 < FX_MAX_IT;
       if (left && !more) {
         const unsigned mine = ((1u << N) - 1u) << first;
-        if (live && p == 0 && finite && (left & mine)) hard[HARD_LIST + atomicAdd(hard, 1u)] = (unsigned)gq;
+        if (live && p == 0 && (left & mine)) hard[HARD_LIST + atomicAdd(hard, 1u)] = (unsigned)gq;
       }
       __syncwarp();
       // E = U [(U^T R U)_ab / (s_a + s_b)] U^T, row by row; R is symmetric (column = row)
@@ -662,8 +664,8 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
         } else {
           // packed upper triangle through shared memory (over M)
           const double bad = __longlong_as_double(0x7ff8000000000000ll);
-          if (hx && o < N) op[packed_index(min(r, cx), max(r, cx), NM)] = finite ? fx_to_double(n0, e2) : bad;
-          if (hy && o > 0) op[packed_index(min(r, cy), max(r, cy), NM)] = finite ? fx_to_double(n1, e2) : bad;
+          if (hx && o < N) op[packed_index(min(r, cx), max(r, cx), NM)] = small != ALWAYS ? fx_to_double(n0, e2) : bad;
+          if (hy && o > 0) op[packed_index(min(r, cy), max(r, cy), NM)] = small != ALWAYS ? fx_to_double(n1, e2) : bad;
         }
       }
       if (!more) break;
