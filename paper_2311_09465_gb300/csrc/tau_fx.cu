@@ -59,10 +59,10 @@ constexpr float FX_LAMBDA = 9.5367431640625e-7f;
 // Pivots of the FP32 factor below this mean a point for the list: a pivot is no smaller
 // than the smallest eigenvalue, and FP32 rounding, n 2^-24, is about as large
 constexpr float FX_PIVOT = 0.25f * FX_LAMBDA;
-// |R| of the start (2-norm, bounded by n times its largest entry) up to which the corrections
-// converge to M^{-1/2}: with a smallest eigenvalue of k times its FP32 value R has 1 - k, and
-// a correction leaves |1 - sqrt k| of the error (k = 4 would end at the negative root)
-constexpr float FX_START = 0.5f;
+// Bound of |R| (2-norm, as n times the largest entry) in a correction.  With a smallest
+// eigenvalue of k times its FP32 value y = X M^{1/2} starts at k^{1/2} in its direction and goes
+// to y + k^{1/2} (1 - y^2) / 2: unbounded, k = 4 would end at -1, a negative root of M^{-1}
+constexpr float FX_STEP = 0.5f;
 // Smallest diagonal entry that this form takes.  Where a mode hardly couples to the
 // others (a cosine without a mean, N = 2: its sine) the entry is an eigenvalue, which
 // floating point has to a relative 2^-53 and fixed point to 2^-54 of the scale: 1e-14
@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
     // what is left to correct; never reached (negative) at a point for the list, always
     // (infinite) at one that is not finite
     constexpr float NEVER = -1.f, ALWAYS = 3e38f;
-    float small = !finite ? ALWAYS : on_list ? NEVER : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
+    const float small = !finite ? ALWAYS : on_list ? NEVER : fmaxf(1e-10f, ldexpf(64.f, 2 * xe - 58));
     // ---- corrections
 #pragma unroll 1
     for (int it = 0;; ++it) {
@@ -555,8 +555,9 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
           const int r = half_row(o);
           i64 v0, v1;
           fx_dot2<NM>(reinterpret_cast<const int4*>(Xs + r * LDQ), pa, pb, pah, pbh, v0, v1);
-          const float r0 = fx_float((r == cx ? one : 0) - v0) * rscale;
-          const float r1 = fx_float((r == cy ? one : 0) - v1) * rscale;
+          constexpr float LIM = FX_STEP / NM;
+          const float r0 = fminf(fmaxf(fx_float((r == cx ? one : 0) - v0) * rscale, -LIM), LIM);
+          const float r1 = fminf(fmaxf(fx_float((r == cy ? one : 0) - v1) * rscale, -LIM), LIM);
           if (hx && o < N) {
             rmax = fmaxf(rmax, fabsf(r0));
             F[r * LDF + cx + 1] = r0;
@@ -568,10 +569,6 @@ __global__ void __launch_bounds__(128, N <= 3 ? 6 : N <= 5 ? 4 : N == 7 ? 3 : 1)
             F[cy * LDF + r + 1] = r1;
           }
         }
-      }
-      if (it == 0) {
-        const unsigned off = __ballot_sync(0xffffffffu, rmax > FX_START / NM);
-        if (off & (((1u << N) - 1u) << first) && small != ALWAYS) small = NEVER;
       }
       const unsigned left = __ballot_sync(0xffffffffu, live && rmax > small);
       const bool more = __any_sync(0xffffffffu, live && rmax > small && small > 0.f) && it + 1 < FX_MAX_IT;
