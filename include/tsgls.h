@@ -66,9 +66,13 @@ extern "C" {
 /* ts_problem_option keys and values (implementation choices, not physics) */
 #define TS_OPT_TAU64        1  /* how the FP64 residual computes tau (eq. 3D-tau):          */
 #define TS_TAU64_REFINE     0  /*   FP32 Jacobi eigenvectors + FP64 refinement             */
-#define TS_TAU64_DOUBLEFLOAT 1 /*   the same refinement in double-float (FP32 pair)         */
-                               /*   arithmetic (default): meets the FP64 bar, 2.4x faster  */
-                               /*   where FP64 runs at 1/64 of the FP32 rate               */
+#define TS_TAU64_DOUBLEFLOAT 1 /*   default: FP32 eigenpairs + Newton corrections with     */
+                               /*   residuals in 58-bit fixed point (named after the form  */
+                               /*   before it); points whose smallest eigenvalue is below  */
+                               /*   2^-20 of the scale, or whose corrections do not end,   */
+                               /*   by the FP64 refinement with Jacobi sweeps.  Meets the  */
+                               /*   FP64 bar, ten times faster than TS_TAU64_REFINE on     */
+                               /*   flows with a mean                                      */
 #define TS_TAU64_JACOBI     2  /*   FP64 Jacobi eigenpairs                                 */
 #define TS_OPT_FP32_TANGENT 2  /* FP32 tangent products: 0 single launch with vector       */
                                /* atomics (default), 1 colour-ordered launches            */
@@ -251,7 +255,9 @@ int  ts_initial_guess(ts_problem* prob, void* y, int precision, void* stream);
  * (device, layout above, precision 32 or 64).  Momentum rows of Dirichlet
  * nodes and Im(mode 0) are zero.  Also freezes the linearisation used by
  * ts_jvp: the convolution matrices A_j of y, tau at every quadrature point
- * (eq. 3D-tau, computed by a Jacobi eigensolver), and tau L_i(y).
+ * (eq. 3D-tau, from eigenpairs; TS_OPT_TAU64 for FP64), and tau L_i(y).  In FP32
+ * tau, and with it the rows of its nodes, is NaN at a point whose smallest
+ * eigenvalue FP32 does not resolve (condition number above about 1e7).
  * y and r may not alias. */
 int  ts_residual(ts_problem* prob, const void* y, void* r, int precision, void* stream);
 
@@ -468,8 +474,9 @@ int  ts_tracer_set_dirichlet(ts_tracer* tracer, int tag);
 /* r(phi) for the advecting velocity a: caller-owned device arrays of the
  * given precision, a [V][3][N][2] (the velocity part of a modal field), phi and
  * r [V][N][2] (one field of the modal layout).  Computes tau at every point
- * (FP64: the fixed-point refinement; FP32: FP32 Jacobi) into library-owned
- * buffers allocated at the first call.  r may not alias a or phi. */
+ * (as TS_TAU64_DOUBLEFLOAT in FP64, as ts_residual in FP32) into library-owned
+ * buffers allocated at the first call, which calls on one tracer share: they
+ * must be ordered.  r may not alias a or phi. */
 int  ts_tracer_residual(ts_tracer* tracer, const void* a, const void* phi, void* r, int precision,
                         void* stream);
 

@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(128)
 // in registers; the records are updated in place by the warp that owns the row.
 // 52,650 tetrahedra, N = 3 / 5 / 7: 0.47 / 0.83 / 1.81 ms (1.47 / 3.09 / 6.53 ms with one
 // output a lane and both operands in shared memory); bound by shared-memory reads
-// (81% at N = 5).
+// (81% at N = 5); 128 registers, at N = 7 with 4 to 6 words spilled.
 template <int N>
 struct NodalAssembly {
   using D = Nodal<N>;

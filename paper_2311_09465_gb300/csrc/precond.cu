@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(128)
 // N = 7, 52,650 tetrahedra, with inverse: 1.16 ms (8.4 ms before: the sums were two
 // shared-memory loads a multiply-add and the elimination one warp's passes over
 // 3136 entries); the inverse is 0.04 ms of it.  Bound by issue and shared memory
-// at 8 warps an SM (254 registers hold the five n x n sums of a group).
+// at 8 warps an SM (255 registers hold the five n x n sums of a group; the inverting form
+// spills 17 words at N = 7).
 constexpr float PIVOT_OK = 0.1f;
 
 template <int N>

@@ -201,8 +201,9 @@ __device__ __forceinline__ void load_row(const float* src, float (&dst)[W]) {
 }
 
 // Blocks an SM asked of the compiler: at N = 5 it takes 111 registers by itself, and 96
-// with 5 blocks are faster (187,266 tetrahedra: 0.89 ms against 0.98); its own choice (0) is the
-// fastest elsewhere.
+// with 5 blocks are faster (187,266 tetrahedra: 0.89 ms against 0.98), at N = 7 128, and 96 with
+// 12 words spilled are faster (52,650: 744 us against 767); its own choice (0) is the fastest
+// elsewhere.
 constexpr int tau32_blocks(int N) { return N == 5 || N == 7 ? 5 : 0; }
 
 template <int N>
